@@ -81,9 +81,21 @@ __host__ __device__ inline int blk_pitch(int bmax) {
 
 // Offset of slot 0's entry d = 0 in the window (elements).
 constexpr int kWndOff = 3;
+// Elements between the NB rows of one ring block and the next.  A tile row
+// of the update is NB ring rows, and NB rows of any pitch span a multiple of
+// eight 16-byte groups, so without the gap the lanes of one column of tiles
+// all meet one bank group; with it consecutive tile rows are one group apart
+// (two for FP64).
+constexpr int kBlkPad = 4;
+// Element offset of ring slot `slot` (entry d = 0 at kWndOff past it).
+template <int NB>
+__host__ __device__ __forceinline__ int wnd_row(int slot, int PW) {
+  return slot * PW + (int)((unsigned)slot / NB) * kBlkPad;
+}
 
 __host__ __device__ inline int blk_wnd_elems(int NB, int bmax) {
-  const int a = kWndOff + blk_ring_rows(NB, bmax) * blk_pitch(bmax), b = 2 * (NB + bmax) * NB;
+  const int rw = blk_ring_rows(NB, bmax);
+  const int a = kWndOff + rw * blk_pitch(bmax) + (rw / NB) * kBlkPad, b = 2 * (NB + bmax) * NB;
   return a > b ? a : b;
 }
 
@@ -241,7 +253,7 @@ __device__ __forceinline__ void blk_fill_raw(const Gen& gen, const BlkSmem<T>& s
     T e[5], rh[NR];
     gen.template make<T, NR>(r, raw, e, rh);
     const int slot = ring(slot0 + gl, s.RW);
-    T* row = s.wnd + kWndOff + slot * s.PW;
+    T* row = s.wnd + kWndOff + wnd_row<G / 2>(slot, s.PW);
     if (mx >= 3 && mx + 1 <= b) {
       // offsets 0, 1, mx-1, mx, mx+1 are distinct: plain stores
       row[0] = e[0];
@@ -400,6 +412,180 @@ __device__ __forceinline__ void panel_pair(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T
   }
 }
 
+// ---- trailing update with 8-row tiles (FP32, two systems per warp, panels
+// of at most 48 rows: half bandwidths 25..40).
+//
+// What bounds the 4 x 4 tiles below is the issue rate: of about 230
+// instructions a tile 128 are FMAs, the rest its index, its zeroing, its
+// loads (two per column and 16 FMAs) and its write-back; and 55 tiles (b =
+// 40) take four rounds of the 16 lanes.  Here every lane owns one tile of
+// the window for the whole factorisation: 8 x 8 (b > 32, 15 tiles), or 8 x
+// 4 halves of the off-diagonal 8 x 8 tiles and the lower triangles of the
+// diagonal ones (8 x 4 and 4 x 4) for b <= 32, 16 tiles.  Two FMAs go into
+// one instruction (fma.rn.f32x2, each half rounded as a scalar FMA): a pair
+// of rows times a pair of columns gives the products (r0 c0, r1 c1), with
+// the columns swapped (r0 c1, r1 c0).  The sums of each entry run over the
+// block's columns in the same order as in the 4 x 4 tiles, and are
+// subtracted from the window once: the results are the same bits.
+// The panel is stored with its rows reversed (row ia at RP - 1 - ia), so a
+// 16-byte group of it and one of a window row list the columns alike.
+struct Tile8 {
+  int ti, g0;   // rows 8 ti .. 8 ti + 7, first column group (4 columns each)
+  int ng;       // column groups: 2 (8 x 8), 1 (8 x 4), 0 (no tile)
+  bool diag;    // on the diagonal
+};
+
+//
+// 1024^2, H/h = 32, oversampling 0..4, 32 samples: 10.40 -> 8.67 ms; 2048^2,
+// contrast 1e4, no oversampling, 4 samples: 2.89 -> 2.27 ms; 345^2, H/h =
+// 23, Petrov-Galerkin with oscillatory data, 37 samples: 1.92 -> 1.66 ms.
+// The form with FP64 solutions (refinement) keeps the 4 x 4 tiles: 14.1 ms
+// with either for 8 samples of the first, the larger code costing what the
+// tiles save.
+template <int G, typename T, int RPL, typename TS>
+__host__ __device__ constexpr bool tiles8_form() {
+  return G == 16 && sizeof(T) == 4 && RPL == 3 && sizeof(TS) == 4;
+}
+
+// Lane gl's tile.  The lane order puts tiles whose window rows share a bank
+// group (ti - g0 mod 8 alike, kBlkPad) into different quarters of the warp
+// where their number allows it.
+__device__ __forceinline__ Tile8 tile8_of(int gl, int b) {
+  Tile8 t;
+  const int sh = 4 * (gl & 7);
+  if (b > 32) {
+    t.ti = ((gl < 8 ? 0x12343210u : 0x04443432u) >> sh) & 15;
+    const int tj = ((gl < 8 ? 0x12300000u : 0x02432111u) >> sh) & 15;
+    t.diag = t.ti == tj;
+    t.g0 = 2 * tj;
+    t.ng = gl < 15 ? 2 : 0;
+  } else {
+    t.ti = ((gl < 8 ? 0x13213210u : 0x33333222u) >> sh) & 15;
+    t.g0 = ((gl < 8 ? 0x10006420u : 0x54321321u) >> sh) & 15;
+    t.diag = gl < 4;
+    t.ng = 8 * t.ti < b ? 1 : 0;
+  }
+  return t;
+}
+
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_swap(uint64_t a) {
+  uint64_t d;
+  asm("{\n.reg .b32 lo, hi;\nmov.b64 {lo, hi}, %1;\nmov.b64 %0, {hi, lo};\n}" : "=l"(d) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ float f2_lo(uint64_t a) { return __uint_as_float((uint32_t)a); }
+__device__ __forceinline__ float f2_hi(uint64_t a) { return __uint_as_float((uint32_t)(a >> 32)); }
+
+// Products of NRP row pairs (descending rows) with NCP column pairs.
+template <int NRP, int NCP>
+struct Pair2 {
+  uint64_t same[NRP][NCP], cross[NRP][NCP];
+  template <bool FIRST>
+  __device__ __forceinline__ void add(const uint64_t* r, const uint64_t* c) {
+#pragma unroll
+    for (int y = 0; y < NCP; ++y) {
+      const uint64_t cs = f2_swap(c[y]);
+#pragma unroll
+      for (int x = 0; x < NRP; ++x) {
+        same[x][y] = FIRST ? f2_mul(r[x], c[y]) : f2_fma(r[x], c[y], same[x][y]);
+        cross[x][y] = FIRST ? f2_mul(r[x], cs) : f2_fma(r[x], cs, cross[x][y]);
+      }
+    }
+  }
+  // window row of pair x (hi: its second row), column pairs y0, y0 + 1:
+  // columns past `last` (counted from the group's first) stay unchanged
+  __device__ __forceinline__ void sub(float* w, int x, bool hi, int y0, int last) const {
+    float v[4];
+    ld_grp4(w, v);
+    const float s[4] = {hi ? f2_hi(cross[x][y0]) : f2_lo(same[x][y0]), hi ? f2_hi(same[x][y0]) : f2_lo(cross[x][y0]),
+                        hi ? f2_hi(cross[x][y0 + 1]) : f2_lo(same[x][y0 + 1]),
+                        hi ? f2_hi(same[x][y0 + 1]) : f2_lo(cross[x][y0 + 1])};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (3 - k <= last) v[k] -= s[k];
+    st_grp4(w, v);
+  }
+};
+
+__device__ __forceinline__ void ld_pairs(const float* p, uint64_t& a, uint64_t& b) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  a = v.x;
+  b = v.y;
+}
+
+// Window rows [K + 8, K + 8 + nt) -= the panel's products; tslot: ring slot
+// of the tile's first row (8-row tiles never wrap: RW is a multiple of 8).
+__device__ __forceinline__ void tiles8_update(const Tile8& t, int b, const float* __restrict__ pt,
+                                              const BlkSmem<float>& s, int tslot, int nt) {
+  if (t.ng == 0 || 8 * t.ti >= nt) return;
+  const int RP = s.RP;
+  const float* pr = pt + RP - 8 - 8 * t.ti;  // rows 8 ti + 7 .. 8 ti
+  const int rows = nt - 8 * t.ti;            // live rows of the tile (8 or more: all)
+  // entry (row a, column group g0, column 3 of the group)
+  float* w = s.wnd + kWndOff + wnd_row<8>(tslot, s.PW) + (8 * t.ti - 4 * t.g0 - 3);
+  const int ws = s.PW + 1;  // to the same columns of the next row
+  uint64_t r[4], c[4];
+  if (b > 32) {
+    const float* pc = pt + RP - 8 - 4 * t.g0;  // columns 4 g0 + 7 .. 4 g0
+    Pair2<4, 4> A;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      ld_pairs(pr + p * RP, r[0], r[1]);
+      ld_pairs(pr + p * RP + 4, r[2], r[3]);
+      ld_pairs(pc + p * RP, c[0], c[1]);
+      ld_pairs(pc + p * RP + 4, c[2], c[3]);
+      if (p == 0)
+        A.template add<true>(r, c);
+      else
+        A.template add<false>(r, c);
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      if (a < rows) {
+        const int x = 3 - a / 2;  // pair 0 holds rows 7, 6; hi: the even row
+        const bool hi = (a & 1) == 0;
+        A.sub(w + a * ws, x, hi, 2, t.diag ? a : 7);
+        // columns 4..7 of a diagonal tile's rows 0..3 lie above the diagonal
+        if (a >= 4 || !t.diag) A.sub(w + a * ws - 4, x, hi, 0, t.diag ? a - 4 : 7);
+      }
+    }
+  } else {
+    const float* pc = pt + RP - 4 - 4 * t.g0;
+    Pair2<4, 2> A;
+    Pair2<2, 2> D;  // diagonal tiles: rows 4..7 times columns 4..7
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      ld_pairs(pr + p * RP, r[0], r[1]);
+      ld_pairs(pr + p * RP + 4, r[2], r[3]);
+      ld_pairs(pc + p * RP, c[0], c[1]);
+      if (p == 0) {
+        A.template add<true>(r, c);
+        D.template add<true>(r, r);
+      } else {
+        A.template add<false>(r, c);
+        D.template add<false>(r, r);
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      if (a < rows) {
+        A.sub(w + a * ws, 3 - a / 2, (a & 1) == 0, 0, t.diag ? a : 7);
+        if (a >= 4 && t.diag) D.sub(w + a * ws - 4, 3 - a / 2, (a & 1) == 0, 0, a - 4);
+      }
+    }
+  }
+}
+
 // Factorise (and forward-substitute NR rhs).  Lg: blocks of (NB+bmax) x NB;
 // yg[k*NR + c] receives the forward solution.  Returns -1 or the first
 // failing pivot index (the factorisation runs to the end either way).
@@ -415,7 +601,9 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
   constexpr int NB = G / 2;
   const int LBS = (NB + bmax) * NB;
   const int RW = s.RW;
-  blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + RW * s.PW)) / 16), gl);
+  constexpr bool kTiles8 = tiles8_form<G, T, RPL, TS>();
+  const Tile8 tile = kTiles8 ? tile8_of(gl, b) : Tile8{0, 0, 0, false};
+  blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + wnd_row<NB>(RW, s.PW))) / 16), gl);
   __syncwarp();
   int fail = -1;
   // first window: rows [0, min(n, NB + b)) in slots 0.. (no wrap), generated directly
@@ -454,28 +642,33 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     T rh[RPL][NR];
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
+      // rows i >= np read slots inside the window too (kslot + i < 2 RW);
+      // their values stay in their own lane's row and are never stored
       const int i = gl + G * q;
-      const bool in = i < np;
-      const int slot = ring(kslot + (in ? i : 0), RW);
-      const T* row = s.wnd + kWndOff + slot * s.PW;
+      const int slot = ring(kslot + i, RW);
+      const T* row = s.wnd + kWndOff + wnd_row<NB>(slot, s.PW);
       // entries d = i - p, p < NB, as NB / 4 aligned groups: group g4 holds
-      // d = i - 4 g4 - 3 .. i - 4 g4 (p = 4 g4 + 3 .. 4 g4); entries outside
-      // [0, b] (the neighbouring rows' ends and the gaps) are masked
+      // d = i - 4 g4 - 3 .. i - 4 g4 (p = 4 g4 + 3 .. 4 g4); the entries
+      // above the diagonal (d < 0, rows i < NB only) hold a neighbour's
+      // values, which the column steps never use
 #pragma unroll
       for (int g4 = 0; g4 < NB / 4; ++g4) {
         const int d0 = i - 4 * g4 - 3;
         T v[4] = {T(0), T(0), T(0), T(0)};
-        if (in && d0 + 3 >= 0 && d0 <= b) ld_grp4(row + d0, v);
+        if (q > 0 || d0 + 3 >= 0) ld_grp4(row + d0, v);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int p = 4 * g4 + 3 - k, d = d0 + k;
-          pr[q][p] = (p < nb && d >= 0 && d <= b) ? v[k] : T(0);
-        }
+        for (int k = 0; k < 4; ++k) pr[q][4 * g4 + 3 - k] = v[k];
+      }
+      // entries past the band (d > b) hold the next row's and are zero
+      if (G * q + G - 1 > b) {
+#pragma unroll
+        for (int p = 0; p < NB; ++p)
+          if (i - p > b) pr[q][p] = T(0);
       }
       T x4[4];
       ld_row4(s.rhs + slot * 4, x4);
 #pragma unroll
-      for (int c = 0; c < NR; ++c) rh[q][c] = in ? x4[c] : T(0);
+      for (int c = 0; c < NR; ++c) rh[q][c] = x4[c];
     }
     if (nb == NB)
       panel_pair<0, G, T, NR, RPL>(pr, rh, s.lb, gl, K, fail);
@@ -487,7 +680,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     T* Lb = Lg + (size_t)kb * LBS;
     // the transposed trailing panel: 16-byte aligned inside the retired
     // rows' span [kWndOff + kslot PW, kWndOff + (kslot + NB) PW)
-    T* pt = s.wnd + kslot * s.PW + 4;
+    T* pt = s.wnd + wnd_row<NB>(kslot, s.PW) + 4;
     const bool store_blk = K + NB > store_from;
     __syncwarp();
 #pragma unroll
@@ -503,14 +696,15 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
 #pragma unroll
           for (int v = 0; v < NB / 4; ++v)
             reinterpret_cast<float4*>(dst)[v] =
-                make_float4(4 * v <= i ? pr[q][4 * v] : 0.f, 4 * v + 1 <= i ? pr[q][4 * v + 1] : 0.f,
-                            4 * v + 2 <= i ? pr[q][4 * v + 2] : 0.f,
-                            4 * v + 3 <= i ? pr[q][4 * v + 3] : 0.f);
+                make_float4(q > 0 || 4 * v <= i ? pr[q][4 * v] : 0.f,
+                            q > 0 || 4 * v + 1 <= i ? pr[q][4 * v + 1] : 0.f,
+                            q > 0 || 4 * v + 2 <= i ? pr[q][4 * v + 2] : 0.f,
+                            q > 0 || 4 * v + 3 <= i ? pr[q][4 * v + 3] : 0.f);
         } else {
 #pragma unroll
           for (int v = 0; v < NB / 2; ++v)
             reinterpret_cast<double2*>(dst)[v] = make_double2(
-                2 * v <= i ? pr[q][2 * v] : 0.0, 2 * v + 1 <= i ? pr[q][2 * v + 1] : 0.0);
+                q > 0 || 2 * v <= i ? pr[q][2 * v] : 0.0, q > 0 || 2 * v + 1 <= i ? pr[q][2 * v + 1] : 0.0);
         }
         if (i < nb) {
           if constexpr (FWD_ONLY) {
@@ -532,14 +726,17 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
         } else {
           st_row4<NR>(s.rhs + ring(kslot + i, RW) * 4, rh[q]);
 #pragma unroll
-          for (int p = 0; p < NB; ++p) pt[p * s.RP + (i - nb)] = pr[q][p];
+          for (int p = 0; p < NB; ++p) pt[p * s.RP + (kTiles8 ? s.RP - 1 - (i - nb) : i - nb)] = pr[q][p];
         }
       }
     }
     __syncwarp();
     // ---- 2. trailing update A22 -= L21 L21^T with 4x4 register tiles
     const int nt = np - nb;
-    if (nt > 0) {
+    if constexpr (kTiles8) {
+      // (nt > 0 only after a full block: nb = NB)
+      if (nt > 0) tiles8_update(tile, b, pt, s, ring(kslot + NB + 8 * tile.ti, RW), nt);
+    } else if (nt > 0) {
       const int T4 = (nt + 3) >> 2;
       const int ntiles = T4 * (T4 + 1) / 2;
       const int tslot = ring(kslot + nb, RW);  // slot of row K + nb
@@ -587,7 +784,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
         for (int a = 0; a < 4; ++a) {
           const int ia = 4 * ti + a;
           if (ia < nt) {
-            T* wr = s.wnd + kWndOff + ring(tslot + ia, RW) * s.PW + (ia - 4 * tj - 3);
+            T* wr = s.wnd + kWndOff + wnd_row<NB>(ring(tslot + ia, RW), s.PW) + (ia - 4 * tj - 3);
             T v[4];
             ld_grp4(wr, v);
 #pragma unroll
@@ -601,7 +798,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     __syncwarp();
     // the retired rows' slots (which held the trailing panel) are cleared for
     // the rows that will occupy them
-    blk_zero_span<G>(s.wnd + kWndOff + kslot * s.PW, NB * s.PW, gl);
+    blk_zero_span<G>(s.wnd + kWndOff + wnd_row<NB>(kslot, s.PW), NB * s.PW, gl);
     __syncwarp();
   }
   return fail;
@@ -660,13 +857,24 @@ __device__ void blk_backward(int n, int b, int bmax, const BlkSmem<T>& s, const 
 #pragma unroll
       for (int c = 0; c < NR; ++c) acc[c] = T(0);
       const int p = gl & (NB - 1);
+      // rows up to the ring's end, then from its start (no index per row)
+      const T* lp = tb + p;
+      int i = nb + gl / NB;
+      const int turn = min(np, RW - kslot);
 #pragma unroll 4
-      for (int i = nb + gl / NB; i < np; i += G / NB) {
-        const T l = tb[i * NB + p];
+      for (; i < turn; i += G / NB) {
         T xi[4];
-        ld_row4(xr + ring(kslot + i, RW) * 4, xi);
+        ld_row4(xr + (kslot + i) * 4, xi);
 #pragma unroll
-        for (int c = 0; c < NR; ++c) acc[c] += l * xi[c];
+        for (int c = 0; c < NR; ++c) acc[c] += lp[i * NB] * xi[c];
+      }
+      const T* xw = xr + (kslot - RW) * 4;
+#pragma unroll 4
+      for (; i < np; i += G / NB) {
+        T xi[4];
+        ld_row4(xw + i * 4, xi);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) acc[c] += lp[i * NB] * xi[c];
       }
 #pragma unroll
       for (int c = 0; c < NR; ++c) {
