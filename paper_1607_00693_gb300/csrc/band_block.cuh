@@ -59,8 +59,7 @@ struct BlkSmem {
            // p-major: pt[p*RP + (i - nb)] = L[K+i][K+p]
   T* tb;   // 2 x [NB + bmax][NB] factor block staging (aliases wnd)
   T* rhs;  // [RW][4]
-  T* lb;   // 2 x 2 x [NB] broadcast of the block-row multipliers; [NB][4]
-           // block solution in the stored forward substitution
+  T* lb;   // 2 x 2 x [NB] broadcast of the block-row multipliers
   double* raw;  // [NB][RAWD] generator values of the next rows (prefetched)
   int RW, PW, RP, RAWD;
 };
@@ -978,51 +977,58 @@ __device__ void blk_forward_stored(int n, int b, int bmax, const BlkSmem<T>& s, 
 #pragma unroll
       for (int c = 0; c < NR; ++c) yv[c] = (gl < nb) ? x4[c] : T(0);
     }
+    // this lane's rows of the block (multipliers of columns p < NB) and the
+    // sums of their products; every lane forms each y_p for the columns
+    // below it, so the rows past the block take them from registers
+    T l[RPL][NB], acc[RPL][NR];
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+      const int i = gl + G * q;
+#pragma unroll
+      for (int c = 0; c < NR; ++c) acc[q][c] = T(0);
+#pragma unroll
+      for (int p = 0; p < NB; p += 4) {
+        T v[4] = {T(0), T(0), T(0), T(0)};
+        if (i < np) ld_grp4(tb + i * NB + p, v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) l[q][p + k] = v[k];
+      }
+    }
 #pragma unroll
     for (int p = 0; p < NB; ++p) {
       if (p < nb) {
-        const T iLpp = tb[p * NB + p];
+        const T iLpp = gshfl<G>(l[0][p], p);
         T yp[NR];
 #pragma unroll
         for (int c = 0; c < NR; ++c) yp[c] = gshfl<G>(yv[c], p) * iLpp;
         if (gl > p && gl < nb) {
-          const T l = tb[gl * NB + p];
 #pragma unroll
-          for (int c = 0; c < NR; ++c) yv[c] -= l * yp[c];
+          for (int c = 0; c < NR; ++c) yv[c] -= l[0][p] * yp[c];
         }
         if (gl == p) {
 #pragma unroll
           for (int c = 0; c < NR; ++c) yv[c] = yp[c];
         }
+#pragma unroll
+        for (int q = 0; q < RPL; ++q)
+#pragma unroll
+          for (int c = 0; c < NR; ++c) acc[q][c] += l[q][p] * yp[c];
       }
     }
-    T* yb = s.lb;  // block solution broadcast
     if (gl < nb) {
 #pragma unroll
-      for (int c = 0; c < NR; ++c) {
-        rg[(size_t)(K + gl) * NR + c] = (double)yv[c];
-        yb[gl * NR + c] = yv[c];
-      }
+      for (int c = 0; c < NR; ++c) rg[(size_t)(K + gl) * NR + c] = (double)yv[c];
     }
-    __syncwarp();
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
       const int i = gl + G * q;
       if (i >= nb && i < np) {
-        T acc[NR];
-#pragma unroll
-        for (int c = 0; c < NR; ++c) acc[c] = T(0);
-        for (int p = 0; p < nb; ++p) {
-          const T l = tb[i * NB + p];
-#pragma unroll
-          for (int c = 0; c < NR; ++c) acc[c] += l * yb[p * NR + c];
-        }
         T* row = rr + ring(kslot + i, RW) * 4;
-        T x4[4];
+        T x4[4], r[NR];
         ld_row4(row, x4);
 #pragma unroll
-        for (int c = 0; c < NR; ++c) acc[c] = x4[c] - acc[c];
-        st_row4<NR>(row, acc);
+        for (int c = 0; c < NR; ++c) r[c] = x4[c] - acc[q][c];
+        st_row4<NR>(row, r);
       }
     }
     __syncwarp();
