@@ -1,0 +1,304 @@
+// Banded SPD solver for 9-point-stencil matrices, one system per CTA of four
+// warps, FP64, one right-hand side: the coarse systems, the same with mixed
+// boundary data, and the small fine-grid systems.
+//
+// Right-looking banded L D L^T in column blocks of 8.  Per block
+//   1. warp 0 factorises the panel in registers: lanes 0..7 hold the rows of
+//      the diagonal block, lane 8 the right-hand side as one more row (its
+//      multipliers are the forward solution already divided by D), and every
+//      lane one row (RS = 1, half bandwidths up to 32) or two below it; the
+//      multipliers l and the unscaled columns c = l d go to shared memory,
+//      l also to global scratch;
+//   2. all warps update the trailing window, W -= l c^T, in 2 x 2 tiles,
+//      while the last warp clears the retired ring rows and writes the next
+//      8 rows, whose values it loaded one block earlier.
+// The back substitution is warp 0's, with the factor blocks copied back two
+// blocks ahead.  Rows past the end are identity rows, so every block is full.
+//
+// What bounds it is the FP64 pipe (one warp instruction per 16 clocks of an
+// SM, whatever its lanes do), so the split is made for full lanes and few
+// FP64 instructions: a right-hand side that rides along as a row costs none
+// in the panel, 1 / d takes three (see recip), 2 x 2 tiles waste 3 % of the
+// lanes of a 32-row triangle where 4 x 4 tiles in whole rounds of a warp
+// waste 35 %, and their four loads per four FMAs cost nothing here (shared
+// memory serves a tile's operands in a tenth of its FMAs' time).  Four warps
+// per system, not one, because the batches are small: 512 systems leave an
+// SM three or four, and one warp alone reaches a quarter of the pipe.
+// 512 coarse systems of 32^2 cells with moments: 2.79 ms with a warp per
+// sample and column blocks of 16, 1.54 ms here.
+//
+// Row generator interface (Gen): typename Raw; load(r, Raw&); template
+// make<double, 1>(r, raw, e, rhs) as in band_block.cuh; mx.
+#pragma once
+#include "band_block.cuh"
+#include "common.cuh"
+
+namespace stomsfem {
+
+constexpr int kCtaThreads = 128;
+constexpr int kCtaPerSm = 4;  // CTAs an SM holds at least (128 registers a thread)
+constexpr int kCtaNB = 8;
+constexpr int kCtaStages = 3;  // factor blocks of the back substitution in flight or in use
+
+// Shared memory of one system: window rows of even pitch P >= b + 1 (lanes
+// one row apart then read entries an odd number of doubles apart), the two
+// panels [8][PB], the right-hand sides of the window rows.  The back
+// substitution's staging and its ring of solutions reuse the window.
+struct CtaBand {
+  double *W, *Lp, *Cp, *rh;
+  int RW, P, PB, LP;  // LP: pitch of a stored factor block's columns
+};
+
+__host__ __device__ inline int cta_ring_rows(int b) { return (kCtaNB + b + kCtaNB - 1) / kCtaNB * kCtaNB; }
+__host__ __device__ inline int cta_lp(int b) { return (kCtaNB + b + 1) & ~1; }
+__host__ __device__ inline int cta_wnd_elems(int b) {
+  const int w = cta_ring_rows(b) * ((b + 2) & ~1), s = kCtaStages * kCtaNB * cta_lp(b) + cta_ring_rows(b);
+  return w > s ? w : s;
+}
+__host__ __device__ inline size_t cta_smem_bytes(int b) {
+  return sizeof(double) * (size_t)(((cta_wnd_elems(b) + 1) & ~1) + 2 * kCtaNB * ((b + 2) & ~1) + cta_ring_rows(b));
+}
+__device__ inline CtaBand make_cta_band(unsigned char* smem, int b) {
+  CtaBand s;
+  s.RW = cta_ring_rows(b);
+  s.P = (b + 2) & ~1;
+  s.PB = (b + 2) & ~1;
+  s.LP = cta_lp(b);
+  s.W = reinterpret_cast<double*>(smem);
+  s.Lp = s.W + ((cta_wnd_elems(b) + 1) & ~1);
+  s.Cp = s.Lp + kCtaNB * s.PB;
+  s.rh = s.Cp + kCtaNB * s.PB;
+  return s;
+}
+
+// 1 / d: the FP32 reciprocal (relative error below 2^-22) with one cubic
+// step r (1 + e + e^2), e = 1 - d r, whose error e^3 is below 2^-66; outside
+// the FP32 range the FP64 division.
+__device__ __forceinline__ double recip(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d);
+  // exponents -90 .. 90 (d is positive here)
+  if (hi - (933u << 20) > (180u << 20)) return 1.0 / d;
+  const double r = (double)__frcp_rn((float)d);
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+__device__ __forceinline__ double shfl_d(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// Row r of the system into ring slot `slot` (cleared before); r >= n: the
+// identity.
+template <class Gen>
+__device__ __forceinline__ void cta_put_row(const Gen& gen, const CtaBand& s, int r, int n, int b, int slot,
+                                            const typename Gen::Raw& raw) {
+  double* row = s.W + slot * s.P;
+  if (r >= n) {
+    row[0] = 1.0;
+    s.rh[slot] = 0.0;
+    return;
+  }
+  double e[5], rh[1];
+  gen.template make<double, 1>(r, raw, e, rh);
+  const int mx = gen.mx;
+  row[0] += e[0];
+  if (r >= 1 && 1 <= b) row[1] += e[1];
+  if (mx - 1 >= 0 && r >= mx - 1 && mx - 1 <= b) row[mx - 1] += e[2];
+  if (r >= mx && mx <= b) row[mx] += e[3];
+  if (r >= mx + 1 && mx + 1 <= b) row[mx + 1] += e[4];
+  s.rh[slot] = rh[0];
+}
+
+// Solves the system into x[n] (global); Lg: ceil(n / 8) * 8 * LP doubles of
+// global scratch.  Every thread of the CTA calls it.  Returns false when a
+// pivot was not positive (x then holds no solution).
+template <int RS, class Gen>
+__device__ bool cta_band_solve(const Gen& gen, int n, int b, const CtaBand& s, double* __restrict__ Lg,
+                               double* __restrict__ x) {
+  constexpr int NB = kCtaNB;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int RW = s.RW, P = s.P, PB = s.PB, LP = s.LP;
+  const int nkb = (n + NB - 1) / NB;
+  const bool filler = warp == kCtaThreads / 32 - 1;
+  bool ok = true;  // warp 0's
+  for (int q = tid; q < RW * P; q += kCtaThreads) s.W[q] = 0.0;
+  __syncthreads();
+  for (int r = tid; r < NB + b; r += kCtaThreads) {
+    typename Gen::Raw raw;
+    if (r < n) gen.load(r, raw);
+    cta_put_row(gen, s, r, n, b, r, raw);
+  }
+  typename Gen::Raw next;  // of row K + NB + b + lane (lanes 0..7 of the filling warp)
+  if (filler && lane < NB && NB + b + lane < n) gen.load(NB + b + lane, next);
+  __syncthreads();
+  const int nt2 = (b + 1) >> 1, ntiles = nt2 * (nt2 + 1) / 2;
+  int kslot = 0;
+  for (int kb = 0; kb < nkb; ++kb, kslot = ring(kslot + NB, RW)) {
+    const int K = kb * NB;
+    if (warp == 0) {
+      // ---- panel
+      double dg[NB], a[RS][NB], y[RS];
+#pragma unroll
+      for (int p = 0; p < NB; ++p) {
+        dg[p] = lane < NB && lane >= p && lane - p <= b ? s.W[(kslot + lane) * P + lane - p]
+                                                        : (lane == NB ? s.rh[kslot + p] : 0.0);
+      }
+      int slot[RS];
+#pragma unroll
+      for (int q = 0; q < RS; ++q) {
+        const int i = lane + 32 * q;
+        slot[q] = ring(kslot + NB + min(i, b - 1), RW);
+        y[q] = s.rh[slot[q]];
+#pragma unroll
+        for (int p = 0; p < NB; ++p)
+          a[q][p] = i < b && NB + i - p <= b ? s.W[slot[q] * P + NB + i - p] : 0.0;
+      }
+      double* Lb = Lg + (size_t)kb * NB * LP;
+#pragma unroll
+      for (int J = 0; J < NB; ++J) {
+        double d = shfl_d(dg[J], J);
+        const long long bits = __double_as_longlong(d);  // positive and not NaN, by the bit pattern
+        if (bits <= 0 || bits > 0x7ff0000000000000ll) {
+          ok = false;
+          d = 1.0;
+        }
+        const double r = recip(d);
+        const double lg = dg[J] * r, yJ = shfl_d(dg[J], NB);
+        if (lane > J && lane < NB) Lb[J * LP + lane] = lg;
+        if (lane == NB && K + J < n) x[K + J] = lg;
+        double l[RS];
+#pragma unroll
+        for (int q = 0; q < RS; ++q) {
+          const int i = lane + 32 * q;
+          l[q] = a[q][J] * r;
+          y[q] = fma(-l[q], yJ, y[q]);
+          if (i < b) {
+            Lb[J * LP + NB + i] = l[q];
+            s.Lp[J * PB + i] = l[q];
+            s.Cp[J * PB + i] = a[q][J];
+          }
+        }
+#pragma unroll
+        for (int p = J + 1; p < NB; ++p) {
+          const double c = shfl_d(dg[J], p);
+          dg[p] = fma(-lg, c, dg[p]);
+#pragma unroll
+          for (int q = 0; q < RS; ++q) a[q][p] = fma(-l[q], c, a[q][p]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < RS; ++q)
+        if (lane + 32 * q < b) s.rh[slot[q]] = y[q];
+    }
+    __syncthreads();
+    // ---- trailing update: rows and columns K + NB .. K + NB + b - 1
+    for (int t = tid; t < ntiles; t += kCtaThreads) {
+      int ti = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+      if ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+      if (ti * (ti + 1) / 2 > t) --ti;
+      const int tj = t - ti * (ti + 1) / 2;
+      const int i0 = 2 * ti, j0 = 2 * tj;
+      double* w0 = s.W + ring(kslot + NB + i0, RW) * P + (i0 - j0);              // (i0, j0); (i0, j0 + 1) at -1
+      double* w1 = s.W + ring(kslot + NB + min(i0 + 1, b - 1), RW) * P + (i0 + 1 - j0);
+      const bool up = ti != tj, lo = i0 + 1 < b;
+      double v00 = w0[0], v01 = up ? w0[-1] : 0.0, v10 = lo ? w1[0] : 0.0, v11 = lo ? w1[-1] : 0.0;
+#pragma unroll
+      for (int p = 0; p < NB; ++p) {
+        const double2 l2 = *reinterpret_cast<const double2*>(s.Lp + p * PB + i0);
+        const double2 c2 = *reinterpret_cast<const double2*>(s.Cp + p * PB + j0);
+        v00 = fma(-l2.x, c2.x, v00);
+        v01 = fma(-l2.x, c2.y, v01);
+        v10 = fma(-l2.y, c2.x, v10);
+        v11 = fma(-l2.y, c2.y, v11);
+      }
+      w0[0] = v00;
+      if (up) w0[-1] = v01;
+      if (lo) {
+        w1[0] = v10;
+        w1[-1] = v11;
+      }
+    }
+    // ---- the retired rows' slots take rows K + NB + b ..  (RW = NB + b
+    // rounded up: slots past K + NB + b - 1 stay free until then)
+    if (filler) {
+      const int r0 = K + NB + b, fslot = ring(kslot + NB + b, RW);
+      // rows r0 .. r0 + 7 lie in slots fslot ..: the retired ones and, before
+      // them, the free ones, all clear or retired by now
+      for (int q = lane; q < NB * P; q += 32) {
+        const int k = q / P;
+        s.W[ring(fslot + k, RW) * P + q - k * P] = 0.0;
+      }
+      __syncwarp();
+      if (lane < NB) cta_put_row(gen, s, r0 + lane, n, b, ring(fslot + lane, RW), next);
+      if (lane < NB && r0 + NB + lane < n) gen.load(r0 + NB + lane, next);
+    }
+    __syncthreads();
+  }
+  ok = __syncthreads_and(ok);
+  if (warp == 0) {
+    // ---- back substitution: x_p = z_p - sum_{i > p} l_ip x_i
+    double* stg = s.W;
+    double* xr = s.W + kCtaStages * NB * LP;  // ring of solution rows, zero past the end
+    for (int q = lane; q < RW; q += 32) xr[q] = 0.0;
+    const int chunks = NB * LP / 2;
+    auto stage = [&](int kb) {
+      if (kb >= 0) {
+        const double* src = Lg + (size_t)kb * NB * LP;
+        double* dst = stg + (kb % kCtaStages) * NB * LP;
+        for (int v = lane; v < chunks; v += 32) cp_async16(dst + 2 * v, src + 2 * v);
+      }
+      cp_async_commit();
+    };
+    stage(nkb - 1);
+    stage(nkb - 2);
+    const int pl = lane >> 2;  // this lane's column
+    double zn = (nkb - 1) * NB + pl < n ? x[(nkb - 1) * NB + pl] : 0.0;
+    int ks = ((nkb - 1) * NB) % RW;
+    for (int kb = nkb - 1; kb >= 0; --kb, ks = ks >= NB ? ks - NB : ks - NB + RW) {
+      const int K = kb * NB;
+      stage(kb - 2);
+      cp_async_wait<kCtaStages - 1>();
+      __syncwarp();
+      const double* L = stg + (kb % kCtaStages) * NB * LP;
+      const double z = zn;
+      if (kb > 0) zn = x[K - NB + pl];
+      double acc[NB];
+#pragma unroll
+      for (int q = 0; q < RS; ++q) {
+        const int i = lane + 32 * q;
+        const bool in = i < b;
+        const double xi = in ? xr[ring(ks + NB + i, RW)] : 0.0;
+#pragma unroll
+        for (int p = 0; p < NB; ++p) {
+          const double li = in ? L[p * LP + NB + i] : 0.0;
+          acc[p] = q == 0 ? li * xi : fma(li, xi, acc[p]);
+        }
+      }
+      // sums over the lanes, halving the columns a lane carries
+#pragma unroll
+      for (int h = 4, m = 16; h >= 1; h >>= 1, m >>= 1) {
+        const bool upper = lane & m;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+          const double send = upper ? acc[k] : acc[k + h], keep = upper ? acc[k + h] : acc[k];
+          acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+      }
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+      double t = z - acc[0];
+#pragma unroll
+      for (int q = NB - 1; q > 0; --q) {
+        const double xq = shfl_d(t, 4 * q);
+        if (pl < q) t = fma(-L[pl * LP + q], xq, t);
+      }
+      if ((lane & 3) == 0) {
+        xr[ks + pl] = t;
+        if (K + pl < n) x[K + pl] = t;
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  return ok;
+}
+
+}  // namespace stomsfem

@@ -1,11 +1,10 @@
 // Coarse assembly and solve (Eq. upscaleSUF) and Monte Carlo moments
 // (Eq. MCestimate); the same with mixed boundary data (Sec. 5.2, Eqs.
-// xsquarewave / ysquarewave).  One warp per sample: the coarse matrix over the
+// xsquarewave / ysquarewave).  One CTA per sample: the coarse matrix over the
 // (nc-1)^2 interior coarse nodes is again a 9-point-stencil SPD matrix,
 // assembled row by row from the K_e of the four cells around each node
-// and factorised in FP64 with the blocked banded Cholesky of the cell
-// problems (column blocks of 16, rows generated one block ahead).
-#include "band_block.cuh"
+// and factorised in FP64 by the banded solver of band_cta.cuh.
+#include "band_cta.cuh"
 #include "common.cuh"
 
 namespace stomsfem {
@@ -18,13 +17,11 @@ __device__ __forceinline__ int kidx(int l, int lp) {
 
 // Row generator of the coarse system for the blocked solver: a row's five
 // band entries and its load, summed from the K_e and b_e of the four cells
-// around the node (loads issued one block ahead by prefetch, which stores
-// the six sums in the row's raw slot).
+// around the node.
 struct CoarseBlkGen {
   const double* Ke;  // this sample [nc*nc][10]
   const double* be;  // [nc*nc][4]
   int nc, mx;        // mx = nc - 1 interior nodes per row
-  static constexpr int kRaw = 8;
   struct Raw {
     double e[5], rhs;
   };
@@ -43,18 +40,6 @@ struct CoarseBlkGen {
     w.rhs = __ldg(be + (size_t)((J - 1) * nc + I - 1) * 4 + 2) + __ldg(be + (size_t)((J - 1) * nc + I) * 4 + 3) +
             __ldg(be + (size_t)(J * nc + I) * 4 + 0) + __ldg(be + (size_t)(J * nc + I - 1) * 4 + 1);
   }
-  __device__ __forceinline__ void prefetch(int r, double* dst) const {
-    Raw w;
-    load(r, w);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) dst[k] = w.e[k];
-    dst[5] = w.rhs;
-  }
-  __device__ __forceinline__ void from_smem(const double* src, Raw& w) const {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) w.e[k] = src[k];
-    w.rhs = src[5];
-  }
   template <typename T, int NR = 1>
   __device__ __forceinline__ void make(int, const Raw& w, T e[5], T* rh) const {
 #pragma unroll
@@ -63,7 +48,8 @@ struct CoarseBlkGen {
   }
 };
 
-constexpr int kCoarseBlkWarps = 2;
+// Least workspace of the coarse and small fine-grid solves, in slots.
+constexpr int kCoarseMinSlots = 2;
 
 // Row generator of the standard Q1 FEM on the fine grid (the u_h of the
 // two-level estimator, Eq. MCmean2level): the element matrices are
@@ -73,7 +59,6 @@ struct FineFemGen {
   const double* a;  // this sample [nf][nf]
   int nf, mx;       // mx = nf - 1 interior nodes per row
   double fh2;       // f h^2
-  static constexpr int kRaw = 4;
   struct Raw {
     double sw, se, ne, nw;
   };
@@ -83,20 +68,6 @@ struct FineFemGen {
     w.se = __ldg(a + (size_t)(J - 1) * nf + I);
     w.ne = __ldg(a + (size_t)J * nf + I);
     w.nw = __ldg(a + (size_t)J * nf + I - 1);
-  }
-  __device__ __forceinline__ void prefetch(int r, double* dst) const {
-    Raw w;
-    load(r, w);
-    dst[0] = w.sw;
-    dst[1] = w.se;
-    dst[2] = w.ne;
-    dst[3] = w.nw;
-  }
-  __device__ __forceinline__ void from_smem(const double* src, Raw& w) const {
-    w.sw = src[0];
-    w.se = src[1];
-    w.ne = src[2];
-    w.nw = src[3];
   }
   // K_ref = [4 -1 -2 -1; -1 4 -1 -2; -2 -1 4 -1; -1 -2 -1 4] / 6 (SW, SE, NE, NW)
   template <typename T, int NR = 1>
@@ -112,37 +83,35 @@ struct FineFemGen {
   }
 };
 
-template <int RPL>
-__global__ void __launch_bounds__(kCoarseBlkWarps * 32)
+// u [(N+1)^2] from the interior solution x [(N-1)^2] (NaN where the
+// factorisation failed), zero on the boundary; the whole CTA.
+__device__ __forceinline__ void write_interior(int N, bool ok, const double* __restrict__ x, double* __restrict__ us) {
+  const int NN = N + 1;
+  for (int q = threadIdx.x; q < NN * NN; q += kCtaThreads) {
+    const int I = q % NN, J = q / NN;
+    double v = 0.0;
+    if (I > 0 && J > 0 && I < N && J < N)
+      v = ok ? x[(J - 1) * (N - 1) + (I - 1)] : __longlong_as_double(0x7ff8000000000000ll);
+    us[q] = v;
+  }
+  __syncthreads();
+}
+
+template <int RS>
+__global__ void __launch_bounds__(kCtaThreads, kCtaPerSm)
 fine_fem_kernel(int nf, int S, double f, const double* __restrict__ a, double* __restrict__ u, unsigned char* ws,
                 size_t slot_bytes, size_t l_bytes) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int mx = nf - 1, n = mx * mx, b = nf;
-  const BlkSmem<double> sm = make_blk<double>(smem + wib * blk_smem_bytes<double>(16, b), 16, b);
-  const int gw = blockIdx.x * kCoarseBlkWarps + wib, nw = gridDim.x * kCoarseBlkWarps;
-  unsigned char* slot = ws + (size_t)gw * slot_bytes;
+  const CtaBand sm = make_cta_band(smem, b);
+  unsigned char* slot = ws + (size_t)blockIdx.x * slot_bytes;
   double* Lg = reinterpret_cast<double*>(slot);
   double* x = reinterpret_cast<double*>(slot + l_bytes);
-  const int NN = nf + 1;
   const double h = 1.0 / nf;
-  for (int s = gw; s < S; s += nw) {
+  for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const FineFemGen gen{a + (size_t)s * nf * nf, nf, mx, f * h * h};
-    int fail = -1;
-    if (n > 0) {
-      fail = blk_factor<32, double, 1, RPL>(gen, n, b, b, sm, Lg, x, lane);
-      blk_backward<32, double, 1>(n, b, b, sm, Lg, x, lane);
-    }
-    __syncwarp();
-    double* us = u + (size_t)s * NN * NN;
-    const double nanv = __longlong_as_double(0x7ff8000000000000ll);
-    for (int q = lane; q < NN * NN; q += 32) {
-      const int I = q % NN, J = q / NN;
-      double v = 0.0;
-      if (I > 0 && J > 0 && I < nf && J < nf) v = fail < 0 ? x[(J - 1) * mx + (I - 1)] : nanv;
-      us[q] = v;
-    }
-    __syncwarp();
+    const bool ok = n > 0 ? cta_band_solve<RS>(gen, n, b, sm, Lg, x) : true;
+    write_interior(nf, ok, x, u + (size_t)s * (nf + 1) * (nf + 1));
   }
 }
 
@@ -161,37 +130,20 @@ __global__ void restrict_kernel(int nf, int nc, int S, const double* __restrict_
   }
 }
 
-template <int RPL>
-__global__ void __launch_bounds__(kCoarseBlkWarps * 32)
+template <int RS>
+__global__ void __launch_bounds__(kCtaThreads, kCtaPerSm)
 coarse_blk_kernel(int nc, int S, const double* __restrict__ Ke, const double* __restrict__ be,
                   double* __restrict__ u, unsigned char* ws, size_t slot_bytes, size_t l_bytes) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int mx = nc - 1, n = mx * mx, b = nc;
-  const BlkSmem<double> sm =
-      make_blk<double>(smem + wib * blk_smem_bytes<double>(16, b, CoarseBlkGen::kRaw), 16, b, CoarseBlkGen::kRaw);
-  const int gw = blockIdx.x * kCoarseBlkWarps + wib, nw = gridDim.x * kCoarseBlkWarps;
-  unsigned char* slot = ws + (size_t)gw * slot_bytes;
+  const CtaBand sm = make_cta_band(smem, b);
+  unsigned char* slot = ws + (size_t)blockIdx.x * slot_bytes;
   double* Lg = reinterpret_cast<double*>(slot);
   double* x = reinterpret_cast<double*>(slot + l_bytes);
-  const int NN = nc + 1;
-  for (int s = gw; s < S; s += nw) {
+  for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const CoarseBlkGen gen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, nc, mx};
-    int fail = -1;
-    if (n > 0) {
-      fail = blk_factor<32, double, 1, RPL>(gen, n, b, b, sm, Lg, x, lane);
-      blk_backward<32, double, 1>(n, b, b, sm, Lg, x, lane);
-    }
-    __syncwarp();
-    double* us = u + (size_t)s * NN * NN;
-    const double nanv = __longlong_as_double(0x7ff8000000000000ll);
-    for (int q = lane; q < NN * NN; q += 32) {
-      const int I = q % NN, J = q / NN;
-      double v = 0.0;
-      if (I > 0 && J > 0 && I < nc && J < nc) v = fail < 0 ? x[(J - 1) * mx + (I - 1)] : nanv;
-      us[q] = v;
-    }
-    __syncwarp();
+    const bool ok = n > 0 ? cta_band_solve<RS>(gen, n, b, sm, Lg, x) : true;
+    write_interior(nc, ok, x, u + (size_t)s * (nc + 1) * (nc + 1));
   }
 }
 
@@ -208,7 +160,6 @@ struct CoarseBcGen {
   const uint8_t* dm;  // [(nc+1)^2] nonzero: prescribed value
   const double* gv;   // [(nc+1)^2] the prescribed values
   int nc, mx;         // mx = nc + 1 nodes per row
-  static constexpr int kRaw = 8;
   using Raw = CoarseBlkGen::Raw;
   __device__ __forceinline__ double K(int cx, int cy, int l, int lp) const {
     return __ldg(Ke + (size_t)(cy * nc + cx) * 10 + kidx(l, lp));
@@ -278,18 +229,6 @@ struct CoarseBcGen {
     w.e[0] = d;
     w.rhs = f;
   }
-  __device__ __forceinline__ void prefetch(int r, double* dst) const {
-    Raw w;
-    load(r, w);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) dst[k] = w.e[k];
-    dst[5] = w.rhs;
-  }
-  __device__ __forceinline__ void from_smem(const double* src, Raw& w) const {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) w.e[k] = src[k];
-    w.rhs = src[5];
-  }
   template <typename T, int NR = 1>
   __device__ __forceinline__ void make(int, const Raw& w, T e[5], T* rh) const {
 #pragma unroll
@@ -298,47 +237,62 @@ struct CoarseBcGen {
   }
 };
 
-// One warp per sample, as coarse_blk_kernel, over all (nc+1)^2 nodes.
-template <int RPL>
-__global__ void __launch_bounds__(kCoarseBlkWarps * 32)
+// One CTA per sample, as coarse_blk_kernel, over all (nc+1)^2 nodes.
+template <int RS>
+__global__ void __launch_bounds__(kCtaThreads, kCtaPerSm)
 coarse_bc_kernel(int nc, int S, const double* __restrict__ Ke, const double* __restrict__ be,
                  const uint8_t* __restrict__ dm, const double* __restrict__ gv, double* __restrict__ u,
                  unsigned char* ws, size_t slot_bytes, size_t l_bytes) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int mx = nc + 1, n = mx * mx, b = mx + 1;
-  const BlkSmem<double> sm =
-      make_blk<double>(smem + wib * blk_smem_bytes<double>(16, b, CoarseBcGen::kRaw), 16, b, CoarseBcGen::kRaw);
-  const int gw = blockIdx.x * kCoarseBlkWarps + wib, nw = gridDim.x * kCoarseBlkWarps;
-  unsigned char* slot = ws + (size_t)gw * slot_bytes;
+  const CtaBand sm = make_cta_band(smem, b);
+  unsigned char* slot = ws + (size_t)blockIdx.x * slot_bytes;
   double* Lg = reinterpret_cast<double*>(slot);
   double* x = reinterpret_cast<double*>(slot + l_bytes);
-  for (int s = gw; s < S; s += nw) {
+  for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const CoarseBcGen gen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, dm, gv, nc, mx};
-    const int fail = blk_factor<32, double, 1, RPL>(gen, n, b, b, sm, Lg, x, lane);
-    blk_backward<32, double, 1>(n, b, b, sm, Lg, x, lane);
-    __syncwarp();
+    const bool ok = cta_band_solve<RS>(gen, n, b, sm, Lg, x);
     double* us = u + (size_t)s * n;
-    const double nanv = __longlong_as_double(0x7ff8000000000000ll);
-    for (int q = lane; q < n; q += 32) us[q] = fail < 0 ? x[q] : nanv;
-    __syncwarp();
+    for (int q = threadIdx.x; q < n; q += kCtaThreads) us[q] = ok ? x[q] : __longlong_as_double(0x7ff8000000000000ll);
+    __syncthreads();
   }
 }
 
 // Merge this batch's moments into the running ones (pairwise update of
 // Chan, Golub and LeVeque): batch mean/M2 two-pass, then combine.
-__global__ void moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double* m2,
-                               const double* count) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nn) return;
+// A CTA takes kMomNodes nodes, kMomGroups threads each sharing the node's
+// samples (one thread per node left a batch of 512 on 9 CTAs, each thread
+// in two chains of 512 dependent additions).
+constexpr int kMomNodes = 16, kMomGroups = 32;
+
+__global__ void __launch_bounds__(kMomNodes * kMomGroups)
+moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double* m2, const double* count) {
+  __shared__ double part[kMomGroups][kMomNodes + 1];
+  const int c = threadIdx.x % kMomNodes, g = threadIdx.x / kMomNodes;
+  const int q = blockIdx.x * kMomNodes + c;
+  auto total = [&](double v) {  // sum of the node's groups, in every thread
+    part[g][c] = v;
+    __syncthreads();
+    for (int h = kMomGroups / 2; h > 0; h >>= 1) {
+      if (g < h) part[g][c] += part[g + h][c];
+      __syncthreads();
+    }
+    const double t = part[0][c];
+    __syncthreads();
+    return t;
+  };
   double mb = 0.0;
-  for (int s = 0; s < S; ++s) mb += u[(size_t)s * nn + q];
-  mb /= S;
+  if (q < nn)
+    for (int s = g; s < S; s += kMomGroups) mb += u[(size_t)s * nn + q];
+  mb = total(mb) / S;
   double M2b = 0.0;
-  for (int s = 0; s < S; ++s) {
-    const double d = u[(size_t)s * nn + q] - mb;
-    M2b += d * d;
-  }
+  if (q < nn)
+    for (int s = g; s < S; s += kMomGroups) {
+      const double d = u[(size_t)s * nn + q] - mb;
+      M2b += d * d;
+    }
+  M2b = total(M2b);
+  if (q >= nn || g != 0) return;
   const double na = count[0], nb = (double)S, nt = na + nb;
   const double delta = mb - mean[q];
   mean[q] = mean[q] + delta * (nb / nt);
@@ -640,7 +594,7 @@ extern "C" int stomsfem_coarse_workspace_size(const stomsfem_grid* grid, int32_t
   const int sms = device_sm_count();
   long long slots = (long long)(sms > 0 ? sms : 152) * 8;
   if (slots > S) slots = S;
-  if (slots < kCoarseBlkWarps) slots = kCoarseBlkWarps;
+  if (slots < kCoarseMinSlots) slots = kCoarseMinSlots;
   *bytes = coarse_slot_bytes(grid->nc) * (size_t)slots;
   return STOMSFEM_OK;
 }
@@ -659,25 +613,21 @@ extern "C" int stomsfem_coarse_solve(const stomsfem_grid* grid, const double* Ke
     return set_error(STOMSFEM_EINVAL, "mean, m2 and count must be given together");
   const size_t sb = coarse_slot_bytes(grid->nc);
   long long slots = (long long)(workspace_bytes / sb);
-  if (slots < kCoarseBlkWarps)
+  if (slots < kCoarseMinSlots)
     return set_error(STOMSFEM_ENOMEM, "coarse workspace %zu < %d slots of %zu", workspace_bytes,
-                     kCoarseBlkWarps, sb);
-  long long blocks = slots / kCoarseBlkWarps;
-  const long long need = ((long long)S + kCoarseBlkWarps - 1) / kCoarseBlkWarps;
-  if (blocks > need) blocks = need;
+                     kCoarseMinSlots, sb);
+  const long long blocks = slots < S ? slots : S;  // one sample per CTA
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int nc = grid->nc;
-  const size_t smem = blk_smem_bytes<double>(16, nc, CoarseBlkGen::kRaw) * kCoarseBlkWarps;
-  const int rpl = (16 + nc + 31) / 32;
-  auto kern = rpl <= 1 ? coarse_blk_kernel<1> : rpl == 2 ? coarse_blk_kernel<2> : coarse_blk_kernel<3>;
+  const size_t smem = cta_smem_bytes(nc);
+  auto kern = nc <= 32 ? coarse_blk_kernel<1> : coarse_blk_kernel<2>;
   STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)blocks, kCoarseBlkWarps * 32, smem, st>>>(nc, S, Ke, be, u,
-                                                              static_cast<unsigned char*>(workspace), sb,
-                                                              coarse_l_bytes(nc));
+  kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, Ke, be, u, static_cast<unsigned char*>(workspace), sb,
+                                                    coarse_l_bytes(nc));
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   if (mom) {
     const int nn = (grid->nc + 1) * (grid->nc + 1);
-    moments_kernel<<<(nn + 127) / 128, 128, 0, st>>>(nn, S, u, mean, m2, count);
+    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     count_kernel<<<1, 1, 0, st>>>(count, S);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
@@ -724,7 +674,7 @@ extern "C" int stomsfem_coarse_solve_pg(const stomsfem_grid* grid, const double*
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   if (mom) {
     const int nn = (grid->nc + 1) * (grid->nc + 1);
-    moments_kernel<<<(nn + 127) / 128, 128, 0, st>>>(nn, S, u, mean, m2, count);
+    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     count_kernel<<<1, 1, 0, st>>>(count, S);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
@@ -740,7 +690,7 @@ extern "C" int stomsfem_coarse_bc_workspace_size(const stomsfem_grid* grid, int3
   if (!grid || grid->nc <= 0 || S < 0 || !bytes || (pg != 0 && pg != 1))
     return set_error(STOMSFEM_EINVAL, "bad arguments");
   const int sms = device_sm_count();
-  const int warps = pg ? kCoarsePgWarps : kCoarseBlkWarps;
+  const int warps = pg ? kCoarsePgWarps : kCoarseMinSlots;
   long long slots = (long long)(sms > 0 ? sms : 152) * (pg ? 4 : 8);
   if (slots > S) slots = S;
   if (slots < warps) slots = warps;
@@ -764,13 +714,14 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
   if (mom && !(mean && m2 && count))
     return set_error(STOMSFEM_EINVAL, "mean, m2 and count must be given together");
   const int nc = grid->nc;
-  const int warps = pg ? kCoarsePgWarps : kCoarseBlkWarps;
+  const int warps = pg ? kCoarsePgWarps : kCoarseMinSlots;
   const size_t sb = pg ? coarse_pg_slot_bytes(nc, true) : coarse_bc_slot_bytes(nc);
   long long slots = (long long)(workspace_bytes / sb);
   if (slots < warps)
     return set_error(STOMSFEM_ENOMEM, "coarse workspace %zu < %d slots of %zu", workspace_bytes, warps, sb);
-  long long blocks = slots / warps;
-  const long long need = ((long long)S + warps - 1) / warps;
+  // Petrov-Galerkin: a warp per sample, two per CTA; Galerkin: a CTA per sample
+  long long blocks = pg ? slots / warps : slots;
+  const long long need = pg ? ((long long)S + warps - 1) / warps : S;
   if (blocks > need) blocks = need;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -781,17 +732,15 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
     coarse_pg_kernel<true><<<(unsigned)blocks, kCoarsePgWarps * 32, smem, st>>>(nc, S, K, b, dirichlet, g, u, ws, sb);
   } else {
     const int bnd = nc + 2;
-    const size_t smem = blk_smem_bytes<double>(16, bnd, CoarseBcGen::kRaw) * kCoarseBlkWarps;
-    const int rpl = (16 + bnd + 31) / 32;
-    auto kern = rpl <= 1 ? coarse_bc_kernel<1> : rpl == 2 ? coarse_bc_kernel<2> : coarse_bc_kernel<3>;
+    const size_t smem = cta_smem_bytes(bnd);
+    auto kern = bnd <= 32 ? coarse_bc_kernel<1> : coarse_bc_kernel<2>;
     STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(unsigned)blocks, kCoarseBlkWarps * 32, smem, st>>>(nc, S, K, b, dirichlet, g, u, ws, sb,
-                                                                coarse_bc_l_bytes(nc));
+    kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, K, b, dirichlet, g, u, ws, sb, coarse_bc_l_bytes(nc));
   }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   if (mom) {
     const int nn = (nc + 1) * (nc + 1);
-    moments_kernel<<<(nn + 127) / 128, 128, 0, st>>>(nn, S, u, mean, m2, count);
+    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     count_kernel<<<1, 1, 0, st>>>(count, S);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
@@ -815,7 +764,7 @@ extern "C" int stomsfem_fine_fem_workspace_size(const stomsfem_grid* grid, int32
   const int sms = device_sm_count();
   long long slots = (long long)(sms > 0 ? sms : 152) * 8;
   if (slots > S) slots = S;
-  if (slots < kCoarseBlkWarps) slots = kCoarseBlkWarps;
+  if (slots < kCoarseMinSlots) slots = kCoarseMinSlots;
   *bytes = coarse_slot_bytes(grid->nf) * (size_t)slots;
   return STOMSFEM_OK;
 }
@@ -838,17 +787,14 @@ extern "C" int stomsfem_fine_fem(const stomsfem_grid* grid, const double* a, int
   }
   const size_t sb = coarse_slot_bytes(nf);
   long long slots = (long long)(workspace_bytes / sb);
-  if (slots < kCoarseBlkWarps)
-    return set_error(STOMSFEM_ENOMEM, "fine FEM workspace %zu < %d slots of %zu", workspace_bytes, kCoarseBlkWarps, sb);
-  long long blocks = slots / kCoarseBlkWarps;
-  const long long need = ((long long)S + kCoarseBlkWarps - 1) / kCoarseBlkWarps;
-  if (blocks > need) blocks = need;
-  const size_t smem = blk_smem_bytes<double>(16, nf) * kCoarseBlkWarps;
-  const int rpl = (16 + nf + 31) / 32;
-  auto kern = rpl <= 1 ? fine_fem_kernel<1> : rpl == 2 ? fine_fem_kernel<2> : fine_fem_kernel<3>;
+  if (slots < kCoarseMinSlots)
+    return set_error(STOMSFEM_ENOMEM, "fine FEM workspace %zu < %d slots of %zu", workspace_bytes, kCoarseMinSlots, sb);
+  const long long blocks = slots < S ? slots : S;  // one sample per CTA
+  const size_t smem = cta_smem_bytes(nf);
+  auto kern = nf <= 32 ? fine_fem_kernel<1> : fine_fem_kernel<2>;
   STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)blocks, kCoarseBlkWarps * 32, smem, st>>>(nf, S, grid->f, a, u, static_cast<unsigned char*>(workspace),
-                                                             sb, coarse_l_bytes(nf));
+  kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nf, S, grid->f, a, u, static_cast<unsigned char*>(workspace), sb,
+                                                    coarse_l_bytes(nf));
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   return STOMSFEM_OK;
 }
@@ -875,7 +821,7 @@ extern "C" int stomsfem_mc_moments(int32_t n, int32_t S, const double* u, double
   if (S == 0) return STOMSFEM_OK;
   if (!u || !mean || !m2 || !count) return set_error(STOMSFEM_EINVAL, "NULL device pointer");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  moments_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, S, u, mean, m2, count);
+  moments_kernel<<<(n + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(n, S, u, mean, m2, count);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   count_kernel<<<1, 1, 0, st>>>(count, S);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
