@@ -139,21 +139,23 @@ __device__ __forceinline__ int ring(int x, int RW) { return x >= RW ? x - RW : x
 
 // Reciprocal of the pivot, 1 / sqrt(a) (the factor keeps only this).
 // FP32: the hardware reciprocal square root (a few ulp).  FP64: the FP32
-// estimate refined by two Newton steps y <- y + y (1 - a y^2) / 2, whose
-// relative error squares each step (2^-23 -> 2^-45 -> below 2^-53 before the
-// final roundings): about ten FP64 operations instead of a correctly rounded
-// square root and division, on a part whose FP64 pipe is narrow.  Outside
-// the FP32 range the library routines are used.
+// estimate y and one cubic step y (1 + e / 2 + 3 e^2 / 8), e = 1 - a y^2 (|e|
+// below 2^-21, the next term of the series 5 e^3 / 16 below 2^-64): five
+// FP64 operations on a part whose FP64 pipe is narrow, and the range test on
+// the bits.  Outside the FP32 range the library routines are used.
 __device__ __forceinline__ float pivot_rsqrt(float a) { return rsqrtf(a); }
 __device__ __forceinline__ double pivot_rsqrt(double a) {
-  if (!(a > 1e-30 && a < 1e30)) return 1.0 / sqrt(a);
-  double y = (double)rsqrtf((float)a);
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double e = fma(-a * y, y, 1.0);
-    y = fma(0.5 * y, e, y);
-  }
-  return y;
+  // exponents -90 .. 90 (a is positive here)
+  if ((unsigned)__double2hiint(a) - (933u << 20) > (180u << 20)) return 1.0 / sqrt(a);
+  const double y = (double)rsqrtf((float)a);
+  const double e = fma(-a * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+// a > 0 and not NaN: FP64 by the bit pattern (no FP64 compare).
+__device__ __forceinline__ bool pivot_ok(float a) { return a > 0.f; }
+__device__ __forceinline__ bool pivot_ok(double a) {
+  const long long b = __double_as_longlong(a);
+  return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
 template <int G, typename T>
@@ -301,8 +303,9 @@ __device__ __forceinline__ void panel_col(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T*
   if constexpr (J < NB) {
     if (J < nb) {
       const T dj = gshfl<G>(pr[0][J], J);
-      if (!(dj > T(0)) && fail < 0) fail = K + J;
-      const T dinv = pivot_rsqrt(dj > T(0) ? dj : T(1));
+      const bool ok = pivot_ok(dj);
+      if (!ok && fail < 0) fail = K + J;
+      const T dinv = pivot_rsqrt(ok ? dj : T(1));
       T yj[NR];
 #pragma unroll
       for (int c = 0; c < NR; ++c) yj[c] = gshfl<G>(rh[0][c], J) * dinv;
@@ -353,12 +356,14 @@ __device__ __forceinline__ void panel_pair(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T
     const T a00 = gshfl<G>(pr[0][J], J);
     const T a10 = gshfl<G>(pr[0][J], J1);
     const T a11 = gshfl<G>(pr[0][J1], J1);
-    if (!(a00 > T(0)) && fail < 0) fail = K + J;
-    const T i0 = pivot_rsqrt(a00 > T(0) ? a00 : T(1));
+    const bool ok0 = pivot_ok(a00);
+    if (!ok0 && fail < 0) fail = K + J;
+    const T i0 = pivot_rsqrt(ok0 ? a00 : T(1));
     const T l10 = a10 * i0;
     const T s11 = a11 - l10 * l10;
-    if (!(s11 > T(0)) && fail < 0) fail = K + J1;
-    const T i1 = pivot_rsqrt(s11 > T(0) ? s11 : T(1));
+    const bool ok1 = pivot_ok(s11);
+    if (!ok1 && fail < 0) fail = K + J1;
+    const T i1 = pivot_rsqrt(ok1 ? s11 : T(1));
     T y0[NR], y1[NR];
 #pragma unroll
     for (int c = 0; c < NR; ++c) {
@@ -467,24 +472,6 @@ __device__ __forceinline__ Tile8 tile8_of(int gl, int b) {
   return t;
 }
 
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_swap(uint64_t a) {
-  uint64_t d;
-  asm("{\n.reg .b32 lo, hi;\nmov.b64 {lo, hi}, %1;\nmov.b64 %0, {hi, lo};\n}" : "=l"(d) : "l"(a));
-  return d;
-}
-__device__ __forceinline__ float f2_lo(uint64_t a) { return __uint_as_float((uint32_t)a); }
-__device__ __forceinline__ float f2_hi(uint64_t a) { return __uint_as_float((uint32_t)(a >> 32)); }
-
 // Products of NRP row pairs (descending rows) with NCP column pairs.
 template <int NRP, int NCP>
 struct Pair2 {
@@ -581,6 +568,51 @@ __device__ __forceinline__ void tiles8_update(const Tile8& t, int b, const float
         A.sub(w + a * ws, 3 - a / 2, (a & 1) == 0, 0, t.diag ? a : 7);
         if (a >= 4 && t.diag) D.sub(w + a * ws - 4, 3 - a / 2, (a & 1) == 0, 0, a - 4);
       }
+    }
+  }
+}
+
+// ---- trailing update of the FP64 systems, in 1 x 4 tiles (one row, one
+// group of four columns).  A DFMA holds the FP64 pipe of the SM for 16
+// clocks whatever its lanes do, while a tile's loads, indices and stores
+// cost issue slots that nothing else needs: what counts is how many lanes of
+// the rounds hold entries of the triangle.  b = 8: 12 tiles, one round of 32
+// FMAs (4 x 4 tiles: 3, one round of 128 and 16 subtractions); b = 32: 144
+// tiles, 9 rounds (36, 3: 288 against 432 FP64 instructions); b = 40: 220,
+// 14 rounds (55, 4: 448 against 576).  The products are subtracted from the
+// window's values as they come.  With the cheaper pivots and the epilogue of
+// upscale_impl.cuh: 64 samples of the 64^2 / 8^2 grid (b = 8) 497 -> 340 us,
+// 1024^2, H/h = 32, 4 samples 27.9 -> 25.4 ms.
+template <int G>
+__device__ __forceinline__ void tiles1x4_update(const double* __restrict__ pt, const BlkSmem<double>& s, int tslot,
+                                                int nt, int nb, int gl) {
+  constexpr int NB = G / 2;
+  // rows 4 R .. 4 R + 3 have R + 1 groups each: 2 R (R + 1) tiles before them
+  const int Rn = nt >> 2, ntiles = (Rn + 1) * (2 * Rn + (nt & 3));
+  for (int t = gl; t < ntiles; t += G) {
+    int R = (int)((sqrtf(2.0f * t + 1.0f) - 1.0f) * 0.5f);
+    if (2 * (R + 1) * (R + 2) <= t) ++R;
+    if (2 * R * (R + 1) > t) --R;
+    const int rem = t - 2 * R * (R + 1), a = rem / (R + 1), g = rem - a * (R + 1), i = 4 * R + a;
+    // entries d = i - 4 g - 3 .. i - 4 g: element k is column 4 g + 3 - k
+    double* w = s.wnd + kWndOff + wnd_row<NB>(ring(tslot + i, s.RW), s.PW) + (i - 4 * g - 3);
+    double v[4];
+    ld_grp4(w, v);
+    const double* col = pt;
+#pragma unroll 4
+    for (int p = 0; p < nb; ++p, col += s.RP) {
+      const double l = -col[i];
+      double c[4];
+      ld_grp4(col + 4 * g, c);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = fma(l, c[3 - k], v[k]);
+    }
+    if (g < R) {
+      st_grp4(w, v);
+    } else {  // the diagonal's group: columns up to i
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (3 - k <= a) w[k] = v[k];
     }
   }
 }
@@ -735,6 +767,8 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     if constexpr (kTiles8) {
       // (nt > 0 only after a full block: nb = NB)
       if (nt > 0) tiles8_update(tile, b, pt, s, ring(kslot + NB + 8 * tile.ti, RW), nt);
+    } else if constexpr (sizeof(T) == 8) {
+      if (nt > 0) tiles1x4_update<G>(pt, s, ring(kslot + nb, RW), nt, nb, gl);
     } else if (nt > 0) {
       const int T4 = (nt + 3) >> 2;
       const int ntiles = T4 * (T4 + 1) / 2;
@@ -756,19 +790,8 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
 #pragma unroll 4
         for (int p = p0; p < nb; ++p, col += s.RP) {
           T va[4], vc[4];
-          if constexpr (sizeof(T) == 4) {
-            const float4 A4 = *reinterpret_cast<const float4*>(col + 4 * ti);
-            const float4 C4 = *reinterpret_cast<const float4*>(col + 4 * tj);
-            va[0] = A4.x; va[1] = A4.y; va[2] = A4.z; va[3] = A4.w;
-            vc[0] = C4.x; vc[1] = C4.y; vc[2] = C4.z; vc[3] = C4.w;
-          } else {
-            const double2 A0 = *reinterpret_cast<const double2*>(col + 4 * ti);
-            const double2 A1 = *reinterpret_cast<const double2*>(col + 4 * ti + 2);
-            const double2 C0 = *reinterpret_cast<const double2*>(col + 4 * tj);
-            const double2 C1 = *reinterpret_cast<const double2*>(col + 4 * tj + 2);
-            va[0] = A0.x; va[1] = A0.y; va[2] = A1.x; va[3] = A1.y;
-            vc[0] = C0.x; vc[1] = C0.y; vc[2] = C1.x; vc[3] = C1.y;
-          }
+          ld_grp4(col + 4 * ti, va);
+          ld_grp4(col + 4 * tj, vc);
 #pragma unroll
           for (int a = 0; a < 4; ++a)
 #pragma unroll

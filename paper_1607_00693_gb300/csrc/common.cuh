@@ -64,6 +64,30 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
     if (_rc != STOMSFEM_OK) return _rc;                          \
   } while (0)
 
+// Pairs of FP32 values in a 64-bit register (two values per instruction,
+// each rounded as the scalar operation).
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_swap(uint64_t a) {
+  uint64_t d;
+  asm("{\n.reg .b32 lo, hi;\nmov.b64 {lo, hi}, %1;\nmov.b64 %0, {hi, lo};\n}" : "=l"(d) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ float f2_lo(uint64_t a) { return __uint_as_float((uint32_t)a); }
+__device__ __forceinline__ float f2_hi(uint64_t a) { return __uint_as_float((uint32_t)(a >> 32)); }
+__device__ __forceinline__ uint64_t f2_both(float a) {
+  const uint64_t b = __float_as_uint(a);
+  return b | (b << 32);
+}
+
 // Full-warp sum (every lane receives the total).
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

@@ -693,6 +693,51 @@ upscale_kernel(UpscaleArgs A) {
       iNx = (TA)pg.iNxd;
       iNy = (TA)pg.iNyd;
     }
+    if constexpr (sizeof(TA) == 8 && !PG && !fwd_only) {
+      // FP64 sums: 6 u^T K_ref v = 3 s s' + 3 t t' + q q' (the eigenvectors of
+      // K_ref: s = u_0 - u_2, t = u_1 - u_3, q = u_0 - u_1 + u_2 - u_3), and a
+      // lane runs up its share of the cell's columns, so an element brings two
+      // new nodes, not four: 64 FP64 operations per element instead of 130
+      // with the six differences and four nodes of the form below.
+      // FP32 + refinement, 1024^2, 8 samples: 12.7 -> 12.1 ms.
+      const int total = A.rho * A.rho, chunk = (total + G - 1) / G;
+      const int e1 = min(total, (gl + 1) * chunk);
+      TA c0[3], c1[3], c2[3], c3[3];
+      int ex = 0, ey = -1;
+      for (int e = gl * chunk; e < e1; ++e, ++ey) {
+        if (ey < 0 || ey == A.rho) {  // the lane's first element, or the next column's
+          ex = e / A.rho;
+          ey = e - ex * A.rho;
+          const TA Y0 = (TA)(g.cy0 + ey) * iNy;
+          psi_node(g.cx0 + ex, g.cy0 + ey, (TA)(g.cx0 + ex) * iNx, Y0, c0, true);
+          psi_node(g.cx0 + ex + 1, g.cy0 + ey, (TA)(g.cx0 + ex + 1) * iNx, Y0, c1, true);
+        }
+        const int i0 = g.cx0 + ex, j0 = g.cy0 + ey;
+        const TA Y1 = (TA)(j0 + 1) * iNy;
+        psi_node(i0, j0 + 1, (TA)i0 * iNx, Y1, c3, true);
+        psi_node(i0 + 1, j0 + 1, (TA)(i0 + 1) * iNx, Y1, c2, true);
+        const TA ae = (TA)pg.ael(i0, j0), ae3 = TA(3) * ae;
+        TA s3[3], t3[3], q1[3], sd[3], td[3], qd[3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+          const TA u = c0[l] + c2[l], v = c1[l] + c3[l];
+          sd[l] = c0[l] - c2[l];
+          td[l] = c1[l] - c3[l];
+          qd[l] = u - v;
+          m[l] += u + v;
+          s3[l] = ae3 * sd[l];
+          t3[l] = ae3 * td[l];
+          q1[l] = ae * qd[l];
+          c0[l] = c3[l];
+          c1[l] = c2[l];
+        }
+        int q = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+#pragma unroll
+          for (int lp = l; lp < 3; ++lp, ++q) M[q] = fma(s3[l], sd[lp], fma(t3[l], td[lp], fma(q1[l], qd[lp], M[q])));
+      }
+    } else
     for (int e = gl; e < A.rho * A.rho; e += G) {
       const int ex = e % A.rho, ey = e / A.rho;
       const int i0 = g.cx0 + ex, j0 = g.cy0 + ey;
