@@ -626,22 +626,44 @@ __global__ void pod_affine_parts_kernel(PodDims d, const double* __restrict__ W,
 
 // a [S][nf][nf] -> Ab [cell][Spad][Kp] BF16 and its remainder Ablo = BF16(a -
 // Ab) (zero padded rows and columns)
-__global__ void pod_gather_kernel(PodDims d, const double* __restrict__ a, int S, int Spad,
-                                  __nv_bfloat16* __restrict__ Ab, __nv_bfloat16* __restrict__ Ablo) {
-  const long long total = (long long)d.ncell * Spad * d.Kp;
+// A thread converts eight consecutive elements of one (cell, sample) row and
+// stores them as one 16-byte vector per part (element by element, each with
+// its own 64-bit index divisions, the kernel ran at 2.1 TB/s).
+__global__ void __launch_bounds__(256) pod_gather_kernel(PodDims d, const double* __restrict__ a, int S, int Spad,
+                                                         __nv_bfloat16* __restrict__ Ab,
+                                                         __nv_bfloat16* __restrict__ Ablo) {
+  const unsigned per_row = d.Kp / 8;
+  const long long total = (long long)d.ncell * Spad * per_row;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
-    const int e = (int)(idx % d.Kp);
-    const long long t = idx / d.Kp;
+    const int e0 = (int)(idx % per_row) * 8;
+    const long long t = idx / per_row;
     const int s = (int)(t % Spad), cell = (int)(t / Spad);
-    float v = 0.f;
-    if (s < S && e < d.ne) {
-      const int cx = cell % d.nc, cy = cell / d.nc, ex = e % d.rho, ey = e / d.rho;
-      v = (float)a[((size_t)s * d.nf + cy * d.rho + ey) * d.nf + cx * d.rho + ex];
+    const int cx = cell % d.nc, cy = cell / d.nc;
+    int ey = e0 / d.rho, ex = e0 - ey * d.rho;
+    const double* as = a + ((size_t)s * d.nf + cy * d.rho) * d.nf + cx * d.rho;
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k] = s < S && e0 + k < d.ne ? (float)as[(size_t)ey * d.nf + ex] : 0.f;
+      if (++ex == d.rho) {
+        ex = 0;
+        ++ey;
+      }
     }
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    Ab[idx] = hi;
-    Ablo[idx] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    uint4 hi, lo;
+    uint32_t* h = reinterpret_cast<uint32_t*>(&hi);
+    uint32_t* l = reinterpret_cast<uint32_t*>(&lo);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * k]), h1 = __float2bfloat16_rn(v[2 * k + 1]);
+      const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * k] - __bfloat162float(h0));
+      const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * k + 1] - __bfloat162float(h1));
+      h[k] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+      l[k] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+    }
+    reinterpret_cast<uint4*>(Ab)[idx] = hi;
+    reinterpret_cast<uint4*>(Ablo)[idx] = lo;
   }
 }
 
@@ -655,10 +677,12 @@ constexpr uint32_t kWaitLimit = 1u << 24;  // about 2 s
 // overwrites the buffers.  split: both operands as BF16 pairs (hi, lo =
 // BF16 of the remainder) and three products per step, Ab T + Ab Tlo + Ablo
 // T (the dropped Ablo Tlo is below 2^-16 relative), so G carries about
-// 16 bits instead of BF16's 8; one product otherwise.
+// 16 bits instead of BF16's 8; one product otherwise.  units: G goes out as
+// [cell][32-sample tile][Ppad][32] (for one unit per thread) instead of
+// [cell][s][Ppad].
 __global__ void __launch_bounds__(128, 1)
 pod_gemm_kernel(PodDims d, int Spad, const __nv_bfloat16* __restrict__ Ab, const __nv_bfloat16* __restrict__ Ablo,
-                const __nv_bfloat16* __restrict__ T, const __nv_bfloat16* __restrict__ Tlo, int split,
+                const __nv_bfloat16* __restrict__ T, const __nv_bfloat16* __restrict__ Tlo, int split, int units,
                 float* __restrict__ G, int32_t* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -735,14 +759,148 @@ pod_gemm_kernel(PodDims d, int Spad, const __nv_bfloat16* __restrict__ Ab, const
     if (tid == 0) atomicOr(err, 2);
   } else {
     float* Grow = G + ((size_t)cell * Spad + s0 + warp * 32 + lane) * d.Ppad;
+    float* Gt = G + ((size_t)cell * Spad + s0 + warp * 32) * d.Ppad + lane;
     for (int col = 0; col < d.Ppad; col += 16) {
       float v[16];
       tc::tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + col, v);
+      if (units) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        reinterpret_cast<float4*>(Grow + col)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < 16; ++q)
+          if (col + q < d.P) Gt[(size_t)(col + q) * 32] = v[q];
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          reinterpret_cast<float4*>(Grow + col)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
     }
   }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(taddr_s, ncols);
+}
+
+// The same products for cells of one K step (at most 64 elements), G laid
+// out for one unit per thread: [cell][32-sample tile][Ppad][32], the samples
+// of a tile side by side.
+//
+// With a CTA per 128-sample tile and cell, each CTA staged 160 KB of
+// operands (four fifths of it the cell's T, the same for every tile), waited,
+// multiplied for 2 us, waited, and stored 250 KB in 16-byte pieces of 128
+// different rows: 16 us a tile where its bytes take 6.  Here a CTA walks a
+// range of (cell, tile), keeps T in shared memory while the cell stays the
+// same, copies the next tile's A while it works, and computes the columns in
+// two halves, so that the tensor core fills one half of the accumulator while
+// the warps empty the other; a store writes one column of 32 samples, 128
+// bytes.
+// 10^4 samples of the 64^2 / 8^2 grid, with the gather and solves reading
+// along: the online call 1.78 -> 1.33 ms.
+__global__ void __launch_bounds__(128, 1)
+pod_gemm_stream_kernel(PodDims d, int Spad, const __nv_bfloat16* __restrict__ Ab, const __nv_bfloat16* __restrict__ Ablo,
+                       const __nv_bfloat16* __restrict__ T, const __nv_bfloat16* __restrict__ Tlo, int split,
+                       float* __restrict__ G, int32_t* err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int nparts = split ? 2 : 1;
+  const uint32_t bytesA = kPodTileM * 128, bytesB = (uint32_t)d.Ppad * 128;
+  auto sB = [&](int part) { return smem + part * bytesB; };
+  auto sA = [&](int buf, int part) { return smem + nparts * bytesB + (buf * nparts + part) * bytesA; };
+  __shared__ uint64_t mbar[2];
+  __shared__ uint32_t taddr_s;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nt = Spad / kPodTileM;
+  const long long total = (long long)nt * d.ncell;
+  const int w0 = (int)(total * blockIdx.x / gridDim.x), w1 = (int)(total * (blockIdx.x + 1) / gridDim.x);
+  const int nhalf = d.Ppad > 256 ? 2 : 1;
+  uint32_t ncols = 32;
+  while ((int)ncols < d.Ppad) ncols <<= 1;
+  if (warp == 0) tc::tmem_alloc(&taddr_s, ncols);
+  if (tid == 0) {
+    tc::mbar_init(&mbar[0], 1);
+    tc::mbar_init(&mbar[1], 1);
+  }
+  auto load_a = [&](int w, int buf) {
+    const size_t row0 = (size_t)(w / nt) * Spad + (size_t)(w % nt) * kPodTileM;
+    for (int part = 0; part < nparts; ++part) {
+      const uint4* g = reinterpret_cast<const uint4*>((part ? Ablo : Ab) + row0 * kPodK);
+      for (int c = tid; c < kPodTileM * 8; c += 128)
+        tc::cp_async16(sA(buf, part) + tc::sw128_offset(c >> 3, (c & 7) * 8), g + c);
+    }
+  };
+  auto load_b = [&](int cell) {
+    for (int part = 0; part < nparts; ++part) {
+      const uint4* g = reinterpret_cast<const uint4*>((part ? Tlo : T) + (size_t)cell * d.Ppad * kPodK);
+      for (int c = tid; c < d.Ppad * 8; c += 128)
+        tc::cp_async16(sB(part) + tc::sw128_offset(c >> 3, (c & 7) * 8), g + c);
+    }
+  };
+  // staged operands and freed accumulator columns visible to the tensor core
+  auto publish = [&]() {
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+  };
+  auto issue = [&](int h, int buf) {  // thread 0: the products of half h
+    const int nb = 256 * h, nsz = min(256, d.Ppad - nb);
+    const uint32_t idesc = tc::idesc_bf16_f32(kPodTileM, nsz);
+    const int nprod = split ? 3 : 1;
+    // products (A part, B part): (0, 0), then with split (0, 1) and (1, 0)
+    for (int pr = 0; pr < nprod; ++pr) {
+      const uint32_t a0 = tc::smem_u32(sA(buf, pr == 2)), b0 = tc::smem_u32(sB(pr == 1));
+#pragma unroll
+      for (int kk = 0; kk < kPodK / 16; ++kk)
+        tc::mma_bf16(taddr_s + nb, tc::sdesc_sw128(a0 + kk * 32), tc::sdesc_sw128(b0 + nb * 128 + kk * 32), idesc,
+                     (pr > 0 || kk > 0) ? 1u : 0u);
+    }
+    tc::mma_commit(&mbar[h]);
+  };
+  bool ok = true;
+  if (w0 < w1) {
+    load_b(w0 / nt);
+    load_a(w0, 0);
+    tc::cp_async_wait_all();
+  }
+  publish();
+  const uint32_t taddr = taddr_s;
+  if (w0 < w1 && tid == 0)
+    for (int h = 0; h < nhalf; ++h) issue(h, 0);
+  for (int w = w0; w < w1 && ok; ++w) {
+    const int i = w - w0, buf = i & 1, cell = w / nt;
+    const bool next = w + 1 < w1, same = next && (w + 1) / nt == cell;
+    if (next) load_a(w + 1, buf ^ 1);
+    float* Gt = G + ((size_t)cell * (Spad / 32) + (size_t)(w % nt) * (kPodTileM / 32) + warp) * d.Ppad * 32 + lane;
+    for (int h = 0; h < nhalf; ++h) {
+      if (tid == 0) s_ok = tc::mbar_wait_bounded(&mbar[h], i & 1, kWaitLimit) ? 1 : 0;
+      __syncthreads();
+      tc::fence_after_sync();
+      if (!s_ok) {
+        ok = false;
+        break;
+      }
+      const int c1 = min(256 * h + 256, d.P);
+      for (int col = 256 * h; col < c1; col += 16) {
+        float v[16];
+        tc::tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + col, v);
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (col + q < c1) Gt[(size_t)(col + q) * 32] = v[q];
+      }
+      if (h == 0 && next) tc::cp_async_wait_all();
+      publish();
+      if (same && tid == 0) issue(h, buf ^ 1);
+    }
+    if (ok && next && !same) {
+      load_b((w + 1) / nt);
+      tc::cp_async_wait_all();
+      publish();
+      if (tid == 0)
+        for (int h = 0; h < nhalf; ++h) issue(h, buf ^ 1);
+    }
+  }
+  if (!ok && tid == 0) atomicOr(err, 2);
+  tc::cp_async_wait_all();
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(taddr_s, ncols);
@@ -851,7 +1009,8 @@ __device__ __forceinline__ void small_bwd(const float (&Mq)[32], float (&Fq)[4],
 struct PodSolveArgs {
   PodDims d;
   int S, Spad, refine;
-  const float* G;         // [cell][Spad][Ppad] reduced quantities, or NULL with Gaff
+  const float* G;         // reduced quantities, or NULL with Gaff: [cell][Spad][Ppad], or for one unit per thread
+                          // [cell][Spad / 32][Ppad][32]
   const float* Gaff;      // affine parts [cell][kPodAffParts][Ppad] (Eq. localAF), or NULL
   const double* xi;       // [S][K] parameters (affine mode)
   const int* aff_var;     // [cell][16] local parameter ids, -1 padded
@@ -1184,25 +1343,10 @@ pod_solve_kernel(PodSolveArgs A) {
 constexpr int kPuTiles = 7;                                    // 4 x 4 tiles per side (rank <= 28)
 constexpr int kPuFSlot = 4 * (kPuTiles * (kPuTiles + 1) / 2);  // first slot of the right-hand sides
 constexpr int kPuSlots = kPuFSlot + 4 * kPuTiles;
-constexpr int kPuPitch = 132;  // floats per slot: 32 units x 4, and 4 of padding
+constexpr int kPuPitch = 128;  // floats per slot: 32 units x 4
 constexpr size_t kPuSmem = sizeof(float) * kPuSlots * kPuPitch;
 
 __host__ __device__ constexpr int pu_tile(int I, int J) { return 4 * (I * (I + 1) / 2 + J); }  // slot of its row 0
-
-// Float offset (unit 0) of packed entry p of G, or -1 (G_pp, the first
-// pass's other entries: a < 4 go to the right-hand sides).
-__device__ __forceinline__ int pu_offset(int p, int P0) {
-  int a = 0, row = P0;  // packed row a holds entries (a, a) .. (a, P0 - 1)
-  while (p >= row) {
-    p -= row;
-    --row;
-    ++a;
-  }
-  const int b = a + p;
-  if (a < 4) return b < 4 ? -1 : (kPuFSlot + b - 4) * kPuPitch + a;
-  const int i = b - 4, j = a - 4;
-  return (pu_tile(i >> 2, j >> 2) + (i & 3)) * kPuPitch + (j & 3);
-}
 
 __device__ __forceinline__ void pu_cp_async4(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -1233,26 +1377,36 @@ __global__ void __launch_bounds__(32) pod_solve_units_kernel(PodSolveArgs A) {
   const double nanv = __longlong_as_double(0x7ff8000000000000ll);
   float* m = pu_smem + 4 * lane;  // this unit's column of the slots
   const bool timeout = A.err[0] != 0;
-  // where this lane's packed entries p = lane + 32 t go
-  int off[16];
-#pragma unroll
-  for (int t = 0; t < 16; ++t) off[t] = lane + 32 * t < d.P ? pu_offset(lane + 32 * t, P0) : -1;
-  const int npp = 4 * P0 - 6;  // packed rows 0..3
   for (int w = blockIdx.x; w < ntile * d.ncell; w += gridDim.x) {
     const int cell = w / ntile, s0 = (w - cell * ntile) * 32, s = s0 + lane;
     if (s0 >= A.S) continue;
     const bool live = s < A.S;
     const size_t u = (size_t)s * d.ncell + cell;
-    const float* g = A.G + ((size_t)cell * A.Spad + s0) * d.Ppad;
+    // this unit's packed entries, 32 floats apart (row a of the packed upper
+    // triangle starts at pu_row(a))
+    const float* g = A.G + (size_t)w * d.Ppad * 32 + lane;
+    auto pu_row = [&](int a) { return a * P0 - a * (a - 1) / 2; };
     const int r = A.ranks[cell], nb = (r + 3) >> 2;
+    // load weights: lane q holds wl[4 + q], lanes 28..31 wl[0..3]
+    const double* wl = A.wl + (size_t)cell * P0;
+    const float wq = lane < r ? (float)wl[4 + lane] : lane >= 28 ? (float)wl[lane - 28] : 0.f;
     if (!timeout) {
+      for (int a = 0; a < 4; ++a) {
+        const float* src = g + (size_t)(pu_row(a) + 4 - a) * 32;
+        float* dst = m + kPuFSlot * kPuPitch + a;
+#pragma unroll 4
+        for (int q = 0; q < r; ++q) pu_cp_async4(dst + q * kPuPitch, src + q * 32);
+      }
+      for (int j = 0; j < r; ++j) {
+        const int J = j >> 2;
+        const float* src = g + (size_t)(pu_row(4 + j) - j) * 32;  // entry (j, i) at i * 32
+        for (int I = J; I < nb; ++I) {
+          float* dst = m + pu_tile(I, J) * kPuPitch + (j & 3);
 #pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        if (off[t] >= 0) {
-          const float* src = g + lane + 32 * t;
-          float* dst = pu_smem + off[t];
-#pragma unroll 8
-          for (int k = 0; k < 32; ++k) pu_cp_async4(dst + 4 * k, src + (size_t)k * d.Ppad);
+          for (int k = 0; k < 4; ++k) {
+            const int i = 4 * I + k;
+            if (i >= j && i < r) pu_cp_async4(dst + k * kPuPitch, src + i * 32);
+          }
         }
       }
       pu_wait();
@@ -1366,23 +1520,14 @@ __global__ void __launch_bounds__(32) pod_solve_units_kernel(PodSolveArgs A) {
     // once more (from L2), entry (a, b) at slot b, component a
     __syncwarp();
     if (!timeout) {
-      for (int t = 0; 32 * t < npp; ++t) {
-        int p = lane + 32 * t, a = 0;
-        if (p < npp) {
-          const float* src = g + p;
-          while (p >= P0 - a) {
-            p -= P0 - a;
-            ++a;
-          }
-          float* dst = pu_smem + (a + p) * kPuPitch + a;
-#pragma unroll 8
-          for (int k = 0; k < 32; ++k) pu_cp_async4(dst + 4 * k, src + (size_t)k * d.Ppad);
-        }
+      for (int a = 0; a < 4; ++a) {
+        const float* src = g + (size_t)(pu_row(a) - a) * 32;  // entry (a, b) at b * 32
+#pragma unroll 4
+        for (int b = a; b < 4 + r; ++b) pu_cp_async4(m + b * kPuPitch + a, src + b * 32);
       }
       pu_wait();
     }
     __syncwarp();
-    const double* wl = A.wl + (size_t)cell * P0;
     // the sums over q as the warp's butterfly forms them: q with q + 16, then
     // + 8, + 4, + 2, + 1; zero past the rank
     float acc[4][14];
@@ -1394,21 +1539,23 @@ __global__ void __launch_bounds__(32) pod_solve_units_kernel(PodSolveArgs A) {
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
           const int q = c + 4 * h + 8 * x;
+          if (q >= 4 * kPuTiles) {
 #pragma unroll
-          for (int k = 0; k < 14; ++k) v[x][k] = 0.f;
-          if (q < r) {
-            const float4 gq = *reinterpret_cast<const float4*>(m + (4 + q) * kPuPitch);
-            const float4 fq = *reinterpret_cast<const float4*>(m + (kPuFSlot + q) * kPuPitch);
-            const float gv[4] = {gq.x, gq.y, gq.z, gq.w}, fv[4] = {fq.x, fq.y, fq.z, fq.w};
-            const float wv = (float)wl[4 + q];
-            int k = 0;
-#pragma unroll
-            for (int l = 0; l < 4; ++l)
-#pragma unroll
-              for (int lp = l; lp < 4; ++lp) v[x][k++] = __fmul_rn(gv[l], fv[lp]);
-#pragma unroll
-            for (int l = 0; l < 4; ++l) v[x][10 + l] = __fmul_rn(wv, fv[l]);
+            for (int k = 0; k < 14; ++k) v[x][k] = 0.f;
+            continue;
           }
+          const bool in = q < r;
+          const float4 gq = *reinterpret_cast<const float4*>(m + (4 + q) * kPuPitch);
+          const float4 fq = *reinterpret_cast<const float4*>(m + (kPuFSlot + q) * kPuPitch);
+          const float gv[4] = {gq.x, gq.y, gq.z, gq.w}, fv[4] = {fq.x, fq.y, fq.z, fq.w};
+          const float wv = __shfl_sync(0xffffffffu, wq, q);
+          int k = 0;
+#pragma unroll
+          for (int l = 0; l < 4; ++l)
+#pragma unroll
+            for (int lp = l; lp < 4; ++lp, ++k) v[x][k] = in ? __fmul_rn(gv[l], fv[lp]) : 0.f;
+#pragma unroll
+          for (int l = 0; l < 4; ++l) v[x][10 + l] = in ? __fmul_rn(wv, fv[l]) : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < 14; ++k) {
@@ -1417,6 +1564,9 @@ __global__ void __launch_bounds__(32) pod_solve_units_kernel(PodSolveArgs A) {
         }
       }
     }
+    float wl4[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) wl4[l] = __shfl_sync(0xffffffffu, wq, 28 + l);
     if (live) {
       double* Ke = A.Ke + u * 10;
       double* be = A.be + u * 4;
@@ -1432,7 +1582,7 @@ __global__ void __launch_bounds__(32) pod_solve_units_kernel(PodSolveArgs A) {
 #pragma unroll
       for (int l = 0; l < 4; ++l) {
         const float t = __fadd_rn(__fadd_rn(acc[0][10 + l], acc[2][10 + l]), __fadd_rn(acc[1][10 + l], acc[3][10 + l]));
-        be[l] = timeout || bad ? nanv : (double)__fadd_rn((float)wl[l], t);
+        be[l] = timeout || bad ? nanv : (double)__fadd_rn(wl4[l], t);
       }
       if (A.status) A.status[u] = timeout ? STOMSFEM_ETIMEOUT : bad ? STOMSFEM_ENOTSPD : 0;
     }
@@ -1798,12 +1948,26 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
   pod_gather_kernel<<<sms * 8, 256, 0, st>>>(d, a, S, Spad, Ab, Ablo);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   const int parts = pod->split ? 2 : 1;
-  const size_t smem = 1024 + parts * ((size_t)kPodTileM * 128 + (size_t)d.Ppad * 128);
+  // one unit per thread in the solves: the unrefined form of the shared basis
+  const bool per_thread = refine_iters == 0 && !d.per_l;
+  // one K step: the streaming product, whose G layout those solves read
+  const bool stream_gemm = per_thread && d.Kp == kPodK;
+  const size_t bytes_b = (size_t)d.Ppad * 128, bytes_a = (size_t)kPodTileM * 128;
+  const size_t smem = 1024 + parts * (bytes_b + (stream_gemm ? 2 : 1) * bytes_a);
   const size_t smem_req = smem < 120 * 1024 ? 120 * 1024 : smem;  // one CTA per SM (TMEM)
-  STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(pod_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_req));
-  dim3 grd(Spad / kPodTileM, d.ncell);
-  pod_gemm_kernel<<<grd, 128, smem_req, st>>>(d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, G, pod->err);
+  if (stream_gemm) {
+    const long long tiles = (long long)(Spad / kPodTileM) * d.ncell;
+    STOMSFEM_TRY_CUDA(
+        cudaFuncSetAttribute(pod_gemm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_req));
+    pod_gemm_stream_kernel<<<(unsigned)(tiles < sms ? tiles : sms), 128, smem_req, st>>>(
+        d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, G, pod->err);
+  } else {
+    STOMSFEM_TRY_CUDA(
+        cudaFuncSetAttribute(pod_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_req));
+    dim3 grd(Spad / kPodTileM, d.ncell);
+    pod_gemm_kernel<<<grd, 128, smem_req, st>>>(d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, per_thread ? 1 : 0, G,
+                                                pod->err);
+  }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   PodSolveArgs A;
   A.d = d;
@@ -1824,7 +1988,7 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
   A.be = be;
   A.status = unit_status;
   A.err = pod->err;
-  if (A.refine == 0 && !d.per_l) {
+  if (per_thread) {
     // one unit per thread (see pod_solve_units_kernel); the refined and the
     // per-l forms keep a warp per unit
     const long long work = (long long)(Spad / 32) * d.ncell;
