@@ -9,9 +9,10 @@
 // ln2/64 by fused multiply-adds, and exp(r) - 1 by its degree-5 Taylor
 // polynomial (truncation below r^6/720 < 3.6e-17).  The 64 table values
 // 2^(j/64) live in shared memory (the caller fills them with exp_table_fill).
-// Error: below about 1.5 ulp for |t| <= 700; outside that range the CUDA
-// library exp is used.  About 11 FP64 operations against the library's
-// general-purpose routine, which matters on a part with a small FP64 pipe.
+// Error: below about 1.5 ulp for |t| < 704; outside that range the CUDA
+// library exp is used.  Ten FP64 operations (the range test and the scaling
+// by 2^m work on the bits) against the library's general-purpose routine,
+// which matters on a part with a small FP64 pipe.
 #pragma once
 #include "common.cuh"
 
@@ -30,7 +31,8 @@ __device__ __forceinline__ void exp_table_fill(double* tab) {
 }
 
 __device__ __forceinline__ double fexp(double t, const double* tab) {
-  if (!(fabs(t) <= 700.0)) return exp(t);  // also NaN
+  // |t| < 704 by the high word (0x40860000 is that of 704); also NaN
+  if (((unsigned)__double2hiint(t) & 0x7fffffffu) >= 0x40860000u) return exp(t);
   const double ks = fma(t, k64ByLn2, kRoundShift);
   const int k = __double2loint(ks);        // low word = the rounded integer (two's complement)
   const double kd = ks - kRoundShift;
@@ -42,9 +44,9 @@ __device__ __forceinline__ double fexp(double t, const double* tab) {
   q = fma(r, q, 1.0);
   const double p = r * q;                  // exp(r) - 1
   const double tj = tab[k & 63];
-  const double v = fma(tj, p, tj);
-  const int m = k >> 6;                    // floor(k / 64)
-  return v * __longlong_as_double((long long)(m + 1023) << 52);
+  const double v = fma(tj, p, tj);         // in [0.99, 2)
+  const int m = k >> 6;                    // floor(k / 64), |m| <= 1016: the exponent stays normal
+  return __hiloint2double(__double2hiint(v) + (m << 20), __double2loint(v));
 }
 
 }  // namespace stomsfem
