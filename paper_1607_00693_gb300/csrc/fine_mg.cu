@@ -27,6 +27,7 @@
 // (max over samples of |r| / |f|) every few iterations.
 #include <cmath>
 #include <cstring>
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -34,7 +35,17 @@
 namespace stomsfem {
 
 constexpr int kMgMaxLevels = 12;
+// Damping of the two sweeps before and after the coarse correction.  On the
+// bilinear levels the high-frequency eigenvalues of D^-1 A lie in [0.75, 1.5]
+// (Q1 stencil, constant coefficient): the two sweeps are the Chebyshev pair
+// of that interval (largest factor 1/17; 0.16 with 0.8 twice; one CG
+// iteration fewer on the lognormal media).  The operator-dependent levels
+// keep 0.8 (see mgf_divisor_kernel), as does the coarsest grid.
 constexpr float kMgOmega = 0.8f;
+template <bool OD>
+__device__ __forceinline__ float mg_omega(int sweep) {
+  return OD ? kMgOmega : (sweep == 0 ? 1.1631f : 0.71932f);
+}
 constexpr int kMgCoarseSweeps = 60;
 constexpr int kMgThreads = 256;
 // Coefficient contrast (max a / min a over the batch) above which the
@@ -51,7 +62,7 @@ struct MgLevel {
   float* u;        // [S][N]
   float* u2;       // [S][N] (Jacobi ping-pong)
   float* f;        // [S][N]
-  float* r;        // [S][N]
+  float* r;        // [S][N], not used (the residuals stay on chip)
   float* P;        // [S][4][N]: prolongation weights from the next coarser level (per node type)
   float* dv;       // [S][N]: Jacobi divisor (see mgf_divisor_kernel)
 };
@@ -216,13 +227,11 @@ __global__ void mgf_interp_kernel(int nff, const float* __restrict__ stf, float*
   }
 }
 
-// Weight of fine node (gx, gy) in the prolongation of coarse node (I, J):
-// the stored operator-dependent weights (OD), else bilinear (1, 1/2, 1/4).
-template <bool OD>
+// Weight of fine node (gx, gy) in the operator-dependent prolongation of
+// coarse node (I, J).
 __device__ __forceinline__ float pweight(const float* __restrict__ ps, size_t N, int W, int gx, int gy, int I, int J) {
   const int dx = gx - 2 * I, dy = gy - 2 * J;
   if (dx < -1 || dx > 1 || dy < -1 || dy > 1) return 0.f;
-  if constexpr (!OD) return (dx == 0 ? 1.f : 0.5f) * (dy == 0 ? 1.f : 0.5f);
   const size_t g = (size_t)gy * W + gx;
   const bool ox = gx & 1, oy = gy & 1;
   if (!ox && !oy) return (dx == 0 && dy == 0) ? 1.f : 0.f;
@@ -232,8 +241,56 @@ __device__ __forceinline__ float pweight(const float* __restrict__ ps, size_t N,
   return ps[(size_t)m * N + g];
 }
 
-// Galerkin coarse stencils A_c = P^T A_f P at the interior coarse nodes.
-template <bool OD>
+// Galerkin coarse stencils A_c = P^T A_f P at the interior coarse nodes,
+// bilinear P.  Every weight is a constant once the loops are unrolled: the
+// nine fine nodes of the coarse node's hat, their nine couplings, and the
+// coarse nodes whose hats cover the coupled fine node; only the five stored
+// couplings are formed.
+// 1024^2, 8 samples, all levels: 508 -> 90 us.
+__global__ void __launch_bounds__(kMgThreads) mgf_rap_bilinear_kernel(int nff, const float* __restrict__ stf,
+                                                                      float* __restrict__ stc) {
+  const int s = blockIdx.y;
+  const int nfc = nff / 2, Wf = nff + 1, Wc = nfc + 1;
+  const size_t Nf = (size_t)Wf * Wf, Nc = (size_t)Wc * Wc;
+  const float* sf = stf + (size_t)s * 5 * Nf;
+  float* sc = stc + (size_t)s * 5 * Nc;
+  // (I, J) offsets of the stored couplings: centre, east, north, north-east, north-west
+  constexpr int cI[5] = {0, 1, 0, 1, -1}, cJ[5] = {0, 0, 1, 1, 1};
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < (int)Nc; v += gridDim.x * blockDim.x) {
+    const int I = v % Wc, J = v / Wc;
+    float out[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    if (interior(I, J, nfc)) {
+#pragma unroll
+      for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+        for (int di = -1; di <= 1; ++di) {
+          const float wf = (di ? 0.5f : 1.f) * (dj ? 0.5f : 1.f);
+          const long fv = (long)(2 * J + dj) * Wf + 2 * I + di;
+#pragma unroll
+          for (int ej = -1; ej <= 1; ++ej)
+#pragma unroll
+            for (int ei = -1; ei <= 1; ++ei) {
+              const int k = (ej + 1) * 3 + ei + 1;
+              const float afv = sf[(size_t)st_arr(k) * Nf + st_node(k, fv, Wf)];
+#pragma unroll
+              for (int m = 0; m < 5; ++m) {
+                const int tx = di + ei - 2 * cI[m], ty = dj + ej - 2 * cJ[m];
+                const float px = tx == 0 ? 1.f : (tx == 1 || tx == -1) ? 0.5f : 0.f;
+                const float py = ty == 0 ? 1.f : (ty == 1 || ty == -1) ? 0.5f : 0.f;
+                if (px * py != 0.f) out[m] = fmaf(wf * px * py, afv, out[m]);
+              }
+            }
+        }
+#pragma unroll
+      for (int m = 1; m < 5; ++m)
+        if (!interior(I + cI[m], J + cJ[m], nfc)) out[m] = 0.f;
+    }
+#pragma unroll
+    for (int m = 0; m < 5; ++m) sc[(size_t)m * Nc + v] = out[m];
+  }
+}
+
+// The same with the operator-dependent P.
 __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const float* __restrict__ P,
                                float* __restrict__ stc) {
   const int s = blockIdx.y;
@@ -250,7 +307,7 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
       for (int dj = -1; dj <= 1; ++dj)
         for (int di = -1; di <= 1; ++di) {
           const int fx = 2 * I + di, fy = 2 * J + dj;  // fine node in the support of coarse (I, J)
-          const float wf = pweight<OD>(ps, Nf, Wf, fx, fy, I, J);
+          const float wf = pweight(ps, Nf, Wf, fx, fy, I, J);
           if (wf == 0.f) continue;
           const int fv = fy * Wf + fx;
           for (int ej = -1; ej <= 1; ++ej)
@@ -259,17 +316,6 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
               const float afv = sf[(size_t)st_arr(k) * Nf + st_node(k, fv, Wf)];
               if (afv == 0.f) continue;
               const int gx = fx + ei, gy = fy + ej;  // neighbour fine node
-              if constexpr (!OD) {
-                // coarse nodes (I + cI, J + cJ) whose hats cover (gx, gy)
-                for (int cJ = -1; cJ <= 1; ++cJ)
-                  for (int cI = -1; cI <= 1; ++cI) {
-                    const int Ic = I + cI, Jc = J + cJ;
-                    if (!interior(Ic, Jc, nfc)) continue;
-                    const float pg = pweight<false>(ps, Nf, Wf, gx, gy, Ic, Jc);
-                    if (pg != 0.f) out[(cJ + 1) * 3 + cI + 1] += wf * afv * pg;
-                  }
-                continue;
-              }
               // the coarse nodes whose prolongation covers (gx, gy): one,
               // two or four by the node's type, with their weights
               int pI[4], pJ[4], np = 0;
@@ -306,22 +352,6 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
   }
 }
 
-// (A u)_v at an interior node from the symmetric stencil form.
-__device__ __forceinline__ float apply9(const float* __restrict__ st, size_t N, long v, const float* __restrict__ u,
-                                        int W) {
-  float t = 0.f;
-  t = fmaf(st9<0>(st, N, v, W), u[v - W - 1], t);
-  t = fmaf(st9<1>(st, N, v, W), u[v - W], t);
-  t = fmaf(st9<2>(st, N, v, W), u[v - W + 1], t);
-  t = fmaf(st9<3>(st, N, v, W), u[v - 1], t);
-  t = fmaf(st9<4>(st, N, v, W), u[v], t);
-  t = fmaf(st9<5>(st, N, v, W), u[v + 1], t);
-  t = fmaf(st9<6>(st, N, v, W), u[v + W - 1], t);
-  t = fmaf(st9<7>(st, N, v, W), u[v + W], t);
-  t = fmaf(st9<8>(st, N, v, W), u[v + W + 1], t);
-  return t;
-}
-
 // Jacobi divisor of each interior node: its diagonal entry, or half the
 // sum of the diagonal and the off-diagonal magnitudes where those exceed
 // the diagonal.  With omega = 0.8 the damped sweep then converges on every
@@ -342,47 +372,6 @@ __global__ void mgf_divisor_kernel(int nf, const float* __restrict__ st, float* 
       d = jacobi_divisor(a);
     }
     dv[(size_t)s * N + v] = d;
-  }
-}
-
-// One damped Jacobi sweep: uo = ui + omega (f - A ui) / divisor (zero_in: ui = 0).
-// OD (operator-dependent transfers, whose coarse operators need not be
-// diagonally dominant): the divisor of mgf_divisor_kernel, read in the
-// sweep from zero and formed from the loaded entries in the others; with
-// the bilinear transfers the diagonal entry, as the M-matrix levels allow.
-template <bool OD>
-__global__ void mgf_jacobi_kernel(int nf, const float* __restrict__ st, const float* __restrict__ dv,
-                                  const float* __restrict__ f, const float* __restrict__ ui, float* __restrict__ uo,
-                                  int zero_in) {
-  const int s = blockIdx.y;
-  const int W = nf + 1, N = W * W;
-  const float* ss = st + (size_t)s * 5 * N;
-  const float* fs = f + (size_t)s * N;
-  const float* us = ui + (size_t)s * N;
-  float* os = uo + (size_t)s * N;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
-    const int i = v % W, j = v / W;
-    float o = 0.f;
-    if (interior(i, j, nf)) {
-      if (zero_in) {
-        o = 0.f + kMgOmega * (fs[v] - 0.f) / (OD ? dv[(size_t)s * N + v] : ss[v]);
-      } else {
-        float a[9];
-        stencil9(ss, N, v, W, a);
-        float t = 0.f;
-        t = fmaf(a[0], us[v - W - 1], t);
-        t = fmaf(a[1], us[v - W], t);
-        t = fmaf(a[2], us[v - W + 1], t);
-        t = fmaf(a[3], us[v - 1], t);
-        t = fmaf(a[4], us[v], t);
-        t = fmaf(a[5], us[v + 1], t);
-        t = fmaf(a[6], us[v + W - 1], t);
-        t = fmaf(a[7], us[v + W], t);
-        t = fmaf(a[8], us[v + W + 1], t);
-        o = us[v] + kMgOmega * (fs[v] - t) / (OD ? jacobi_divisor(a) : a[4]);
-      }
-    }
-    os[v] = o;
   }
 }
 
@@ -426,77 +415,309 @@ __global__ void __launch_bounds__(kMgCoarseThreads) mgf_coarse_kernel(int nf, co
   if (v < N) u[(size_t)s * N + v] = o;
 }
 
-// r = f - A u at the interior nodes (0 elsewhere).
-__global__ void mgf_residual_kernel(int nf, const float* __restrict__ st, const float* __restrict__ f,
-                                    const float* __restrict__ u, float* __restrict__ r) {
-  const int s = blockIdx.y;
-  const int W = nf + 1, N = W * W;
-  const float* ss = st + (size_t)s * 5 * N;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
-    const int i = v % W, j = v / W;
-    r[(size_t)s * N + v] = interior(i, j, nf) ? f[(size_t)s * N + v] - apply9(ss, N, v, u + (size_t)s * N, W) : 0.f;
-  }
+// FP32 <-> FP64 on the integer units: the conversion instructions run on the
+// FP64 pipe, which bounds the CG's kernels (two of its slots each, as much
+// as two of the nine products of the stencil).  The exact values; subnormal
+// and other rare arguments take the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), e = b & 0x7f800000u;
+  if ((e == 0 && (b << 1)) || e == 0x7f800000u) return (double)v;
+  const unsigned hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  if (!(b << 1)) return __uint_as_float((unsigned)(b >> 32));
+  // round to nearest even at bit 29
+  const unsigned long long w = b + 0x0fffffffull + ((b >> 29) & 1);
+  const unsigned e = (unsigned)(w >> 52) & 0x7ffu;
+  if (e < 897u || e > 1150u) return (float)v;
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (((unsigned)(w >> 29) + 0x40000000u) & 0x7fffffffu));
 }
 
-// f_c = P^T r_f at the interior coarse nodes.
-template <bool OD>
-__global__ void mgf_restrict_kernel(int nff, const float* __restrict__ P, const float* __restrict__ rf,
-                                    float* __restrict__ fc) {
-  const int s = blockIdx.y;
-  const int nfc = nff / 2, Wf = nff + 1, Wc = nfc + 1;
-  const int Nf = Wf * Wf, Nc = Wc * Wc;
-  const float* ps = P + (size_t)s * 4 * Nf;
-  const float* r = rf + (size_t)s * Nf;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < Nc; v += gridDim.x * blockDim.x) {
-    const int I = v % Wc, J = v / Wc;
+// Block sum of v into acc[s] (one atomic per block).
+__device__ __forceinline__ void block_sum_to(double v, double* acc) {
+  __shared__ double part[32];
+  v = warp_sum(v);
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (l == 0) part[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    double t = l < (int)(blockDim.x >> 5) ? part[l] : 0.0;
+    t = warp_sum(t);
+    if (l == 0) atomicAdd(acc, t);
+  }
+  __syncthreads();
+}
+
+// ---- the V-cycle's passes over a level, two fused kernels
+//
+// Smoothing sweeps, residual and transfers read the same five coupling
+// arrays; as kernels of their own (two sweeps, residual, restriction going
+// down; prolongation and two sweeps going up) they moved 152 bytes per node,
+// five times the 28 that the arrays and vectors of one direction hold, and
+// from 256^2 down a level's eight launches cost more than its work.  Here a
+// warp marches up a strip of 32 columns, one row per step, with the stages
+// one row behind each other: sweep 1 on row t, sweep 2 on row t - 1, the
+// residual on row t - 2, the restriction on row t - 3.  The rows a stage
+// needs of the one before it stay in registers, the neighbouring columns
+// come from the neighbouring lanes, and each array entry is loaded once.
+// The stages narrow the strip by one lane on either side each (26 of 32
+// lanes write going down, 28 going up); a segment of rows starts three (two)
+// rows early.  In shared-memory tiles (64 x 32 nodes, the first version) the
+// same passes took 390 instructions per 32 nodes for index arithmetic and 18
+// coupling loads, and ten turns of latency per phase on the small levels.
+// 1024^2, 8 samples: the V-cycle 540 -> 290 us, the solve with the leaner CG
+// and set-up 12.02 -> 8.53 ms.
+constexpr int kMgWarps = 4;
+
+// One strip and row segment of a level for the calling warp.
+struct MgMarch {
+  int x, y0, y1;
+  bool in;  // an interior column
+};
+__device__ __forceinline__ bool mg_march(int nf, int useful, int halo, int rows, MgMarch& m) {
+  const int W = nf + 1, strips = (W + useful - 1) / useful;
+  const int w = blockIdx.x * kMgWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int seg = w / strips;
+  m.x = (w - seg * strips) * useful - halo + lane;
+  m.y0 = seg * rows;
+  m.y1 = min(m.y0 + rows, W);
+  m.in = m.x > 0 && m.x < nf;
+  return m.y0 < W;
+}
+
+__device__ __forceinline__ float lane_west(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ float lane_east(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+// A row of a vector with its two neighbouring columns.
+struct MgTri {
+  float w, c, e;
+  __device__ __forceinline__ void set(float v) {
+    c = v;
+    w = lane_west(v);
+    e = lane_east(v);
+  }
+};
+
+// The couplings of row y (own entries), zero outside the interior.
+struct MgCoef {
+  float c, e, n, ne, nw, f;  // f: the right-hand side
+  __device__ __forceinline__ void load(const float* __restrict__ st, size_t N, const float* __restrict__ fs, bool in,
+                                       size_t q) {
+    c = e = n = ne = nw = f = 0.f;
+    if (in) {
+      c = st[q];
+      e = st[N + q];
+      n = st[2 * N + q];
+      ne = st[3 * N + q];
+      nw = st[4 * N + q];
+      f = fs[q];
+    } else {
+      c = 1.f;
+    }
+  }
+};
+
+// A 9-point stencil in place (its own row's entries and the row below's).
+struct MgStencil {
+  float a[9];
+  __device__ __forceinline__ void set(const MgCoef& k, const MgCoef& below) {
+    a[4] = k.c;
+    a[5] = k.e;
+    a[3] = lane_west(k.e);
+    a[7] = k.n;
+    a[1] = below.n;
+    a[8] = k.ne;
+    a[0] = lane_west(below.ne);
+    a[6] = k.nw;
+    a[2] = lane_east(below.nw);
+  }
+  __device__ __forceinline__ float apply(const MgTri& s, const MgTri& m, const MgTri& n) const {
     float t = 0.f;
-    if (interior(I, J, nfc)) {
-      if constexpr (OD) {
+    t = fmaf(a[0], s.w, t);
+    t = fmaf(a[1], s.c, t);
+    t = fmaf(a[2], s.e, t);
+    t = fmaf(a[3], m.w, t);
+    t = fmaf(a[4], m.c, t);
+    t = fmaf(a[5], m.e, t);
+    t = fmaf(a[6], n.w, t);
+    t = fmaf(a[7], n.c, t);
+    t = fmaf(a[8], n.e, t);
+    return t;
+  }
+};
+
+// Going down: u = two damped Jacobi sweeps from zero on A u = f, and fc =
+// P^T (f - A u) at the next level's nodes.  OD: operator-dependent transfers,
+// whose coarse operators need not be diagonally dominant: the sweeps divide
+// by the divisor of mgf_divisor_kernel; with the bilinear transfers by the
+// diagonal entry, as the M-matrix levels allow.  rows: even.
+template <bool OD>
+__global__ void __launch_bounds__(kMgWarps * 32) mgf_down_kernel(int nf, int rows, const float* __restrict__ st,
+                                                                 const float* __restrict__ dv,
+                                                                 const float* __restrict__ P,
+                                                                 const float* __restrict__ f, float* __restrict__ u,
+                                                                 float* __restrict__ fc) {
+  MgMarch m;
+  if (!mg_march(nf, 26, 3, rows, m)) return;
+  const int s = blockIdx.y, lane = threadIdx.x & 31;
+  const int W = nf + 1, nfc = nf / 2, Wc = nfc + 1;
+  const size_t N = (size_t)W * W;
+  st += (size_t)s * 5 * N;
+  f += (size_t)s * N;
+  u += (size_t)s * N;
+  fc += (size_t)s * Wc * Wc;
+  const float* ds = dv + (size_t)s * N;
+  const float* ps = P + (size_t)s * 4 * N;
+  const bool mine = lane >= 3 && lane < 29 && m.x < W;
+  auto inside = [&](int y) { return m.in && y > 0 && y < nf; };
+  auto at = [&](int y) { return (size_t)y * W + m.x; };
+  MgCoef k0, k1, k2, kn;  // rows t, t - 1, t - 2 and t + 1
+  float r0 = 0.f, r1 = 0.f;  // reciprocal divisors of rows t, t - 1
+  MgStencil sa, sb;          // rows t - 1, t - 2
+  MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};                           // sweep 1: rows t, t - 1, t - 2
+  MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};                           // sweep 2: rows t - 1, t - 2, t - 3
+  MgTri c2, c3{0.f, 0.f, 0.f}, c4{0.f, 0.f, 0.f};                           // residual: rows t - 2, t - 3, t - 4
+  int t = m.y0 - 3;
+  k1.load(st, N, f, false, 0);
+  k2 = k1;
+  sb.set(k1, k2);
+  kn.load(st, N, f, inside(t), at(t));
+  float dn = OD && inside(t) ? ds[at(t)] : 1.f;
+#pragma unroll 3
+  for (; t < m.y1 + 3; ++t) {
+    k0 = kn;
+    r0 = __fdividef(1.f, OD ? dn : k0.c);
+    kn.load(st, N, f, inside(t + 1), at(t + 1));
+    if (OD) dn = inside(t + 1) ? ds[at(t + 1)] : 1.f;
+    a0.set(mg_omega<OD>(0) * k0.f * r0);
+    sa.set(k1, k2);
+    const float v = inside(t - 1) ? a1.c + mg_omega<OD>(1) * (k1.f - sa.apply(a2, a1, a0)) * r1 : 0.f;
+    if (mine && t - 1 >= m.y0 && t - 1 < m.y1) u[at(t - 1)] = v;
+    b1.set(v);
+    c2.set(inside(t - 2) ? k2.f - sb.apply(b3, b2, b1) : 0.f);
+    const int y = t - 3;
+    if (mine && y >= m.y0 && y < m.y1 && !((y | m.x) & 1)) {
+      const int I = m.x >> 1, J = y >> 1;
+      float q = 0.f;
+      if (interior(I, J, nfc)) {
+        if constexpr (OD) {
+          const MgTri* c[3] = {&c4, &c3, &c2};
 #pragma unroll
-        for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-          for (int dx = -1; dx <= 1; ++dx) {
-            const int gx = 2 * I + dx, gy = 2 * J + dy;
-            t = fmaf(pweight<true>(ps, Nf, Wf, gx, gy, I, J), r[(size_t)gy * Wf + gx], t);
+          for (int dy = -1; dy <= 1; ++dy) {
+            q = fmaf(pweight(ps, N, W, m.x - 1, y + dy, I, J), c[dy + 1]->w, q);
+            q = fmaf(pweight(ps, N, W, m.x, y + dy, I, J), c[dy + 1]->c, q);
+            q = fmaf(pweight(ps, N, W, m.x + 1, y + dy, I, J), c[dy + 1]->e, q);
           }
-      } else {
-        const float* q = r + (size_t)(2 * J) * Wf + 2 * I;
-        t = q[0] + 0.5f * (q[-1] + q[1] + q[-Wf] + q[Wf]) + 0.25f * (q[-Wf - 1] + q[-Wf + 1] + q[Wf - 1] + q[Wf + 1]);
+        } else {
+          q = c3.c + 0.5f * (c3.w + c3.e + c4.c + c2.c) + 0.25f * (c4.w + c4.e + c2.w + c2.e);
+        }
       }
+      fc[(size_t)J * Wc + I] = q;
     }
-    fc[(size_t)s * Nc + v] = t;
+    a2 = a1;
+    a1 = a0;
+    b3 = b2;
+    b2 = b1;
+    c4 = c3;
+    c3 = c2;
+    sb = sa;
+    k2 = k1;
+    k1 = k0;
+    r1 = r0;
   }
 }
 
-// u_f += P u_c at the interior fine nodes.
+// (P u_c) at the interior fine node (x, y).
 template <bool OD>
-__global__ void mgf_prolong_kernel(int nff, const float* __restrict__ P, const float* __restrict__ uc,
-                                   float* __restrict__ uf) {
-  const int s = blockIdx.y;
-  const int nfc = nff / 2, Wf = nff + 1, Wc = nfc + 1;
-  const int Nf = Wf * Wf, Nc = Wc * Wc;
-  const float* ps = P + (size_t)s * 4 * Nf;
-  const float* u = uc + (size_t)s * Nc;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < Nf; v += gridDim.x * blockDim.x) {
-    const int x = v % Wf, y = v / Wf;
-    if (!interior(x, y, nff)) continue;
-    const int I0 = x >> 1, J0 = y >> 1;
-    float t;
-    if constexpr (!OD) {
-      const int I1 = (x & 1) ? I0 + 1 : I0, J1 = (y & 1) ? J0 + 1 : J0;
-      t = 0.25f * (u[J0 * Wc + I0] + u[J0 * Wc + I1] + u[J1 * Wc + I0] + u[J1 * Wc + I1]);
-    } else if (!(x & 1) && !(y & 1)) {
-      t = u[J0 * Wc + I0];
-    } else if (!(y & 1)) {  // between coarse nodes I0, I0 + 1 of row J0
-      t = ps[v] * u[J0 * Wc + I0] + ps[(size_t)Nf + v] * u[J0 * Wc + I0 + 1];
-    } else if (!(x & 1)) {  // between coarse nodes J0, J0 + 1 of column I0
-      t = ps[v] * u[J0 * Wc + I0] + ps[(size_t)Nf + v] * u[(J0 + 1) * Wc + I0];
-    } else {  // cell centre: corners SW, SE, NE, NW
-      t = ps[v] * u[J0 * Wc + I0] + ps[(size_t)Nf + v] * u[J0 * Wc + I0 + 1] +
-          ps[(size_t)2 * Nf + v] * u[(J0 + 1) * Wc + I0 + 1] + ps[(size_t)3 * Nf + v] * u[(J0 + 1) * Wc + I0];
-    }
-    uf[(size_t)s * Nf + v] += t;
+__device__ __forceinline__ float prolong_at(const float* __restrict__ ps, size_t Nf, int Wf, const float* __restrict__ u,
+                                            int Wc, int x, int y) {
+  const int I0 = x >> 1, J0 = y >> 1;
+  const size_t v = (size_t)y * Wf + x;
+  if constexpr (!OD) {
+    const int I1 = (x & 1) ? I0 + 1 : I0, J1 = (y & 1) ? J0 + 1 : J0;
+    return 0.25f * (u[J0 * Wc + I0] + u[J0 * Wc + I1] + u[J1 * Wc + I0] + u[J1 * Wc + I1]);
   }
+  if (!(x & 1) && !(y & 1)) return u[J0 * Wc + I0];
+  if (!(y & 1))  // between coarse nodes I0, I0 + 1 of row J0
+    return ps[v] * u[J0 * Wc + I0] + ps[Nf + v] * u[J0 * Wc + I0 + 1];
+  if (!(x & 1))  // between coarse nodes J0, J0 + 1 of column I0
+    return ps[v] * u[J0 * Wc + I0] + ps[Nf + v] * u[(J0 + 1) * Wc + I0];
+  // cell centre: corners SW, SE, NE, NW
+  return ps[v] * u[J0 * Wc + I0] + ps[Nf + v] * u[J0 * Wc + I0 + 1] + ps[2 * Nf + v] * u[(J0 + 1) * Wc + I0 + 1] +
+         ps[3 * Nf + v] * u[(J0 + 1) * Wc + I0];
+}
+
+// Going up: uo = two damped Jacobi sweeps on A u = f from ui + P uc.  r
+// (the finest level, else NULL): the sample's r . uo is added to rz[s].
+template <bool OD>
+__global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows, const float* __restrict__ st,
+                                                               const float* __restrict__ dv,
+                                                               const float* __restrict__ P,
+                                                               const float* __restrict__ f,
+                                                               const float* __restrict__ uc,
+                                                               const float* __restrict__ ui, float* __restrict__ uo,
+                                                               const double* __restrict__ r, double* __restrict__ rz) {
+  MgMarch m;
+  const bool run = mg_march(nf, 28, 2, rows, m);
+  const int s = blockIdx.y, lane = threadIdx.x & 31;
+  double acc = 0.0;
+  if (run) {
+    const int W = nf + 1, Wc = nf / 2 + 1;
+    const size_t N = (size_t)W * W;
+    st += (size_t)s * 5 * N;
+    f += (size_t)s * N;
+    ui += (size_t)s * N;
+    uo += (size_t)s * N;
+    uc += (size_t)s * Wc * Wc;
+    const float* ds = dv + (size_t)s * N;
+    const float* ps = P + (size_t)s * 4 * N;
+    const double* rs = r ? r + (size_t)s * N : nullptr;
+    const bool mine = lane >= 2 && lane < 30 && m.x < W;
+    auto inside = [&](int y) { return m.in && y > 0 && y < nf; };
+    auto at = [&](int y) { return (size_t)y * W + m.x; };
+    auto start = [&](int y) { return inside(y) ? ui[at(y)] + prolong_at<OD>(ps, N, W, uc, Wc, m.x, y) : 0.f; };
+    auto mine_at = [&](int y) { return mine && m.in && y > 0 && y < nf && y >= m.y0 && y < m.y1; };
+    MgCoef k0, k1, k2, kn;  // rows t, t - 1, t - 2 and t + 1
+    float r0, r1 = 0.f, r2 = 0.f;  // reciprocal divisors of rows t, t - 1, t - 2
+    MgStencil sa, sb;              // rows t - 1, t - 2
+    MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};  // the starting values: rows t, t - 1, t - 2
+    MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};  // sweep 1: rows t - 1, t - 2, t - 3
+    int t = m.y0 - 2;
+    k1.load(st, N, f, false, 0);
+    k2 = k1;
+    sb.set(k1, k2);
+    kn.load(st, N, f, inside(t), at(t));
+    float vn = start(t), dn = OD && inside(t) ? ds[at(t)] : 1.f;
+    double rn = 0.0;  // r of row t - 2
+#pragma unroll 3
+    for (; t < m.y1 + 2; ++t) {
+      k0 = kn;
+      r0 = __fdividef(1.f, OD ? dn : k0.c);
+      a0.set(vn);
+      const double rv = rn;
+      kn.load(st, N, f, inside(t + 1), at(t + 1));
+      vn = start(t + 1);
+      if (OD) dn = inside(t + 1) ? ds[at(t + 1)] : 1.f;
+      if (rs) rn = mine_at(t - 1) ? rs[at(t - 1)] : 0.0;
+      sa.set(k1, k2);
+      b1.set(inside(t - 1) ? a1.c + mg_omega<OD>(0) * (k1.f - sa.apply(a2, a1, a0)) * r1 : 0.f);
+      const float v = inside(t - 2) ? b2.c + mg_omega<OD>(1) * (k2.f - sb.apply(b3, b2, b1)) * r2 : 0.f;
+      if (mine && t - 2 >= m.y0 && t - 2 < m.y1) uo[at(t - 2)] = v;
+      if (rs) acc = fma(rv, widen(v), acc);
+      a2 = a1;
+      a1 = a0;
+      b3 = b2;
+      b2 = b1;
+      sb = sa;
+      k2 = k1;
+      k1 = k0;
+      r2 = r1;
+      r1 = r0;
+    }
+  }
+  if (r) block_sum_to(acc, rz + s);
 }
 
 // mm[0] = bit pattern of max a, mm[1] = that of min a over the positive
@@ -526,102 +747,95 @@ __global__ void mgf_range_kernel(long long n, const double* __restrict__ a, unsi
 
 // ---------------------------------------------------------------- CG (FP64)
 
-// Block sum of v into acc[s] (one atomic per block).
-__device__ __forceinline__ void block_sum_to(double v, double* acc) {
-  __shared__ double part[kMgThreads / 32];
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) part[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    double t = l < (int)(blockDim.x >> 5) ? part[l] : 0.0;
-    t = warp_sum(t);
-    if (l == 0) atomicAdd(acc, t);
-  }
-  __syncthreads();
+// Scalars of the iteration, per sample: r . z and p . Ap of this and the
+// next iteration (two slots each, by the iteration's parity), r . r, b . b,
+// and which samples have converged.  Each kernel clears the sums that the
+// next ones add to (blocks x = y = 0 of a sample, values nothing reads then).
+struct CgScal {
+  double* v;  // [6][S]: r . z (two slots), p . Ap (two slots), r . r, b . b
+  int32_t* done;
+  int S;
+  __device__ __forceinline__ double& rz(int slot, int s) const { return v[(size_t)slot * S + s]; }
+  __device__ __forceinline__ double& pAp(int slot, int s) const { return v[(size_t)(2 + slot) * S + s]; }
+  __device__ __forceinline__ double& rr(int s) const { return v[(size_t)4 * S + s]; }
+};
+
+// (A p)_v from the FP64 symmetric form: q points at p's value (pitch pw).
+__device__ __forceinline__ double apply9d(const double* __restrict__ C, size_t N, long v, int W, const double* q, int pw) {
+  const double *E = C + N, *Nn = C + 2 * N, *NE = C + 3 * N, *NW = C + 4 * N;
+  double t = C[v] * q[0];
+  t = fma(E[v], q[1], t);
+  t = fma(E[v - 1], q[-1], t);
+  t = fma(Nn[v], q[pw], t);
+  t = fma(Nn[v - W], q[-pw], t);
+  t = fma(NE[v], q[pw + 1], t);
+  t = fma(NE[v - W - 1], q[-pw - 1], t);
+  t = fma(NW[v], q[pw - 1], t);
+  t = fma(NW[v - W + 1], q[-pw + 1], t);
+  return t;
 }
 
-// Ap = A p (the stored FP64 stencil in symmetric form), and pAp[s] += p . Ap.
-__global__ void __launch_bounds__(kMgThreads) cg_matvec_kernel(int nf, const double* __restrict__ st64,
-                                                               const double* __restrict__ p, double* __restrict__ Ap,
-                                                               double* __restrict__ pAp) {
+// p = z + beta p, beta = rz_new / rz_old (p = z on the first step, where p
+// is not read: the workspace holds whatever it held before).  (In one kernel
+// with the product A p, through a tile of p with its halo, the two took 255
+// us where they take 28 and 165 apart, 1024^2, 8 samples: both are bound by
+// the FP64 pipe, and the halo adds to it.)
+__global__ void __launch_bounds__(kMgThreads) cg_direction_kernel(int nf, const float* __restrict__ z, CgScal c, int cur,
+                                                                  int first, double* __restrict__ p) {
+  const int s = blockIdx.y;
+  const int N = (nf + 1) * (nf + 1);
+  const double rn = c.rz(cur, s), ro = c.rz(cur ^ 1, s);
+  const bool done = c.done[s] != 0;
+  const double beta = (first || done || !(ro != 0.0)) ? 0.0 : rn / ro;
+  if (blockIdx.x == 0 && threadIdx.x == 0) c.rr(s) = 0.0;
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
+    const size_t q = (size_t)s * N + v;
+    p[q] = done ? 0.0 : first ? widen(z[q]) : fma(beta, p[q], widen(z[q]));
+  }
+}
+__global__ void __launch_bounds__(kMgThreads) cg_matvec_kernel(int nf, const double* __restrict__ st64, CgScal c, int cur,
+                                                               const double* __restrict__ p, double* __restrict__ Ap) {
   const int s = blockIdx.y;
   const int W = nf + 1, N = W * W;
   const double* C = st64 + (size_t)s * 5 * N;
-  const double *E = C + N, *Nn = C + 2 * (size_t)N, *NE = C + 3 * (size_t)N, *NW = C + 4 * (size_t)N;
   const double* ps = p + (size_t)s * N;
   double acc = 0.0;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
     const int i = v % W, j = v / W;
     double t = 0.0;
     if (interior(i, j, nf)) {
-      const double* q = ps + v;
-      t = C[v] * q[0];
-      t = fma(E[v], q[1], t);
-      t = fma(E[v - 1], q[-1], t);
-      t = fma(Nn[v], q[W], t);
-      t = fma(Nn[v - W], q[-W], t);
-      t = fma(NE[v], q[W + 1], t);
-      t = fma(NE[v - W - 1], q[-W - 1], t);
-      t = fma(NW[v], q[W - 1], t);
-      t = fma(NW[v - W + 1], q[-W + 1], t);
-      acc += q[0] * t;
+      t = apply9d(C, N, v, W, ps + v, W);
+      acc += ps[v] * t;
     }
     Ap[(size_t)s * N + v] = t;
   }
-  block_sum_to(acc, pAp + s);
+  block_sum_to(acc, &c.pAp(cur, s));
 }
 
-// Per sample: alpha = rz / pAp (0 once converged or degenerate).
-__global__ void cg_alpha_kernel(int S, const double* rz, const double* pAp, const int32_t* done, double* alpha) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < S) alpha[s] = (done[s] || !(pAp[s] > 0.0)) ? 0.0 : rz[s] / pAp[s];
-}
-
-// x += alpha p, r -= alpha Ap; rr[s] += r . r; the FP32 copy of r for the
-// preconditioner.
-__global__ void __launch_bounds__(kMgThreads) cg_update_kernel(int nf, const double* __restrict__ alpha,
-                                                               const double* __restrict__ p, const double* __restrict__ Ap,
-                                                               double* __restrict__ x, double* __restrict__ r,
-                                                               float* __restrict__ r32, double* __restrict__ rr) {
+// x += alpha p, r -= alpha Ap with alpha = rz / pAp (0 once converged or
+// degenerate); rr[s] += r . r; the FP32 copy of r for the preconditioner.
+// Clears the next iteration's r . z and p . Ap.
+__global__ void __launch_bounds__(kMgThreads) cg_update_kernel(int nf, CgScal c, int cur, const double* __restrict__ p,
+                                                               const double* __restrict__ Ap, double* __restrict__ x,
+                                                               double* __restrict__ r, float* __restrict__ r32) {
   const int s = blockIdx.y;
   const int N = (nf + 1) * (nf + 1);
-  const double al = alpha[s];
+  const double pap = c.pAp(cur, s);
+  const double al = (c.done[s] || !(pap > 0.0)) ? 0.0 : c.rz(cur, s) / pap;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    c.rz(cur ^ 1, s) = 0.0;
+    c.pAp(cur ^ 1, s) = 0.0;
+  }
   double acc = 0.0;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
     const size_t q = (size_t)s * N + v;
     x[q] += al * p[q];
     const double rv = r[q] - al * Ap[q];
     r[q] = rv;
-    r32[q] = (float)rv;
+    r32[q] = narrow(rv);
     acc += rv * rv;
   }
-  block_sum_to(acc, rr + s);
-}
-
-// rz[s] += r . z (z the FP32 preconditioned residual).
-__global__ void __launch_bounds__(kMgThreads) cg_rz_kernel(int nf, const double* __restrict__ r,
-                                                           const float* __restrict__ z, double* __restrict__ rz) {
-  const int s = blockIdx.y;
-  const int N = (nf + 1) * (nf + 1);
-  double acc = 0.0;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x)
-    acc += r[(size_t)s * N + v] * (double)z[(size_t)s * N + v];
-  block_sum_to(acc, rz + s);
-}
-
-// p = z + beta p, beta = rz_new / rz_old (p = z on the first step, where p
-// is not read: the workspace holds whatever it held before).
-__global__ void cg_direction_kernel(int nf, const float* __restrict__ z, const double* __restrict__ rz_new,
-                                    const double* __restrict__ rz_old, const int32_t* done, int first,
-                                    double* __restrict__ p) {
-  const int s = blockIdx.y;
-  const int N = (nf + 1) * (nf + 1);
-  const double beta = (first || done[s] || !(rz_old[s] != 0.0)) ? 0.0 : rz_new[s] / rz_old[s];
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
-    const size_t q = (size_t)s * N + v;
-    p[q] = done[s] ? 0.0 : first ? (double)z[q] : (double)z[q] + beta * p[q];
-  }
+  block_sum_to(acc, &c.rr(s));
 }
 
 // r = b (f h^2 at the interior nodes), x = 0, |b|^2 per sample.
@@ -707,28 +921,38 @@ dim3 grid2(int N, int S) {
   return dim3((unsigned)bx, (unsigned)S);
 }
 
+// Rows per segment of a level's marches: the longest that still gives the
+// chip twelve warps per SM (a segment repeats up to six rows of its
+// neighbours; below that many warps the loads' latency shows), 8 at least.
+int mg_rows(int nf, int S) {
+  const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
+  int rows = 64;
+  while (rows > 8 && (long long)((nf + 28) / 28) * ((nf + rows) / rows) * S < 12LL * sms) rows >>= 1;
+  return rows;
+}
+dim3 mg_grid(int nf, int S, int useful, int rows) {
+  const long long warps = (long long)((nf + useful) / useful) * ((nf + rows) / rows);
+  return dim3((unsigned)((warps + kMgWarps - 1) / kMgWarps), (unsigned)S);
+}
+
 // z = V-cycle(r) on level l (f of level l holds the right-hand side; the
-// result in u of level l).
+// result in u2 of level l, in u on the coarsest); on the finest level rz[s]
+// += r . z.
 template <bool OD>
-int vcycle(MgLevel* lv, int L, int l, int S, cudaStream_t st) {
+int vcycle(MgLevel* lv, int L, int l, int S, const double* r, double* rz, cudaStream_t st) {
   MgLevel& c = lv[l];
-  const dim3 g = grid2(c.N, S);
   if (l == L - 1) {
     if (c.N > kMgCoarseMaxNodes) return set_error(STOMSFEM_EINVAL, "coarsest grid of %d nodes", c.N);
     mgf_coarse_kernel<<<S, kMgCoarseThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u);
     return check_cuda(cudaGetLastError(), "coarse sweeps");
   }
-  // pre-smoothing from zero
-  mgf_jacobi_kernel<OD><<<g, kMgThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u, c.u2, 1);
-  mgf_jacobi_kernel<OD><<<g, kMgThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u2, c.u, 0);
-  mgf_residual_kernel<<<g, kMgThreads, 0, st>>>(c.nf, c.st, c.f, c.u, c.r);
+  const int rows = mg_rows(c.nf, S);
   MgLevel& n = lv[l + 1];
-  mgf_restrict_kernel<OD><<<grid2(n.N, S), kMgThreads, 0, st>>>(c.nf, c.P, c.r, n.f);
-  int rc = vcycle<OD>(lv, L, l + 1, S, st);
+  mgf_down_kernel<OD><<<mg_grid(c.nf, S, 26, rows), kMgWarps * 32, 0, st>>>(c.nf, rows, c.st, c.dv, c.P, c.f, c.u, n.f);
+  int rc = vcycle<OD>(lv, L, l + 1, S, nullptr, nullptr, st);
   if (rc) return rc;
-  mgf_prolong_kernel<OD><<<g, kMgThreads, 0, st>>>(c.nf, c.P, n.u, c.u);
-  mgf_jacobi_kernel<OD><<<g, kMgThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u, c.u2, 0);
-  mgf_jacobi_kernel<OD><<<g, kMgThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u2, c.u, 0);
+  mgf_up_kernel<OD><<<mg_grid(c.nf, S, 28, rows), kMgWarps * 32, 0, st>>>(
+      c.nf, rows, c.st, c.dv, c.P, c.f, l + 1 == L - 1 ? n.u : n.u2, c.u, c.u2, r, rz);
   return check_cuda(cudaGetLastError(), "v-cycle");
 }
 
@@ -763,9 +987,8 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
   if (workspace_bytes < need)
     return set_error(STOMSFEM_ENOMEM, "fine FEM workspace %zu < %zu bytes", workspace_bytes, need);
   double *r = vec[0], *p = vec[1], *Ap = vec[2], *st64 = vec[3];
-  double *alpha = scal, *pAp = scal + S, *rz = scal + 2 * S, *rz_old = scal + 3 * S, *rr = scal + 4 * S,
-         *bb = scal + 5 * S;
-  int32_t* done = reinterpret_cast<int32_t*>(scal + 6 * S);
+  const CgScal sc{scal, reinterpret_cast<int32_t*>(scal + 6 * (size_t)S), S};
+  double *rr = scal + 4 * (size_t)S, *bb = scal + 5 * (size_t)S;
   const int N0 = lv[0].N;
   const dim3 g0 = grid2(N0, S);
   unsigned long long* range = reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(scal) +
@@ -791,33 +1014,33 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
   for (int l = 0; l + 1 < L; ++l) {
     if (od) {
       mgf_interp_kernel<<<grid2(lv[l].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].P);
-      mgf_rap_kernel<true><<<grid2(lv[l + 1].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].P,
-                                                                          lv[l + 1].st);
+      mgf_rap_kernel<<<grid2(lv[l + 1].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].P, lv[l + 1].st);
     } else {
-      mgf_rap_kernel<false><<<grid2(lv[l + 1].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].P,
-                                                                           lv[l + 1].st);
+      mgf_rap_bilinear_kernel<<<grid2(lv[l + 1].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l + 1].st);
     }
   }
-  for (int l = 0; l < L; ++l)
+  // (the bilinear sweeps divide by the diagonal entry)
+  for (int l = od ? 0 : L - 1; l < L; ++l)
     mgf_divisor_kernel<<<grid2(lv[l].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].dv);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
-  auto cycle = [&]() { return od ? vcycle<true>(lv, L, 0, S, st) : vcycle<false>(lv, L, 0, S, st); };
-  // z = M r, rz = r . z, p = z
-  int rc = cycle();
+  // z = M r, rz[cur] += r . z
+  auto cycle = [&](int cur) {
+    return od ? vcycle<true>(lv, L, 0, S, r, scal + (size_t)cur * S, st) : vcycle<false>(lv, L, 0, S, r, scal + (size_t)cur * S, st);
+  };
+  const float* z = lv[0].u2;
+  int rc = cycle(0);
   if (rc) return rc;
-  cg_rz_kernel<<<g0, kMgThreads, 0, st>>>(nf, r, lv[0].u, rz);
-  cg_direction_kernel<<<g0, kMgThreads, 0, st>>>(nf, lv[0].u, rz, rz_old, done, 1, p);
-  STOMSFEM_TRY_CUDA(cudaGetLastError());
   double worst = 1.0;
-  int it = 0;
+  // the next iteration whose residual the host reads: the fourth, then where
+  // the reduction so far predicts the end, within four iterations
+  int it = 0, check = 4;
   for (it = 1; it <= max_iters; ++it) {
-    STOMSFEM_TRY_CUDA(cudaMemsetAsync(pAp, 0, sizeof(double) * S, st));
-    STOMSFEM_TRY_CUDA(cudaMemsetAsync(rr, 0, sizeof(double) * S, st));
-    cg_matvec_kernel<<<g0, kMgThreads, 0, st>>>(nf, st64, p, Ap, pAp);
-    cg_alpha_kernel<<<(S + 127) / 128, 128, 0, st>>>(S, rz, pAp, done, alpha);
-    cg_update_kernel<<<g0, kMgThreads, 0, st>>>(nf, alpha, p, Ap, u, r, lv[0].f, rr);
+    const int cur = (it - 1) & 1;  // slot of this iteration's scalars
+    cg_direction_kernel<<<g0, kMgThreads, 0, st>>>(nf, z, sc, cur, it == 1, p);
+    cg_matvec_kernel<<<g0, kMgThreads, 0, st>>>(nf, st64, sc, cur, p, Ap);
+    cg_update_kernel<<<g0, kMgThreads, 0, st>>>(nf, sc, cur, p, Ap, u, r, lv[0].f);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
-    if (it % 4 == 0 || it == max_iters) {
+    if (it == check || it == max_iters) {
       STOMSFEM_TRY_CUDA(cudaMemcpyAsync(hr.data(), rr, sizeof(double) * S, cudaMemcpyDeviceToHost, st));
       STOMSFEM_TRY_CUDA(cudaStreamSynchronize(st));
       worst = 0.0;
@@ -832,15 +1055,12 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
       if (!finite)
         return set_error(STOMSFEM_ENOTSPD, "fine FEM CG: non-finite residual after %d iterations", it);
       if (all) break;
-      STOMSFEM_TRY_CUDA(cudaMemcpyAsync(done, hd.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, st));
+      const double rate = std::log(worst) / it, left = rate < 0.0 ? (std::log(rtol) - std::log(worst)) / rate : 4.0;
+      check = it + (left < 4.0 ? std::max(1, (int)left) : 4);
+      STOMSFEM_TRY_CUDA(cudaMemcpyAsync(sc.done, hd.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, st));
     }
-    rc = cycle();
+    rc = cycle(cur ^ 1);
     if (rc) return rc;
-    STOMSFEM_TRY_CUDA(cudaMemcpyAsync(rz_old, rz, sizeof(double) * S, cudaMemcpyDeviceToDevice, st));
-    STOMSFEM_TRY_CUDA(cudaMemsetAsync(rz, 0, sizeof(double) * S, st));
-    cg_rz_kernel<<<g0, kMgThreads, 0, st>>>(nf, r, lv[0].u, rz);
-    cg_direction_kernel<<<g0, kMgThreads, 0, st>>>(nf, lv[0].u, rz, rz_old, done, 0, p);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
   }
   if (res) *res = worst;
   if (iters) *iters = it > max_iters ? max_iters : it;
