@@ -158,6 +158,13 @@ __device__ __forceinline__ bool pivot_ok(double a) {
   return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
+// v - (a b + c d).  FP64: two operations of the narrow pipe (the expression
+// as written takes three); FP32: as written.
+__device__ __forceinline__ float sub2(float v, float a, float b, float c, float d) { return v - (a * b + c * d); }
+__device__ __forceinline__ double sub2(double v, double a, double b, double c, double d) {
+  return fma(-c, d, fma(-a, b, v));
+}
+
 template <int G, typename T>
 __device__ __forceinline__ T gshfl(T v, int src) {
   return __shfl_sync(0xffffffffu, v, src, G);
@@ -378,7 +385,7 @@ __device__ __forceinline__ void panel_pair(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T
       const T l0 = b0 ? pr[q][J] * i0 : T(0);
       const T l1 = b1 ? (pr[q][J1] - l0 * l10) * i1 : T(0);
 #pragma unroll
-      for (int c = 0; c < NR; ++c) rh[q][c] -= l0 * y0[c] + l1 * y1[c];
+      for (int c = 0; c < NR; ++c) rh[q][c] = sub2(rh[q][c], l0, y0[c], l1, y1[c]);
       pr[q][J] = l0;
       pr[q][J1] = l1;
       if (q == 0) {
@@ -409,7 +416,7 @@ __device__ __forceinline__ void panel_pair(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T
 #pragma unroll
       for (int p = J1 + 1; p < NB; ++p) {
 #pragma unroll
-        for (int q = 0; q < RPL; ++q) pr[q][p] -= l0q[q] * L0[p] + l1q[q] * L1[p];
+        for (int q = 0; q < RPL; ++q) pr[q][p] = sub2(pr[q][p], l0q[q], L0[p], l1q[q], L1[p]);
       }
     }
     panel_pair<J + 2, G, T, NR, RPL, NB>(pr, rh, lb, gl, K, fail);
@@ -921,7 +928,7 @@ __device__ void blk_backward(int n, int b, int bmax, const BlkSmem<T>& s, const 
         if (gl < p - 1) {
           const T l1 = tb[p * NB + gl], l0 = tb[(p - 1) * NB + gl];
 #pragma unroll
-          for (int c = 0; c < NR; ++c) yv[c] -= l1 * x1[c] + l0 * x0[c];
+          for (int c = 0; c < NR; ++c) yv[c] = sub2(yv[c], l1, x1[c], l0, x0[c]);
         }
         if (gl == p) {
 #pragma unroll
