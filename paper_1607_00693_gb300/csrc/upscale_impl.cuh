@@ -426,7 +426,12 @@ struct UpscaleTuning {
   int blocks_per_sm = 0;  // 0: as many as fit
   int split_fp32 = 1;     // FP32 form: separate forward-only launch for the cells without oversampling
   int engine = 0;         // FP32 forms: factorisation engine (kEngine*; 0 = the default for the patch size)
-  int order = 0;          // STOMSFEM_ORDER_*: unit order of the persistent launches
+  // STOMSFEM_ORDER_*: unit order of the persistent launches; negative: by
+  // patch size where the lists fit (a warp then ends on small patches, and
+  // those in flight are of one size).  1024^2, oversampling 0..4, cell against
+  // patch order: FP64, 4 samples, 23.1 -> 18.8 ms; FP32 + refinement, 8, 12.2
+  // -> 10.2; FP32, 32, 8.5 -> 8.0.
+  int order = -1;
 };
 
 // Upscale launch modes: 0 every unit (back-substitution route), 1 the
@@ -436,43 +441,78 @@ struct UpscaleTuning {
 // doubled and cost more than the forward-only route saved.
 enum { kModeAll = 0, kModeFwd = 1, kModeRest = 2 };
 
-// Cell lists of the launches (one warp, ballot compaction): list0 the
-// cells without oversampling, list1 the others (cells with an oversampling
+// Cell lists of the launches (one block, counting sort): list0 the cells
+// without oversampling, list1 the others (cells with an oversampling
 // outside [0, max_o] included: the kernel flags them), listall every cell;
 // counts = {|list0|, |list1|, |listall|}.  sorted = 0: ascending cell index
 // (listall unused); sorted = 1: by patch size, largest first (decreasing
 // oversampling, the flagged cells last), ascending cell index within one
 // size, so that a launch that walks its list with the samples fastest
-// takes the longest units first.
-static __global__ void upscale_cell_lists_kernel(const int8_t* __restrict__ oversample, int ncell, int max_o,
-                                          int sorted, int32_t* __restrict__ list0, int32_t* __restrict__ list1,
-                                          int32_t* __restrict__ listall, int32_t* __restrict__ counts) {
-  const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  int n0 = 0, n1 = 0, na = 0;
-  // pass k: sorted, k = max_o .. 0 the cells of oversampling k, then k = -1
-  // the flagged ones; unsorted, one pass (k = -2) over all cells
-  for (int k = sorted ? max_o : -2; k >= (sorted ? -1 : -2); --k) {
-    for (int c0 = 0; c0 < ncell; c0 += 32) {
-      const int c = c0 + lane;
-      const bool valid = c < ncell;
-      const int v = valid ? (int)oversample[c] : 0;
-      const bool take = valid && (k == -2 || (k >= 0 ? v == k : (v < 0 || v > max_o)));
-      const bool z = take && v == 0;
-      const unsigned m0 = __ballot_sync(0xffffffffu, z), m1 = __ballot_sync(0xffffffffu, take && !z);
-      const unsigned ma = __ballot_sync(0xffffffffu, take);
-      if (z) list0[n0 + __popc(m0 & below)] = c;
-      if (take && !z) list1[n1 + __popc(m1 & below)] = c;
-      if (sorted && take) listall[na + __popc(ma & below)] = c;
-      n0 += __popc(m0);
-      n1 += __popc(m1);
-      na += __popc(ma);
+// takes the longest units first.  (One warp took a pass over the cells per
+// size: 10 us unsorted, 50 us sorted for 32^2 cells.)
+constexpr int kListThreads = 1024;
+constexpr int kListKeys = kMaxBand / 2 + 2;  // oversampling 0 .. kMaxBand / 2, and the flagged cells
+static __global__ void __launch_bounds__(kListThreads)
+upscale_cell_lists_kernel(const int8_t* __restrict__ oversample, int ncell, int max_o, int sorted,
+                          int32_t* __restrict__ list0, int32_t* __restrict__ list1, int32_t* __restrict__ listall,
+                          int32_t* __restrict__ counts) {
+  __shared__ int base[kListKeys], warp_n[kListThreads / 32][kListKeys], total[kListKeys];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // key 0: without oversampling; unsorted, 1: the others; sorted, o: that
+  // oversampling, kListKeys - 1: flagged
+  auto key_of = [&](int c) {
+    const int v = (int)oversample[c];
+    if (v == 0) return 0;
+    if (!sorted) return 1;
+    return v < 0 || v > max_o ? kListKeys - 1 : min(v, kListKeys - 2);  // (patches clipped to a small grid)
+  };
+  if (tid < kListKeys) total[tid] = 0;
+  __syncthreads();
+  for (int c = tid; c < ncell; c += kListThreads) atomicAdd(&total[key_of(c)], 1);
+  __syncthreads();
+  if (tid == 0) {
+    // starts: list0 (key 0) on its own; list1 by decreasing key, the flagged last
+    int n1 = 0;
+    for (int k = kListKeys - 2; k >= 1; --k) {
+      base[k] = n1;
+      n1 += total[k];
     }
+    base[kListKeys - 1] = n1;
+    base[0] = 0;
+    counts[0] = total[0];
+    counts[1] = n1 + total[kListKeys - 1];
+    counts[2] = sorted ? ncell : 0;
   }
-  if (lane == 0) {
-    counts[0] = n0;
-    counts[1] = n1;
-    counts[2] = na;
+  __syncthreads();
+  const int n0 = total[0], flagged0 = base[kListKeys - 1];
+  __syncthreads();
+  for (int c0 = 0; c0 < ncell; c0 += kListThreads) {
+    const int c = c0 + tid;
+    const bool valid = c < ncell;
+    const int k = valid ? key_of(c) : -1;
+    for (int q = tid; q < (kListThreads / 32) * kListKeys; q += kListThreads) (&warp_n[0][0])[q] = 0;
+    __syncthreads();
+    const unsigned same = __match_any_sync(0xffffffffu, k);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (valid && rank == 0) warp_n[warp][k] = __popc(same);
+    __syncthreads();
+    if (tid < kListKeys) {  // exclusive sums over the warps
+      int t = base[tid];
+      for (int w = 0; w < kListThreads / 32; ++w) {
+        const int n = warp_n[w][tid];
+        warp_n[w][tid] = t;
+        t += n;
+      }
+      base[tid] = t;
+    }
+    __syncthreads();
+    if (valid) {
+      const int pos = warp_n[warp][k] + rank;
+      (k == 0 ? list0 : list1)[pos] = c;
+      // every cell: the larger ones, then those without oversampling, then the flagged
+      if (sorted) listall[k == 0 ? flagged0 + pos : pos < flagged0 ? pos : pos + n0] = c;
+    }
+    __syncthreads();
   }
 }
 
@@ -1120,7 +1160,6 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   A.cell_list = nullptr;
   A.cell_count = nullptr;
   A.blocks_per_sm_cap = tune.blocks_per_sm;
-  A.order = tune.order;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // cell lists at the end of the workspace (the split launch, or the order
   // by patch size), when the slots of one block still fit before them
@@ -1133,7 +1172,8 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   int32_t* list1 = list0 + ncell;
   int32_t* listall = list1 + ncell;
   int32_t* counts = listall + ncell;
-  const bool sorted = tune.order == 1 && lists_fit;
+  const bool sorted = tune.order != 0 && lists_fit;
+  A.order = tune.order < 0 ? (sorted ? 1 : 0) : tune.order;
   const long long mb = lists_fit && max_blocks > slots2 / slots_per_block ? slots2 / slots_per_block : max_blocks;
   // the oscillatory data: every cell by back substitution in one launch
   // (the forward-only route never forms psi0, which the Petrov-Galerkin
@@ -1144,7 +1184,7 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
       // forward-only route in a launch of their own, the others follow
       if (!oversample) return launch_fp32<float, kModeFwd, PG, OSC>(engine, A, max_blocks, st);
       if (lists_fit) {
-        upscale_cell_lists_kernel<<<1, 32, 0, st>>>(oversample, ncell, mo, sorted ? 1 : 0, list0, list1, listall,
+        upscale_cell_lists_kernel<<<1, kListThreads, 0, st>>>(oversample, ncell, mo, sorted ? 1 : 0, list0, list1, listall,
                                                     counts);
         STOMSFEM_TRY_CUDA(cudaGetLastError());
         A.cell_list = list0;
@@ -1159,7 +1199,7 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   }
   if (sorted) {
     // one launch over every cell, largest patches first
-    upscale_cell_lists_kernel<<<1, 32, 0, st>>>(oversample, ncell, mo, 1, list0, list1, listall, counts);
+    upscale_cell_lists_kernel<<<1, kListThreads, 0, st>>>(oversample, ncell, mo, 1, list0, list1, listall, counts);
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     A.cell_list = listall;
     A.cell_count = counts + 2;
