@@ -28,9 +28,9 @@
 
 namespace stomsfem {
 
-// Warps per block: 4, except 2 for two FP64 units per warp (whose 36 KB of
-// shared memory per warp then fit three blocks on an SM).
-__host__ __device__ constexpr int upscale_warps(bool fp64, int G) { return fp64 && G == 16 ? 2 : 4; }
+// Warps per block: 4, except 2 for two or four FP64 units per warp (two: the
+// 36 KB of shared memory per warp then fit three blocks on an SM).
+__host__ __device__ constexpr int upscale_warps(bool fp64, int G) { return fp64 && G <= 16 ? 2 : 4; }
 constexpr int kMaxBand = 64;       // half bandwidth limit (mx + 1)
 
 struct UnitGeom {
@@ -542,7 +542,7 @@ __device__ inline BlkSmem<TK> unit_blk(unsigned char* base, const TcSmem& tsm, i
 // list).  G = 16: a warp takes one cell of two consecutive samples, whose
 // patches have the same shape, so its two halves run the same loop bounds
 // in lockstep (an odd last sample is mirrored by the idle half, which
-// writes nothing).
+// writes nothing).  G = 8 (FP64, small bands): the same with four samples.
 // OSC: the oscillatory boundary data of the cell problems (PatchGenOsc).
 // TC > 0 (FP32 factor, G = 32): the factorisation of band_tc.cuh (window
 // in mma accumulator registers, trailing update on the tensor cores with
@@ -550,7 +550,7 @@ __device__ inline BlkSmem<TK> unit_blk(unsigned char* base, const TcSmem& tsm, i
 // substitutions read its 8-column blocks.
 template <typename TK, typename TA, int RPL, int G, int MODE, bool PG, bool OSC = false, int TC = 0>
 __global__ void __launch_bounds__(upscale_warps(sizeof(TK) == 8, G) * 32,
-                                  sizeof(TK) == 4 ? (G == 16 ? 3 : 4) : (G == 16 ? 3 : 2))
+                                  sizeof(TK) == 4 ? (G == 16 ? 3 : 4) : (G == 8 ? 6 : G == 16 ? 3 : 2))
 upscale_kernel(UpscaleArgs A) {
   // the oscillatory data run every cell by back substitution (one launch)
   static_assert(!OSC || MODE == kModeAll, "oscillatory data: back-substitution route only");
@@ -579,30 +579,29 @@ upscale_kernel(UpscaleArgs A) {
 
   // cells of this launch (MODE 1, 2: a device list, or all cells when none)
   const int nlc = A.cell_list ? A.cell_count[0] : ncell;
-  // work items: (sample, cell) for G = 32, (pair of samples, cell) for G = 16;
-  // with a unit list, one entry (G = 32) or two consecutive entries (G = 16:
-  // the list holds cells without oversampling only, all of one patch shape,
-  // so the two halves of a warp run in lockstep)
-  const long long npair = G == 32 ? (long long)A.S : (long long)((A.S + 1) / 2);
+  // work items: (GPW consecutive samples, cell); with a unit list, GPW
+  // consecutive entries (the list holds cells without oversampling only, all
+  // of one patch shape, so the groups of a warp run in lockstep)
+  const long long npair = ((long long)A.S + GPW - 1) / GPW;
   const long long nlist = A.unit_list ? (long long)A.unit_count[0] : 0;
-  const long long nwork = A.unit_list ? (G == 32 ? nlist : (nlist + 1) / 2) : npair * nlc;
+  const long long nwork = A.unit_list ? (nlist + GPW - 1) / GPW : npair * nlc;
   for (long long w = gw; w < nwork; w += nw) {
     long long u;
-    bool dup = false;  // this half mirrors the other half's unit
+    bool dup = false;  // this group mirrors another group's unit
     const int ci = A.order ? (int)(w / npair) : (int)(w % nlc);
     const long long pw = A.order ? w % npair : w / nlc;
     const int cell_w = A.cell_list ? A.cell_list[ci] : ci;
     if (G == 32) {
       u = A.unit_list ? (long long)A.unit_list[w] : pw * ncell + cell_w;
     } else if (A.unit_list) {
-      long long li = 2 * w + grp;
+      long long li = GPW * w + grp;
       if (li >= nlist) {
         li = nlist - 1;
         dup = true;
       }
       u = (long long)A.unit_list[li];
     } else {
-      int sp = 2 * (int)pw + grp;
+      int sp = GPW * (int)pw + grp;
       if (sp >= A.S) {
         sp = A.S - 1;
         dup = true;
@@ -1021,10 +1020,13 @@ static int launch_upscale(const UpscaleArgs& A, long long max_blocks, cudaStream
 
 template <typename TK, typename TA, int G, int MODE = kModeAll, bool PG = false, bool OSC = false>
 static int launch_rpl(const UpscaleArgs& A, long long max_blocks, cudaStream_t st) {
-  const int rpl = (G / 2 + A.bmax + G - 1) / G;  // <= 3 (G = 32) or 5 (G = 16) for bmax <= 64
+  // <= 3 (G = 32), 5 (G = 16) for bmax <= 64, 2 (G = 8) for bmax <= kQuadBand
+  const int rpl = (G / 2 + A.bmax + G - 1) / G;
   if (rpl <= 1) return launch_upscale<TK, TA, 1, G, MODE, PG, OSC>(A, max_blocks, st);
   if (rpl == 2) return launch_upscale<TK, TA, 2, G, MODE, PG, OSC>(A, max_blocks, st);
-  if (rpl == 3) return launch_upscale<TK, TA, 3, G, MODE, PG, OSC>(A, max_blocks, st);
+  if constexpr (G > 8) {
+    if (rpl == 3) return launch_upscale<TK, TA, 3, G, MODE, PG, OSC>(A, max_blocks, st);
+  }
   if constexpr (G == 16) {
     if (rpl == 4) return launch_upscale<TK, TA, 4, G, MODE, PG, OSC>(A, max_blocks, st);
     return launch_upscale<TK, TA, 5, G, MODE, PG, OSC>(A, max_blocks, st);
@@ -1036,8 +1038,15 @@ static int launch_rpl(const UpscaleArgs& A, long long max_blocks, cudaStream_t s
 // FP32 launch.
 static size_t cell_list_bytes(const stomsfem_grid* g) { return round256(sizeof(int32_t) * (3 * (size_t)g->nc * g->nc + 4)); }
 
-// Lanes per unit of each form: two units per warp.
-constexpr int group_lanes(int) { return 16; }
+// FP64: four units per warp (8 lanes each, column blocks of 4) up to this half
+// bandwidth, two beyond.  A small patch leaves most of 16 lanes without
+// entries, and the pivots and substitutions, whose FP64 instructions cost the
+// same however many lanes they serve, then serve four units: about 790 against
+// 1,125 warp instructions of the FP64 pipe a unit at b = 8.  From b = 13 the
+// panel takes three rows a lane and the update's rounds fill 16 lanes.
+// 64 samples of the 64^2 / 8^2 grid, whole step: 401 ->
+// 312 us.
+constexpr int kQuadBand = 12;
 
 // Factorisation engines of the FP32 forms: the two-units-per-warp FMA
 // factorisation of band_block.cuh in column blocks of 8 (any bandwidth),
@@ -1122,14 +1131,18 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   const long long units = (long long)S * grid->nc * grid->nc;
   const long long slots = (long long)(workspace_bytes / sb);
   const int engine = upscale_engine(tune.engine, precision, grid->nf / grid->nc, bmax);
-  const int G = upscale_engine_lanes(engine);
+  int G = upscale_engine_lanes(engine);
   const int WPB = upscale_warps(precision == STOMSFEM_FP64, G);
+  // four FP64 units per warp: where the workspace holds a block of them and
+  // three samples at least share a warp
+  if (precision == STOMSFEM_FP64 && bmax <= kQuadBand && S >= 3 && slots >= WPB * 4) G = 8;
   const int slots_per_block = WPB * (32 / G);
   if (slots < slots_per_block)
     return set_error(STOMSFEM_ENOMEM, "workspace %zu bytes < %d slots of %zu bytes", workspace_bytes,
                      slots_per_block, sb);
   long long max_blocks = slots / slots_per_block;
-  const long long items = G == 32 ? units : (long long)((S + 1) / 2) * grid->nc * grid->nc;
+  const int GPW = 32 / G;
+  const long long items = ((long long)S + GPW - 1) / GPW * grid->nc * grid->nc;
   const long long need = (items + WPB - 1) / WPB;
   if (max_blocks > need) max_blocks = need;
 
@@ -1206,7 +1219,8 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
     max_blocks = mb;
   }
   if (precision == STOMSFEM_FP64)
-    return launch_rpl<double, double, group_lanes(STOMSFEM_FP64), kModeAll, PG, OSC>(A, max_blocks, st);
+    return G == 8 ? launch_rpl<double, double, 8, kModeAll, PG, OSC>(A, max_blocks, st)
+                  : launch_rpl<double, double, 16, kModeAll, PG, OSC>(A, max_blocks, st);
   if (precision == STOMSFEM_FP32_REFINED) return launch_fp32<double, kModeAll, PG, OSC>(engine, A, max_blocks, st);
   return launch_fp32<float, kModeAll, PG, OSC>(engine, A, max_blocks, st);
 }
