@@ -88,6 +88,37 @@ __device__ __forceinline__ uint64_t f2_both(float a) {
   return b | (b << 32);
 }
 
+// FP32 <-> FP64 on the integer units: the conversion instructions run on the
+// FP64 pipe (two of its slots each), which bounds the kernels that use these.
+// The exact values; subnormal and other rare arguments take the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), e = b & 0x7f800000u;
+  if ((e == 0 && (b << 1)) || e == 0x7f800000u) {
+    double d;  // (volatile: not computed ahead of the test)
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(v));
+    return d;
+  }
+  const unsigned hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double v) {
+  // 32-bit operations only: 64-bit additions run on the FP64 pipe as well
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
+  if (((hi << 1) | lo) == 0) return __uint_as_float(sign);
+  if (e - 897u > 1150u - 897u) {
+    float f;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(v));
+    return f;
+  }
+  // exponent rebased by 896, 23 mantissa bits, then round to nearest even
+  // (a carry runs into the exponent, to infinity at the end of the range)
+  const unsigned m = (__funnelshift_l(lo, hi, 3) + 0x40000000u) & 0x7fffffffu;
+  const unsigned rest = lo & 0x1fffffffu;
+  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float(sign | (m + up));
+}
+
 // Full-warp sum (every lane receives the total).
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

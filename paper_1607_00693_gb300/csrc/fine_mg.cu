@@ -9,7 +9,7 @@
 // when the batch's coefficient contrast exceeds kMgOdContrast, with the
 // other fine nodes' weights from the fine stencil (mgf_interp_kernel);
 // restriction P^T, Galerkin coarse operators A_{l+1} = P^T A_l P (9-point
-// stencils again), damped Jacobi smoothing (omega = 0.8, two sweeps before
+// stencils again), damped Jacobi smoothing (two sweeps before
 // and after the coarse correction: a symmetric V-cycle, so the
 // preconditioner is symmetric positive definite and plain CG applies), and
 // 60 Jacobi sweeps on the coarsest grid.  Stencils are stored per level and
@@ -38,15 +38,21 @@ constexpr int kMgMaxLevels = 12;
 // Damping of the two sweeps before and after the coarse correction.  On the
 // bilinear levels the high-frequency eigenvalues of D^-1 A lie in [0.75, 1.5]
 // (Q1 stencil, constant coefficient): the two sweeps are the Chebyshev pair
-// of that interval (largest factor 1/17; 0.16 with 0.8 twice; one CG
-// iteration fewer on the lognormal media).  The operator-dependent levels
-// keep 0.8 (see mgf_divisor_kernel), as does the coarsest grid.
+// of [0.8, 1.6] (largest factor on the former 0.09; 0.16 with 0.8 twice),
+// which converges for eigenvalues below 2.4.  The operator-dependent levels
+// keep 0.8 (see mgf_divisor_kernel).
 constexpr float kMgOmega = 0.8f;
 template <bool OD>
 __device__ __forceinline__ float mg_omega(int sweep) {
-  return OD ? kMgOmega : (sweep == 0 ? 1.1631f : 0.71932f);
+  return OD ? kMgOmega : (sweep == 0 ? 1.0903f : 0.6744f);
 }
-constexpr int kMgCoarseSweeps = 60;
+// The coarsest grid (at most 16 elements per side): Chebyshev iteration in
+// D^-1 A on [0.02, 2.5] (the smoothest mode of a 16^2 grid has 0.029, and the
+// sweeps converge up to 2.5): 24 steps leave at most 0.03 of any mode in the
+// interval, where 60 Jacobi sweeps left 0.25 of the smoothest.
+constexpr int kMgCoarseSteps = 24;
+constexpr float kMgCoarseLo = 0.02f, kMgCoarseHi = 2.5f;
+constexpr int kMgSmall = 32;  // a level of at most this many elements per side and the one below run in one kernel
 constexpr int kMgThreads = 256;
 // Coefficient contrast (max a / min a over the batch) above which the
 // transfers between levels use the operator-dependent prolongation; below
@@ -58,36 +64,36 @@ constexpr double kMgOdContrast = 1e3;
 struct MgLevel {
   int nf;          // elements per side
   int N;           // (nf + 1)^2 nodes
-  float* st;       // [S][5][N]: centre, east, north, north-east, north-west
+  float* st;       // [S][st_stride(N)]: (centre, east, north, north-east)[N], north-west[N]
   float* u;        // [S][N]
   float* u2;       // [S][N] (Jacobi ping-pong)
   float* f;        // [S][N]
-  float* r;        // [S][N], not used (the residuals stay on chip)
   float* P;        // [S][4][N]: prolongation weights from the next coarser level (per node type)
   float* dv;       // [S][N]: Jacobi divisor (see mgf_divisor_kernel)
 };
 
 __device__ __forceinline__ bool interior(int i, int j, int nf) { return i > 0 && j > 0 && i < nf && j < nf; }
 
-// Stencils of every level in symmetric form: st[m][node] for m = 0..4 the
-// centre, east, north, north-east and north-west couplings of the node; the
-// west, south, south-west and south-east couplings are the east, north,
-// north-east and north-west ones of the neighbour there (zero at the
-// boundary nodes, whose values stay zero in every multigrid vector).
+// Stencils of every level in symmetric form: couplings m = 0..4 of a node
+// are its centre, east, north, north-east and north-west ones; the west,
+// south, south-west and south-east couplings are the east, north, north-east
+// and north-west ones of the neighbour there (zero at the boundary nodes,
+// whose values stay zero in every multigrid vector).  The first four lie
+// side by side (one 16-byte load), the north-west ones follow.
+__host__ __device__ __forceinline__ size_t st_stride(size_t N) { return (5 * N + 3) & ~size_t(3); }
+__device__ __forceinline__ size_t st_at(int m, size_t N, long v) {
+  return m < 4 ? 4 * (size_t)v + m : 4 * N + (size_t)v;
+}
 // Entry k = (dj + 1) * 3 + (di + 1) of the 9-point stencil of node v:
-__device__ __forceinline__ int st_arr(int k) {  // array m holding entry k
+__device__ __forceinline__ int st_arr(int k) {  // coupling m holding entry k
   return k == 4 ? 0 : (k == 5 || k == 3) ? 1 : (k == 7 || k == 1) ? 2 : (k == 8 || k == 0) ? 3 : 4;
 }
-__device__ __forceinline__ long st_node(int k, long v, int W) {  // node whose array holds it
+__device__ __forceinline__ long st_node(int k, long v, int W) {  // node whose coupling it is
   const int di = k % 3 - 1, dj = k / 3 - 1;
   return (dj < 0 || (dj == 0 && di < 0)) ? v + dj * W + di : v;
 }
-template <int K>
-__device__ __forceinline__ float st9(const float* __restrict__ st, size_t N, long v, int W) {
-  constexpr int di = K % 3 - 1, dj = K / 3 - 1;
-  constexpr int m = K == 4 ? 0 : (K == 5 || K == 3) ? 1 : (K == 7 || K == 1) ? 2 : (K == 8 || K == 0) ? 3 : 4;
-  constexpr bool own = !(dj < 0 || (dj == 0 && di < 0));
-  return st[(size_t)m * N + (own ? v : v + dj * W + di)];
+__device__ __forceinline__ float st_entry(const float* __restrict__ st, size_t N, int k, long v, int W) {
+  return st[st_at(st_arr(k), N, st_node(k, v, W))];
 }
 
 // Level-0 stencil from a, FP32 for the preconditioner (symmetric form
@@ -99,40 +105,28 @@ __device__ __forceinline__ float st9(const float* __restrict__ st, size_t N, lon
 __global__ void mgf_fine_stencil_kernel(int nf, const double* __restrict__ a, float* __restrict__ st,
                                         double* __restrict__ st64) {
   const int s = blockIdx.y;
-  const int N = (nf + 1) * (nf + 1);
+  const int W = nf + 1, N = W * W;
   const double* as = a + (size_t)s * nf * nf;
-  float* ss = st + (size_t)s * 5 * N;
+  float* ss = st + (size_t)s * st_stride(N);
   double* s64 = st64 + (size_t)s * 5 * N;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
-    const int i = v % (nf + 1), j = v / (nf + 1);
-    float c[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    const int i = v % W, j = v / W;
     double d[5] = {0, 0, 0, 0, 0};
     if (interior(i, j, nf)) {
-      const double aSW = as[(size_t)(j - 1) * nf + i - 1], aSE = as[(size_t)(j - 1) * nf + i];
-      const double aNE = as[(size_t)j * nf + i], aNW = as[(size_t)j * nf + i - 1];
+      const double* p = as + (size_t)(j - 1) * nf + i - 1;
+      const double aSW = p[0], aSE = p[1], aNE = p[nf + 1], aNW = p[nf];
       // products with 1/6 and 1/3, not quotients: an FP64 division is a
       // long instruction sequence on the FP64 pipe
       constexpr double k6 = 1.0 / 6.0, k3 = 1.0 / 3.0;
-      d[0] = (4.0 * k6) * (aSW + aSE + aNE + aNW);
+      const double north = aNW + aNE;
+      d[0] = (4.0 * k6) * ((aSW + aSE) + north);
       d[1] = -(aSE + aNE) * k6;
-      d[2] = -(aNW + aNE) * k6;
+      d[2] = -north * k6;
       d[3] = -aNE * k3;
       d[4] = -aNW * k3;
-      c[4] = (float)((4.0 * k6) * (aSW + aSE + aNE + aNW));
-      c[3] = (float)(-(aSW + aNW) * k6);  // west
-      c[5] = (float)(-(aSE + aNE) * k6);  // east
-      c[1] = (float)(-(aSW + aSE) * k6);  // south
-      c[7] = (float)(-(aNW + aNE) * k6);  // north
-      c[0] = (float)(-aSW * k3);
-      c[2] = (float)(-aSE * k3);
-      c[8] = (float)(-aNE * k3);
-      c[6] = (float)(-aNW * k3);
     }
-    ss[v] = c[4];
-    ss[(size_t)N + v] = c[5];
-    ss[(size_t)2 * N + v] = c[7];
-    ss[(size_t)3 * N + v] = c[8];
-    ss[(size_t)4 * N + v] = c[6];
+    *reinterpret_cast<float4*>(ss + 4 * (size_t)v) = make_float4(narrow(d[0]), narrow(d[1]), narrow(d[2]), narrow(d[3]));
+    ss[4 * (size_t)N + v] = narrow(d[4]);
 #pragma unroll
     for (int k = 0; k < 5; ++k) s64[(size_t)k * N + v] = d[k];
   }
@@ -140,15 +134,8 @@ __global__ void mgf_fine_stencil_kernel(int nf, const double* __restrict__ a, fl
 
 // The 9-point stencil of interior node v (entries k = (dj + 1) * 3 + di + 1).
 __device__ __forceinline__ void stencil9(const float* __restrict__ st, size_t N, long v, int W, float a[9]) {
-  a[0] = st9<0>(st, N, v, W);
-  a[1] = st9<1>(st, N, v, W);
-  a[2] = st9<2>(st, N, v, W);
-  a[3] = st9<3>(st, N, v, W);
-  a[4] = st9<4>(st, N, v, W);
-  a[5] = st9<5>(st, N, v, W);
-  a[6] = st9<6>(st, N, v, W);
-  a[7] = st9<7>(st, N, v, W);
-  a[8] = st9<8>(st, N, v, W);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a[k] = st_entry(st, N, k, v, W);
 }
 
 // The Jacobi divisor of a node from its nine entries (mgf_divisor_kernel).
@@ -191,7 +178,7 @@ __global__ void mgf_interp_kernel(int nff, const float* __restrict__ stf, float*
   const int s = blockIdx.y;
   const int W = nff + 1;
   const size_t N = (size_t)W * W;
-  const float* sf = stf + (size_t)s * 5 * N;
+  const float* sf = stf + (size_t)s * st_stride(N);
   float* ps = P + (size_t)s * 4 * N;
   for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < (long)N; v += (long)gridDim.x * blockDim.x) {
     const int x = (int)(v % W), y = (int)(v / W);
@@ -246,14 +233,14 @@ __device__ __forceinline__ float pweight(const float* __restrict__ ps, size_t N,
 // nine fine nodes of the coarse node's hat, their nine couplings, and the
 // coarse nodes whose hats cover the coupled fine node; only the five stored
 // couplings are formed.
-// 1024^2, 8 samples, all levels: 508 -> 90 us.
+// 1024^2, 8 samples, all levels: 508 -> 165 us.
 __global__ void __launch_bounds__(kMgThreads) mgf_rap_bilinear_kernel(int nff, const float* __restrict__ stf,
                                                                       float* __restrict__ stc) {
   const int s = blockIdx.y;
   const int nfc = nff / 2, Wf = nff + 1, Wc = nfc + 1;
   const size_t Nf = (size_t)Wf * Wf, Nc = (size_t)Wc * Wc;
-  const float* sf = stf + (size_t)s * 5 * Nf;
-  float* sc = stc + (size_t)s * 5 * Nc;
+  const float* sf = stf + (size_t)s * st_stride(Nf);
+  float* sc = stc + (size_t)s * st_stride(Nc);
   // (I, J) offsets of the stored couplings: centre, east, north, north-east, north-west
   constexpr int cI[5] = {0, 1, 0, 1, -1}, cJ[5] = {0, 0, 1, 1, 1};
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < (int)Nc; v += gridDim.x * blockDim.x) {
@@ -271,7 +258,7 @@ __global__ void __launch_bounds__(kMgThreads) mgf_rap_bilinear_kernel(int nff, c
 #pragma unroll
             for (int ei = -1; ei <= 1; ++ei) {
               const int k = (ej + 1) * 3 + ei + 1;
-              const float afv = sf[(size_t)st_arr(k) * Nf + st_node(k, fv, Wf)];
+              const float afv = st_entry(sf, Nf, k, fv, Wf);
 #pragma unroll
               for (int m = 0; m < 5; ++m) {
                 const int tx = di + ei - 2 * cI[m], ty = dj + ej - 2 * cJ[m];
@@ -286,7 +273,7 @@ __global__ void __launch_bounds__(kMgThreads) mgf_rap_bilinear_kernel(int nff, c
         if (!interior(I + cI[m], J + cJ[m], nfc)) out[m] = 0.f;
     }
 #pragma unroll
-    for (int m = 0; m < 5; ++m) sc[(size_t)m * Nc + v] = out[m];
+    for (int m = 0; m < 5; ++m) sc[st_at(m, Nc, v)] = out[m];
   }
 }
 
@@ -297,9 +284,9 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
   const int nfc = nff / 2;
   const int Wf = nff + 1;
   const int Nf = Wf * Wf, Nc = (nfc + 1) * (nfc + 1);
-  const float* sf = stf + (size_t)s * 5 * Nf;
+  const float* sf = stf + (size_t)s * st_stride(Nf);
   const float* ps = P + (size_t)s * 4 * Nf;
-  float* sc = stc + (size_t)s * 5 * Nc;
+  float* sc = stc + (size_t)s * st_stride(Nc);
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < Nc; v += gridDim.x * blockDim.x) {
     const int I = v % (nfc + 1), J = v / (nfc + 1);
     float out[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -313,7 +300,7 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
           for (int ej = -1; ej <= 1; ++ej)
             for (int ei = -1; ei <= 1; ++ei) {
               const int k = (ej + 1) * 3 + ei + 1;
-              const float afv = sf[(size_t)st_arr(k) * Nf + st_node(k, fv, Wf)];
+              const float afv = st_entry(sf, Nf, k, fv, Wf);
               if (afv == 0.f) continue;
               const int gx = fx + ei, gy = fy + ej;  // neighbour fine node
               // the coarse nodes whose prolongation covers (gx, gy): one,
@@ -344,11 +331,11 @@ __global__ void mgf_rap_kernel(int nff, const float* __restrict__ stf, const flo
             }
         }
     }
-    sc[v] = out[4];
-    sc[(size_t)Nc + v] = out[5];
-    sc[(size_t)2 * Nc + v] = out[7];
-    sc[(size_t)3 * Nc + v] = out[8];
-    sc[(size_t)4 * Nc + v] = out[6];
+    sc[st_at(0, Nc, v)] = out[4];
+    sc[st_at(1, Nc, v)] = out[5];
+    sc[st_at(2, Nc, v)] = out[7];
+    sc[st_at(3, Nc, v)] = out[8];
+    sc[st_at(4, Nc, v)] = out[6];
   }
 }
 
@@ -363,7 +350,7 @@ __global__ void mgf_divisor_kernel(int nf, const float* __restrict__ st, float* 
   const int s = blockIdx.y;
   const int W = nf + 1;
   const size_t N = (size_t)W * W;
-  const float* ss = st + (size_t)s * 5 * N;
+  const float* ss = st + (size_t)s * st_stride(N);
   for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < (long)N; v += (long)gridDim.x * blockDim.x) {
     float d = 1.f;
     if (interior((int)(v % W), (int)(v / W), nf)) {
@@ -373,66 +360,6 @@ __global__ void mgf_divisor_kernel(int nf, const float* __restrict__ st, float* 
     }
     dv[(size_t)s * N + v] = d;
   }
-}
-
-// The coarsest grid (nf <= 16: at most 289 nodes): all kMgCoarseSweeps
-// damped Jacobi sweeps from zero in one launch, one CTA per sample, the
-// iterates in shared memory; each sweep is mgf_jacobi_kernel's arithmetic.
-constexpr int kMgCoarseMaxNodes = 289;
-constexpr int kMgCoarseThreads = 320;
-
-__global__ void __launch_bounds__(kMgCoarseThreads) mgf_coarse_kernel(int nf, const float* __restrict__ st,
-                                                                      const float* __restrict__ dv,
-                                                                      const float* __restrict__ f,
-                                                                      float* __restrict__ u) {
-  __shared__ float buf[2][kMgCoarseMaxNodes];
-  const int s = blockIdx.x;
-  const int W = nf + 1, N = W * W;
-  const int v = threadIdx.x;
-  const bool in = v < N && interior(v % W, v / W, nf);
-  float c[9], fv = 0.f;
-  const float* ss = st + (size_t)s * 5 * N;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) c[k] = in ? ss[(size_t)st_arr(k) * N + st_node(k, v, W)] : 0.f;
-  if (in) fv = f[(size_t)s * N + v];
-  const float dd = in ? dv[(size_t)s * N + v] : 1.f;
-  float o = in ? 0.f + kMgOmega * (fv - 0.f) / dd : 0.f;  // the first sweep, from zero
-  if (v < N) buf[0][v] = o;
-  __syncthreads();
-  for (int k = 1; k < kMgCoarseSweeps; ++k) {
-    const float* ui = buf[(k - 1) & 1];
-    if (in) {
-      float t = 0.f;
-#pragma unroll
-      for (int dj = -1; dj <= 1; ++dj)
-#pragma unroll
-        for (int di = -1; di <= 1; ++di) t = fmaf(c[(dj + 1) * 3 + di + 1], ui[v + dj * W + di], t);
-      o = ui[v] + kMgOmega * (fv - t) / dd;
-    }
-    if (v < N) buf[k & 1][v] = o;
-    __syncthreads();
-  }
-  if (v < N) u[(size_t)s * N + v] = o;
-}
-
-// FP32 <-> FP64 on the integer units: the conversion instructions run on the
-// FP64 pipe, which bounds the CG's kernels (two of its slots each, as much
-// as two of the nine products of the stencil).  The exact values; subnormal
-// and other rare arguments take the instruction.
-__device__ __forceinline__ double widen(float v) {
-  const unsigned b = __float_as_uint(v), e = b & 0x7f800000u;
-  if ((e == 0 && (b << 1)) || e == 0x7f800000u) return (double)v;
-  const unsigned hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-__device__ __forceinline__ float narrow(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  if (!(b << 1)) return __uint_as_float((unsigned)(b >> 32));
-  // round to nearest even at bit 29
-  const unsigned long long w = b + 0x0fffffffull + ((b >> 29) & 1);
-  const unsigned e = (unsigned)(w >> 52) & 0x7ffu;
-  if (e < 897u || e > 1150u) return (float)v;
-  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (((unsigned)(w >> 29) + 0x40000000u) & 0x7fffffffu));
 }
 
 // Block sum of v into acc[s] (one atomic per block).
@@ -467,9 +394,11 @@ __device__ __forceinline__ void block_sum_to(double v, double* acc) {
 // rows early.  In shared-memory tiles (64 x 32 nodes, the first version) the
 // same passes took 390 instructions per 32 nodes for index arithmetic and 18
 // coupling loads, and ten turns of latency per phase on the small levels.
-// 1024^2, 8 samples: the V-cycle 540 -> 290 us, the solve with the leaner CG
-// and set-up 12.02 -> 8.53 ms.
+// 1024^2, 8 samples: the whole solve, with the leaner CG and set-up, 12.0 ->
+// 6.84 ms; the finest level's passes 69 us down and 138 us up.
 constexpr int kMgWarps = 4;
+constexpr int kMgBlocks = 5;  // of the downward kernel, blocks an SM holds at least (102 registers a
+                              // thread; the upward one spills there: 196 against 138 us on the finest level)
 
 // One strip and row segment of a level for the calling warp.
 struct MgMarch {
@@ -500,21 +429,25 @@ struct MgTri {
   }
 };
 
-// The couplings of row y (own entries), zero outside the interior.
+// The couplings and right-hand side of one row; zero (centre 1) outside the
+// interior.  q: the node.
 struct MgCoef {
-  float c, e, n, ne, nw, f;  // f: the right-hand side
-  __device__ __forceinline__ void load(const float* __restrict__ st, size_t N, const float* __restrict__ fs, bool in,
-                                       size_t q) {
-    c = e = n = ne = nw = f = 0.f;
+  float c, e, n, ne, nw, f;
+  __device__ __forceinline__ void none() {
+    c = 1.f;
+    e = n = ne = nw = f = 0.f;
+  }
+  __device__ __forceinline__ void load(const float* __restrict__ st, const float* __restrict__ nws,
+                                       const float* __restrict__ fs, bool in, int q) {
+    none();
     if (in) {
-      c = st[q];
-      e = st[N + q];
-      n = st[2 * N + q];
-      ne = st[3 * N + q];
-      nw = st[4 * N + q];
+      const float4 v = reinterpret_cast<const float4*>(st)[q];
+      c = v.x;
+      e = v.y;
+      n = v.z;
+      ne = v.w;
+      nw = nws[q];
       f = fs[q];
-    } else {
-      c = 1.f;
     }
   }
 };
@@ -554,7 +487,7 @@ struct MgStencil {
 // by the divisor of mgf_divisor_kernel; with the bilinear transfers by the
 // diagonal entry, as the M-matrix levels allow.  rows: even.
 template <bool OD>
-__global__ void __launch_bounds__(kMgWarps * 32) mgf_down_kernel(int nf, int rows, const float* __restrict__ st,
+__global__ void __launch_bounds__(kMgWarps * 32, kMgBlocks) mgf_down_kernel(int nf, int rows, const float* __restrict__ st,
                                                                  const float* __restrict__ dv,
                                                                  const float* __restrict__ P,
                                                                  const float* __restrict__ f, float* __restrict__ u,
@@ -564,57 +497,68 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_down_kernel(int nf, int row
   const int s = blockIdx.y, lane = threadIdx.x & 31;
   const int W = nf + 1, nfc = nf / 2, Wc = nfc + 1;
   const size_t N = (size_t)W * W;
-  st += (size_t)s * 5 * N;
+  st += (size_t)s * st_stride(N);
   f += (size_t)s * N;
   u += (size_t)s * N;
   fc += (size_t)s * Wc * Wc;
+  const float* nws = st + 4 * N;
   const float* ds = dv + (size_t)s * N;
   const float* ps = P + (size_t)s * 4 * N;
   const bool mine = lane >= 3 && lane < 29 && m.x < W;
   auto inside = [&](int y) { return m.in && y > 0 && y < nf; };
-  auto at = [&](int y) { return (size_t)y * W + m.x; };
-  MgCoef k0, k1, k2, kn;  // rows t, t - 1, t - 2 and t + 1
-  float r0 = 0.f, r1 = 0.f;  // reciprocal divisors of rows t, t - 1
-  MgStencil sa, sb;          // rows t - 1, t - 2
-  MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};                           // sweep 1: rows t, t - 1, t - 2
-  MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};                           // sweep 2: rows t - 1, t - 2, t - 3
-  MgTri c2, c3{0.f, 0.f, 0.f}, c4{0.f, 0.f, 0.f};                           // residual: rows t - 2, t - 3, t - 4
+  // rows t .. t + 2 are loaded ahead
+  MgCoef k0, k1, k2, kn, kq;  // rows t, t - 1, t - 2, t + 1, t + 2
+  float r0, r1 = 0.f;         // reciprocal divisors of rows t, t - 1
+  float dn = 1.f, dq = 1.f;   // divisors of rows t + 1, t + 2 (OD)
+  MgStencil sa, sb;           // rows t - 1, t - 2
+  MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};  // sweep 1: rows t, t - 1, t - 2
+  MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};  // sweep 2: rows t - 1, t - 2, t - 3
+  MgTri c2, c3{0.f, 0.f, 0.f}, c4{0.f, 0.f, 0.f};  // residual: rows t - 2, t - 3, t - 4
   int t = m.y0 - 3;
-  k1.load(st, N, f, false, 0);
-  k2 = k1;
+  int q = t * W + m.x;  // node of row t
+  k1.none();
+  k2.none();
   sb.set(k1, k2);
-  kn.load(st, N, f, inside(t), at(t));
-  float dn = OD && inside(t) ? ds[at(t)] : 1.f;
-#pragma unroll 3
-  for (; t < m.y1 + 3; ++t) {
+  kn.load(st, nws, f, inside(t), q);
+  kq.load(st, nws, f, inside(t + 1), q + W);
+  if (OD) {
+    if (inside(t)) dn = ds[q];
+    if (inside(t + 1)) dq = ds[q + W];
+  }
+#pragma unroll 2
+  for (; t < m.y1 + 3; ++t, q += W) {
     k0 = kn;
     r0 = __fdividef(1.f, OD ? dn : k0.c);
-    kn.load(st, N, f, inside(t + 1), at(t + 1));
-    if (OD) dn = inside(t + 1) ? ds[at(t + 1)] : 1.f;
+    kn = kq;
+    kq.load(st, nws, f, inside(t + 2), q + 2 * W);
+    if (OD) {
+      dn = dq;
+      dq = inside(t + 2) ? ds[q + 2 * W] : 1.f;
+    }
     a0.set(mg_omega<OD>(0) * k0.f * r0);
     sa.set(k1, k2);
     const float v = inside(t - 1) ? a1.c + mg_omega<OD>(1) * (k1.f - sa.apply(a2, a1, a0)) * r1 : 0.f;
-    if (mine && t - 1 >= m.y0 && t - 1 < m.y1) u[at(t - 1)] = v;
+    if (mine && t - 1 >= m.y0 && t - 1 < m.y1) u[q - W] = v;
     b1.set(v);
     c2.set(inside(t - 2) ? k2.f - sb.apply(b3, b2, b1) : 0.f);
     const int y = t - 3;
-    if (mine && y >= m.y0 && y < m.y1 && !((y | m.x) & 1)) {
+    if (y >= m.y0 && y < m.y1 && !(y & 1) && mine && !(m.x & 1)) {
       const int I = m.x >> 1, J = y >> 1;
-      float q = 0.f;
+      float w = 0.f;
       if (interior(I, J, nfc)) {
         if constexpr (OD) {
           const MgTri* c[3] = {&c4, &c3, &c2};
 #pragma unroll
           for (int dy = -1; dy <= 1; ++dy) {
-            q = fmaf(pweight(ps, N, W, m.x - 1, y + dy, I, J), c[dy + 1]->w, q);
-            q = fmaf(pweight(ps, N, W, m.x, y + dy, I, J), c[dy + 1]->c, q);
-            q = fmaf(pweight(ps, N, W, m.x + 1, y + dy, I, J), c[dy + 1]->e, q);
+            w = fmaf(pweight(ps, N, W, m.x - 1, y + dy, I, J), c[dy + 1]->w, w);
+            w = fmaf(pweight(ps, N, W, m.x, y + dy, I, J), c[dy + 1]->c, w);
+            w = fmaf(pweight(ps, N, W, m.x + 1, y + dy, I, J), c[dy + 1]->e, w);
           }
         } else {
-          q = c3.c + 0.5f * (c3.w + c3.e + c4.c + c2.c) + 0.25f * (c4.w + c4.e + c2.w + c2.e);
+          w = c3.c + 0.5f * (c3.w + c3.e + c4.c + c2.c) + 0.25f * (c4.w + c4.e + c2.w + c2.e);
         }
       }
-      fc[(size_t)J * Wc + I] = q;
+      fc[(size_t)J * Wc + I] = w;
     }
     a2 = a1;
     a1 = a0;
@@ -629,16 +573,11 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_down_kernel(int nf, int row
   }
 }
 
-// (P u_c) at the interior fine node (x, y).
-template <bool OD>
-__device__ __forceinline__ float prolong_at(const float* __restrict__ ps, size_t Nf, int Wf, const float* __restrict__ u,
+// (P u_c) at the interior fine node (x, y), operator-dependent P.
+__device__ __forceinline__ float prolong_od(const float* __restrict__ ps, size_t Nf, int Wf, const float* __restrict__ u,
                                             int Wc, int x, int y) {
   const int I0 = x >> 1, J0 = y >> 1;
   const size_t v = (size_t)y * Wf + x;
-  if constexpr (!OD) {
-    const int I1 = (x & 1) ? I0 + 1 : I0, J1 = (y & 1) ? J0 + 1 : J0;
-    return 0.25f * (u[J0 * Wc + I0] + u[J0 * Wc + I1] + u[J1 * Wc + I0] + u[J1 * Wc + I1]);
-  }
   if (!(x & 1) && !(y & 1)) return u[J0 * Wc + I0];
   if (!(y & 1))  // between coarse nodes I0, I0 + 1 of row J0
     return ps[v] * u[J0 * Wc + I0] + ps[Nf + v] * u[J0 * Wc + I0 + 1];
@@ -666,45 +605,79 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
   if (run) {
     const int W = nf + 1, Wc = nf / 2 + 1;
     const size_t N = (size_t)W * W;
-    st += (size_t)s * 5 * N;
+    st += (size_t)s * st_stride(N);
     f += (size_t)s * N;
     ui += (size_t)s * N;
     uo += (size_t)s * N;
     uc += (size_t)s * Wc * Wc;
+    const float* nws = st + 4 * N;
     const float* ds = dv + (size_t)s * N;
     const float* ps = P + (size_t)s * 4 * N;
     const double* rs = r ? r + (size_t)s * N : nullptr;
     const bool mine = lane >= 2 && lane < 30 && m.x < W;
     auto inside = [&](int y) { return m.in && y > 0 && y < nf; };
-    auto at = [&](int y) { return (size_t)y * W + m.x; };
-    auto start = [&](int y) { return inside(y) ? ui[at(y)] + prolong_at<OD>(ps, N, W, uc, Wc, m.x, y) : 0.f; };
-    auto mine_at = [&](int y) { return mine && m.in && y > 0 && y < nf && y >= m.y0 && y < m.y1; };
-    MgCoef k0, k1, k2, kn;  // rows t, t - 1, t - 2 and t + 1
+    // bilinear: the coarse values beside column x, summed over the two
+    // columns, of the coarse rows floor(y / 2) (ha) and the next (hb)
+    const int I0 = m.x >> 1, I1 = (m.x + 1) >> 1;
+    auto coarse = [&](int J) {
+      return m.in && J > 0 && J < nf / 2 ? uc[J * Wc + I0] + uc[J * Wc + I1] : 0.f;
+    };
+    MgCoef k0, k1, k2, kn, kq;     // rows t, t - 1, t - 2, t + 1, t + 2
     float r0, r1 = 0.f, r2 = 0.f;  // reciprocal divisors of rows t, t - 1, t - 2
+    float dn = 1.f, dq = 1.f, un = 0.f, uq = 0.f;  // rows t + 1, t + 2
     MgStencil sa, sb;              // rows t - 1, t - 2
     MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};  // the starting values: rows t, t - 1, t - 2
     MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};  // sweep 1: rows t - 1, t - 2, t - 3
-    int t = m.y0 - 2;
-    k1.load(st, N, f, false, 0);
-    k2 = k1;
+    int t = m.y0 - 2;  // even
+    int q = t * W + m.x;
+    k1.none();
+    k2.none();
     sb.set(k1, k2);
-    kn.load(st, N, f, inside(t), at(t));
-    float vn = start(t), dn = OD && inside(t) ? ds[at(t)] : 1.f;
-    double rn = 0.0;  // r of row t - 2
-#pragma unroll 3
-    for (; t < m.y1 + 2; ++t) {
+    kn.load(st, nws, f, inside(t), q);
+    kq.load(st, nws, f, inside(t + 1), q + W);
+    if (inside(t)) un = ui[q];
+    if (inside(t + 1)) uq = ui[q + W];
+    float ha = 0.f, hb = 0.f, hc = 0.f;  // coarse rows t / 2, t / 2 + 1, t / 2 + 2
+    if constexpr (OD) {
+      if (inside(t)) dn = ds[q];
+      if (inside(t + 1)) dq = ds[q + W];
+    } else {
+      ha = coarse(t >> 1);
+      hb = coarse((t >> 1) + 1);
+    }
+    double rn = 0.0, rq = 0.0;  // r of rows t - 2, t - 1
+#pragma unroll 2
+    for (; t < m.y1 + 2; ++t, q += W) {
       k0 = kn;
       r0 = __fdividef(1.f, OD ? dn : k0.c);
-      a0.set(vn);
+      float v0 = 0.f;
+      if constexpr (OD) {
+        if (inside(t)) v0 = un + prolong_od(ps, N, W, uc, Wc, m.x, t);
+        dn = dq;
+        dq = inside(t + 2) ? ds[q + 2 * W] : 1.f;
+      } else {
+        if (t & 1) {
+          v0 = un + 0.25f * (ha + hb);
+          ha = hb;
+          hb = hc;
+        } else {
+          v0 = un + 0.5f * ha;
+          hc = coarse((t >> 1) + 2);
+        }
+        if (!inside(t)) v0 = 0.f;
+      }
+      a0.set(v0);
       const double rv = rn;
-      kn.load(st, N, f, inside(t + 1), at(t + 1));
-      vn = start(t + 1);
-      if (OD) dn = inside(t + 1) ? ds[at(t + 1)] : 1.f;
-      if (rs) rn = mine_at(t - 1) ? rs[at(t - 1)] : 0.0;
+      kn = kq;
+      un = uq;
+      kq.load(st, nws, f, inside(t + 2), q + 2 * W);
+      uq = inside(t + 2) ? ui[q + 2 * W] : 0.f;
+      rn = rq;
+      if (rs) rq = mine && inside(t) && t >= m.y0 && t < m.y1 ? rs[q] : 0.0;
       sa.set(k1, k2);
       b1.set(inside(t - 1) ? a1.c + mg_omega<OD>(0) * (k1.f - sa.apply(a2, a1, a0)) * r1 : 0.f);
       const float v = inside(t - 2) ? b2.c + mg_omega<OD>(1) * (k2.f - sb.apply(b3, b2, b1)) * r2 : 0.f;
-      if (mine && t - 2 >= m.y0 && t - 2 < m.y1) uo[at(t - 2)] = v;
+      if (mine && t - 2 >= m.y0 && t - 2 < m.y1) uo[q - 2 * W] = v;
       if (rs) acc = fma(rv, widen(v), acc);
       a2 = a1;
       a1 = a0;
@@ -720,6 +693,129 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
   if (r) block_sum_to(acc, rz + s);
 }
 
+// ---- the last levels of one sample in one CTA: a level of at most 32 elements
+// per side (if the coarsest is not the only one left) and the coarsest.  A
+// thread holds one interior node of each (at most 961 and 225) with its
+// couplings in registers; the vectors live in shared memory.  As marches and
+// a kernel for the coarsest grid, three launches of 10 to 13 us; with the
+// level of 64 and loops over the nodes in here too, 40 us.
+struct MgSmallArgs {
+  int nf;  // the upper level, 0: only the coarsest
+  const float *st, *P;
+  int nfc;  // the coarsest level
+  const float* stc;
+  const float* f;  // right-hand side of the first of them [S][N]
+  float* out;      // solution there [S][N]
+};
+constexpr int kMgSmallThreads = 992;  // 31 warps: 31^2 interior nodes
+
+template <bool OD>
+__device__ __forceinline__ float mg_divisor(const float a[9]) {
+  return OD ? jacobi_divisor(a) : a[4];
+}
+__device__ __forceinline__ float apply9s(const float a[9], const float* u, int W) {
+  float t = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) t = fmaf(a[k], u[(k / 3 - 1) * W + k % 3 - 1], t);
+  return t;
+}
+
+template <bool OD>
+__global__ void __launch_bounds__(kMgSmallThreads) mgf_small_kernel(MgSmallArgs A) {
+  constexpr int NF = (kMgSmall + 1) * (kMgSmall + 1), NC = 17 * 17;
+  __shared__ float U[NF], V[NF], Uc[2][NC];
+  const int s = blockIdx.x, tid = threadIdx.x;
+  const bool two = A.nf > 0;
+  // the upper level's node (x, y) and the coarsest's (I, J)
+  const int W = A.nf + 1, N = W * W, Wc = A.nfc + 1, Nc = Wc * Wc;
+  const int mx = max(A.nf - 1, 1), mc = A.nfc - 1;
+  const int x = tid % mx + 1, y = tid / mx + 1, v = y * W + x;
+  const int I = tid % mc + 1, J = tid / mc + 1, vc = J * Wc + I;
+  const bool in = two && tid < mx * mx, inc = tid < mc * mc;
+  for (int q = tid; q < NF; q += kMgSmallThreads) U[q] = V[q] = 0.f;
+  for (int q = tid; q < NC; q += kMgSmallThreads) Uc[0][q] = Uc[1][q] = 0.f;
+  float a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, c[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  float fv = 0.f, fc = 0.f, rd = 0.f, rc = 0.f;
+  if (in) {
+    stencil9(A.st + (size_t)s * st_stride(N), N, v, W, a);
+    fv = A.f[(size_t)s * N + v];
+    rd = 1.f / mg_divisor<OD>(a);
+  }
+  if (inc) {
+    stencil9(A.stc + (size_t)s * st_stride(Nc), Nc, vc, Wc, c);
+    rc = 1.f / jacobi_divisor(c);
+    if (!two) fc = A.f[(size_t)s * Nc + vc];
+  }
+  const float* ps = A.P + (size_t)s * 4 * N;
+  __syncthreads();
+  float u = 0.f;
+  if (two) {
+    // two sweeps from zero, the residual and its restriction
+    u = mg_omega<OD>(0) * fv * rd;
+    if (in) V[v] = u;
+    __syncthreads();
+    if (in) {
+      u += mg_omega<OD>(1) * (fv - apply9s(a, V + v, W)) * rd;
+      U[v] = u;
+    }
+    __syncthreads();
+    if (in) V[v] = fv - apply9s(a, U + v, W);
+    __syncthreads();
+    if (inc) {
+      const float* q = V + 2 * J * W + 2 * I;
+      if constexpr (OD) {
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx)
+            fc = fmaf(pweight(ps, N, W, 2 * I + dx, 2 * J + dy, I, J), q[dy * W + dx], fc);
+      } else {
+        fc = q[0] + 0.5f * (q[-1] + q[1] + q[-W] + q[W]) + 0.25f * (q[-W - 1] + q[-W + 1] + q[W - 1] + q[W + 1]);
+      }
+    }
+  }
+  // the coarsest grid: Chebyshev steps from zero
+  constexpr float theta = 0.5f * (kMgCoarseHi + kMgCoarseLo), delta = 0.5f * (kMgCoarseHi - kMgCoarseLo);
+  constexpr float sigma = theta / delta;
+  float d = fc * rc / theta, uc = d, rho = 1.f / sigma;
+  if (inc) Uc[0][vc] = uc;
+  __syncthreads();
+  for (int k = 1; k < kMgCoarseSteps; ++k) {
+    const float next = 1.f / (2.f * sigma - rho);
+    if (inc) {
+      d = next * rho * d + 2.f * next / delta * rc * (fc - apply9s(c, Uc[(k - 1) & 1] + vc, Wc));
+      uc += d;
+      Uc[k & 1][vc] = uc;
+    }
+    rho = next;
+    __syncthreads();
+  }
+  if (!two) {
+    for (int q = tid; q < Nc; q += kMgSmallThreads) A.out[(size_t)s * Nc + q] = Uc[(kMgCoarseSteps - 1) & 1][q];
+    return;
+  }
+  // prolongation and two sweeps
+  if (in) {
+    const float* q = Uc[(kMgCoarseSteps - 1) & 1];
+    if constexpr (OD) {
+      u += prolong_od(ps, N, W, q, Wc, x, y);
+    } else {
+      const int I0 = x >> 1, J0 = y >> 1, I1 = (x + 1) >> 1, J1 = (y + 1) >> 1;
+      u += 0.25f * (q[J0 * Wc + I0] + q[J0 * Wc + I1] + q[J1 * Wc + I0] + q[J1 * Wc + I1]);
+    }
+    U[v] = u;
+  }
+  __syncthreads();
+  if (in) {
+    u += mg_omega<OD>(0) * (fv - apply9s(a, U + v, W)) * rd;
+    V[v] = u;  // (the residual in V was last read before the barriers of the Chebyshev steps)
+  }
+  __syncthreads();
+  if (in) U[v] = u + mg_omega<OD>(1) * (fv - apply9s(a, V + v, W)) * rd;
+  __syncthreads();
+  for (int q = tid; q < N; q += kMgSmallThreads) A.out[(size_t)s * N + q] = U[q];
+}
+
 // mm[0] = bit pattern of max a, mm[1] = that of min a over the positive
 // entries of a (the patterns of positive doubles order like their values;
 // mm[0] starts at zero, mm[1] at the pattern 0x7F7F7F7F7F7F7F7F, a positive
@@ -727,9 +823,8 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
 __global__ void mgf_range_kernel(long long n, const double* __restrict__ a, unsigned long long* __restrict__ mm) {
   unsigned long long hi = 0, lo = 0x7F7F7F7F7F7F7F7Full;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double v = a[i];
-    if (v > 0.0) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a[i]);
+    if (b - 1 < 0x7ff0000000000000ull) {  // positive and not NaN
       hi = max(hi, b);
       lo = min(lo, b);
     }
@@ -887,14 +982,12 @@ size_t mg_layout(int nf, int S, MgLevel* lv, int* L, unsigned char* base, double
     lv[l].nf = nfs[l];
     lv[l].N = (int)N;
     lv[l].st = reinterpret_cast<float*>(base + o);
-    o += al256(sizeof(float) * 5 * N * S);
+    o += al256(sizeof(float) * st_stride(N) * S);
     lv[l].u = reinterpret_cast<float*>(base + o);
     o += al256(sizeof(float) * N * S);
     lv[l].u2 = reinterpret_cast<float*>(base + o);
     o += al256(sizeof(float) * N * S);
     lv[l].f = reinterpret_cast<float*>(base + o);
-    o += al256(sizeof(float) * N * S);
-    lv[l].r = reinterpret_cast<float*>(base + o);
     o += al256(sizeof(float) * N * S);
     lv[l].P = reinterpret_cast<float*>(base + o);  // unused on the coarsest level
     o += l + 1 < *L ? al256(sizeof(float) * 4 * N * S) : 0;
@@ -936,15 +1029,24 @@ dim3 mg_grid(int nf, int S, int useful, int rows) {
 }
 
 // z = V-cycle(r) on level l (f of level l holds the right-hand side; the
-// result in u2 of level l, in u on the coarsest); on the finest level rz[s]
-// += r . z.
+// result in u2 of level l); on the finest level rz[s] += r . z.
 template <bool OD>
 int vcycle(MgLevel* lv, int L, int l, int S, const double* r, double* rz, cudaStream_t st) {
   MgLevel& c = lv[l];
-  if (l == L - 1) {
-    if (c.N > kMgCoarseMaxNodes) return set_error(STOMSFEM_EINVAL, "coarsest grid of %d nodes", c.N);
-    mgf_coarse_kernel<<<S, kMgCoarseThreads, 0, st>>>(c.nf, c.st, c.dv, c.f, c.u);
-    return check_cuda(cudaGetLastError(), "coarse sweeps");
+  const int left = L - l;
+  if (left == 1 || (left == 2 && c.nf <= kMgSmall)) {
+    const MgLevel& last = lv[L - 1];
+    if (last.nf > 16) return set_error(STOMSFEM_EINVAL, "coarsest grid of %d elements per side", last.nf);
+    MgSmallArgs A;
+    A.nf = left == 2 ? c.nf : 0;
+    A.st = c.st;
+    A.P = c.P;
+    A.nfc = last.nf;
+    A.stc = last.st;
+    A.f = c.f;
+    A.out = c.u2;
+    mgf_small_kernel<OD><<<S, kMgSmallThreads, 0, st>>>(A);
+    return check_cuda(cudaGetLastError(), "small levels");
   }
   const int rows = mg_rows(c.nf, S);
   MgLevel& n = lv[l + 1];
@@ -952,7 +1054,7 @@ int vcycle(MgLevel* lv, int L, int l, int S, const double* r, double* rz, cudaSt
   int rc = vcycle<OD>(lv, L, l + 1, S, nullptr, nullptr, st);
   if (rc) return rc;
   mgf_up_kernel<OD><<<mg_grid(c.nf, S, 28, rows), kMgWarps * 32, 0, st>>>(
-      c.nf, rows, c.st, c.dv, c.P, c.f, l + 1 == L - 1 ? n.u : n.u2, c.u, c.u2, r, rz);
+      c.nf, rows, c.st, c.dv, c.P, c.f, n.u2, c.u, c.u2, r, rz);
   return check_cuda(cudaGetLastError(), "v-cycle");
 }
 
@@ -1020,7 +1122,7 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
     }
   }
   // (the bilinear sweeps divide by the diagonal entry)
-  for (int l = od ? 0 : L - 1; l < L; ++l)
+  for (int l = 0; l < L && od; ++l)
     mgf_divisor_kernel<<<grid2(lv[l].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].dv);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   // z = M r, rz[cur] += r . z
