@@ -3,23 +3,25 @@
 // The bumps are Gaussians on a tensor lattice, so
 //   z(x, y) = sum_bx gx_bx(x) * U_bx(y),   U_bx(y) = sum_by xi[by][bx] gy_by(y),
 // with gx_bx(x) = exp(-(x - cx_bx)^2 / w^2) (and gy likewise).  A block
-// handles one sample and a strip of R element rows: gy of the strip and then
-// U are built once in shared memory, each thread keeps gx of its column in
+// handles strips of R element rows of kCoefCols columns: gy of the strip and
+// then U are built in shared memory, each thread keeps gx of its column in
 // registers and sweeps the strip, so the work per element is at most nbx
-// FMAs plus the final exponential (the table-driven FP64 exp of fexp.cuh);
-// the strip height R amortises the nbx exponentials of gx over R elements.
+// FMAs plus the final exponential (the table-driven FP64 exp of fexp.cuh).
 //
-// The FP64 kernel is bound by the FP64 pipe.  Bumps further than kCoefReach
-// widths from a warp's columns are left out, four at a time: exp(-7.5^2) =
-// 3.7e-25, so with amplitudes below kCoefAmp (of the exponent) what they add
-// stays below 3e-17, less than the exponential's rounding; a strip with a
-// larger one, or with one that is not finite, sums them all.  On the 1024^2 workload
-// (16 bumps a row, spacing one width) 12 of 16 products remain, with 32
-// bumps of 3/4 of the spacing 15 of 32.  A block takes kCoefCols columns,
-// so that the blocks' number evens out over the SMs, and where a batch gives
-// fewer than four blocks an SM the strips get shorter.
-// 32 samples of the 1024^2 grid: 2.25 -> 2.12 ms; the 64-sample step of the
-// 64^2 grid (64 blocks before): 52 us less.
+// The FP64 kernel is bound by the FP64 pipe.  gx and gy depend on the place
+// only, so a block takes the samples of one place one after the other and
+// makes them once; and the blocks are as many as fit the chip, with equal
+// shares of the (place, sample) pairs (as a grid of strips, 6.7 blocks an SM
+// left it idle a fifth of the time, and gx cost 1.8 of 28 operations an
+// element).  Bumps further than kCoefReach widths from a warp's columns are
+// left out, four at a time: exp(-7.5^2) = 3.7e-25, so with amplitudes below
+// kCoefAmp (of the exponent) what they add stays below 3e-17, less than the
+// exponential's rounding; a strip with a larger one, or with one that is not
+// finite, sums them all.  On the 1024^2 workload (16 bumps a row, spacing one
+// width) 12 of 16 products remain, with 32 bumps of 3/4 of the spacing 15 of
+// 32.  Where a batch gives fewer than four pairs a block the strips get
+// shorter.
+// 32 samples of the 1024^2 grid: 2.25 -> 1.72 ms.
 #include "common.cuh"
 #include "fexp.cuh"
 
@@ -30,7 +32,7 @@ constexpr int kCoefThreads = 128;
 constexpr size_t kCoefSmem = 48 * 1024;
 constexpr double kCoefReach = 7.5;  // in widths
 constexpr double kCoefAmp = 1e6;
-constexpr int kCoefCols = 256;      // columns per block (FP64)
+constexpr int kCoefCols = 256;      // columns and threads per block (FP64)
 
 __host__ __device__ inline int coef_rows(int nbx, int nby) {
   int R = 128;
@@ -54,73 +56,83 @@ __device__ __forceinline__ double sigmoid_scaled(double clog, double e) {
 }
 
 template <int NBX>
-__global__ void __launch_bounds__(kCoefThreads)
-sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, double w, double scale, double clog,
-                   double gain, const double* __restrict__ xi, double* __restrict__ a) {
+__global__ void __launch_bounds__(kCoefCols, NBX <= 32 ? 2 : 1)
+sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int S, long long npair, double w, double scale,
+                   double clog, double gain, const double* __restrict__ xi, double* __restrict__ a) {
   extern __shared__ double csm[];
   __shared__ int large;                  // an amplitude beyond kCoefAmp
   double* tab = csm;                     // [64] 2^(j/64)
   double* gy = csm + 64;                 // [nby][R]
   double* U = gy + (size_t)nby * R;      // [nbx][R]
-  const int s = blockIdx.y;
-  const int nstrip = (nf + R - 1) / R, strip = blockIdx.x % nstrip, col0 = (blockIdx.x / nstrip) * kCoefCols;
-  const int ey0 = strip * R;
-  const int rows = min(R, nf - ey0);
+  const int tid = threadIdx.x;
   const double h = 1.0 / nf;
   const double iw2 = 1.0 / (w * w);
-  const double* xs = xi + (size_t)s * nbx * nby;
   const double gain_z = kind == STOMSFEM_FIELD_EXP_SIGMOID ? 0.25 * fabs(clog * gain) : fabs(scale);
   const double amp = gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp;
-  if (threadIdx.x == 0) large = 0;
-  exp_table_fill(tab);
-  __syncthreads();
-  for (int q = threadIdx.x; q < nby * rows; q += blockDim.x) {
-    const int by = q / rows, r = q % rows;
-    const double dy = (ey0 + r + 0.5) * h - (by + 0.5) / nby;
-    gy[by * R + r] = fexp(-dy * dy * iw2, tab);
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nbx * rows; q += blockDim.x) {
-    const int bx = q / rows, r = q % rows;
-    double acc = 0.0;
-    for (int by = 0; by < nby; ++by) acc = fma(__ldg(xs + by * nbx + bx), gy[by * R + r], acc);
-    U[bx * R + r] = acc;
-    if (!(fabs(acc) <= amp)) large = 1;
-  }
-  __syncthreads();
   // narrow grids: the threads split into row groups of a power of two of
   // columns (32 at least)
-  int cols = kCoefThreads;
+  int cols = kCoefCols;
   while (cols > 32 && cols / 2 >= nf) cols >>= 1;
-  const int rg = threadIdx.x / cols, nrg = kCoefThreads / cols;
-  const int col1 = min(nf, col0 + kCoefCols);
-  for (int ex = col0 + threadIdx.x % cols; ex < col1; ex += cols) {
-    const double x = (ex + 0.5) * h;
-    // groups of four bumps within reach of the warp's 32 columns
-    unsigned near = 0xffffffffu;
-    if (!large) {
-      near = 0;
+  const int rg = tid / cols, nrg = kCoefCols / cols;
+  exp_table_fill(tab);
+  // this block's (place, sample) pairs, the samples fastest
+  const long long u0 = npair * blockIdx.x / gridDim.x, u1 = npair * (blockIdx.x + 1) / gridDim.x;
+  int place = -1, ey0 = 0, rows = 0, ex = 0;
+  unsigned near = 0;    // groups of four bumps within reach of the warp's 32 columns
+  unsigned have = 0;    // those that gx holds
+  double gx[NBX];
+  for (long long u = u0; u < u1; ++u) {
+    const int t = (int)(u / S), s = (int)(u - (long long)t * S);
+    __syncthreads();  // (the table; gy and U of the pair before are no longer read)
+    if (t != place) {
+      place = t;
+      const int strip = t % nstrip, col0 = t / nstrip * kCoefCols;
+      ey0 = strip * R;
+      rows = min(R, nf - ey0);
+      ex = col0 + tid % cols;
+      for (int q = tid; q < nby * rows; q += kCoefCols) {
+        const int by = q / rows, r = q % rows;
+        const double dy = (ey0 + r + 0.5) * h - (by + 0.5) / nby;
+        gy[by * R + r] = fexp(-dy * dy * iw2, tab);
+      }
       const int e0 = ex & ~31;
       const float lo = (float)((e0 + 0.5) * h - kCoefReach * w), hi = (float)((e0 + 31.5) * h + kCoefReach * w);
+      near = have = 0;
 #pragma unroll
       for (int g = 0; g < NBX / 4; ++g)
         if ((4 * g + 3.5f) / nbx >= lo && (4 * g + 0.5f) / nbx <= hi) near |= 1u << g;
     }
-    double gx[NBX];
+    if (tid == 0) large = 0;
+    __syncthreads();
+    const double* xs = xi + (size_t)s * nbx * nby;
+    for (int q = tid; q < nbx * rows; q += kCoefCols) {
+      const int bx = q / rows, r = q % rows;
+      double acc = 0.0;
+      for (int by = 0; by < nby; ++by) acc = fma(__ldg(xs + by * nbx + bx), gy[by * R + r], acc);
+      U[bx * R + r] = acc;
+      if (!(fabs(acc) <= amp)) large = 1;
+    }
+    __syncthreads();
+    if (ex >= nf) continue;  // (every thread comes back to the barriers above)
+    const unsigned use = large ? 0xffffffffu : near;
+    if (use & ~have) {
+      have = use;
 #pragma unroll
-    for (int bx = 0; bx < NBX; ++bx) {
-      gx[bx] = 0.0;
-      if (bx < nbx && (near >> (bx / 4) & 1)) {
-        const double dx = x - (bx + 0.5) / nbx;
-        gx[bx] = fexp(-dx * dx * iw2, tab);
+      for (int bx = 0; bx < NBX; ++bx) {
+        gx[bx] = 0.0;
+        if (bx < nbx && (use >> (bx / 4) & 1)) {
+          const double dx = (ex + 0.5) * h - (bx + 0.5) / nbx;
+          gx[bx] = fexp(-dx * dx * iw2, tab);
+        }
       }
     }
-    double* arow = a + ((size_t)s * nf + ey0) * nf + ex;
-    for (int r = rg; r < rows; r += nrg) {
+    double* arow = a + ((size_t)s * nf + ey0 + rg) * nf + ex;
+    const size_t astep = (size_t)nrg * nf;
+    for (int r = rg; r < rows; r += nrg, arow += astep) {
       double z = 0.0;
 #pragma unroll
       for (int g = 0; g < NBX / 4; ++g)
-        if (near >> g & 1) {
+        if (use >> g & 1) {
 #pragma unroll
           for (int bx = 4 * g; bx < 4 * g + 4; ++bx)
             if (bx < nbx) z = fma(gx[bx], U[bx * R + r], z);
@@ -132,7 +144,7 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, double w, double s
         v = fma(scale, z, gain);
       else
         v = fexp(sigmoid_scaled(clog, fexp(-gain * z, tab)), tab);
-      arow[(size_t)r * nf] = v;
+      *arow = v;
     }
   }
 }
@@ -210,33 +222,42 @@ static int sample_coef_impl(const stomsfem_grid* grid, const stomsfem_field* fie
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int nbx = field->nbx;
   int R = coef_rows(field->nbx, field->nby);
-  const int ncol = (grid->nf + kCoefCols - 1) / kCoefCols;
-  if (precision == STOMSFEM_FP64) {
-    // at least four blocks per SM, down to strips of 8 rows
-    const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
-    while (R > 8 && (long long)((grid->nf + R - 1) / R) * ncol * S < 4LL * sms) R >>= 1;
-  }
-  const size_t smem = precision == STOMSFEM_FP64
-                          ? (64 + (size_t)(field->nbx + field->nby) * R) * sizeof(double)
-                          : (size_t)(field->nbx + field->nby) * R * sizeof(float);
+  const size_t smem = (size_t)(field->nbx + field->nby) * R * sizeof(float);
   const size_t K = (size_t)field->nbx * field->nby;
+  const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
+  if (precision == STOMSFEM_FP64) {
+    const int nchunk = (grid->nf + kCoefCols - 1) / kCoefCols;
+    auto pairs = [&](int r) { return (long long)((grid->nf + r - 1) / r) * nchunk * S; };
+    const long long blocks = 2LL * sms;
+    if (R > 64) R = 64;
+    while (R > 8 && pairs(R) < 4 * blocks) R >>= 1;
+    const int nstrip = (grid->nf + R - 1) / R;
+    const long long npair = pairs(R);
+    const size_t bytes = (64 + (size_t)(field->nbx + field->nby) * R) * sizeof(double);
+    const unsigned grd = (unsigned)(npair < blocks ? npair : blocks);
+#define LAUNCH(N)                                                                                               \
+  sample_coef_kernel<N><<<grd, kCoefCols, bytes, st>>>(grid->nf, field->kind, nbx, field->nby, R, nstrip, S, npair, \
+                                                       field->width, field->scale, field->contrast_log,         \
+                                                       field->gain, xi, a)
+    if (nbx <= 4) LAUNCH(4);
+    else if (nbx <= 8) LAUNCH(8);
+    else if (nbx <= 16) LAUNCH(16);
+    else if (nbx <= 32) LAUNCH(32);
+    else LAUNCH(64);
+#undef LAUNCH
+    STOMSFEM_TRY_CUDA(cudaGetLastError());
+    return STOMSFEM_OK;
+  }
   // the sample index runs over gridDim.y (at most 65535 per launch)
   for (int s0 = 0; s0 < S; s0 += 65535) {
     const int Sc = S - s0 < 65535 ? S - s0 : 65535;
-    dim3 grd((grid->nf + R - 1) / R * (precision == STOMSFEM_FP64 ? ncol : 1), Sc);
+    dim3 grd((grid->nf + R - 1) / R, Sc);
     const double* xs = xi + (size_t)s0 * K;
     double* as = a + (size_t)s0 * grid->nf * grid->nf;
-#define LAUNCH(N)                                                                                        \
-  do {                                                                                                   \
-    if (precision == STOMSFEM_FP64)                                                                      \
-      sample_coef_kernel<N><<<grd, kCoefThreads, smem, st>>>(grid->nf, field->kind, nbx, field->nby, R,  \
-                                                             field->width, field->scale,                 \
-                                                             field->contrast_log, field->gain, xs, as);  \
-    else                                                                                                 \
-      sample_coef_f32_kernel<N><<<grd, kCoefThreads, smem, st>>>(                                        \
-          grid->nf, field->kind, nbx, field->nby, R, (float)field->width, (float)field->scale,            \
-          (float)field->contrast_log, (float)field->gain, xs, as);                                       \
-  } while (0)
+#define LAUNCH(N)                                                                                         \
+  sample_coef_f32_kernel<N><<<grd, kCoefThreads, smem, st>>>(grid->nf, field->kind, nbx, field->nby, R,   \
+                                                             (float)field->width, (float)field->scale,    \
+                                                             (float)field->contrast_log, (float)field->gain, xs, as)
     if (nbx <= 4) LAUNCH(4);
     else if (nbx <= 8) LAUNCH(8);
     else if (nbx <= 16) LAUNCH(16);
