@@ -1,0 +1,222 @@
+"""The tiled kernels at the sizes where their rules turn, against the FP64
+oracle: the FP32 trailing update's 8-row tiles (half bandwidths around 24, 32
+and 40, and pitches that are not multiples of 8), the FP64 forms with four and
+two units per warp, the unit order by patch size with flagged cells and
+oversampling clipped to a small grid, the CTA-wide banded solves, the
+multigrid's level counts, the reduced solves at every tile remainder of the
+rank and the sampling's bump groups.
+
+Tolerances as in the parity tests: FP64 1e-11 (relative Frobenius of a unit's
+K_e and b_e), refinement 1e-10, FP32 1e-5; coarse solutions 1e-9 and the
+multigrid solutions 1e-10 in relative L2; a sampled coefficient within the
+rounding of its exponent, 4 (g sum psi 8 eps + 4 eps)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_1607_00693_gb300 import api
+
+DEV = "cuda:0"
+TOL = {api.FP64: 1e-11, api.FP32_REFINED: 1e-10, api.FP32: 1e-5}
+
+
+@pytest.fixture(scope="module")
+def orc():
+    from paper_1607_00693_gb300.build import build_library
+    import oracle
+    build_library()
+    oracle.build()
+    return oracle
+
+
+def _t(x, dtype=None):
+    return torch.from_numpy(np.ascontiguousarray(x, dtype=dtype)).to(DEV)
+
+
+def _rel(x, y):
+    return float(np.max(np.linalg.norm(x - y, axis=-1) / np.linalg.norm(y, axis=-1)))
+
+
+def _coef(S, nf, seed, s=1.0):
+    return np.exp(np.random.default_rng(seed).uniform(-s, s, size=(S, nf, nf)))
+
+
+def _upscale(nf, nc, a, ov, mo, precision, slots=None):
+    g = api.grid(nf, nc)
+    S, cells = a.shape[0], nc * nc
+    Ke = torch.zeros((S, cells, 10), dtype=torch.float64, device=DEV)
+    be = torch.zeros((S, cells, 4), dtype=torch.float64, device=DEV)
+    st = torch.full((S, cells), 99, dtype=torch.int32, device=DEV)
+    ws = None
+    if slots:
+        ws = torch.zeros(api.stomsfem_upscale_workspace_size(g, mo, precision)[0] * slots, dtype=torch.uint8, device=DEV)
+    api.stomsfem_upscale(g, _t(a), Ke, be, oversample=None if ov is None else _t(ov, np.int8), max_oversample=mo,
+                         precision=precision, unit_status=st, workspace=ws)
+    torch.cuda.synchronize()
+    return Ke.cpu().numpy(), be.cpu().numpy(), st.cpu().numpy()
+
+
+# half bandwidth = rho + 2 o inside the domain: 17 .. 41 with mixed patches
+@pytest.mark.parametrize("rho,mo", [(17, 0), (21, 2), (24, 0), (25, 0), (24, 4), (29, 0), (32, 0), (33, 0), (30, 3),
+                                    (32, 4), (36, 0), (37, 1), (40, 0), (41, 0)])
+@pytest.mark.parametrize("precision", [api.FP32, api.FP32_REFINED])
+def test_fp32_tiles_at_the_band_edges(orc, rho, mo, precision):
+    nc, S = 2 + (mo > 0), 3
+    nf = nc * rho
+    a = _coef(S, nf, 100 + rho)
+    ov = np.random.default_rng(rho).integers(0, mo + 1, size=nc * nc).astype(np.int8) if mo else None
+    Ko, bo = orc.upscale(nf, nc, 1.0, a, ov)
+    Kg, bg, st = _upscale(nf, nc, a, ov, mo, precision)
+    assert not st.any()
+    assert _rel(Kg, Ko) <= TOL[precision] and _rel(bg, bo) <= TOL[precision]
+
+
+# four units per warp up to b = 12 from three samples on; two below, beyond,
+# or with a workspace of less than a block of eight slots
+@pytest.mark.parametrize("rho,mo", [(1, 0), (2, 0), (3, 0), (4, 0), (5, 1), (8, 0), (8, 2), (12, 0), (13, 0)])
+@pytest.mark.parametrize("S,slots", [(1, None), (3, None), (5, None), (9, 8), (5, 4)])
+def test_fp64_units_per_warp(orc, rho, mo, S, slots):
+    nc = 5
+    nf = nc * rho
+    a = _coef(S, nf, 200 + rho)
+    ov = np.random.default_rng(rho).integers(0, mo + 1, size=nc * nc).astype(np.int8) if mo else None
+    Ko, bo = orc.upscale(nf, nc, 1.0, a, ov)
+    Kg, bg, st = _upscale(nf, nc, a, ov, mo, api.FP64, slots)
+    assert not st.any()
+    assert _rel(Kg, Ko) <= 1e-11 and _rel(bg, bo) <= 1e-11
+
+
+@pytest.mark.parametrize("nf,nc,mo", [(48, 8, 3), (8, 4, 100), (70, 35, 2)])
+@pytest.mark.parametrize("precision", [api.FP64, api.FP32])
+def test_order_by_patch_size_with_flagged_cells(orc, nf, nc, mo, precision):
+    """More cells than a pass of the list kernel (35^2), cells outside [0, mo]
+    and an oversampling far beyond the grid."""
+    a = _coef(2, nf, nf)
+    ov = np.random.default_rng(nf).integers(0, min(mo, 4) + 1, size=nc * nc).astype(np.int8)
+    if mo == 100:
+        ov[1::3] = 100
+    ok = np.ones(nc * nc, dtype=bool)
+    bad = ov.copy()
+    bad[2::5] = -1
+    bad[3::7] = 127
+    ok[2::5] = ok[3::7] = False
+    Ko, bo = orc.upscale(nf, nc, 1.0, a, ov)
+    Kg, bg, st = _upscale(nf, nc, a, bad, mo, precision)
+    assert not st[:, ok].any() and (st[:, ~ok] == -1).all() and np.isnan(Kg[:, ~ok]).all()
+    assert _rel(Kg[:, ok], Ko[:, ok]) <= TOL[precision] and _rel(bg[:, ok], bo[:, ok]) <= TOL[precision]
+
+
+@pytest.mark.parametrize("nc", [1, 2, 3, 4, 9, 16, 31, 32, 33, 47, 63])
+def test_coarse_solve_sizes(orc, nc):
+    """Last blocks of every remainder, one and two rows per lane, S above and
+    below the workspace's slots, an indefinite sample beside sound ones."""
+    S = 5
+    a = _coef(S, 2 * nc, nc)
+    K, b = orc.upscale(2 * nc, nc, 1.0, a)
+    uo = orc.coarse_solve(nc, K, b)
+    g = api.grid(2 * nc, nc)
+    for slots in (None, 2):
+        ws = None if slots is None else torch.zeros(
+            api.stomsfem_coarse_workspace_size(g, 2), dtype=torch.uint8, device=DEV)
+        u = torch.zeros((S, (nc + 1) ** 2), dtype=torch.float64, device=DEV)
+        mean, m2 = (torch.zeros((nc + 1) ** 2, dtype=torch.float64, device=DEV) for _ in range(2))
+        cnt = torch.zeros(1, dtype=torch.float64, device=DEV)
+        api.stomsfem_coarse_solve(g, _t(K), _t(b), u, mean, m2, cnt, workspace=ws)
+        ug = u.cpu().numpy()
+        assert np.linalg.norm(ug - uo) <= 1e-9 * max(np.linalg.norm(uo), 1e-300)
+        mo, vo = uo.mean(0), ((uo - uo.mean(0)) ** 2).sum(0)
+        assert np.allclose(mean.cpu().numpy(), mo, rtol=1e-9, atol=1e-12)
+        assert np.allclose(m2.cpu().numpy(), vo, rtol=1e-8, atol=1e-14) and float(cnt[0]) == S
+    if nc > 2:
+        K[2] = -K[2]
+        api.stomsfem_coarse_solve(g, _t(K), _t(b), u)
+        ug = u.cpu().numpy()
+        inner = uo[2] != 0
+        assert np.isnan(ug[2][inner]).all()
+        keep = [0, 1, 3, 4]
+        assert np.linalg.norm(ug[keep] - uo[keep]) <= 1e-9 * np.linalg.norm(uo[keep])
+
+
+# levels 66, 33 is odd: not offered; one to four levels below the finest
+@pytest.mark.parametrize("nf", [2, 9, 33, 64, 72, 80, 96, 112, 128, 240])
+@pytest.mark.parametrize("contrast", [False, True])
+def test_fine_solver_levels(orc, nf, contrast):
+    r = np.random.default_rng(nf)
+    a = np.exp(r.uniform(-1.0, 1.0, size=(2, nf, nf)))
+    if contrast:
+        a[:, nf // 3: nf // 3 + 2, :] = 2e3
+    g = api.grid(nf, 1)
+    u = torch.zeros((2, (nf + 1) ** 2), dtype=torch.float64, device=DEV)
+    api.stomsfem_fine_fem(g, _t(a), u)
+    for s in range(2):
+        uo = orc.fine_fem(nf, 1.0, a[s]).reshape(-1)
+        assert np.linalg.norm(u[s].cpu().numpy() - uo) <= 1e-10 * np.linalg.norm(uo)
+
+
+@pytest.mark.parametrize("rank", [1, 2, 3, 4, 5, 7, 8, 26, 27])
+def test_reduced_solves_at_every_remainder(orc, rank):
+    """Rank remainders of the 4 x 4 tiles and ragged sample counts against the
+    FP64-refined online stage, within the unrefined stage's 5e-3."""
+    nf, nc, Ns, S = 16, 2, 12, 131
+    a_tr, a = _coef(Ns, nf, 1, 0.3), _coef(S, nf, 2, 0.3)
+    g = api.grid(nf, nc)
+    phi = _t(orc.upscale(nf, nc, 1.0, a_tr, want_phi=True)[2])
+    h, rk = api.stomsfem_pod_build(g, phi, _t(a_tr), ranks=[rank, max(1, rank - 1), rank, 1])
+    try:
+        out = []
+        for refine in (0, 4):
+            Ke = torch.zeros((S, nc * nc, 10), dtype=torch.float64, device=DEV)
+            be = torch.zeros((S, nc * nc, 4), dtype=torch.float64, device=DEV)
+            st = torch.full((S, nc * nc), 9, dtype=torch.int32, device=DEV)
+            api.stomsfem_pod_upscale(h, g, _t(a), Ke, be, refine_iters=refine, unit_status=st)
+            assert not st.cpu().numpy().any()
+            out.append((Ke.cpu().numpy(), be.cpu().numpy()))
+        assert _rel(out[0][0], out[1][0]) <= 5e-3 and _rel(out[0][1], out[1][1]) <= 5e-3
+        for n in (1, 31, 32, 33):  # a sample's result does not depend on the batch
+            Ke = torch.zeros((n, nc * nc, 10), dtype=torch.float64, device=DEV)
+            be = torch.zeros((n, nc * nc, 4), dtype=torch.float64, device=DEV)
+            api.stomsfem_pod_upscale(h, g, _t(a[:n]), Ke, be)
+            assert np.array_equal(Ke.cpu().numpy(), out[0][0][:n]) and np.array_equal(be.cpu().numpy(), out[0][1][:n])
+    finally:
+        api.stomsfem_pod_destroy(h)
+
+
+@pytest.mark.parametrize("nf,nbx,nby,width,S", [(1, 1, 1, 0.3, 3), (7, 3, 5, 0.02, 2), (33, 4, 4, 0.1, 40),
+                                                (64, 17, 2, 0.01, 3), (257, 33, 9, 0.02, 2), (300, 5, 64, 0.004, 2),
+                                                (520, 64, 3, 0.5, 1)])
+@pytest.mark.parametrize("kind", [api.FIELD_EXP, api.FIELD_EXP_SIGMOID])
+def test_sampling_bump_groups(orc, nf, nbx, nby, width, S, kind):
+    fld = dict(kind=kind, nbx=nbx, nby=nby, width=width, scale=0.7, contrast_log=np.log(1e3), gain=2.0)
+    xi = np.random.default_rng(nf).uniform(-1, 1, size=(S, nbx * nby))
+    ref = orc.sample_coef(nf, fld, xi)
+    a = torch.zeros((S, nf, nf), dtype=torch.float64, device=DEV)
+    api.stomsfem_sample_coef(api.grid(nf, 1), api.field_from_dict(fld), _t(xi), a)
+    x = (np.arange(nf) + 0.5) / nf
+    psi = [np.exp(-((x[:, None] - (np.arange(n) + 0.5) / n) / width) ** 2).sum(1).max() for n in (nbx, nby)]
+    gain = 0.7 if kind == api.FIELD_EXP else np.log(1e3) * 2.0 / 4
+    eps = np.finfo(float).eps
+    bound = 4 * (gain * psi[0] * psi[1] * 8 * eps + 4 * eps) + (0 if kind == api.FIELD_EXP else 8 * np.log(1e3) * eps)
+    assert np.max(np.abs(a.cpu().numpy() / ref - 1)) <= bound
+
+
+def test_sampling_large_and_non_finite_amplitudes():
+    """Far bumps are left out only below the amplitude bound: a large one is
+    summed everywhere, and a NaN reaches every element of its sample."""
+    nf, n, width = 64, 16, 0.01
+    fld = api.field(api.FIELD_AFFINE, n, n, width, 1.0, 0.0, 2.0)
+    xi = torch.zeros((3, n * n), dtype=torch.float64, device=DEV)
+    xi[1, 0] = 1e200
+    xi[2, 5] = float("nan")
+    a = torch.zeros((3, nf, nf), dtype=torch.float64, device=DEV)
+    api.stomsfem_sample_coef(api.grid(nf, 1), fld, xi, a)
+    got = a.cpu().numpy()
+    x = (np.arange(nf) + 0.5) / nf
+    b = np.exp(-((x - 0.5 / n) / width) ** 2)
+    want = 2.0 + 1e200 * b[:, None] * b[None, :]
+    assert np.array_equal(got[0], np.full((nf, nf), 2.0))
+    near = want < 1e300
+    assert np.allclose(got[1][near], want[near], rtol=1e-10)
+    assert np.isnan(got[2]).all()
