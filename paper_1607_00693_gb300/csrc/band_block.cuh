@@ -968,11 +968,11 @@ __device__ void blk_backward(int n, int b, int bmax, const BlkSmem<T>& s, const 
   }
 }
 
-// Forward substitution with the stored factor: rg [n][NR] double holds the
+// Forward substitution with the stored factor: rg [n][NR] holds the
 // right-hand side on entry and the forward solution y on exit.
 template <int G, typename T, int NR, int RPL, int NB = G / 2>
 __device__ void blk_forward_stored(int n, int b, int bmax, const BlkSmem<T>& s, const T* __restrict__ Lg,
-                                   double* __restrict__ rg, int gl) {
+                                   T* __restrict__ rg, int gl) {
   const int RW = s.RW;
   const int stg = (NB + bmax) * NB;
   const int nbk = (n + NB - 1) / NB;
@@ -988,7 +988,7 @@ __device__ void blk_forward_stored(int n, int b, int bmax, const BlkSmem<T>& s, 
     for (int r = filled + gl; r < need; r += G) {
       T v[NR];
 #pragma unroll
-      for (int c = 0; c < NR; ++c) v[c] = (T)rg[(size_t)r * NR + c];
+      for (int c = 0; c < NR; ++c) v[c] = rg[(size_t)r * NR + c];
       st_row4<NR>(rr + ring(kslot + (r - K), RW) * 4, v);
     }
     filled = max(filled, need);
@@ -1047,7 +1047,7 @@ __device__ void blk_forward_stored(int n, int b, int bmax, const BlkSmem<T>& s, 
     }
     if (gl < nb) {
 #pragma unroll
-      for (int c = 0; c < NR; ++c) rg[(size_t)(K + gl) * NR + c] = (double)yv[c];
+      for (int c = 0; c < NR; ++c) rg[(size_t)(K + gl) * NR + c] = yv[c];
     }
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
@@ -1078,8 +1078,7 @@ __device__ __noinline__ void blk_backward_outlined(int n, int b, int bmax, const
 }
 template <int G, typename T, int NR, int RPL, int NB = G / 2>
 __device__ __noinline__ void blk_forward_stored_outlined(int n, int b, int bmax, const BlkSmem<T> s,
-                                                         const T* __restrict__ Lg, double* __restrict__ rg,
-                                                         int gl) {
+                                                         const T* __restrict__ Lg, T* __restrict__ rg, int gl) {
   blk_forward_stored<G, T, NR, RPL, NB>(n, b, bmax, s, Lg, rg, gl);
 }
 
