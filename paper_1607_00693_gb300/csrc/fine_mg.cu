@@ -437,20 +437,51 @@ struct MgCoef {
     c = 1.f;
     e = n = ne = nw = f = 0.f;
   }
-  __device__ __forceinline__ void load(const float* __restrict__ st, const float* __restrict__ nws,
-                                       const float* __restrict__ fs, bool in, int q) {
-    none();
-    if (in) {
-      const float4 v = reinterpret_cast<const float4*>(st)[q];
-      c = v.x;
-      e = v.y;
-      n = v.z;
-      ne = v.w;
-      nw = nws[q];
-      f = fs[q];
-    }
-  }
 };
+
+// Rows in flight.  A warp's marches are bound by the latency of its rows (16
+// warps an SM at about 100 registers): each lane copies its own entries of
+// the row kMgAhead steps ahead into its own places of a ring in shared
+// memory, which costs no registers and needs no barrier.
+constexpr int kMgRing = 8, kMgAhead = kMgRing - 1;
+struct MgRing {
+  float4 st[kMgRing][32];
+  float nw[kMgRing][32], f[kMgRing][32];
+};
+struct MgRingUp : MgRing {
+  float u[kMgRing][32];
+  double r[kMgRing][32];
+};
+template <int BYTES>
+__device__ __forceinline__ void mg_cp(void* dst, const void* src) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(BYTES)
+                 : "memory");
+}
+__device__ __forceinline__ void mg_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void mg_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kMgAhead - 1) : "memory"); }
+__device__ __forceinline__ void mg_fetch(MgRing& g, int slot, int lane, const float* st, const float* nws, const float* f,
+                                         int q) {
+  mg_cp<16>(&g.st[slot][lane], reinterpret_cast<const float4*>(st) + q);
+  mg_cp<4>(&g.nw[slot][lane], nws + q);
+  mg_cp<4>(&g.f[slot][lane], f + q);
+}
+__device__ __forceinline__ void mg_take(const MgRing& g, int slot, int lane, bool in, MgCoef& k) {
+  k.none();
+  if (in) {
+    const float4 v = g.st[slot][lane];
+    k.c = v.x;
+    k.e = v.y;
+    k.n = v.z;
+    k.ne = v.w;
+    k.nw = g.nw[slot][lane];
+    k.f = g.f[slot][lane];
+  }
+}
 
 // A 9-point stencil in place (its own row's entries and the row below's).
 struct MgStencil {
@@ -506,10 +537,11 @@ __global__ void __launch_bounds__(kMgWarps * 32, kMgBlocks) mgf_down_kernel(int 
   const float* ps = P + (size_t)s * 4 * N;
   const bool mine = lane >= 3 && lane < 29 && m.x < W;
   auto inside = [&](int y) { return m.in && y > 0 && y < nf; };
-  // rows t .. t + 2 are loaded ahead
-  MgCoef k0, k1, k2, kn, kq;  // rows t, t - 1, t - 2, t + 1, t + 2
+  __shared__ MgRing rings[kMgWarps];
+  MgRing& ring = rings[threadIdx.x >> 5];
+  MgCoef k0, k1, k2;          // rows t, t - 1, t - 2
   float r0, r1 = 0.f;         // reciprocal divisors of rows t, t - 1
-  float dn = 1.f, dq = 1.f;   // divisors of rows t + 1, t + 2 (OD)
+  float dn = 1.f, dq = 1.f;   // divisors of rows t, t + 1 (OD)
   MgStencil sa, sb;           // rows t - 1, t - 2
   MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};  // sweep 1: rows t, t - 1, t - 2
   MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};  // sweep 2: rows t - 1, t - 2, t - 3
@@ -519,18 +551,24 @@ __global__ void __launch_bounds__(kMgWarps * 32, kMgBlocks) mgf_down_kernel(int 
   k1.none();
   k2.none();
   sb.set(k1, k2);
-  kn.load(st, nws, f, inside(t), q);
-  kq.load(st, nws, f, inside(t + 1), q + W);
+#pragma unroll
+  for (int k = 0; k < kMgAhead; ++k) {
+    if (inside(t + k)) mg_fetch(ring, k, lane, st, nws, f, q + k * W);
+    mg_commit();
+  }
   if (OD) {
     if (inside(t)) dn = ds[q];
     if (inside(t + 1)) dq = ds[q + W];
   }
+  int slot = 0;
 #pragma unroll 2
-  for (; t < m.y1 + 3; ++t, q += W) {
-    k0 = kn;
+  for (; t < m.y1 + 3; ++t, q += W, slot = (slot + 1) & (kMgRing - 1)) {
+    mg_wait();
+    mg_take(ring, slot, lane, inside(t), k0);
     r0 = __fdividef(1.f, OD ? dn : k0.c);
-    kn = kq;
-    kq.load(st, nws, f, inside(t + 2), q + 2 * W);
+    if (t + kMgAhead < m.y1 + 3 && inside(t + kMgAhead))
+      mg_fetch(ring, (slot + kMgAhead) & (kMgRing - 1), lane, st, nws, f, q + kMgAhead * W);
+    mg_commit();
     if (OD) {
       dn = dq;
       dq = inside(t + 2) ? ds[q + 2 * W] : 1.f;
@@ -622,9 +660,11 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
     auto coarse = [&](int J) {
       return m.in && J > 0 && J < nf / 2 ? uc[J * Wc + I0] + uc[J * Wc + I1] : 0.f;
     };
-    MgCoef k0, k1, k2, kn, kq;     // rows t, t - 1, t - 2, t + 1, t + 2
+    __shared__ MgRingUp rings[kMgWarps];
+    MgRingUp& ring = rings[threadIdx.x >> 5];
+    MgCoef k0, k1, k2;             // rows t, t - 1, t - 2
     float r0, r1 = 0.f, r2 = 0.f;  // reciprocal divisors of rows t, t - 1, t - 2
-    float dn = 1.f, dq = 1.f, un = 0.f, uq = 0.f;  // rows t + 1, t + 2
+    float dn = 1.f, dq = 1.f;      // rows t, t + 1
     MgStencil sa, sb;              // rows t - 1, t - 2
     MgTri a0, a1{0.f, 0.f, 0.f}, a2{0.f, 0.f, 0.f};  // the starting values: rows t, t - 1, t - 2
     MgTri b1, b2{0.f, 0.f, 0.f}, b3{0.f, 0.f, 0.f};  // sweep 1: rows t - 1, t - 2, t - 3
@@ -633,10 +673,19 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
     k1.none();
     k2.none();
     sb.set(k1, k2);
-    kn.load(st, nws, f, inside(t), q);
-    kq.load(st, nws, f, inside(t + 1), q + W);
-    if (inside(t)) un = ui[q];
-    if (inside(t + 1)) uq = ui[q + W];
+    auto fetch = [&](int y, int slot, int node) {
+      if (inside(y)) {
+        mg_fetch(ring, slot, lane, st, nws, f, node);
+        mg_cp<4>(&ring.u[slot][lane], ui + node);
+        if (rs) mg_cp<8>(&ring.r[slot][lane], rs + node);
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < kMgAhead; ++k) {
+      fetch(t + k, k, q + k * W);
+      mg_commit();
+    }
+    int slot = 0;
     float ha = 0.f, hb = 0.f, hc = 0.f;  // coarse rows t / 2, t / 2 + 1, t / 2 + 2
     if constexpr (OD) {
       if (inside(t)) dn = ds[q];
@@ -645,10 +694,15 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
       ha = coarse(t >> 1);
       hb = coarse((t >> 1) + 1);
     }
-    double rn = 0.0, rq = 0.0;  // r of rows t - 2, t - 1
+    double ra = 0.0, rb = 0.0;  // r of rows t - 1, t - 2
 #pragma unroll 2
-    for (; t < m.y1 + 2; ++t, q += W) {
-      k0 = kn;
+    for (; t < m.y1 + 2; ++t, q += W, slot = (slot + 1) & (kMgRing - 1)) {
+      mg_wait();
+      mg_take(ring, slot, lane, inside(t), k0);
+      const float un = inside(t) ? ring.u[slot][lane] : 0.f;
+      const double rt = rs && mine && inside(t) && t >= m.y0 && t < m.y1 ? ring.r[slot][lane] : 0.0;
+      if (t + kMgAhead < m.y1 + 2) fetch(t + kMgAhead, (slot + kMgAhead) & (kMgRing - 1), q + kMgAhead * W);
+      mg_commit();
       r0 = __fdividef(1.f, OD ? dn : k0.c);
       float v0 = 0.f;
       if constexpr (OD) {
@@ -667,18 +721,13 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
         if (!inside(t)) v0 = 0.f;
       }
       a0.set(v0);
-      const double rv = rn;
-      kn = kq;
-      un = uq;
-      kq.load(st, nws, f, inside(t + 2), q + 2 * W);
-      uq = inside(t + 2) ? ui[q + 2 * W] : 0.f;
-      rn = rq;
-      if (rs) rq = mine && inside(t) && t >= m.y0 && t < m.y1 ? rs[q] : 0.0;
       sa.set(k1, k2);
       b1.set(inside(t - 1) ? a1.c + mg_omega<OD>(0) * (k1.f - sa.apply(a2, a1, a0)) * r1 : 0.f);
       const float v = inside(t - 2) ? b2.c + mg_omega<OD>(1) * (k2.f - sb.apply(b3, b2, b1)) * r2 : 0.f;
       if (mine && t - 2 >= m.y0 && t - 2 < m.y1) uo[q - 2 * W] = v;
-      if (rs) acc = fma(rv, widen(v), acc);
+      if (rs) acc = fma(rb, widen(v), acc);
+      rb = ra;
+      ra = rt;
       a2 = a1;
       a1 = a0;
       b3 = b2;
