@@ -141,13 +141,28 @@ __device__ __forceinline__ int ring(int x, int RW) { return x >= RW ? x - RW : x
 // FP32: the hardware reciprocal square root (a few ulp).  FP64: the FP32
 // estimate y and one cubic step y (1 + e / 2 + 3 e^2 / 8), e = 1 - a y^2 (|e|
 // below 2^-21, the next term of the series 5 e^3 / 16 below 2^-64): five
-// FP64 operations on a part whose FP64 pipe is narrow, and the range test on
+// FP64 operations on a part whose FP64 pipe is narrow; the range test and the
+// estimate's conversions (which would take two more of its slots) work on
 // the bits.  Outside the FP32 range the library routines are used.
 __device__ __forceinline__ float pivot_rsqrt(float a) { return rsqrtf(a); }
+// Exponents -90 .. 90 (a is positive).
+__device__ __forceinline__ bool in_f32_range(double a) {
+  return (unsigned)__double2hiint(a) - (933u << 20) <= (180u << 20);
+}
+// A positive double in that range rounded to FP32 (to nearest even), and a
+// positive normal FP32 value as a double.
+__device__ __forceinline__ float near_f32(double a) {
+  const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
+  const unsigned m = __funnelshift_l(lo, hi, 3) + 0x40000000u, rest = lo & 0x1fffffffu;
+  return __uint_as_float(m + (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u));
+}
+__device__ __forceinline__ double exact_f64(float a) {
+  const unsigned b = __float_as_uint(a);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
 __device__ __forceinline__ double pivot_rsqrt(double a) {
-  // exponents -90 .. 90 (a is positive here)
-  if ((unsigned)__double2hiint(a) - (933u << 20) > (180u << 20)) return 1.0 / sqrt(a);
-  const double y = (double)rsqrtf((float)a);
+  if (!in_f32_range(a)) return 1.0 / sqrt(a);
+  const double y = exact_f64(rsqrtf(near_f32(a)));
   const double e = fma(-a * y, y, 1.0);
   return fma(y * e, fma(e, 0.375, 0.5), y);
 }

@@ -9,7 +9,7 @@
 //      lane one row (RS = 1, half bandwidths up to 32) or two below it; the
 //      multipliers l and the unscaled columns c = l d go to shared memory,
 //      l also to global scratch;
-//   2. all warps update the trailing window, W -= l c^T, in 2 x 2 tiles,
+//   2. all warps update the trailing window, W -= l c^T, in 1 x 2 tiles,
 //      while the last warp clears the retired ring rows and writes the next
 //      8 rows, whose values it loaded one block earlier.
 // The back substitution is warp 0's, with the factor blocks copied back two
@@ -18,14 +18,14 @@
 // What bounds it is the FP64 pipe (one warp instruction per 16 clocks of an
 // SM, whatever its lanes do), so the split is made for full lanes and few
 // FP64 instructions: a right-hand side that rides along as a row costs none
-// in the panel, 1 / d takes three (see recip), 2 x 2 tiles waste 3 % of the
-// lanes of a 32-row triangle where 4 x 4 tiles in whole rounds of a warp
-// waste 35 %, and their four loads per four FMAs cost nothing here (shared
-// memory serves a tile's operands in a tenth of its FMAs' time).  Four warps
+// in the panel, 1 / d takes three (see recip), 1 x 2 tiles fill 272 of 288
+// lanes of a 32-row triangle's rounds where 4 x 4 tiles in whole rounds of a
+// warp fill 36 of 64, and their two loads per two FMAs cost nothing here
+// (shared memory serves a tile's operands in a tenth of its FMAs' time).  Four warps
 // per system, not one, because the batches are small: 512 systems leave an
 // SM three or four, and one warp alone reaches a quarter of the pipe.
 // 512 coarse systems of 32^2 cells with moments: 2.79 ms with a warp per
-// sample and column blocks of 16, 1.54 ms here.
+// sample and column blocks of 16, 1.45 ms here.
 //
 // Row generator interface (Gen): typename Raw; load(r, Raw&); template
 // make<double, 1>(r, raw, e, rhs) as in band_block.cuh; mx.
@@ -72,13 +72,12 @@ __device__ inline CtaBand make_cta_band(unsigned char* smem, int b) {
 }
 
 // 1 / d: the FP32 reciprocal (relative error below 2^-22) with one cubic
-// step r (1 + e + e^2), e = 1 - d r, whose error e^3 is below 2^-66; outside
-// the FP32 range the FP64 division.
+// step r (1 + e + e^2), e = 1 - d r, whose error e^3 is below 2^-66; the
+// conversions work on the bits (band_block.cuh).  Outside the FP32 range the
+// FP64 division.
 __device__ __forceinline__ double recip(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d);
-  // exponents -90 .. 90 (d is positive here)
-  if (hi - (933u << 20) > (180u << 20)) return 1.0 / d;
-  const double r = (double)__frcp_rn((float)d);
+  if (!in_f32_range(d)) return 1.0 / d;
+  const double r = exact_f64(__frcp_rn(near_f32(d)));
   const double e = fma(-d, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
@@ -129,7 +128,7 @@ __device__ bool cta_band_solve(const Gen& gen, int n, int b, const CtaBand& s, d
   typename Gen::Raw next;  // of row K + NB + b + lane (lanes 0..7 of the filling warp)
   if (filler && lane < NB && NB + b + lane < n) gen.load(NB + b + lane, next);
   __syncthreads();
-  const int nt2 = (b + 1) >> 1, ntiles = nt2 * (nt2 + 1) / 2;
+  const int ntiles = ((b >> 1) + 1) * ((b >> 1) + (b & 1));
   int kslot = 0;
   for (int kb = 0; kb < nkb; ++kb, kslot = ring(kslot + NB, RW)) {
     const int K = kb * NB;
@@ -190,31 +189,25 @@ __device__ bool cta_band_solve(const Gen& gen, int n, int b, const CtaBand& s, d
     }
     __syncthreads();
     // ---- trailing update: rows and columns K + NB .. K + NB + b - 1
+    // in 1 x 2 tiles: rows 2 R and 2 R + 1 have R + 1 pairs of columns each,
+    // R (R + 1) tiles before them
     for (int t = tid; t < ntiles; t += kCtaThreads) {
-      int ti = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
-      if ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-      if (ti * (ti + 1) / 2 > t) --ti;
-      const int tj = t - ti * (ti + 1) / 2;
-      const int i0 = 2 * ti, j0 = 2 * tj;
-      double* w0 = s.W + ring(kslot + NB + i0, RW) * P + (i0 - j0);              // (i0, j0); (i0, j0 + 1) at -1
-      double* w1 = s.W + ring(kslot + NB + min(i0 + 1, b - 1), RW) * P + (i0 + 1 - j0);
-      const bool up = ti != tj, lo = i0 + 1 < b;
-      double v00 = w0[0], v01 = up ? w0[-1] : 0.0, v10 = lo ? w1[0] : 0.0, v11 = lo ? w1[-1] : 0.0;
+      int R = (int)((sqrtf(4.0f * t + 1.0f) - 1.0f) * 0.5f);
+      if ((R + 1) * (R + 2) <= t) ++R;
+      if (R * (R + 1) > t) --R;
+      const int rem = t - R * (R + 1), odd = rem > R, i = 2 * R + odd, j = 2 * (rem - odd * (R + 1));
+      double* w = s.W + ring(kslot + NB + i, RW) * P + (i - j);  // (i, j); (i, j + 1) at -1
+      const bool two = j + 1 <= i;
+      double v0 = w[0], v1 = two ? w[-1] : 0.0;
 #pragma unroll
       for (int p = 0; p < NB; ++p) {
-        const double2 l2 = *reinterpret_cast<const double2*>(s.Lp + p * PB + i0);
-        const double2 c2 = *reinterpret_cast<const double2*>(s.Cp + p * PB + j0);
-        v00 = fma(-l2.x, c2.x, v00);
-        v01 = fma(-l2.x, c2.y, v01);
-        v10 = fma(-l2.y, c2.x, v10);
-        v11 = fma(-l2.y, c2.y, v11);
+        const double l = -s.Lp[p * PB + i];
+        const double2 c2 = *reinterpret_cast<const double2*>(s.Cp + p * PB + j);
+        v0 = fma(l, c2.x, v0);
+        v1 = fma(l, c2.y, v1);
       }
-      w0[0] = v00;
-      if (up) w0[-1] = v01;
-      if (lo) {
-        w1[0] = v10;
-        w1[-1] = v11;
-      }
+      w[0] = v0;
+      if (two) w[-1] = v1;
     }
     // ---- the retired rows' slots take rows K + NB + b ..  (RW = NB + b
     // rounded up: slots past K + NB + b - 1 stay free until then)
