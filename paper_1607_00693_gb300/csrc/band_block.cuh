@@ -476,10 +476,11 @@ __host__ __device__ constexpr bool tiles8_form() {
 // Lane gl's tile.  The lane order puts tiles whose window rows share a bank
 // group (ti - g0 mod 8 alike, kBlkPad) into different quarters of the warp
 // where their number allows it.
+template <bool TIGHT>
 __device__ __forceinline__ Tile8 tile8_of(int gl, int b) {
   Tile8 t;
   const int sh = 4 * (gl & 7);
-  if (b > 32) {
+  if (!TIGHT && b > 32) {
     t.ti = ((gl < 8 ? 0x12343210u : 0x04443432u) >> sh) & 15;
     const int tj = ((gl < 8 ? 0x12300000u : 0x02432111u) >> sh) & 15;
     t.diag = t.ti == tj;
@@ -533,6 +534,8 @@ __device__ __forceinline__ void ld_pairs(const float* p, uint64_t& a, uint64_t& 
 
 // Window rows [K + 8, K + 8 + nt) -= the panel's products; tslot: ring slot
 // of the tile's first row (8-row tiles never wrap: RW is a multiple of 8).
+// TIGHT: b <= 32 (only the smaller tiles are compiled).
+template <bool TIGHT>
 __device__ __forceinline__ void tiles8_update(const Tile8& t, int b, const float* __restrict__ pt,
                                               const BlkSmem<float>& s, int tslot, int nt) {
   if (t.ng == 0 || 8 * t.ti >= nt) return;
@@ -543,7 +546,7 @@ __device__ __forceinline__ void tiles8_update(const Tile8& t, int b, const float
   float* w = s.wnd + kWndOff + wnd_row<8>(tslot, s.PW) + (8 * t.ti - 4 * t.g0 - 3);
   const int ws = s.PW + 1;  // to the same columns of the next row
   uint64_t r[4], c[4];
-  if (b > 32) {
+  if (!TIGHT && b > 32) {
     const float* pc = pt + RP - 8 - 4 * t.g0;  // columns 4 g0 + 7 .. 4 g0
     Pair2<4, 4> A;
 #pragma unroll
@@ -648,14 +651,14 @@ __device__ __forceinline__ void tiles1x4_update(const double* __restrict__ pt, c
 // over the rows it finishes, y0 y0, y0 y1, y0 y2, y1 y1, y1 y2, y2 y2 and
 // y3 y0, y3 y1, y3 y2 into yy[0..8] (FP64), for the caller to sum over the
 // group.
-template <int G, typename T, int NR, int RPL, class Gen, typename TS, bool FWD_ONLY = false>
+template <int G, typename T, int NR, int RPL, class Gen, typename TS, bool FWD_ONLY = false, bool TIGHT = false>
 __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<T>& s, T* __restrict__ Lg,
                           TS* __restrict__ yg, int gl, double* yy = nullptr, int store_from = 0) {
   constexpr int NB = G / 2;
   const int LBS = (NB + bmax) * NB;
   const int RW = s.RW;
   constexpr bool kTiles8 = tiles8_form<G, T, RPL, TS>();
-  const Tile8 tile = kTiles8 ? tile8_of(gl, b) : Tile8{0, 0, 0, false};
+  const Tile8 tile = kTiles8 ? tile8_of<TIGHT>(gl, b) : Tile8{0, 0, 0, false};
   blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + wnd_row<NB>(RW, s.PW))) / 16), gl);
   __syncwarp();
   int fail = -1;
@@ -788,7 +791,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     const int nt = np - nb;
     if constexpr (kTiles8) {
       // (nt > 0 only after a full block: nb = NB)
-      if (nt > 0) tiles8_update(tile, b, pt, s, ring(kslot + NB + 8 * tile.ti, RW), nt);
+      if (nt > 0) tiles8_update<TIGHT>(tile, b, pt, s, ring(kslot + NB + 8 * tile.ti, RW), nt);
     } else if constexpr (sizeof(T) == 8) {
       if (nt > 0) tiles1x4_update<G>(pt, s, ring(kslot + nb, RW), nt, nb, gl);
     } else if (nt > 0) {

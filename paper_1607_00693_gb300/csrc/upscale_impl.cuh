@@ -547,9 +547,15 @@ __device__ inline BlkSmem<TK> unit_blk(unsigned char* base, const TcSmem& tsm, i
 // in mma accumulator registers, trailing update on the tensor cores with
 // operands split into TC TF32 parts, column blocks of 8), b <= 40; the
 // substitutions read its 8-column blocks.
-template <typename TK, typename TA, int RPL, int G, int MODE, bool PG, bool OSC = false, int TC = 0>
+// TIGHT (FP32 form, forward-only route, two units per warp, half bandwidths
+// 25..32): only the smaller update tiles are compiled, 128 registers, so
+// that four blocks fit an SM instead of three (their windows take 54 KB).
+// 2048^2, H/h = 32, 4 samples: 2.27 -> 2.08 ms.  (The back-substitution
+// route spills more at 128 registers: 345^2, H/h = 23, oscillatory data, 1.36
+// -> 1.39 ms; it keeps three blocks.)
+template <typename TK, typename TA, int RPL, int G, int MODE, bool PG, bool OSC = false, int TC = 0, bool TIGHT = false>
 __global__ void __launch_bounds__(upscale_warps(sizeof(TK) == 8, G) * 32,
-                                  sizeof(TK) == 4 ? (G == 16 ? 3 : 4) : (G == 8 ? 6 : G == 16 ? 3 : 2))
+                                  sizeof(TK) == 4 ? (G == 16 && !TIGHT ? 3 : 4) : (G == 8 ? 6 : G == 16 ? 3 : 2))
 upscale_kernel(UpscaleArgs A) {
   // the oscillatory data run every cell by back substitution (one launch)
   static_assert(!OSC || MODE == kModeAll, "oscillatory data: back-substitution route only");
@@ -665,7 +671,7 @@ upscale_kernel(UpscaleArgs A) {
           fail = tc_factor<4, true, Gen, TS, TC>(pg, g.n, g.b, A.bmax, tsm, reinterpret_cast<float*>(Lg), psi0, gl,
                                                  yy);
         else
-          fail = blk_factor<G, TK, 4, RPL, Gen, TS, true>(pg, g.n, g.b, A.bmax, sm, Lg, psi0, gl, yy);
+          fail = blk_factor<G, TK, 4, RPL, Gen, TS, true, TIGHT>(pg, g.n, g.b, A.bmax, sm, Lg, psi0, gl, yy);
       }
     } else if (g.n > 0) {
       // without refinement only psi on the cell's nodes is read: the rows
@@ -675,7 +681,7 @@ upscale_kernel(UpscaleArgs A) {
       if constexpr (TC > 0)
         fail = tc_factor<3, false, Gen, TS, TC>(pg, g.n, g.b, A.bmax, tsm, reinterpret_cast<float*>(Lg), psi0, gl);
       else
-        fail = blk_factor<G, TK, 3, RPL>(pg, g.n, g.b, A.bmax, sm, Lg, psi0, gl, nullptr, need_from);
+        fail = blk_factor<G, TK, 3, RPL, Gen, TS, false, TIGHT>(pg, g.n, g.b, A.bmax, sm, Lg, psi0, gl, nullptr, need_from);
       // the factor-and-refine form (FP32 factor, FP64 solutions) calls the
       // substitutions out of line: one copy of each for all its passes
       constexpr bool outlined = sizeof(TK) == 4 && std::is_same<TA, double>::value;
@@ -1001,9 +1007,9 @@ static void patch_limits(const stomsfem_grid* g, int max_o, int* nmax, int* bmax
   *bmax = m + 1;
 }
 
-template <typename TK, typename TA, int RPL, int G, int MODE, bool PG, bool OSC = false, int TC = 0>
+template <typename TK, typename TA, int RPL, int G, int MODE, bool PG, bool OSC = false, int TC = 0, bool TIGHT = false>
 static int launch_upscale(const UpscaleArgs& A, long long max_blocks, cudaStream_t st) {
-  auto kern = upscale_kernel<TK, TA, RPL, G, MODE, PG, OSC, TC>;
+  auto kern = upscale_kernel<TK, TA, RPL, G, MODE, PG, OSC, TC, TIGHT>;
   constexpr int WPB = upscale_warps(sizeof(TK) == 8, G);
   // (oscillatory data: each unit's edge tables after all the windows)
   const size_t unit_smem = TC > 0 ? kTcSmemWarp : blk_smem_bytes<TK>(G / 2, A.bmax);
@@ -1028,6 +1034,8 @@ static int launch_rpl(const UpscaleArgs& A, long long max_blocks, cudaStream_t s
   if (rpl <= 1) return launch_upscale<TK, TA, 1, G, MODE, PG, OSC>(A, max_blocks, st);
   if (rpl == 2) return launch_upscale<TK, TA, 2, G, MODE, PG, OSC>(A, max_blocks, st);
   if constexpr (G > 8) {
+    if constexpr (G == 16 && sizeof(TK) == 4 && sizeof(TA) == 4 && MODE == kModeFwd)
+      if (rpl == 3 && A.bmax <= 32) return launch_upscale<TK, TA, 3, G, MODE, PG, OSC, 0, true>(A, max_blocks, st);
     if (rpl == 3) return launch_upscale<TK, TA, 3, G, MODE, PG, OSC>(A, max_blocks, st);
   }
   if constexpr (G == 16) {
@@ -1203,10 +1211,13 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
         upscale_cell_lists_kernel<<<1, kListThreads, 0, st>>>(oversample, ncell, mo, sorted ? 1 : 0, list0, list1, listall,
                                                     counts);
         STOMSFEM_TRY_CUDA(cudaGetLastError());
+        // (these patches are the cells themselves: half bandwidth rho)
         A.cell_list = list0;
         A.cell_count = counts;
+        A.bmax = A.rho;
         rc = launch_fp32<float, kModeFwd, PG, OSC>(engine, A, mb, st);
         if (rc) return rc;
+        A.bmax = bmax;
         A.cell_list = list1;
         A.cell_count = counts + 1;
         return launch_fp32<float, kModeRest, PG, OSC>(engine, A, mb, st);
