@@ -465,12 +465,10 @@ struct Tile8 {
 // 1024^2, H/h = 32, oversampling 0..4, 32 samples: 10.40 -> 8.67 ms; 2048^2,
 // contrast 1e4, no oversampling, 4 samples: 2.89 -> 2.27 ms; 345^2, H/h =
 // 23, Petrov-Galerkin with oscillatory data, 37 samples: 1.92 -> 1.66 ms.
-// The form with FP64 solutions (refinement) keeps the 4 x 4 tiles: 14.1 ms
-// with either for 8 samples of the first, the larger code costing what the
-// tiles save.
-template <int G, typename T, int RPL, typename TS>
+// With refinement, 8 samples of the first: 9.46 -> 9.18 ms.
+template <int G, typename T, int RPL>
 __host__ __device__ constexpr bool tiles8_form() {
-  return G == 16 && sizeof(T) == 4 && RPL == 3 && sizeof(TS) == 4;
+  return G == 16 && sizeof(T) == 4 && RPL == 3;
 }
 
 // Lane gl's tile.  The lane order puts tiles whose window rows share a bank
@@ -657,7 +655,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
   constexpr int NB = G / 2;
   const int LBS = (NB + bmax) * NB;
   const int RW = s.RW;
-  constexpr bool kTiles8 = tiles8_form<G, T, RPL, TS>();
+  constexpr bool kTiles8 = tiles8_form<G, T, RPL>();
   const Tile8 tile = kTiles8 ? tile8_of<TIGHT>(gl, b) : Tile8{0, 0, 0, false};
   blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + wnd_row<NB>(RW, s.PW))) / 16), gl);
   __syncwarp();
