@@ -1967,8 +1967,11 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
   }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   const int parts = pod->split ? 2 : 1;
-  // one unit per thread in the solves: the unrefined form of the shared basis
-  const bool per_thread = refine_iters == 0 && !d.per_l;
+  // one unit per thread in the solves: the unrefined form of the shared basis,
+  // beyond one tile of 32 samples (a warp per unit has the shorter chain, and
+  // the same bits: 5 samples of the 64^2 / 8^2 grid 38 us against 44, 31 samples 42
+  // against 44, 130 samples 80 against 67)
+  const bool per_thread = refine_iters == 0 && !d.per_l && S > 32;
   // one K step: the streaming product, whose G layout those solves read
   const bool stream_gemm = per_thread && d.Kp == kPodK;
   const size_t bytes_b = (size_t)d.Ppad * 128, bytes_a = (size_t)kPodTileM * 128;
@@ -2009,7 +2012,7 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
   A.err = pod->err;
   if (per_thread) {
     // one unit per thread (see pod_solve_units_kernel); the refined and the
-    // per-l forms keep a warp per unit
+    // per-l forms and small batches keep a warp per unit
     const long long work = (long long)(Spad / 32) * d.ncell;
     const long long most = (long long)sms * 3;
     STOMSFEM_TRY_CUDA(
@@ -2020,7 +2023,7 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
     long long blocks = (units + kPodSolveWarps - 1) / kPodSolveWarps;
     if (blocks > (long long)sms * 16) blocks = (long long)sms * 16;
     auto kern = A.refine > 0 ? (d.per_l ? pod_solve_kernel<true, true> : pod_solve_kernel<true, false>)
-                             : pod_solve_kernel<false, true>;
+                             : (d.per_l ? pod_solve_kernel<false, true> : pod_solve_kernel<false, false>);
     kern<<<(unsigned)blocks, kPodSolveWarps * 32, 0, st>>>(A);
   }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
