@@ -32,7 +32,14 @@ __device__ __forceinline__ void exp_table_fill(double* tab) {
 
 __device__ __forceinline__ double fexp(double t, const double* tab) {
   // |t| < 704 by the high word (0x40860000 is that of 704); also NaN
-  if (((unsigned)__double2hiint(t) & 0x7fffffffu) >= 0x40860000u) return exp(t);
+  const unsigned hi = (unsigned)__double2hiint(t);
+  if ((hi & 0x7fffffffu) >= 0x40860000u) {
+    // -746 (high word 0xc0875000) .. -infinity: the result is 0 (the smallest
+    // subnormal is exp(-745.1)); distant narrow bumps come here, and a warp that
+    // called the library for them spent longer there than on all near ones
+    if (hi >= 0xc0875000u && hi < 0xfff00000u) return 0.0;
+    return exp(t);
+  }
   const double ks = fma(t, k64ByLn2, kRoundShift);
   const int k = __double2loint(ks);        // low word = the rounded integer (two's complement)
   const double kd = ks - kRoundShift;

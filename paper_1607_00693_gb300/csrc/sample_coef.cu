@@ -3,10 +3,11 @@
 // The bumps are Gaussians on a tensor lattice, so
 //   z(x, y) = sum_bx gx_bx(x) * U_bx(y),   U_bx(y) = sum_by xi[by][bx] gy_by(y),
 // with gx_bx(x) = exp(-(x - cx_bx)^2 / w^2) (and gy likewise).  A block
-// handles strips of R element rows of kCoefCols columns: gy of the strip and
-// then U are built in shared memory, each thread keeps gx of its column in
-// registers and sweeps the strip, so the work per element is at most nbx
-// FMAs plus the final exponential (the table-driven FP64 exp of fexp.cuh).
+// handles strips of R element rows of up to kCoefCols columns: gy of the
+// strip and then U are built in shared memory, each thread keeps gx of its
+// column in registers and sweeps its rows of the strip, so the work per
+// element is at most nbx FMAs plus the final exponential (the table-driven FP64
+// exp of fexp.cuh).
 //
 // The FP64 kernel is bound by the FP64 pipe.  gx and gy depend on the place
 // only, so a block takes the samples of one place one after the other and
@@ -20,8 +21,12 @@
 // finite, sums them all.  On the 1024^2 workload (16 bumps a row, spacing one
 // width) 12 of 16 products remain, with 32 bumps of 3/4 of the spacing 15 of
 // 32.  Where a batch gives fewer than four pairs a block the strips get
-// shorter.
-// 32 samples of the 1024^2 grid: 2.25 -> 1.72 ms.
+// shorter.  A block's width follows the grid's (see the rule at the launch),
+// narrow ones split the rows among their warps and share gx through shared
+// memory, and the strips are of equal height.
+// 32 samples of the 1024^2 grid: 2.25 -> 1.65 ms; 60 samples of 513^2 1.31 ->
+// 1.05 ms (1.43 with 256 columns in every block and strips of 64 rows); 64
+// samples of 32^2 with 32^2 narrow bumps 161 -> 89 us (187 without shared gx).
 #include "common.cuh"
 #include "fexp.cuh"
 
@@ -32,7 +37,7 @@ constexpr int kCoefThreads = 128;
 constexpr size_t kCoefSmem = 48 * 1024;
 constexpr double kCoefReach = 7.5;  // in widths
 constexpr double kCoefAmp = 1e6;
-constexpr int kCoefCols = 256;      // columns and threads per block (FP64)
+constexpr int kCoefCols = 256;      // threads per block, and its columns at most (FP64)
 
 __host__ __device__ inline int coef_rows(int nbx, int nby) {
   int R = 128;
@@ -57,23 +62,22 @@ __device__ __forceinline__ double sigmoid_scaled(double clog, double e) {
 
 template <int NBX>
 __global__ void __launch_bounds__(kCoefCols, NBX <= 32 ? 2 : 1)
-sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int S, long long npair, double w, double scale,
+sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw, int share, int S, long long npair, double w, double scale,
                    double clog, double gain, const double* __restrict__ xi, double* __restrict__ a) {
   extern __shared__ double csm[];
   __shared__ int large;                  // an amplitude beyond kCoefAmp
   double* tab = csm;                     // [64] 2^(j/64)
   double* gy = csm + 64;                 // [nby][R]
   double* U = gy + (size_t)nby * R;      // [nbx][R]
+  double* gxs = U + (size_t)nbx * R;     // share: [nbx][32 kw]
   const int tid = threadIdx.x;
   const double h = 1.0 / nf;
   const double iw2 = 1.0 / (w * w);
   const double gain_z = kind == STOMSFEM_FIELD_EXP_SIGMOID ? 0.25 * fabs(clog * gain) : fabs(scale);
   const double amp = gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp;
-  // narrow grids: the threads split into row groups of a power of two of
-  // columns (32 at least)
-  int cols = kCoefCols;
-  while (cols > 32 && cols / 2 >= nf) cols >>= 1;
-  const int rg = tid / cols, nrg = kCoefCols / cols;
+  // the warps split into row groups of kw warps (32 kw columns); those left
+  // over only help with the tables
+  const int cols = 32 * kw, nrg = kCoefCols / cols, rg = tid / cols, col = tid - rg * cols;
   exp_table_fill(tab);
   // this block's (place, sample) pairs, the samples fastest
   const long long u0 = npair * blockIdx.x / gridDim.x, u1 = npair * (blockIdx.x + 1) / gridDim.x;
@@ -86,15 +90,21 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int S,
     __syncthreads();  // (the table; gy and U of the pair before are no longer read)
     if (t != place) {
       place = t;
-      const int strip = t % nstrip, col0 = t / nstrip * kCoefCols;
+      const int strip = t % nstrip, col0 = t / nstrip * cols;
       ey0 = strip * R;
       rows = min(R, nf - ey0);
-      ex = col0 + tid % cols;
+      ex = col0 + col;
       for (int q = tid; q < nby * rows; q += kCoefCols) {
         const int by = q / rows, r = q % rows;
         const double dy = (ey0 + r + 0.5) * h - (by + 0.5) / nby;
         gy[by * R + r] = fexp(-dy * dy * iw2, tab);
       }
+      if (share)
+        for (int q = tid; q < nbx * cols; q += kCoefCols) {
+          const int bx = q / cols;
+          const double dx = (col0 + (q - bx * cols) + 0.5) * h - (bx + 0.5) / nbx;
+          gxs[q] = fexp(-dx * dx * iw2, tab);
+        }
       const int e0 = ex & ~31;
       const float lo = (float)((e0 + 0.5) * h - kCoefReach * w), hi = (float)((e0 + 31.5) * h + kCoefReach * w);
       near = have = 0;
@@ -113,7 +123,7 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int S,
       if (!(fabs(acc) <= amp)) large = 1;
     }
     __syncthreads();
-    if (ex >= nf) continue;  // (every thread comes back to the barriers above)
+    if (ex >= nf || rg >= nrg) continue;  // (every thread comes back to the barriers above)
     const unsigned use = large ? 0xffffffffu : near;
     if (use & ~have) {
       have = use;
@@ -121,8 +131,12 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int S,
       for (int bx = 0; bx < NBX; ++bx) {
         gx[bx] = 0.0;
         if (bx < nbx && (use >> (bx / 4) & 1)) {
-          const double dx = (ex + 0.5) * h - (bx + 0.5) / nbx;
-          gx[bx] = fexp(-dx * dx * iw2, tab);
+          if (share) {
+            gx[bx] = gxs[bx * cols + col];
+          } else {
+            const double dx = (ex + 0.5) * h - (bx + 0.5) / nbx;
+            gx[bx] = fexp(-dx * dx * iw2, tab);
+          }
         }
       }
     }
@@ -226,17 +240,38 @@ static int sample_coef_impl(const stomsfem_grid* grid, const stomsfem_field* fie
   const size_t K = (size_t)field->nbx * field->nby;
   const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
   if (precision == STOMSFEM_FP64) {
-    const int nchunk = (grid->nf + kCoefCols - 1) / kCoefCols;
+    // columns of a block, 32 kw: the kw of the least work, in FP64 warp
+    // instructions per row and sample (an element takes about 14 and one for each
+    // bump within reach, U nbx nby / 32); 256 columns for every grid left a
+    // third of the lanes of 513 past its edge
+    int kw = 1, nchunk = 1;
+    double least = 0.0;
+    for (int k = kCoefCols / 32; k >= 1; --k) {
+      const int n = (grid->nf + 32 * k - 1) / (32 * k);
+      const double cost = n * (k * (14.0 + nbx) + nbx * field->nby / 32.0);
+      if (k == kCoefCols / 32 || cost < least) {
+        least = cost;
+        kw = k;
+        nchunk = n;
+      }
+    }
     auto pairs = [&](int r) { return (long long)((grid->nf + r - 1) / r) * nchunk * S; };
     const long long blocks = 2LL * sms;
     if (R > 64) R = 64;
     while (R > 8 && pairs(R) < 4 * blocks) R >>= 1;
+    // strips of equal height (77 rows as 39 + 38, not 64 + 13: the blocks' shares
+    // count pairs)
     const int nstrip = (grid->nf + R - 1) / R;
     const long long npair = pairs(R);
-    const size_t bytes = (64 + (size_t)(field->nbx + field->nby) * R) * sizeof(double);
+    R = (grid->nf + nstrip - 1) / nstrip;
+    // row groups share the bump values of their columns where these fit
+    const size_t own = (64 + (size_t)(field->nbx + field->nby) * R) * sizeof(double);
+    const size_t shared_gx = (size_t)nbx * 32 * kw * sizeof(double);
+    const int share = kw <= kCoefCols / 64 && own + shared_gx <= kCoefSmem;
+    const size_t bytes = own + (share ? shared_gx : 0);
     const unsigned grd = (unsigned)(npair < blocks ? npair : blocks);
 #define LAUNCH(N)                                                                                               \
-  sample_coef_kernel<N><<<grd, kCoefCols, bytes, st>>>(grid->nf, field->kind, nbx, field->nby, R, nstrip, S, npair, \
+  sample_coef_kernel<N><<<grd, kCoefCols, bytes, st>>>(grid->nf, field->kind, nbx, field->nby, R, nstrip, kw, share, S, npair, \
                                                        field->width, field->scale, field->contrast_log,         \
                                                        field->gain, xi, a)
     if (nbx <= 4) LAUNCH(4);

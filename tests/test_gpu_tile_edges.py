@@ -220,3 +220,20 @@ def test_sampling_large_and_non_finite_amplitudes():
     near = want < 1e300
     assert np.allclose(got[1][near], want[near], rtol=1e-10)
     assert np.isnan(got[2]).all()
+
+
+@pytest.mark.parametrize("nf,nbx,nby,width,S", [(33, 3, 4, 0.2, 300), (77, 16, 5, 0.06, 60), (97, 4, 3, 0.3, 150),
+                                                (130, 20, 8, 0.03, 40), (225, 2, 9, 0.4, 30)])
+def test_sampling_row_groups_and_strips(orc, nf, nbx, nby, width, S):
+    """Column groups of 1..8 warps with shared bump values, strips of uneven
+    rest and blocks that take several (place, sample) pairs; distant narrow
+    bumps whose values are zero."""
+    fld = dict(kind=api.FIELD_EXP, nbx=nbx, nby=nby, width=width, scale=0.7, contrast_log=0.0, gain=1.0)
+    xi = np.random.default_rng(nf).uniform(-1, 1, size=(S, nbx * nby))
+    ref = orc.sample_coef(nf, fld, xi)
+    a = torch.zeros((S, nf, nf), dtype=torch.float64, device=DEV)
+    api.stomsfem_sample_coef(api.grid(nf, 1), api.field_from_dict(fld), _t(xi), a)
+    x = (np.arange(nf) + 0.5) / nf
+    psi = [np.exp(-((x[:, None] - (np.arange(n) + 0.5) / n) / width) ** 2).sum(1).max() for n in (nbx, nby)]
+    eps = np.finfo(float).eps
+    assert np.max(np.abs(a.cpu().numpy() / ref - 1)) <= 4 * (0.7 * psi[0] * psi[1] * 8 * eps + 4 * eps)
