@@ -12,6 +12,7 @@
 
 #include "ckpt.cuh"
 #include "common.cuh"
+#include "tc_gemm.cuh"
 
 namespace stomsfem {
 
@@ -19,8 +20,8 @@ constexpr int kRiMaxDim = 16;         // interpolated directions per cell
 constexpr int kRiMaxNu = 8;           // degree per direction
 constexpr int kRiMaxNodes = kRiMaxNu + 1;
 constexpr int kRiMaxSlots = 64;       // sum over directions of (nu + 1)
-constexpr int kRiUnits = 256;         // units per CTA (one tile)
-constexpr int kRiThreads = 128;       // two units per thread
+constexpr int kRiThreads = 128;
+constexpr int kRiUnits = 2 * kRiThreads;  // units per CTA (one tile) at most: one or two a thread
 constexpr int kRiStagePitch = 15;     // floats per unit of the output staging (odd: no bank conflicts)
 constexpr int kRiMaxBlock = 16;       // grid points of the inner block (weights kept per unit)
 constexpr long long kRiMaxPoints = 2048;  // one family's table in shared memory, 64 B per point
@@ -224,15 +225,27 @@ __global__ void ri_gather_kernel(int n, const int32_t* __restrict__ list, const 
   }
 }
 
-// First tile of every family for S samples (tiles of kRiUnits units).
-__global__ void ri_tiles_kernel(int nfam, const RiFam* __restrict__ fam, int S, int* __restrict__ tile0) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// First tile of every family for S samples (tiles of `units` units), and the
+// direct-upscale count cleared; one warp.
+__global__ void ri_tiles_kernel(int nfam, const RiFam* __restrict__ fam, int S, int units, int* __restrict__ tile0,
+                                int32_t* __restrict__ count) {
+  const int lane = threadIdx.x;
   int t = 0;
-  for (int f = 0; f < nfam; ++f) {
-    tile0[f] = t;
-    t += (int)(((long long)S * fam[f].ncell + kRiUnits - 1) / kRiUnits);
+  for (int f0 = 0; f0 < nfam; f0 += 32) {
+    const int f = f0 + lane;
+    int n = f < nfam ? (int)(((long long)S * fam[f].ncell + units - 1) / units) : 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {  // inclusive sums
+      const int v = __shfl_up_sync(0xffffffffu, n, d);
+      if (lane >= d) n += v;
+    }
+    if (f < nfam) tile0[f + 1] = t + n;
+    t += __shfl_sync(0xffffffffu, n, 31);
   }
-  tile0[nfam] = t;
+  if (lane == 0) {
+    tile0[0] = 0;
+    *count = 0;
+  }
 }
 
 struct RiEvalArgs {
@@ -274,6 +287,7 @@ __device__ __forceinline__ void ri_values(const float* sx, const float* sw, floa
 // Direction of radix n at t: an inner direction multiplies the unit's
 // block weights sW[0..len) into sW[0..n len) (this direction slowest), an
 // outer one stores its values at its node slots of sL.
+template <int UN>
 __device__ __forceinline__ void ri_direction(bool inner, int n, const float* sx, const float* sw, float t,
                                              float* sW, float* sL, int slot0, int q, int len) {
   switch (n) {
@@ -283,10 +297,10 @@ __device__ __forceinline__ void ri_direction(bool inner, int n, const float* sx,
     ri_values<N>(sx, sw, t, l);                                                              \
     if (inner) {                                                                             \
       _Pragma("unroll") for (int j = N - 1; j >= 1; --j) for (int i = 0; i < len; ++i)       \
-          sW[(j * len + i) * kRiUnits + q] = l[j] * sW[i * kRiUnits + q];                     \
-      for (int i = 0; i < len; ++i) sW[i * kRiUnits + q] *= l[0];                            \
+          sW[(j * len + i) * UN       + q] = l[j] * sW[i * UN       + q];                     \
+      for (int i = 0; i < len; ++i) sW[i * UN       + q] *= l[0];                            \
     } else {                                                                                 \
-      _Pragma("unroll") for (int j = 0; j < N; ++j) sL[(slot0 + j) * kRiUnits + q] = l[j];   \
+      _Pragma("unroll") for (int j = 0; j < N; ++j) sL[(slot0 + j) * UN       + q] = l[j];   \
     }                                                                                        \
     break;                                                                                   \
   }
@@ -297,79 +311,81 @@ __device__ __forceinline__ void ri_direction(bool inner, int n, const float* sx,
   }
 }
 
-// Sum over the family's grid for the thread's two units: outer index o
-// (the product of the outer directions' 1-d values, at the node slots
-// sO[o][k] of sL) times the NB inner points (block weights held in
-// registers), table rows broadcast from shared memory.
+// Sum over the family's grid for the thread's U units (unit tid + h
+// kRiThreads): outer index o (the product of the outer directions' 1-d values,
+// at the node slots sO[o][k] of sL) times the NB inner points (block weights
+// held in registers), table rows broadcast from shared memory.
 //
-// The loop is bound by its issue slots, so two entries of a table row share
-// an FMA (fma.rn.f32x2, each half rounded as a scalar FMA; the row's pairs
-// come as they lie in memory), with the units' weights kept as pairs of
-// equal halves: 4 loads, 2 products and 14 FMAs per grid point and two
-// units instead of 4, 2 and 28, the same bits.
-// 10^5 samples of the 64^2 / 8^2 grid, with the staged stores below: 1.31 ->
-// 1.18 ms (the pairs alone: 811 -> 666 M instructions at the same time).
-template <int NB>
+// Two entries of a table row share an FMA (fma.rn.f32x2, each half rounded
+// as a scalar FMA; the row's pairs come as they lie in memory).  What bounds
+// the loop then is shared memory (a broadcast 128-bit load still delivers 512
+// bytes to the warp's registers, 16 clocks of the SM a row, against 3.5 of the
+// FMA pipes a unit) and, with few warps, the latency of the next outer weight,
+// which is therefore formed one index ahead.  Weights as scalars, doubled where
+// used: half the registers of pairs.  Four units a thread take 167 registers
+// and leave too few warps: 448 us where two take 396 (40000 samples).
+// 10^5 samples of the 64^2 / 8^2 grid: 1.31 -> 1.18 ms with paired FMAs and
+// staged stores, 1.00 ms with the outer weights formed ahead, scalar block weights
+// and asynchronous copies of the table; one sample 42 -> 26 us.
+template <int NB, int U>
 __device__ __forceinline__ void ri_accumulate(const float4* __restrict__ sV, const float* __restrict__ sW,
                                               const float* __restrict__ sL, const uint8_t* __restrict__ sO,
-                                              const RiFam& F, int tid,
-                                              float (&acc0)[14], float (&acc1)[14]) {
-  uint64_t w0[NB], w1[NB], a0[7], a1[7];
+                                              const RiFam& F, int tid, uint64_t (&acc)[U][7]) {
+  float w[U][NB];
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    w0[b] = f2_both(sW[b * kRiUnits + tid]);
-    w1[b] = f2_both(sW[b * kRiUnits + tid + kRiThreads]);
-  }
+  for (int h = 0; h < U; ++h)
 #pragma unroll
-  for (int q = 0; q < 7; ++q) a0[q] = a1[q] = 0;
+    for (int b = 0; b < NB; ++b) w[h][b] = sW[b * (kRiThreads * U) + tid + h * kRiThreads];
   const int dout = F.ndim - F.din;
   const int nout = F.npts / NB;
   const ulonglong2* v = reinterpret_cast<const ulonglong2*>(sV);
   const uint8_t* so = sO;
-  for (int o = 0; o < nout; ++o) {
-    float b0 = 1.f, b1 = 1.f;
+  float wo[U], wn[U];  // outer weights of this index and of the next (its loads overlap the sums)
+  auto outer = [&](float (&t)[U]) {
+#pragma unroll
+    for (int h = 0; h < U; ++h) t[h] = 1.f;
     for (int k = 0; k < dout; ++k) {
-      const int sl = so[k] * kRiUnits + tid;
-      b0 *= sL[sl];
-      b1 *= sL[sl + kRiThreads];
+      const int sl = so[k] * (kRiThreads * U) + tid;
+#pragma unroll
+      for (int h = 0; h < U; ++h) t[h] *= sL[sl + h * kRiThreads];
     }
     so += dout;
-    const uint64_t bb0 = f2_both(b0), bb1 = f2_both(b1);
+  };
+  outer(wo);
+  for (int o = 0; o < nout; ++o) {
+    if (o + 1 < nout) outer(wn);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const uint64_t wa = f2_mul(bb0, w0[b]), wb = f2_mul(bb1, w1[b]);
       const ulonglong2 v0 = v[4 * b], v1 = v[4 * b + 1], v2 = v[4 * b + 2];
       const uint64_t v3 = v[4 * b + 3].x;
       const uint64_t e[7] = {v0.x, v0.y, v1.x, v1.y, v2.x, v2.y, v3};
 #pragma unroll
-      for (int q = 0; q < 7; ++q) {
-        a0[q] = f2_fma(wa, e[q], a0[q]);
-        a1[q] = f2_fma(wb, e[q], a1[q]);
+      for (int h = 0; h < U; ++h) {
+        const uint64_t wh = f2_both(wo[h] * w[h][b]);
+#pragma unroll
+        for (int q = 0; q < 7; ++q) acc[h][q] = f2_fma(wh, e[q], acc[h][q]);
       }
     }
     v += 4 * NB;
-  }
 #pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    acc0[2 * q] = f2_lo(a0[q]);
-    acc0[2 * q + 1] = f2_hi(a0[q]);
-    acc1[2 * q] = f2_lo(a1[q]);
-    acc1[2 * q + 1] = f2_hi(a1[q]);
+    for (int h = 0; h < U; ++h) wo[h] = wn[h];
   }
 }
 
-// One tile of 256 units of one family; thread t takes units t and t + 128.
+// One tile of 128 U units of one family; thread t takes units t and (U = 2) t + 128.
 // Shared memory: the family's table [npts][16]; per unit (column q) the
 // inner block weights sW[b][q] (b < nb: products over the last din
 // directions) and the outer directions' 1-d values sL[slot][q]; the outer
 // node slots per outer index sO[o][k] (uniform over the tile).
+template <int U>
 __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
+  constexpr int UN = kRiThreads * U;
   extern __shared__ float4 sV[];
   __shared__ RiFam F;
   __shared__ float sx[kRiMaxSlots], sw[kRiMaxSlots];
   float* sW = reinterpret_cast<float*>(sV + (size_t)A.max_pts * 4);
-  float* sL = sW + (size_t)A.max_nb * kRiUnits;
-  uint8_t* sO = reinterpret_cast<uint8_t*>(sL + (size_t)A.max_slot * kRiUnits);
+  float* sL = sW + (size_t)A.max_nb * UN;
+  uint8_t* sO = reinterpret_cast<uint8_t*>(sL + (size_t)A.max_slot * UN);
   const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   int lo = 0, hi = A.nfam;  // tile0[lo] <= tile < tile0[hi]
@@ -380,14 +396,15 @@ __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
   }
   const int f = lo;
   if (tid == 0) F = A.fam[f];
-  if (tid < kRiMaxSlots) {
-    sx[tid] = A.x[f * kRiMaxSlots + tid];
-    sw[tid] = A.w[f * kRiMaxSlots + tid];
+  for (int i = tid; i < kRiMaxSlots; i += kRiThreads) {
+    sx[i] = A.x[f * kRiMaxSlots + i];
+    sw[i] = A.w[f * kRiMaxSlots + i];
   }
   __syncthreads();
   {
+    // (asynchronous: the weights below are made meanwhile)
     const float4* src = A.tab + F.pt0 * 4;
-    for (int i = tid; i < F.npts * 4; i += kRiThreads) sV[i] = src[i];
+    for (int i = tid; i < F.npts * 4; i += kRiThreads) tc::cp_async16(sV + i, src + i);
   }
   const int D = F.ndim, dout = F.ndim - F.din;
   // node slots of the outer directions per outer index (last outer direction fastest)
@@ -398,12 +415,12 @@ __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
       rem /= F.radix[k];
     }
   }
-  long long u[2];
-  bool run[2], out[2];
+  long long u[U];
+  bool run[U], out[U];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < U; ++h) {
     const int q = tid + h * kRiThreads;
-    const long long r = (long long)(tile - A.tile0[f]) * kRiUnits + q;
+    const long long r = (long long)(tile - A.tile0[f]) * UN + q;
     run[h] = r < (long long)A.S * F.ncell;
     out[h] = false;
     u[h] = 0;
@@ -421,13 +438,14 @@ __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
       const double t = xs[vars[k]];
       if (!(fabs(t) <= 1.0)) out[h] = true;
       const int n = F.radix[k];
-      ri_direction(k >= dout, n, sx + F.slot0[k], sw + F.slot0[k], (float)t, sW, sL, F.slot0[k], q, len);
+      ri_direction<UN>(k >= dout, n, sx + F.slot0[k], sw + F.slot0[k], (float)t, sW, sL, F.slot0[k], q, len);
       if (k >= dout) len *= n;
     }
   }
+  tc::cp_async_wait_all();
   __syncthreads();
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < U; ++h) {
     if (!run[h] || !out[h]) continue;
     if (A.list) {
       A.flag[u[h]] = 1;
@@ -439,17 +457,26 @@ __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
       for (int l = 0; l < 4; ++l) A.be[u[h] * 4 + l] = nanv;
     }
   }
-  float acc0[14], acc1[14];
-  switch (F.nb) {
+  uint64_t acc[U][7];
+#pragma unroll
+  for (int h = 0; h < U; ++h)
+#pragma unroll
+    for (int q = 0; q < 7; ++q) acc[h][q] = 0;
+  if (__any_sync(0xffffffffu, run[0])) {  // (a lane's further units lie behind its first)
+    switch (F.nb) {
 #define RI_NB(N) \
   case N:        \
-    ri_accumulate<N>(sV, sW, sL, sO, F, tid, acc0, acc1); \
+    ri_accumulate<N, U>(sV, sW, sL, sO, F, tid, acc); \
     break;
-    RI_NB(1) RI_NB(2) RI_NB(3) RI_NB(4) RI_NB(5) RI_NB(6) RI_NB(7) RI_NB(8)
-    RI_NB(9) RI_NB(10) RI_NB(12) RI_NB(14) RI_NB(15) RI_NB(16)
+      RI_NB(1) RI_NB(2) RI_NB(3) RI_NB(4) RI_NB(5) RI_NB(6) RI_NB(7) RI_NB(8)
+      RI_NB(9) RI_NB(10) RI_NB(12) RI_NB(14) RI_NB(15) RI_NB(16)
 #undef RI_NB
-    default:
-      for (int q = 0; q < 14; ++q) acc0[q] = acc1[q] = __int_as_float(0x7fc00000);  // unreachable sizes
+      default:
+#pragma unroll
+        for (int h = 0; h < U; ++h)
+#pragma unroll
+          for (int q = 0; q < 7; ++q) acc[h][q] = 0x7fc000007fc00000ull;  // unreachable sizes
+    }
   }
   // The 14 values of a unit go out as two runs of 80 and 32 bytes: through
   // shared memory (the table's, no longer needed), so that the lanes of a
@@ -457,26 +484,28 @@ __global__ void __launch_bounds__(kRiThreads) ri_eval_kernel(RiEvalArgs A) {
   // 28 stores of 32 sectors a warp, a third of the kernel's memory
   // instructions' time.
   __syncthreads();
-  float* stage = reinterpret_cast<float*>(sV);  // [kRiUnits][kRiStagePitch], then the unit ids (-1: none)
-  long long* su = reinterpret_cast<long long*>(stage + kRiUnits * kRiStagePitch);
+  float* stage = reinterpret_cast<float*>(sV);  // [UN][kRiStagePitch], then the unit ids (-1: none)
+  long long* su = reinterpret_cast<long long*>(stage + UN * kRiStagePitch);
 #pragma unroll
-  for (int q = 0; q < 14; ++q) {
-    stage[tid * kRiStagePitch + q] = acc0[q];
-    stage[(tid + kRiThreads) * kRiStagePitch + q] = acc1[q];
-  }
+  for (int h = 0; h < U; ++h)
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+    for (int q = 0; q < 7; ++q) {
+      stage[(tid + h * kRiThreads) * kRiStagePitch + 2 * q] = f2_lo(acc[h][q]);
+      stage[(tid + h * kRiThreads) * kRiStagePitch + 2 * q + 1] = f2_hi(acc[h][q]);
+    }
+#pragma unroll
+  for (int h = 0; h < U; ++h) {
     const bool ok = run[h] && !out[h];
     if (ok) A.flag[u[h]] = 0;
     su[tid + h * kRiThreads] = ok ? u[h] : -1;
   }
   __syncthreads();
-  for (int i = tid; i < kRiUnits * 10; i += kRiThreads) {
+  for (int i = tid; i < UN * 10; i += kRiThreads) {
     const int q = i / 10, k = i - q * 10;
     const long long un = su[q];
     if (un >= 0) A.Ke[(size_t)un * 10 + k] = (double)stage[q * kRiStagePitch + k];
   }
-  for (int i = tid; i < kRiUnits * 4; i += kRiThreads) {
+  for (int i = tid; i < UN * 4; i += kRiThreads) {
     const int q = i >> 2, k = i & 3;
     const long long un = su[q];
     if (un >= 0) A.be[(size_t)un * 4 + k] = (double)stage[q * kRiStagePitch + 10 + k];
@@ -715,9 +744,12 @@ extern "C" int stomsfem_ri_upscale(stomsfem_ri* ri, const double* xi, const doub
   o += 256;
   int32_t* list = reinterpret_cast<int32_t*>(ws + o);
   o += 256 * (((size_t)S * P.ncell * 4 + 255) / 256);
-  long long tiles = 0;
-  for (int f = 0; f < P.nfam; ++f) tiles += ((long long)S * P.F[f].ncell + kRiUnits - 1) / kRiUnits;
-  if (tiles > 0x7fffffffll) return set_error(STOMSFEM_EINVAL, "S too large for one call");
+  auto tiles_of = [&](int units) {
+    long long t = 0;
+    for (int f = 0; f < P.nfam; ++f) t += ((long long)S * P.F[f].ncell + units - 1) / units;
+    return t;
+  };
+  if (tiles_of(kRiUnits) > 0x7fffffffll) return set_error(STOMSFEM_EINVAL, "S too large for one call");
   int maxpts = 0, maxnb = 1, maxslot = 0;
   size_t maxouter = 0;
   for (int f = 0; f < P.nfam; ++f) {
@@ -727,9 +759,16 @@ extern "C" int stomsfem_ri_upscale(stomsfem_ri* ri, const double* xi, const doub
     maxouter = std::max(maxouter, (size_t)(P.F[f].npts / P.F[f].nb) * (P.F[f].ndim - P.F[f].din));
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  STOMSFEM_TRY_CUDA(cudaMemsetAsync(count, 0, 4, st));
-  ri_tiles_kernel<<<1, 32, 0, st>>>(P.nfam, ri->fam_d, S, tile0);
-  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  // Two units a thread halve the loads per unit, one leaves twice the warps.
+  // Few CTAs an SM, or small tables (where the weights and the copies of the
+  // table take the time) go faster with one: 64^2 / 8^2 grid, one against two
+  // units, 161 points a family: 700 samples 29.2, 30.4 us, 3000 51.3, 47.6,
+  // 40000 480, 396; coarser tables (tolerance 1e-2): 40000 213, 228.
+  const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
+  long long points = 0;
+  for (int f = 0; f < P.nfam; ++f) points += (long long)P.F[f].npts * P.F[f].ncell;
+  const int per_thread = tiles_of(kRiThreads) > 4LL * sms && points >= 100LL * P.ncell ? 2 : 1;
+  auto kern = per_thread == 2 ? ri_eval_kernel<2> : ri_eval_kernel<1>;
   RiEvalArgs A;
   A.xi = xi;
   A.K = P.K;
@@ -751,12 +790,19 @@ extern "C" int stomsfem_ri_upscale(stomsfem_ri* ri, const double* xi, const doub
   A.flag = fell_back;
   A.list = a ? list : nullptr;
   A.count = count;
-  const size_t stage = (sizeof(float) * kRiStagePitch + sizeof(long long)) * kRiUnits;
-  size_t smem = (size_t)maxpts * 64 + (size_t)(maxnb + maxslot) * kRiUnits * 4 + ((maxouter + 15) & ~(size_t)15);
-  if (smem < stage) smem = stage;
-  if (smem > 227 * 1024) return set_error(STOMSFEM_EINVAL, "RI tables need %zu B of shared memory", smem);
-  STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(ri_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ri_eval_kernel<<<(unsigned)tiles, kRiThreads, smem, st>>>(A);
+  auto smem_of = [&](int units) {
+    const size_t stage = (sizeof(float) * kRiStagePitch + sizeof(long long)) * units;
+    const size_t b = (size_t)maxpts * 64 + (size_t)(maxnb + maxslot) * units * 4 + ((maxouter + 15) & ~(size_t)15);
+    return b < stage ? stage : b;
+  };
+  if (smem_of(kRiUnits) > 227 * 1024)
+    return set_error(STOMSFEM_EINVAL, "RI tables need %zu B of shared memory", smem_of(kRiUnits));
+  const int units = kRiThreads * per_thread;
+  const size_t smem = smem_of(units);
+  STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ri_tiles_kernel<<<1, 32, 0, st>>>(P.nfam, ri->fam_d, S, units, tile0, count);
+  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  kern<<<(unsigned)tiles_of(units), kRiThreads, smem, st>>>(A);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   if (!a) return STOMSFEM_OK;
   return upscale_list_fp64(&ri->grid, a, S, list, count, Ke, be, ws + o, workspace_bytes - o, st);

@@ -237,3 +237,31 @@ def test_sampling_row_groups_and_strips(orc, nf, nbx, nby, width, S):
     psi = [np.exp(-((x[:, None] - (np.arange(n) + 0.5) / n) / width) ** 2).sum(1).max() for n in (nbx, nby)]
     eps = np.finfo(float).eps
     assert np.max(np.abs(a.cpu().numpy() / ref - 1)) <= 4 * (0.7 * psi[0] * psi[1] * 8 * eps + 4 * eps)
+
+
+@pytest.mark.parametrize("eps", [1e-3, 1e-2])
+def test_interpolation_units_per_thread(eps):
+    """A sample's interpolant does not depend on the batch: one and two units
+    a thread, ragged tiles, a parameter outside the box."""
+    from paper_1607_00693_gb300 import workloads as W
+    w = W.workload("msfem_64")
+    g = api.grid(w["nf"], w["nc"], w["f"])
+    h, _ = api.stomsfem_ri_build(g, api.field_from_dict(w["field"]), eps, 8, api.RI_LEGENDRE)
+    try:
+        S, cells = 5003, w["nc"] ** 2
+        xi = _t(W.draw_xi(w["field"], S, 3))
+        xi[0, 2] = 1.5
+        ref = None
+        for n in (S, 1, 2, 33, 130, 700):
+            Ke = torch.full((n, cells, 10), 7.0, dtype=torch.float64, device=DEV)
+            be = torch.full((n, cells, 4), 7.0, dtype=torch.float64, device=DEV)
+            fb = torch.full((n, cells), 9, dtype=torch.uint8, device=DEV)
+            api.stomsfem_ri_upscale(h, g, xi[:n].contiguous(), None, Ke, be, fb)
+            out = [t.cpu().numpy() for t in (Ke, be, fb)]
+            if ref is None:
+                ref = out
+                assert set(np.unique(out[2])) == {0, 2} and not out[2][1:].any()
+            for x, y in zip(out, ref):
+                assert np.array_equal(x, y[:n], equal_nan=x.dtype.kind == "f")
+    finally:
+        api.stomsfem_ri_destroy(h)
