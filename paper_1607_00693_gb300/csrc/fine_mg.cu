@@ -12,9 +12,8 @@
 // stencils again), damped Jacobi smoothing (two sweeps before
 // and after the coarse correction: a symmetric V-cycle, so the
 // preconditioner is symmetric positive definite and plain CG applies), and
-// 60 Jacobi sweeps on the coarsest grid.  Stencils are stored per level and
-// sample in FP32, structure of arrays over the full (nf_l+1)^2 node grid,
-// in symmetric form: five couplings per node (centre, east, north,
+// Chebyshev steps on the coarsest grid.  Stencils are stored per level and
+// sample in FP32, over the full (nf_l+1)^2 node grid, in symmetric form: five couplings per node (centre, east, north,
 // north-east, north-west), the other four read from the neighbours, so
 // every level's operator is exactly symmetric (boundary nodes carry zero
 // stencils and stay zero).
