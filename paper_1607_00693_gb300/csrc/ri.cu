@@ -326,7 +326,7 @@ __device__ __forceinline__ void ri_direction(bool inner, int n, const float* sx,
 // and leave too few warps: 448 us where two take 396 (40000 samples).
 // 10^5 samples of the 64^2 / 8^2 grid: 1.31 -> 1.18 ms with paired FMAs and
 // staged stores, 1.00 ms with the outer weights formed ahead, scalar block weights
-// and asynchronous copies of the table; one sample 42 -> 26 us.
+// and asynchronous copies of the table; one sample 42 -> 27 us.
 template <int NB, int U>
 __device__ __forceinline__ void ri_accumulate(const float4* __restrict__ sV, const float* __restrict__ sW,
                                               const float* __restrict__ sL, const uint8_t* __restrict__ sO,

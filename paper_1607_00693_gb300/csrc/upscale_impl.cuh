@@ -415,6 +415,7 @@ struct UpscaleArgs {
   double fq, fH2;             // f h^2 / 4 and f H^2 (load scaling)
   const int32_t* cell_list;   // optional: process only these cells (device list)
   const int32_t* cell_count;  // device length of cell_list
+  int32_t* next;              // optional: work taken past each warp's first item (zero at the launch)
   int blocks_per_sm_cap;      // host-side launch shape: at most this many resident CTAs per SM (0: occupancy)
   int order;                  // 0: cells fastest; 1: samples fastest, cells in list order
 };
@@ -443,7 +444,8 @@ enum { kModeAll = 0, kModeFwd = 1, kModeRest = 2 };
 // Cell lists of the launches (one block, counting sort): list0 the cells
 // without oversampling, list1 the others (cells with an oversampling
 // outside [0, max_o] included: the kernel flags them), listall every cell;
-// counts = {|list0|, |list1|, |listall|}.  sorted = 0: ascending cell index
+// counts = {|list0|, |list1|, |listall|, 0}; the last is the launch's work
+// counter (UpscaleArgs::next).  sorted = 0: ascending cell index
 // (listall unused); sorted = 1: by patch size, largest first (decreasing
 // oversampling, the flagged cells last), ascending cell index within one
 // size, so that a launch that walks its list with the samples fastest
@@ -481,6 +483,7 @@ upscale_cell_lists_kernel(const int8_t* __restrict__ oversample, int ncell, int 
     counts[0] = total[0];
     counts[1] = n1 + total[kListKeys - 1];
     counts[2] = sorted ? ncell : 0;
+    counts[3] = 0;
   }
   __syncthreads();
   const int n0 = total[0], flagged0 = base[kListKeys - 1];
@@ -590,7 +593,18 @@ upscale_kernel(UpscaleArgs A) {
   const long long npair = ((long long)A.S + GPW - 1) / GPW;
   const long long nlist = A.unit_list ? (long long)A.unit_count[0] : 0;
   const long long nwork = A.unit_list ? (nlist + GPW - 1) / GPW : npair * nlc;
-  for (long long w = gw; w < nwork; w += nw) {
+  // the next work item of this warp.  In fixed steps a launch of 2.2 items a
+  // warp (4 samples of 1024^2 in FP64, 8 with refinement) gave some warps the
+  // largest, a middle and a small patch, others two middle ones; taken as the
+  // warps come free, the sorted list evens out.  1024^2: FP64, 4 samples, 18.5
+  // -> 16.2 ms; FP32 + refinement, 8, 9.2 -> 8.2; 345^2 with oscillatory data 1.39 -> 1.35.
+  auto following = [&](long long w) {
+    if (!A.next) return w + nw;
+    int c = 0;
+    if (lane == 0) c = atomicAdd(A.next, 1);
+    return nw + __shfl_sync(0xffffffffu, c, 0);
+  };
+  for (long long w = gw; w < nwork; w = following(w)) {
     long long u;
     bool dup = false;  // this group mirrors another group's unit
     const int ci = A.order ? (int)(w / npair) : (int)(w % nlc);
@@ -1183,6 +1197,7 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   A.unit_count = nullptr;
   A.cell_list = nullptr;
   A.cell_count = nullptr;
+  A.next = nullptr;
   A.blocks_per_sm_cap = tune.blocks_per_sm;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // cell lists at the end of the workspace (the split launch, or the order
@@ -1198,6 +1213,7 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   int32_t* counts = listall + ncell;
   const bool sorted = tune.order != 0 && lists_fit;
   A.order = tune.order < 0 ? (sorted ? 1 : 0) : tune.order;
+  const bool by_counter = units < (1LL << 30);  // (a 32-bit counter of work items)
   const long long mb = lists_fit && max_blocks > slots2 / slots_per_block ? slots2 / slots_per_block : max_blocks;
   // the oscillatory data: every cell by back substitution in one launch
   // (the forward-only route never forms psi0, which the Petrov-Galerkin
@@ -1230,6 +1246,7 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     A.cell_list = listall;
     A.cell_count = counts + 2;
+    if (by_counter) A.next = counts + 3;
     max_blocks = mb;
   }
   if (precision == STOMSFEM_FP64)
