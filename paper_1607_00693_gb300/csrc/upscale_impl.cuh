@@ -415,7 +415,7 @@ struct UpscaleArgs {
   double fq, fH2;             // f h^2 / 4 and f H^2 (load scaling)
   const int32_t* cell_list;   // optional: process only these cells (device list)
   const int32_t* cell_count;  // device length of cell_list
-  int32_t* next;              // optional: work taken past each warp's first item (zero at the launch)
+  int32_t* next = nullptr;    // optional: work taken past each warp's first item (zero at the launch)
   int blocks_per_sm_cap;      // host-side launch shape: at most this many resident CTAs per SM (0: occupancy)
   int order;                  // 0: cells fastest; 1: samples fastest, cells in list order
 };
@@ -1197,7 +1197,6 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   A.unit_count = nullptr;
   A.cell_list = nullptr;
   A.cell_count = nullptr;
-  A.next = nullptr;
   A.blocks_per_sm_cap = tune.blocks_per_sm;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // cell lists at the end of the workspace (the split launch, or the order
