@@ -419,8 +419,8 @@ int stomsfem_fine_fem_workspace_size(const stomsfem_grid* grid, int32_t S, size_
 
 /* Standard Q1 FEM on the fine grid with zero Dirichlet data and load f
  * (element matrices a_e K_ref, load f h^2/4 per element corner).
- *  - nf <= 64: one warp per sample on the blocked banded Cholesky of the
- *    coarse solve (NaN for a sample whose matrix is not positive
+ *  - nf <= 64: one CTA per sample on the banded solver of the coarse
+ *    solve (NaN for a sample whose matrix is not positive
  *    definite); stream-ordered.
  *  - nf > 64 (nf = c 2^k, c <= 16): conjugate gradients in FP64 on all S
  *    samples at once, preconditioned by one multigrid V-cycle in FP32

@@ -748,8 +748,8 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
   return STOMSFEM_OK;
 }
 
-// Fine grids up to 64 elements per side: the blocked banded Cholesky (one
-// warp per sample); larger grids: multigrid-preconditioned CG (fine_mg.cu).
+// Fine grids up to 64 elements per side: the banded solver of band_cta.cuh
+// (one CTA per sample); larger grids: multigrid-preconditioned CG (fine_mg.cu).
 constexpr int kFineDirectMax = 64;
 
 extern "C" int stomsfem_fine_fem_workspace_size(const stomsfem_grid* grid, int32_t S, size_t* bytes) {

@@ -1,4 +1,5 @@
-// Simultaneous local upscaling: one warp per (sample, coarse cell) unit.
+// Simultaneous local upscaling of (sample, coarse cell) units: two or four
+// units of one cell per warp (one in the wide and tensor-core engines).
 //
 // Per unit (Eq. MsFEB, Remark on oversampling, Eq. stiffness_local):
 //   1. patch = cell enlarged by o fine elements per side, clipped to [0,1]^2;
