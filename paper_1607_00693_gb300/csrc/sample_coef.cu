@@ -65,7 +65,6 @@ __global__ void __launch_bounds__(kCoefCols, NBX <= 32 ? 2 : 1)
 sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw, int share, int S, long long npair, double w, double scale,
                    double clog, double gain, const double* __restrict__ xi, double* __restrict__ a) {
   extern __shared__ double csm[];
-  __shared__ int large;                  // an amplitude beyond kCoefAmp
   double* tab = csm;                     // [64] 2^(j/64)
   double* gy = csm + 64;                 // [nby][R]
   double* U = gy + (size_t)nby * R;      // [nbx][R]
@@ -112,17 +111,19 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
       for (int g = 0; g < NBX / 4; ++g)
         if ((4 * g + 3.5f) / nbx >= lo && (4 * g + 0.5f) / nbx <= hi) near |= 1u << g;
     }
-    if (tid == 0) large = 0;
     __syncthreads();
     const double* xs = xi + (size_t)s * nbx * nby;
+    int beyond = 0;
     for (int q = tid; q < nbx * rows; q += kCoefCols) {
       const int bx = q / rows, r = q % rows;
       double acc = 0.0;
       for (int by = 0; by < nby; ++by) acc = fma(__ldg(xs + by * nbx + bx), gy[by * R + r], acc);
       U[bx * R + r] = acc;
-      if (!(fabs(acc) <= amp)) large = 1;
+      if (!(fabs(acc) <= amp)) beyond = 1;
     }
-    __syncthreads();
+    // (a flag in shared memory would be static: the host gives the dynamic part
+    // all of the 48 KB that a launch may have without opting in for more)
+    const bool large = __syncthreads_or(beyond);
     if (ex >= nf || rg >= nrg) continue;  // (every thread comes back to the barriers above)
     const unsigned use = large ? 0xffffffffu : near;
     if (use & ~have) {

@@ -239,6 +239,24 @@ def test_sampling_row_groups_and_strips(orc, nf, nbx, nby, width, S):
     assert np.max(np.abs(a.cpu().numpy() / ref - 1)) <= 4 * (0.7 * psi[0] * psi[1] * 8 * eps + 4 * eps)
 
 
+# dynamic shared memory of exactly 48 KB: the bump values of 64-row strips
+# alone (47 + 48 bumps), and with the shared column values (the others)
+@pytest.mark.parametrize("nf,nbx,nby,S", [(1024, 47, 48, 20), (1024, 48, 47, 20), (128, 21, 32, 1000),
+                                          (128, 16, 47, 700), (110, 20, 44, 700)])
+def test_sampling_at_the_shared_memory_limit(orc, nf, nbx, nby, S):
+    width = 0.02
+    fld = dict(kind=api.FIELD_EXP, nbx=nbx, nby=nby, width=width, scale=0.7, contrast_log=0.0, gain=1.0)
+    xi = np.random.default_rng(nf).uniform(-1, 1, size=(S, nbx * nby))
+    a = torch.zeros((S, nf, nf), dtype=torch.float64, device=DEV)
+    api.stomsfem_sample_coef(api.grid(nf, 1), api.field_from_dict(fld), _t(xi), a)
+    some = [0, S // 2, S - 1]
+    ref = orc.sample_coef(nf, fld, xi[some])
+    x = (np.arange(nf) + 0.5) / nf
+    psi = [np.exp(-((x[:, None] - (np.arange(n) + 0.5) / n) / width) ** 2).sum(1).max() for n in (nbx, nby)]
+    eps = np.finfo(float).eps
+    assert np.max(np.abs(a[some].cpu().numpy() / ref - 1)) <= 4 * (0.7 * psi[0] * psi[1] * 8 * eps + 4 * eps)
+
+
 @pytest.mark.parametrize("eps", [1e-3, 1e-2])
 def test_interpolation_units_per_thread(eps):
     """A sample's interpolant does not depend on the batch: one and two units
