@@ -16,12 +16,12 @@
 // left it idle a fifth of the time, and gx cost 1.8 of 28 operations an
 // element).  Bumps further than kCoefReach widths from a warp's columns are
 // left out, four at a time: exp(-7.5^2) = 3.7e-25, so with amplitudes below
-// kCoefAmp (of the exponent) what they add stays below 3e-17, less than the
-// exponential's rounding; a strip with a larger one, or with one that is not
-// finite, sums them all.  On the 1024^2 workload (16 bumps a row, spacing one
-// width) 12 of 16 products remain, with 32 bumps of 3/4 of the spacing 15 of
-// 32.  Where a batch gives fewer than four pairs a block the strips get
-// shorter.  A block's width follows the grid's (see the rule at the launch),
+// kCoefAmp (of the exponent, or of the mean level of an affine field) what they
+// add stays below 3e-17, less than the rounding there; a strip with a larger
+// one, or with one that is not finite, sums them all.  On the 1024^2 workload
+// (16 bumps a row, spacing one width) 12 of 16 products remain, with 32 bumps of
+// 3/4 of the spacing 15 of 32.  Where a batch gives fewer than four pairs a
+// block the strips get shorter.  A block's width follows the grid's (see the rule at the launch),
 // narrow ones split the rows among their warps and share gx through shared
 // memory, and the strips are of equal height.
 // 32 samples of the 1024^2 grid: 2.25 -> 1.65 ms; 60 samples of 513^2 1.31 ->
@@ -72,8 +72,12 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
   const int tid = threadIdx.x;
   const double h = 1.0 / nf;
   const double iw2 = 1.0 / (w * w);
+  // the largest amplitude with which far bumps are left out: what they add
+  // stays below the rounding of the exponent, or of an affine field's mean
+  // level (whose field may be sampled with the mean zero: every bump counts then)
   const double gain_z = kind == STOMSFEM_FIELD_EXP_SIGMOID ? 0.25 * fabs(clog * gain) : fabs(scale);
-  const double amp = gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp;
+  const double amp = kind == STOMSFEM_FIELD_AFFINE ? kCoefAmp * fabs(gain) / gain_z
+                                                   : (gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp);
   // the warps split into row groups of kw warps (32 kw columns); those left
   // over only help with the tables
   const int cols = 32 * kw, nrg = kCoefCols / cols, rg = tid / cols, col = tid - rg * cols;

@@ -257,6 +257,24 @@ def test_sampling_at_the_shared_memory_limit(orc, nf, nbx, nby, S):
     assert np.max(np.abs(a[some].cpu().numpy() / ref - 1)) <= 4 * (0.7 * psi[0] * psi[1] * 8 * eps + 4 * eps)
 
 
+def test_sampling_affine_field_without_mean():
+    """With no mean level beside them the far bumps are the field: every
+    element relative to its own value.  Places, widths and products of the
+    reference differ from the kernel's by roundings of the exponent (at most
+    2 (0.125 / 0.01)^2 = 313): 8 eps each, and of the sums."""
+    nf, n, width, S = 1024, 4, 0.01, 3
+    fld = api.field(api.FIELD_AFFINE, n, n, width, 1.0, 0.0, 0.0)
+    xi = np.random.default_rng(5).uniform(0.5, 1.0, size=(S, n * n))
+    a = torch.zeros((S, nf, nf), dtype=torch.float64, device=DEV)
+    api.stomsfem_sample_coef(api.grid(nf, 1), fld, _t(xi), a)
+    x = (np.arange(nf) + 0.5) / nf
+    t = -((x[:, None] - (np.arange(n) + 0.5) / n) ** 2) / width ** 2
+    b = np.exp(t)
+    want = np.einsum("yj,sji,xi->syx", b, xi.reshape(S, n, n), b)
+    assert want.min() < 1e-100
+    assert np.max(np.abs(a.cpu().numpy() / want - 1)) <= (8 * 313 + 64) * np.finfo(float).eps
+
+
 @pytest.mark.parametrize("eps", [1e-3, 1e-2])
 def test_interpolation_units_per_thread(eps):
     """A sample's interpolant does not depend on the batch: one and two units
