@@ -1094,9 +1094,21 @@ static size_t cell_list_bytes(const stomsfem_grid* g) { return round256(sizeof(i
 // same however many lanes they serve, then serve four units: about 790 against
 // 1,125 warp instructions of the FP64 pipe a unit at b = 8.  From b = 13 the
 // panel takes three rows a lane and the update's rounds fill 16 lanes.
-// 64 samples of the 64^2 / 8^2 grid, whole step: 401 ->
-// 312 us.
+// 64 samples of the 64^2 / 8^2 grid, whole step: 401 -> 312 us.
 constexpr int kQuadBand = 12;
+// A unit of its own takes longer on 8 lanes than on 16, so a call pays for it
+// until two units a warp fill the SMs: as many blocks of pairs a SM as are
+// resident (three), or two where a panel is one row a lane (b <= 4) and the unit
+// hardly longer; with at most one unknown (b <= 2) never.  Four samples of 10^2
+// cells (0.66 blocks of pairs a SM), two against four a warp: H/h = 3 16.9, 19.0
+// us; 5 36.2, 49.7; 8 92.7, 127.5; 8, Petrov-Galerkin with oscillatory data 131,
+// 191.  13 samples (2.3): 3 23.0, 21.0; 4 31.3, 30.0; 5 47.6, 52.1; 8 119, 138; 12
+// 350, 355.  7 samples of 16^2 cells (3.4): 5 59.9, 53.0; 8 150, 138; 12 445, 355.
+static bool quad_units(int bmax, long long pair_blocks) {
+  if (bmax > kQuadBand) return false;
+  const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
+  return pair_blocks > (bmax <= 2 ? 0LL : bmax <= 4 ? 2LL : 3LL) * sms;
+}
 
 // Factorisation engines of the FP32 forms: the two-units-per-warp FMA
 // factorisation of band_block.cuh in column blocks of 8 (any bandwidth),
@@ -1185,7 +1197,8 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   const int WPB = upscale_warps(precision == STOMSFEM_FP64, G);
   // four FP64 units per warp: where the workspace holds a block of them and
   // three samples at least share a warp
-  if (precision == STOMSFEM_FP64 && bmax <= kQuadBand && S >= 3 && slots >= WPB * 4) G = 8;
+  const long long pair_blocks = ((S + 1LL) / 2 * grid->nc * grid->nc + WPB - 1) / WPB;
+  if (precision == STOMSFEM_FP64 && S >= 3 && slots >= WPB * 4 && quad_units(bmax, pair_blocks)) G = 8;
   const int slots_per_block = WPB * (32 / G);
   if (slots < slots_per_block)
     return set_error(STOMSFEM_ENOMEM, "workspace %zu bytes < %d slots of %zu bytes", workspace_bytes,

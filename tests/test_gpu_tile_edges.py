@@ -89,6 +89,21 @@ def test_fp64_units_per_warp(orc, rho, mo, S, slots):
     assert _rel(Kg, Ko) <= 1e-11 and _rel(bg, bo) <= 1e-11
 
 
+# four units per warp need a full chip (about 1000 pairs of units): every
+# remainder of the samples by four, with and without oversampling
+@pytest.mark.parametrize("rho,mo", [(1, 1), (2, 0), (3, 0), (4, 0), (4, 1), (5, 0), (8, 0), (6, 3), (12, 0)])
+@pytest.mark.parametrize("S", [8, 9, 10, 11])
+def test_fp64_four_units_per_warp(orc, rho, mo, S):
+    nc = 16
+    nf = nc * rho
+    a = _coef(S, nf, 300 + rho)
+    ov = np.random.default_rng(rho).integers(0, mo + 1, size=nc * nc).astype(np.int8) if mo else None
+    Ko, bo = orc.upscale(nf, nc, 1.0, a, ov)
+    Kg, bg, st = _upscale(nf, nc, a, ov, mo, api.FP64)
+    assert not st.any()
+    assert _rel(Kg, Ko) <= 1e-11 and _rel(bg, bo) <= 1e-11
+
+
 @pytest.mark.parametrize("nf,nc,mo", [(48, 8, 3), (8, 4, 100), (70, 35, 2)])
 @pytest.mark.parametrize("precision", [api.FP64, api.FP32])
 def test_order_by_patch_size_with_flagged_cells(orc, nf, nc, mo, precision):
