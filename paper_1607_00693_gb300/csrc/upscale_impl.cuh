@@ -428,10 +428,10 @@ struct UpscaleTuning {
   int split_fp32 = 1;     // FP32 form: separate forward-only launch for the cells without oversampling
   int engine = 0;         // FP32 forms: factorisation engine (kEngine*; 0 = the default for the patch size)
   // STOMSFEM_ORDER_*: unit order of the persistent launches; negative: by
-  // patch size where the lists fit (a warp then ends on small patches, and
-  // those in flight are of one size).  1024^2, oversampling 0..4, cell against
-  // patch order: FP64, 4 samples, 23.1 -> 18.8 ms; FP32 + refinement, 8, 12.2
-  // -> 10.2; FP32, 32, 8.5 -> 8.0.
+  // patch size where the lists fit and the call is large enough (a warp then
+  // ends on small patches, and those in flight are of one size).  1024^2,
+  // oversampling 0..4, cell against patch order: FP64, 4 samples, 23.1 -> 18.8
+  // ms; FP32 + refinement, 8, 12.2 -> 10.2; FP32, 32, 8.5 -> 8.0.
   int order = -1;
 };
 
@@ -1248,17 +1248,26 @@ int upscale_run(const stomsfem_grid* grid, const double* a, const int8_t* oversa
   int32_t* list1 = list0 + ncell;
   int32_t* listall = list1 + ncell;
   int32_t* counts = listall + ncell;
-  const bool sorted = tune.order != 0 && lists_fit;
+  // FP32 without phi output: cells without oversampling take the
+  // forward-only route in a launch of their own, the others follow.  Not the
+  // oscillatory data: every cell by back substitution in one launch (the
+  // forward-only route never forms psi0, which the Petrov-Galerkin sums then
+  // need, and one launch mode keeps the compile short)
+  const bool split = !OSC && precision == STOMSFEM_FP32 && !phi && tune.split_fp32;
+  // Unless the caller chose, by patch size: always where the split launches need
+  // lists anyway, else where the call makes more than one block an SM (two of the
+  // smallest FP64 patches); below that the lists' launch costs more than
+  // the order gives.  H/h = 1, oversampling up to 1, FP64, 4 samples of 4^2 cells:
+  // 31.1 us with the lists, 27.2 without; 7 of 10^2 (1.3 blocks an SM) 33.7, 29.2.
+  // FP32 + refinement, one sample of 32^2 (1.7): 42.3, 48.1; H/h = 32 3.10, 3.17 ms.
+  const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
+  const bool worth = split || need > (precision == STOMSFEM_FP64 && bmax <= 4 ? 2 : 1) * sms;
+  const bool sorted = lists_fit && (tune.order > 0 || (tune.order < 0 && worth));
   A.order = tune.order < 0 ? (sorted ? 1 : 0) : tune.order;
   const bool by_counter = units < (1LL << 30);  // (a 32-bit counter of work items)
   const long long mb = lists_fit && max_blocks > slots2 / slots_per_block ? slots2 / slots_per_block : max_blocks;
-  // the oscillatory data: every cell by back substitution in one launch
-  // (the forward-only route never forms psi0, which the Petrov-Galerkin
-  // sums then need, and one launch mode keeps the compile short)
   if constexpr (!OSC) {
-    if (precision == STOMSFEM_FP32 && !phi && tune.split_fp32) {
-      // FP32 without phi output: cells without oversampling take the
-      // forward-only route in a launch of their own, the others follow
+    if (split) {
       if (!oversample) return launch_fp32<float, kModeFwd, PG, OSC>(engine, A, max_blocks, st);
       if (lists_fit) {
         upscale_cell_lists_kernel<<<1, kListThreads, 0, st>>>(oversample, ncell, mo, sorted ? 1 : 0, list0, list1, listall,

@@ -124,6 +124,27 @@ def test_order_by_patch_size_with_flagged_cells(orc, nf, nc, mo, precision):
     assert _rel(Kg[:, ok], Ko[:, ok]) <= TOL[precision] and _rel(bg[:, ok], bo[:, ok]) <= TOL[precision]
 
 
+# (small calls keep the cell order unless told otherwise; the default takes
+# the patch order once there is more than one block an SM)
+@pytest.mark.parametrize("nf,nc,mo,S", [(48, 8, 3, 3), (8, 4, 100, 2), (16, 16, 1, 5), (16, 16, 1, 3), (70, 35, 2, 1)])
+@pytest.mark.parametrize("precision", [api.FP64, api.FP32_REFINED, api.FP32])
+def test_unit_order_does_not_change_the_results(nf, nc, mo, S, precision):
+    a = _t(_coef(S, nf, nf))
+    ov = np.random.default_rng(nf).integers(0, min(mo, 4) + 1, size=nc * nc).astype(np.int8)
+    ov[2::5] = -1
+    if mo == 100:
+        ov[1::3] = 100
+    g, out = api.grid(nf, nc), []
+    for order in (None, api.ORDER_CELL, api.ORDER_PATCH):
+        Ke = torch.full((S, nc * nc, 10), 7.0, dtype=torch.float64, device=DEV)
+        be = torch.full((S, nc * nc, 4), 7.0, dtype=torch.float64, device=DEV)
+        api.stomsfem_upscale(g, a, Ke, be, oversample=_t(ov), max_oversample=mo, precision=precision, order=order)
+        out.append((Ke.cpu().numpy(), be.cpu().numpy()))
+    for K, b in out[1:]:
+        assert np.array_equal(K, out[0][0], equal_nan=True) and np.array_equal(b, out[0][1], equal_nan=True)
+    assert np.isfinite(out[0][0][:, ov >= 0]).all()
+
+
 @pytest.mark.parametrize("nc", [1, 2, 3, 4, 9, 16, 31, 32, 33, 47, 63])
 def test_coarse_solve_sizes(orc, nc):
     """Last blocks of every remainder, one and two rows per lane, S above and
