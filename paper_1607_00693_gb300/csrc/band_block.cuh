@@ -80,16 +80,21 @@ __host__ __device__ inline int blk_pitch(int bmax) {
 
 // Offset of slot 0's entry d = 0 in the window (elements).
 constexpr int kWndOff = 3;
-// Elements between the NB rows of one ring block and the next.  A tile row
-// of the update is NB ring rows, and NB rows of any pitch span a multiple of
-// eight 16-byte groups, so without the gap the lanes of one column of tiles
-// all meet one bank group; with it consecutive tile rows are one group apart
-// (two for FP64).
+// Elements between the NB rows of one ring block and the next, for the forms
+// whose update tiles cover whole blocks of rows or single rows (8-row FP32
+// tiles, 1 x 4 FP64 tiles): NB rows of any pitch span a multiple of eight 16-byte
+// groups, so without the gap the lanes of one column of tiles all meet one bank
+// group; with it consecutive tile rows are one group apart (two for FP64).
+// The 4 x 4 FP32 tiles do without (wnd_pad): lower than a block, they spread
+// over several groups anyway, and the gap only adds index operations to every
+// window access.  With it, without it: 10^2 cells at H/h = 12 49.3, 47.6 us; 64
+// samples of 64^2 cells at H/h = 16 7.28, 7.14 ms; 10^2 cells at H/h = 60 2.82,
+// 2.71 ms.
 constexpr int kBlkPad = 4;
 // Element offset of ring slot `slot` (entry d = 0 at kWndOff past it).
-template <int NB>
+template <int NB, int PAD>
 __host__ __device__ __forceinline__ int wnd_row(int slot, int PW) {
-  return slot * PW + (int)((unsigned)slot / NB) * kBlkPad;
+  return slot * PW + (int)((unsigned)slot / NB) * PAD;
 }
 
 __host__ __device__ inline int blk_wnd_elems(int NB, int bmax) {
@@ -267,7 +272,7 @@ __device__ __forceinline__ void st_grp4(double* p, const double (&v)[4]) {
 // generator's entries and rhs.  The slots are zero on entry (the whole
 // window is cleared when a factorisation starts, and each block's slots
 // again once the block is retired).
-template <int G, typename T, int NR, class Gen>
+template <int G, typename T, int NR, int PAD, class Gen>
 __device__ __forceinline__ void blk_fill_raw(const Gen& gen, const BlkSmem<T>& s, int r0, int r1, int slot0, int b,
                                              int gl, const typename Gen::Raw& raw) {
   const int mx = gen.mx;
@@ -276,7 +281,7 @@ __device__ __forceinline__ void blk_fill_raw(const Gen& gen, const BlkSmem<T>& s
     T e[5], rh[NR];
     gen.template make<T, NR>(r, raw, e, rh);
     const int slot = ring(slot0 + gl, s.RW);
-    T* row = s.wnd + kWndOff + wnd_row<G / 2>(slot, s.PW);
+    T* row = s.wnd + kWndOff + wnd_row<G / 2, PAD>(slot, s.PW);
     if (mx >= 3 && mx + 1 <= b) {
       // offsets 0, 1, mx-1, mx, mx+1 are distinct: plain stores
       row[0] = e[0];
@@ -470,6 +475,11 @@ template <int G, typename T, int RPL>
 __host__ __device__ constexpr bool tiles8_form() {
   return G == 16 && sizeof(T) == 4 && RPL == 3;
 }
+// The window's gap of a form.
+template <int G, typename T, int RPL>
+__host__ __device__ constexpr int wnd_pad() {
+  return sizeof(T) == 8 || tiles8_form<G, T, RPL>() ? kBlkPad : 0;
+}
 
 // Lane gl's tile.  The lane order puts tiles whose window rows share a bank
 // group (ti - g0 mod 8 alike, kBlkPad) into different quarters of the warp
@@ -541,7 +551,7 @@ __device__ __forceinline__ void tiles8_update(const Tile8& t, int b, const float
   const float* pr = pt + RP - 8 - 8 * t.ti;  // rows 8 ti + 7 .. 8 ti
   const int rows = nt - 8 * t.ti;            // live rows of the tile (8 or more: all)
   // entry (row a, column group g0, column 3 of the group)
-  float* w = s.wnd + kWndOff + wnd_row<8>(tslot, s.PW) + (8 * t.ti - 4 * t.g0 - 3);
+  float* w = s.wnd + kWndOff + wnd_row<8, kBlkPad>(tslot, s.PW) + (8 * t.ti - 4 * t.g0 - 3);
   const int ws = s.PW + 1;  // to the same columns of the next row
   uint64_t r[4], c[4];
   if (!TIGHT && b > 32) {
@@ -618,7 +628,7 @@ __device__ __forceinline__ void tiles1x4_update(const double* __restrict__ pt, c
     if (2 * R * (R + 1) > t) --R;
     const int rem = t - 2 * R * (R + 1), a = rem / (R + 1), g = rem - a * (R + 1), i = 4 * R + a;
     // entries d = i - 4 g - 3 .. i - 4 g: element k is column 4 g + 3 - k
-    double* w = s.wnd + kWndOff + wnd_row<NB>(ring(tslot + i, s.RW), s.PW) + (i - 4 * g - 3);
+    double* w = s.wnd + kWndOff + wnd_row<NB, kBlkPad>(ring(tslot + i, s.RW), s.PW) + (i - 4 * g - 3);
     double v[4];
     ld_grp4(w, v);
     const double* col = pt;
@@ -653,11 +663,12 @@ template <int G, typename T, int NR, int RPL, class Gen, typename TS, bool FWD_O
 __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<T>& s, T* __restrict__ Lg,
                           TS* __restrict__ yg, int gl, double* yy = nullptr, int store_from = 0) {
   constexpr int NB = G / 2;
+  constexpr int PAD = wnd_pad<G, T, RPL>();
   const int LBS = (NB + bmax) * NB;
   const int RW = s.RW;
   constexpr bool kTiles8 = tiles8_form<G, T, RPL>();
   const Tile8 tile = kTiles8 ? tile8_of<TIGHT>(gl, b) : Tile8{0, 0, 0, false};
-  blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + wnd_row<NB>(RW, s.PW))) / 16), gl);
+  blk_zero16<G>(s.wnd, (int)(al16(sizeof(T) * (size_t)(kWndOff + wnd_row<NB, PAD>(RW, s.PW))) / 16), gl);
   __syncwarp();
   int fail = -1;
   // first window: rows [0, min(n, NB + b)) in slots 0.. (no wrap), generated directly
@@ -665,7 +676,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
   for (int r0 = 0; r0 < filled; r0 += G) {
     typename Gen::Raw raw;
     if (r0 + gl < filled) gen.load(r0 + gl, raw);
-    blk_fill_raw<G, T, NR>(gen, s, r0, min(filled, r0 + G), r0, b, gl, raw);
+    blk_fill_raw<G, T, NR, PAD>(gen, s, r0, min(filled, r0 + G), r0, b, gl, raw);
   }
   __syncwarp();
   int fslot = ring(filled, RW);  // slot of row `filled` (filled <= RW)
@@ -683,7 +694,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
       __syncwarp();
       typename Gen::Raw pf;
       if (gl < NB) gen.from_smem(s.raw + s.RAWD * gl, pf);
-      blk_fill_raw<G, T, NR>(gen, s, filled, need, fslot, b, gl, pf);
+      blk_fill_raw<G, T, NR, PAD>(gen, s, filled, need, fslot, b, gl, pf);
       fslot = ring(fslot + (need - filled), RW);
       filled = need;
       __syncwarp();
@@ -700,7 +711,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
       // their values stay in their own lane's row and are never stored
       const int i = gl + G * q;
       const int slot = ring(kslot + i, RW);
-      const T* row = s.wnd + kWndOff + wnd_row<NB>(slot, s.PW);
+      const T* row = s.wnd + kWndOff + wnd_row<NB, PAD>(slot, s.PW);
       // entries d = i - p, p < NB, as NB / 4 aligned groups: group g4 holds
       // d = i - 4 g4 - 3 .. i - 4 g4 (p = 4 g4 + 3 .. 4 g4); the entries
       // above the diagonal (d < 0, rows i < NB only) hold a neighbour's
@@ -734,7 +745,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     T* Lb = Lg + (size_t)kb * LBS;
     // the transposed trailing panel: 16-byte aligned inside the retired
     // rows' span [kWndOff + kslot PW, kWndOff + (kslot + NB) PW)
-    T* pt = s.wnd + wnd_row<NB>(kslot, s.PW) + 4;
+    T* pt = s.wnd + wnd_row<NB, PAD>(kslot, s.PW) + 4;
     const bool store_blk = K + NB > store_from;
     __syncwarp();
 #pragma unroll
@@ -829,7 +840,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
         for (int a = 0; a < 4; ++a) {
           const int ia = 4 * ti + a;
           if (ia < nt) {
-            T* wr = s.wnd + kWndOff + wnd_row<NB>(ring(tslot + ia, RW), s.PW) + (ia - 4 * tj - 3);
+            T* wr = s.wnd + kWndOff + wnd_row<NB, PAD>(ring(tslot + ia, RW), s.PW) + (ia - 4 * tj - 3);
             T v[4];
             ld_grp4(wr, v);
 #pragma unroll
@@ -843,7 +854,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
     __syncwarp();
     // the retired rows' slots (which held the trailing panel) are cleared for
     // the rows that will occupy them
-    blk_zero_span<G>(s.wnd + kWndOff + wnd_row<NB>(kslot, s.PW), NB * s.PW, gl);
+    blk_zero_span<G>(s.wnd + kWndOff + wnd_row<NB, PAD>(kslot, s.PW), NB * s.PW, gl);
     __syncwarp();
   }
   return fail;
