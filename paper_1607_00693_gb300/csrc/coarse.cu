@@ -260,20 +260,19 @@ coarse_bc_kernel(int nc, int S, const double* __restrict__ Ke, const double* __r
 
 // Merge this batch's moments into the running ones (pairwise update of
 // Chan, Golub and LeVeque): batch mean/M2 two-pass, then combine.
-// A CTA takes kMomNodes nodes, kMomGroups threads each sharing the node's
-// samples (one thread per node left a batch of 512 on 9 CTAs, each thread
-// in two chains of 512 dependent additions).
-constexpr int kMomNodes = 16, kMomGroups = 32;
-
-__global__ void __launch_bounds__(kMomNodes * kMomGroups)
+// A CTA takes NODES nodes, GROUPS threads each sharing the node's samples.
+template <int NODES, int GROUPS>
+__global__ void __launch_bounds__(NODES * GROUPS)
 moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double* m2, const double* count) {
-  __shared__ double part[kMomGroups][kMomNodes + 1];
-  const int c = threadIdx.x % kMomNodes, g = threadIdx.x / kMomNodes;
-  const int q = blockIdx.x * kMomNodes + c;
+  __shared__ double part[GROUPS][NODES + 1];
+  const int c = threadIdx.x % NODES, g = threadIdx.x / NODES;
+  const int q = blockIdx.x * NODES + c;
+  if (GROUPS == 1 && q >= nn) return;
   auto total = [&](double v) {  // sum of the node's groups, in every thread
+    if constexpr (GROUPS == 1) return v;
     part[g][c] = v;
     __syncthreads();
-    for (int h = kMomGroups / 2; h > 0; h >>= 1) {
+    for (int h = GROUPS / 2; h > 0; h >>= 1) {
       if (g < h) part[g][c] += part[g + h][c];
       __syncthreads();
     }
@@ -283,11 +282,11 @@ moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double
   };
   double mb = 0.0;
   if (q < nn)
-    for (int s = g; s < S; s += kMomGroups) mb += u[(size_t)s * nn + q];
+    for (int s = g; s < S; s += GROUPS) mb += u[(size_t)s * nn + q];
   mb = total(mb) / S;
   double M2b = 0.0;
   if (q < nn)
-    for (int s = g; s < S; s += kMomGroups) {
+    for (int s = g; s < S; s += GROUPS) {
       const double d = u[(size_t)s * nn + q] - mb;
       M2b += d * d;
     }
@@ -300,6 +299,26 @@ moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double
 }
 
 __global__ void count_kernel(double* count, int S) { count[0] += (double)S; }
+
+// Moments of a batch merged, then the count.  One thread per node is bound by
+// its two chains of S dependent additions (about 0.14 us a sample), 32 threads
+// per node by the barriers of their sums, 12 us for a CTA of 16 nodes and more once
+// the SMs hold several: the line lies where the chains have grown past that.  One
+// thread, 32 threads, us: 1089 nodes, 1 sample 6.7, 10.8; 16 8.7, 11.6; 100 20.4,
+// 13.2; 512 74, 19; 4225 nodes, 64 samples 15.3, 16.9; 100 19.8, 17.3; 9409 nodes,
+// 100 samples 20.6, 26.0; 200 32.9, 31.3; 16641 nodes, 16 samples 9.1, 31; 100 21, 39;
+// 512 76, 76; 1025^2 nodes, 16 samples 158, 1348.
+static int merge_moments(int nn, int S, const double* u, double* mean, double* m2, double* count, cudaStream_t st) {
+  constexpr int kNodes = 16, kGroups = 32, kThreads = 128;
+  if (S > 48 + nn / 64)
+    moments_kernel<kNodes, kGroups><<<(nn + kNodes - 1) / kNodes, kNodes * kGroups, 0, st>>>(nn, S, u, mean, m2, count);
+  else
+    moments_kernel<kThreads, 1><<<(nn + kThreads - 1) / kThreads, kThreads, 0, st>>>(nn, S, u, mean, m2, count);
+  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  count_kernel<<<1, 1, 0, st>>>(count, S);
+  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  return STOMSFEM_OK;
+}
 
 // Merge a second set of running moments (mean_b, m2_b, count_b: another
 // rank's, or another stream's) into (mean, m2, count): the same pairwise
@@ -625,14 +644,7 @@ extern "C" int stomsfem_coarse_solve(const stomsfem_grid* grid, const double* Ke
   kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, Ke, be, u, static_cast<unsigned char*>(workspace), sb,
                                                     coarse_l_bytes(nc));
   STOMSFEM_TRY_CUDA(cudaGetLastError());
-  if (mom) {
-    const int nn = (grid->nc + 1) * (grid->nc + 1);
-    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-    count_kernel<<<1, 1, 0, st>>>(count, S);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-  }
-  return STOMSFEM_OK;
+  return mom ? merge_moments((grid->nc + 1) * (grid->nc + 1), S, u, mean, m2, count, st) : STOMSFEM_OK;
 }
 
 extern "C" int stomsfem_coarse_pg_workspace_size(const stomsfem_grid* grid, int32_t S, size_t* bytes) {
@@ -672,14 +684,7 @@ extern "C" int stomsfem_coarse_solve_pg(const stomsfem_grid* grid, const double*
   coarse_pg_kernel<false><<<(unsigned)blocks, kCoarsePgWarps * 32, smem, st>>>(
       grid->nc, S, Kpg, bpg, nullptr, nullptr, u, static_cast<unsigned char*>(workspace), sb);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
-  if (mom) {
-    const int nn = (grid->nc + 1) * (grid->nc + 1);
-    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-    count_kernel<<<1, 1, 0, st>>>(count, S);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-  }
-  return STOMSFEM_OK;
+  return mom ? merge_moments((grid->nc + 1) * (grid->nc + 1), S, u, mean, m2, count, st) : STOMSFEM_OK;
 }
 
 // Largest coarse grid of the solves with mixed boundary data: their half
@@ -738,14 +743,7 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
     kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, K, b, dirichlet, g, u, ws, sb, coarse_bc_l_bytes(nc));
   }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
-  if (mom) {
-    const int nn = (nc + 1) * (nc + 1);
-    moments_kernel<<<(nn + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(nn, S, u, mean, m2, count);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-    count_kernel<<<1, 1, 0, st>>>(count, S);
-    STOMSFEM_TRY_CUDA(cudaGetLastError());
-  }
-  return STOMSFEM_OK;
+  return mom ? merge_moments((nc + 1) * (nc + 1), S, u, mean, m2, count, st) : STOMSFEM_OK;
 }
 
 // Fine grids up to 64 elements per side: the banded solver of band_cta.cuh
@@ -821,11 +819,7 @@ extern "C" int stomsfem_mc_moments(int32_t n, int32_t S, const double* u, double
   if (S == 0) return STOMSFEM_OK;
   if (!u || !mean || !m2 || !count) return set_error(STOMSFEM_EINVAL, "NULL device pointer");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  moments_kernel<<<(n + kMomNodes - 1) / kMomNodes, kMomNodes * kMomGroups, 0, st>>>(n, S, u, mean, m2, count);
-  STOMSFEM_TRY_CUDA(cudaGetLastError());
-  count_kernel<<<1, 1, 0, st>>>(count, S);
-  STOMSFEM_TRY_CUDA(cudaGetLastError());
-  return STOMSFEM_OK;
+  return merge_moments(n, S, u, mean, m2, count, st);
 }
 
 extern "C" int stomsfem_mc_merge(int32_t n, double* mean, double* m2, double* count, const double* mean_b,

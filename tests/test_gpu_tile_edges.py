@@ -176,6 +176,25 @@ def test_coarse_solve_sizes(orc, nc):
         assert np.linalg.norm(ug[keep] - uo[keep]) <= 1e-9 * np.linalg.norm(uo[keep])
 
 
+# one and 32 threads per node; the rule turns at 48 samples and one more for each
+# 64 nodes
+@pytest.mark.parametrize("n", [9, 1089, 9409, 40001])
+@pytest.mark.parametrize("S", [1, 3, 48, 49, 65, 66, 195, 196])
+def test_moments_threads_per_node(n, S):
+    """Two batches against NumPy; values in [0, 1): sums of S terms carry at most S
+    roundings, the squared deviations at most 12 S of their sum."""
+    u = np.random.default_rng(n + S).uniform(size=(2, S, n))
+    mean, m2 = (torch.zeros(n, dtype=torch.float64, device=DEV) for _ in range(2))
+    cnt = torch.zeros(1, dtype=torch.float64, device=DEV)
+    for b in range(2):
+        api.stomsfem_mc_moments(_t(u[b]), mean, m2, cnt)
+    v = u.reshape(2 * S, n)
+    tol = 32 * 2 * S * np.finfo(float).eps
+    assert float(cnt[0]) == 2 * S
+    assert np.allclose(mean.cpu().numpy(), v.mean(0), rtol=tol, atol=tol)
+    assert np.allclose(m2.cpu().numpy(), ((v - v.mean(0)) ** 2).sum(0), rtol=tol, atol=tol * S)
+
+
 # levels 66, 33 is odd: not offered; one to four levels below the finest
 @pytest.mark.parametrize("nf", [2, 9, 33, 64, 72, 80, 96, 112, 128, 240])
 @pytest.mark.parametrize("contrast", [False, True])
