@@ -27,6 +27,8 @@
 // 512 coarse systems of 32^2 cells with moments: 2.79 ms with a warp per
 // sample and column blocks of 16, 1.45 ms here.
 //
+// Systems of at most 16 unknowns: tiny_solve, 16 lanes each (below).
+//
 // Row generator interface (Gen): typename Raw; load(r, Raw&); template
 // make<double, 1>(r, raw, e, rhs) as in band_block.cuh; mx.
 #pragma once
@@ -291,6 +293,69 @@ __device__ bool cta_band_solve(const Gen& gen, int n, int b, const CtaBand& s, d
     }
   }
   __syncthreads();
+  return ok;
+}
+
+// ---- systems of at most 16 unknowns, 16 lanes each
+//
+// A CTA for a system of 1, 4 or 9 unknowns spends its time in barriers and its
+// lanes on identity rows.  Here lane r holds row r of the dense lower triangle in
+// registers, the factor l d l^T goes column by column with shuffles inside the
+// 16 lanes, and l into shared memory (pitch 17) for the back substitution; eight
+// systems a CTA, no barrier between warps and no global scratch.  Coarse systems
+// of 4^2 cells, 20,000: 555 -> 91 us (345 with a warp each and column blocks of 16),
+// one 19.0 -> 12.0; of 2^2 cells 311 -> 43 (86), with mixed boundary data 570 -> 103
+// (363).
+constexpr int kTinyMax = 16;
+constexpr int kTinySystems = kCtaThreads / kTinyMax;  // per CTA
+
+// Returns (in every lane of the system) false when a pivot was not positive; x:
+// the solution of this lane's row.
+template <class Gen>
+__device__ __forceinline__ bool tiny_solve(const Gen& gen, int n, double (*L)[kTinyMax + 1], double& x) {
+  const int r = threadIdx.x % kTinyMax, mx = gen.mx;
+  double e[5] = {1.0, 0.0, 0.0, 0.0, 0.0}, y[1] = {0.0};  // rows past the end: the identity
+  if (r < n) {
+    typename Gen::Raw raw;
+    gen.load(r, raw);
+    gen.template make<double, 1>(r, raw, e, y);
+  }
+  double a[kTinyMax], inv = 1.0;
+#pragma unroll
+  for (int j = 0; j < kTinyMax; ++j) {
+    const int d = r - j;  // (d <= r: the entries of a row that do not exist are never met)
+    a[j] = d == 0 ? e[0] : 0.0;
+    if (d == 1) a[j] += e[1];
+    if (d >= 0 && d == mx - 1) a[j] += e[2];
+    if (d > 0 && d == mx) a[j] += e[3];
+    if (d == mx + 1) a[j] += e[4];
+  }
+  bool ok = true;
+#pragma unroll
+  for (int J = 0; J < kTinyMax; ++J) {
+    if (J < n) {
+      double d = __shfl_sync(0xffffffffu, a[J], J, kTinyMax);
+      const long long bits = __double_as_longlong(d);  // positive and not NaN, by the bit pattern
+      if (bits <= 0 || bits > 0x7ff0000000000000ll) {
+        ok = false;
+        d = 1.0;
+      }
+      const double rd = recip(d), l = a[J] * rd, yJ = __shfl_sync(0xffffffffu, y[0], J, kTinyMax);
+      if (r == J) inv = rd;
+      if (r > J) y[0] = fma(-l, yJ, y[0]);
+#pragma unroll
+      for (int p = J + 1; p < kTinyMax; ++p)
+        if (p < n) a[p] = fma(-l, __shfl_sync(0xffffffffu, a[J], p, kTinyMax), a[p]);
+      L[r][J] = l;
+    }
+  }
+  __syncwarp();
+  double z = y[0] * inv;
+  for (int J = n - 1; J > 0; --J) {
+    const double xJ = __shfl_sync(0xffffffffu, z, J, kTinyMax);
+    if (r < J) z = fma(-L[J][r], xJ, z);
+  }
+  x = z;
   return ok;
 }
 

@@ -1,9 +1,10 @@
 // Coarse assembly and solve (Eq. upscaleSUF) and Monte Carlo moments
 // (Eq. MCestimate); the same with mixed boundary data (Sec. 5.2, Eqs.
-// xsquarewave / ysquarewave).  One CTA per sample: the coarse matrix over the
-// (nc-1)^2 interior coarse nodes is again a 9-point-stencil SPD matrix,
-// assembled row by row from the K_e of the four cells around each node
-// and factorised in FP64 by the banded solver of band_cta.cuh.
+// xsquarewave / ysquarewave).  One CTA per sample (16 lanes where it has at most
+// 16 unknowns): the coarse matrix over the (nc-1)^2 interior coarse nodes is
+// again a 9-point-stencil SPD matrix, assembled row by row from the K_e of the
+// four cells around each node and factorised in FP64 by the solvers of
+// band_cta.cuh.
 #include "band_cta.cuh"
 #include "common.cuh"
 
@@ -84,18 +85,66 @@ struct FineFemGen {
 };
 
 // u [(N+1)^2] from the interior solution x [(N-1)^2] (NaN where the
-// factorisation failed), zero on the boundary; the whole CTA.
-__device__ __forceinline__ void write_interior(int N, bool ok, const double* __restrict__ x, double* __restrict__ us) {
+// factorisation failed), zero on the boundary; thread tid of nt.
+__device__ __forceinline__ void write_interior(int N, bool ok, const double* __restrict__ x, double* __restrict__ us,
+                                               int tid, int nt) {
   const int NN = N + 1;
-  for (int q = threadIdx.x; q < NN * NN; q += kCtaThreads) {
+  for (int q = tid; q < NN * NN; q += nt) {
     const int I = q % NN, J = q / NN;
     double v = 0.0;
     if (I > 0 && J > 0 && I < N && J < N)
       v = ok ? x[(J - 1) * (N - 1) + (I - 1)] : __longlong_as_double(0x7ff8000000000000ll);
     us[q] = v;
   }
-  __syncthreads();
 }
+
+// S systems of at most kTinyMax unknowns, 16 lanes each (none at all on a grid
+// of one element, whose solution is its boundary).  Sys: the batch's unknowns,
+// row generator and output of a sample.
+template <class Sys>
+__global__ void __launch_bounds__(kCtaThreads) tiny_systems_kernel(Sys sys, int S) {
+  __shared__ double L[kTinySystems][kTinyMax][kTinyMax + 1], xs[kTinySystems][kTinyMax];
+  const int g = threadIdx.x / kTinyMax, lane = threadIdx.x % kTinyMax;
+  const int s = blockIdx.x * kTinySystems + g, sc = min(s, S - 1);  // (idle lanes mirror the last system)
+  double x;
+  const bool ok = tiny_solve(sys.gen(sc), sys.n(), L[g], x);
+  xs[g][lane] = x;
+  __syncwarp();
+  if (s < S) sys.write(s, ok, xs[g], lane);
+}
+template <class Sys>
+static int tiny_systems(const Sys& sys, int S, cudaStream_t st) {
+  tiny_systems_kernel<Sys><<<(S - 1) / kTinySystems + 1, kCtaThreads, 0, st>>>(sys, S);
+  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  return STOMSFEM_OK;
+}
+
+struct FineSystems {
+  int nf;
+  double f;
+  const double* a;
+  double* u;
+  __host__ __device__ int n() const { return (nf - 1) * (nf - 1); }
+  __device__ FineFemGen gen(int s) const {
+    const double h = 1.0 / nf;
+    return FineFemGen{a + (size_t)s * nf * nf, nf, nf - 1, f * h * h};
+  }
+  __device__ void write(int s, bool ok, const double* x, int lane) const {
+    write_interior(nf, ok, x, u + (size_t)s * (nf + 1) * (nf + 1), lane, kTinyMax);
+  }
+};
+struct CoarseSystems {
+  int nc;
+  const double *Ke, *be;
+  double* u;
+  __host__ __device__ int n() const { return (nc - 1) * (nc - 1); }
+  __device__ CoarseBlkGen gen(int s) const {
+    return CoarseBlkGen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, nc, nc - 1};
+  }
+  __device__ void write(int s, bool ok, const double* x, int lane) const {
+    write_interior(nc, ok, x, u + (size_t)s * (nc + 1) * (nc + 1), lane, kTinyMax);
+  }
+};
 
 template <int RS>
 __global__ void __launch_bounds__(kCtaThreads, kCtaPerSm)
@@ -110,8 +159,9 @@ fine_fem_kernel(int nf, int S, double f, const double* __restrict__ a, double* _
   const double h = 1.0 / nf;
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const FineFemGen gen{a + (size_t)s * nf * nf, nf, mx, f * h * h};
-    const bool ok = n > 0 ? cta_band_solve<RS>(gen, n, b, sm, Lg, x) : true;
-    write_interior(nf, ok, x, u + (size_t)s * (nf + 1) * (nf + 1));
+    const bool ok = cta_band_solve<RS>(gen, n, b, sm, Lg, x);
+    write_interior(nf, ok, x, u + (size_t)s * (nf + 1) * (nf + 1), threadIdx.x, kCtaThreads);
+    __syncthreads();
   }
 }
 
@@ -142,8 +192,9 @@ coarse_blk_kernel(int nc, int S, const double* __restrict__ Ke, const double* __
   double* x = reinterpret_cast<double*>(slot + l_bytes);
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const CoarseBlkGen gen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, nc, mx};
-    const bool ok = n > 0 ? cta_band_solve<RS>(gen, n, b, sm, Lg, x) : true;
-    write_interior(nc, ok, x, u + (size_t)s * (nc + 1) * (nc + 1));
+    const bool ok = cta_band_solve<RS>(gen, n, b, sm, Lg, x);
+    write_interior(nc, ok, x, u + (size_t)s * (nc + 1) * (nc + 1), threadIdx.x, kCtaThreads);
+    __syncthreads();
   }
 }
 
@@ -257,6 +308,21 @@ coarse_bc_kernel(int nc, int S, const double* __restrict__ Ke, const double* __r
     __syncthreads();
   }
 }
+
+struct BcSystems {
+  int nc;
+  const double *Ke, *be;
+  const uint8_t* dm;
+  const double* gv;
+  double* u;
+  __host__ __device__ int n() const { return (nc + 1) * (nc + 1); }
+  __device__ CoarseBcGen gen(int s) const {
+    return CoarseBcGen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, dm, gv, nc, nc + 1};
+  }
+  __device__ void write(int s, bool ok, const double* x, int lane) const {
+    if (lane < n()) u[(size_t)s * n() + lane] = ok ? x[lane] : __longlong_as_double(0x7ff8000000000000ll);
+  }
+};
 
 // Merge this batch's moments into the running ones (pairwise update of
 // Chan, Golub and LeVeque): batch mean/M2 two-pass, then combine.
@@ -635,15 +701,21 @@ extern "C" int stomsfem_coarse_solve(const stomsfem_grid* grid, const double* Ke
   if (slots < kCoarseMinSlots)
     return set_error(STOMSFEM_ENOMEM, "coarse workspace %zu < %d slots of %zu", workspace_bytes,
                      kCoarseMinSlots, sb);
-  const long long blocks = slots < S ? slots : S;  // one sample per CTA
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int nc = grid->nc;
-  const size_t smem = cta_smem_bytes(nc);
-  auto kern = nc <= 32 ? coarse_blk_kernel<1> : coarse_blk_kernel<2>;
-  STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, Ke, be, u, static_cast<unsigned char*>(workspace), sb,
-                                                    coarse_l_bytes(nc));
-  STOMSFEM_TRY_CUDA(cudaGetLastError());
+  const CoarseSystems sys{nc, Ke, be, u};
+  if (sys.n() <= kTinyMax) {
+    const int rc = tiny_systems(sys, S, st);
+    if (rc) return rc;
+  } else {
+    const long long blocks = slots < S ? slots : S;  // one sample per CTA
+    const size_t smem = cta_smem_bytes(nc);
+    auto kern = nc <= 32 ? coarse_blk_kernel<1> : coarse_blk_kernel<2>;
+    STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<(unsigned)blocks, kCtaThreads, smem, st>>>(nc, S, Ke, be, u, static_cast<unsigned char*>(workspace), sb,
+                                                      coarse_l_bytes(nc));
+    STOMSFEM_TRY_CUDA(cudaGetLastError());
+  }
   return mom ? merge_moments((grid->nc + 1) * (grid->nc + 1), S, u, mean, m2, count, st) : STOMSFEM_OK;
 }
 
@@ -724,7 +796,7 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
   long long slots = (long long)(workspace_bytes / sb);
   if (slots < warps)
     return set_error(STOMSFEM_ENOMEM, "coarse workspace %zu < %d slots of %zu", workspace_bytes, warps, sb);
-  // Petrov-Galerkin: a warp per sample, two per CTA; Galerkin: a CTA per sample
+  // Petrov-Galerkin: a warp per sample, two per CTA; Galerkin: a CTA (or 16 lanes) per sample
   long long blocks = pg ? slots / warps : slots;
   const long long need = pg ? ((long long)S + warps - 1) / warps : S;
   if (blocks > need) blocks = need;
@@ -735,6 +807,9 @@ extern "C" int stomsfem_coarse_solve_bc(const stomsfem_grid* grid, int32_t pg, c
     STOMSFEM_TRY_CUDA(
         cudaFuncSetAttribute(coarse_pg_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     coarse_pg_kernel<true><<<(unsigned)blocks, kCoarsePgWarps * 32, smem, st>>>(nc, S, K, b, dirichlet, g, u, ws, sb);
+  } else if (const BcSystems sys{nc, K, b, dirichlet, g, u}; sys.n() <= kTinyMax) {
+    const int rc = tiny_systems(sys, S, st);
+    if (rc) return rc;
   } else {
     const int bnd = nc + 2;
     const size_t smem = cta_smem_bytes(bnd);
@@ -787,6 +862,8 @@ extern "C" int stomsfem_fine_fem(const stomsfem_grid* grid, const double* a, int
   long long slots = (long long)(workspace_bytes / sb);
   if (slots < kCoarseMinSlots)
     return set_error(STOMSFEM_ENOMEM, "fine FEM workspace %zu < %d slots of %zu", workspace_bytes, kCoarseMinSlots, sb);
+  const FineSystems sys{nf, grid->f, a, u};
+  if (sys.n() <= kTinyMax) return tiny_systems(sys, S, st);
   const long long blocks = slots < S ? slots : S;  // one sample per CTA
   const size_t smem = cta_smem_bytes(nf);
   auto kern = nf <= 32 ? fine_fem_kernel<1> : fine_fem_kernel<2>;

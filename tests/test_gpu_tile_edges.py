@@ -176,6 +176,43 @@ def test_coarse_solve_sizes(orc, nc):
         assert np.linalg.norm(ug[keep] - uo[keep]) <= 1e-9 * np.linalg.norm(uo[keep])
 
 
+# 16 lanes per system up to 16 unknowns (nc = 5, 4^2 interior nodes; nc = 3 with all
+# nodes unknown), a CTA beyond; ragged groups of eight systems
+@pytest.mark.parametrize("nc", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("S", [2, 7, 8, 37])
+def test_small_systems(orc, nc, S):
+    a = _coef(S, 2 * nc, 10 * nc + S)
+    K, b = orc.upscale(2 * nc, nc, 1.0, a)
+    g, nn = api.grid(2 * nc, nc), (nc + 1) ** 2
+    bad = S // 2  # an indefinite sample among sound ones
+    keep = np.arange(S) != bad
+    Kb = K.copy()
+    Kb[bad] = -Kb[bad]
+    u = torch.full((S, nn), 7.0, dtype=torch.float64, device=DEV)
+    api.stomsfem_coarse_solve(g, _t(Kb), _t(b), u)
+    ug, uo = u.cpu().numpy(), orc.coarse_solve(nc, K, b)
+    assert np.linalg.norm((ug - uo)[keep]) <= 1e-9 * np.linalg.norm(uo[keep]) and (ug[keep][uo[keep] == 0] == 0).all()
+    inner = np.zeros((nc + 1, nc + 1), bool)
+    inner[1:-1, 1:-1] = True
+    assert np.isnan(ug[bad][inner.ravel()]).all() and (ug[bad][~inner.ravel()] == 0).all()
+    # mixed data: prescribed left and right, every node an unknown
+    dm = np.zeros((nc + 1, nc + 1), np.uint8)
+    dm[:, 0] = dm[:, -1] = 1
+    gv = np.where(dm, np.arange(nc + 1)[None, :] + 0.5, 0.0)
+    api.stomsfem_coarse_solve_bc(g, 0, _t(Kb), _t(b), _t(dm.ravel()), _t(gv.ravel()), u)
+    ug, uo = u.cpu().numpy(), orc.coarse_solve_bc(nc, K, b, dm.ravel(), gv.ravel())
+    assert np.linalg.norm((ug - uo)[keep]) <= 1e-9 * np.linalg.norm(uo[keep])
+    if nc > 1:
+        assert np.isnan(ug[bad]).all()
+    # the fine grid's own system
+    af = _coef(S, nc, nc + S)
+    uf = torch.full((S, nn), 7.0, dtype=torch.float64, device=DEV)
+    api.stomsfem_fine_fem(api.grid(nc, 1), _t(af), uf)
+    for s in range(S):
+        ref = orc.fine_fem(nc, 1.0, af[s]).reshape(-1) if nc > 1 else np.zeros(nn)
+        assert np.linalg.norm(uf[s].cpu().numpy() - ref) <= 1e-10 * np.linalg.norm(ref) + 1e-300
+
+
 # one and 32 threads per node; the rule turns at 48 samples and one more for each
 # 64 nodes
 @pytest.mark.parametrize("n", [9, 1089, 9409, 40001])
