@@ -688,13 +688,14 @@ constexpr uint32_t kWaitLimit = 1u << 24;  // about 2 s
 // overwrites the buffers.  split: both operands as BF16 pairs (hi, lo =
 // BF16 of the remainder) and three products per step, Ab T + Ab Tlo + Ablo
 // T (the dropped Ablo Tlo is below 2^-16 relative), so G carries about
-// 16 bits instead of BF16's 8; one product otherwise.  units: G goes out as
+// 16 bits instead of BF16's 8; one product otherwise.  UNITS: G goes out as
 // [cell][32-sample tile][Ppad][32] (for one unit per thread) instead of
 // [cell][s][Ppad].
+template <bool UNITS>
 __global__ void __launch_bounds__(128, 1)
 pod_gemm_kernel(PodDims d, int Spad, const __nv_bfloat16* __restrict__ Ab, const __nv_bfloat16* __restrict__ Ablo,
-                const __nv_bfloat16* __restrict__ T, const __nv_bfloat16* __restrict__ Tlo, int split, int units,
-                float* __restrict__ G, int32_t* err) {
+                const __nv_bfloat16* __restrict__ T, const __nv_bfloat16* __restrict__ Tlo, int split, float* __restrict__ G,
+                int32_t* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -774,7 +775,7 @@ pod_gemm_kernel(PodDims d, int Spad, const __nv_bfloat16* __restrict__ Ab, const
     for (int col = 0; col < d.Ppad; col += 16) {
       float v[16];
       tc::tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + col, v);
-      if (units) {
+      if constexpr (UNITS) {
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           if (col + q < d.P) Gt[(size_t)(col + q) * 32] = v[q];
@@ -1968,10 +1969,11 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   const int parts = pod->split ? 2 : 1;
   // one unit per thread in the solves: the unrefined form of the shared basis,
-  // beyond one tile of 32 samples (a warp per unit has the shorter chain, and
-  // the same bits: 5 samples of the 64^2 / 8^2 grid 38 us against 44, 31 samples 42
-  // against 44, 130 samples 80 against 67)
-  const bool per_thread = refine_iters == 0 && !d.per_l && S > 32;
+  // beyond one tile of 32 samples and 2048 units (a warp per unit has the shorter
+  // chain, and the same bits: 5 samples of the 64^2 / 8^2 grid 38 us against 44, 31
+  // samples 42 against 44, 130 samples 80 against 67; 33 samples of 16 cells, H/h =
+  // 16, 37.4 against 39.9)
+  const bool per_thread = refine_iters == 0 && !d.per_l && S > 32 && (long long)S * d.ncell > 2048;
   // one K step: the streaming product, whose G layout those solves read
   const bool stream_gemm = per_thread && d.Kp == kPodK;
   const size_t bytes_b = (size_t)d.Ppad * 128, bytes_a = (size_t)kPodTileM * 128;
@@ -1984,11 +1986,10 @@ extern "C" int stomsfem_pod_upscale(stomsfem_pod* pod, const double* a, int32_t 
     pod_gemm_stream_kernel<<<(unsigned)(tiles < sms ? tiles : sms), 128, smem_req, st>>>(
         d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, G, pod->err);
   } else {
-    STOMSFEM_TRY_CUDA(
-        cudaFuncSetAttribute(pod_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_req));
+    auto kern = per_thread ? pod_gemm_kernel<true> : pod_gemm_kernel<false>;
+    STOMSFEM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_req));
     dim3 grd(Spad / kPodTileM, d.ncell);
-    pod_gemm_kernel<<<grd, 128, smem_req, st>>>(d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, per_thread ? 1 : 0, G,
-                                                pod->err);
+    kern<<<grd, 128, smem_req, st>>>(d, Spad, Ab, Ablo, pod->T, pod->Tlo, pod->split, G, pod->err);
   }
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   PodSolveArgs A;

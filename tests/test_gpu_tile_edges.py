@@ -276,6 +276,47 @@ def test_reduced_solves_at_every_remainder(orc, rank):
         api.stomsfem_pod_destroy(h)
 
 
+# one unit per thread (more than 2048 units) at every remainder of the rank, with one K
+# step (the streaming product: 1500 samples of 64 cells are 768 tiles, five a CTA with
+# a change of cell among them; one half of the accumulator or two) and several (H/h =
+# 16), against batches of 32, which take a warp per unit and the other product
+@pytest.mark.parametrize("rho,nc,rank,S", [(8, 8, 27, 1500), (8, 8, 12, 1500)] +
+                         [(8, 8, r, 131) for r in (1, 2, 3, 4, 5, 7, 8, 26, 27)] + [(16, 4, 5, 200), (16, 4, 27, 200)])
+@pytest.mark.parametrize("split", [1, 0])
+def test_reduced_units_do_not_depend_on_the_batch(rho, nc, rank, S, split):
+    nf, cells, Ns = rho * nc, nc * nc, 12
+    g = api.grid(nf, nc)
+    a_tr, a = _t(_coef(Ns, nf, 1, 0.3)), _t(_coef(S, nf, 2, 0.3))
+    phi = torch.zeros((Ns, cells, 4, (rho + 1) ** 2), dtype=torch.float64, device=DEV)
+    K0, b0 = (torch.zeros((Ns, cells, k), dtype=torch.float64, device=DEV) for k in (10, 4))
+    api.stomsfem_upscale(g, a_tr, K0, b0, phi=phi)
+    h, _ = api.stomsfem_pod_build(g, phi, a_tr, ranks=[max(1, rank - c % 3) for c in range(cells)])
+
+    def online(lo, hi, refine=0):
+        n = hi - lo
+        Ke = torch.full((n, cells, 10), 7.0, dtype=torch.float64, device=DEV)
+        be = torch.full((n, cells, 4), 7.0, dtype=torch.float64, device=DEV)
+        st = torch.full((n, cells), 9, dtype=torch.int32, device=DEV)
+        api.stomsfem_pod_upscale(h, g, a[lo:hi].contiguous(), Ke, be, refine_iters=refine, unit_status=st)
+        assert not st.cpu().numpy().any()
+        return Ke.cpu().numpy(), be.cpu().numpy()
+
+    try:
+        api.stomsfem_pod_set_gemm_split(h, split)
+        Ke, be = online(0, S)
+        for lo in list(range(0, S - 32, 32 if S < 300 else 96)) + [S - 32]:
+            K, b = online(lo, lo + 32)
+            assert np.array_equal(K, Ke[lo:lo + 32]) and np.array_equal(b, be[lo:lo + 32])
+        if rho <= 8:
+            # split: the dropped products are below 2^-16 of the sums, three of
+            # them per entry of K_e, amplified by the solves at most tenfold
+            tol = 5e-4 if split else 5e-3
+            K, b = online(S - 40, S, 4)
+            assert _rel(Ke[S - 40:], K) <= tol and _rel(be[S - 40:], b) <= tol
+    finally:
+        api.stomsfem_pod_destroy(h)
+
+
 @pytest.mark.parametrize("nf,nbx,nby,width,S", [(1, 1, 1, 0.3, 3), (7, 3, 5, 0.02, 2), (33, 4, 4, 0.1, 40),
                                                 (64, 17, 2, 0.01, 3), (257, 33, 9, 0.02, 2), (300, 5, 64, 0.004, 2),
                                                 (520, 64, 3, 0.5, 1)])
