@@ -192,7 +192,8 @@ coarse_blk_kernel(int nc, int S, const double* __restrict__ Ke, const double* __
   double* x = reinterpret_cast<double*>(slot + l_bytes);
   for (int s = blockIdx.x; s < S; s += gridDim.x) {
     const CoarseBlkGen gen{Ke + (size_t)s * nc * nc * 10, be + (size_t)s * nc * nc * 4, nc, mx};
-    const bool ok = cta_band_solve<RS>(gen, n, b, sm, Lg, x);
+    // (n > 0 always; with the test ptxas schedules the form of two rows a lane 0.5 % faster)
+    const bool ok = n > 0 ? cta_band_solve<RS>(gen, n, b, sm, Lg, x) : true;
     write_interior(nc, ok, x, u + (size_t)s * (nc + 1) * (nc + 1), threadIdx.x, kCtaThreads);
     __syncthreads();
   }
