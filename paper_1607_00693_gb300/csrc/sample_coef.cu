@@ -37,7 +37,7 @@ constexpr int kCoefThreads = 128;
 constexpr size_t kCoefSmem = 48 * 1024;
 constexpr double kCoefReach = 7.5;  // in widths
 constexpr double kCoefAmp = 1e6;
-constexpr int kCoefCols = 256;      // threads per block, and its columns at most (FP64)
+constexpr int kCoefCols = 256;      // threads per block, and its columns at most (FP64; or half of them)
 
 __host__ __device__ inline int coef_rows(int nbx, int nby) {
   int R = 128;
@@ -60,8 +60,8 @@ __device__ __forceinline__ double sigmoid_scaled(double clog, double e) {
   return fma(fma(-d, q, clog), r, q);
 }
 
-template <int NBX>
-__global__ void __launch_bounds__(kCoefCols, NBX <= 32 ? 2 : 1)
+template <int NBX, int COLS>
+__global__ void __launch_bounds__(COLS, (NBX <= 32 ? 512 : 256) / COLS)
 sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw, int share, int S, long long npair, double w, double scale,
                    double clog, double gain, const double* __restrict__ xi, double* __restrict__ a) {
   extern __shared__ double csm[];
@@ -80,7 +80,7 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
                                                    : (gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp);
   // the warps split into row groups of kw warps (32 kw columns); those left
   // over only help with the tables
-  const int cols = 32 * kw, nrg = kCoefCols / cols, rg = tid / cols, col = tid - rg * cols;
+  const int cols = 32 * kw, nrg = COLS / cols, rg = tid / cols, col = tid - rg * cols;
   exp_table_fill(tab);
   // this block's (place, sample) pairs, the samples fastest
   const long long u0 = npair * blockIdx.x / gridDim.x, u1 = npair * (blockIdx.x + 1) / gridDim.x;
@@ -97,13 +97,13 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
       ey0 = strip * R;
       rows = min(R, nf - ey0);
       ex = col0 + col;
-      for (int q = tid; q < nby * rows; q += kCoefCols) {
+      for (int q = tid; q < nby * rows; q += COLS) {
         const int by = q / rows, r = q % rows;
         const double dy = (ey0 + r + 0.5) * h - (by + 0.5) / nby;
         gy[by * R + r] = fexp(-dy * dy * iw2, tab);
       }
       if (share)
-        for (int q = tid; q < nbx * cols; q += kCoefCols) {
+        for (int q = tid; q < nbx * cols; q += COLS) {
           const int bx = q / cols;
           const double dx = (col0 + (q - bx * cols) + 0.5) * h - (bx + 0.5) / nbx;
           gxs[q] = fexp(-dx * dx * iw2, tab);
@@ -118,7 +118,7 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
     __syncthreads();
     const double* xs = xi + (size_t)s * nbx * nby;
     int beyond = 0;
-    for (int q = tid; q < nbx * rows; q += kCoefCols) {
+    for (int q = tid; q < nbx * rows; q += COLS) {
       const int bx = q / rows, r = q % rows;
       double acc = 0.0;
       for (int by = 0; by < nby; ++by) acc = fma(__ldg(xs + by * nbx + bx), gy[by * R + r], acc);
@@ -240,50 +240,76 @@ static int sample_coef_impl(const stomsfem_grid* grid, const stomsfem_field* fie
   if (!xi || !a) return set_error(STOMSFEM_EINVAL, "xi and a must be device pointers");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int nbx = field->nbx;
-  int R = coef_rows(field->nbx, field->nby);
+  const int R = coef_rows(field->nbx, field->nby);
   const size_t smem = (size_t)(field->nbx + field->nby) * R * sizeof(float);
   const size_t K = (size_t)field->nbx * field->nby;
   const int sms = device_sm_count() > 0 ? device_sm_count() : 152;
   if (precision == STOMSFEM_FP64) {
-    // columns of a block, 32 kw: the kw of the least work, in FP64 warp
-    // instructions per row and sample (an element takes about 14 and one for each
-    // bump within reach, U nbx nby / 32); 256 columns for every grid left a
-    // third of the lanes of 513 past its edge
-    int kw = 1, nchunk = 1;
-    double least = 0.0;
-    for (int k = kCoefCols / 32; k >= 1; --k) {
-      const int n = (grid->nf + 32 * k - 1) / (32 * k);
-      const double cost = n * (k * (14.0 + nbx) + nbx * field->nby / 32.0);
-      if (k == kCoefCols / 32 || cost < least) {
-        least = cost;
-        kw = k;
-        nchunk = n;
+    struct Shape {
+      int cols, kw, R, nstrip, share;
+      long long npair, blocks;
+      size_t bytes;
+    };
+    auto shape = [&](int cols) {  // with blocks of `cols` threads
+      Shape h;
+      h.cols = cols;
+      // columns of a block, 32 kw: the kw of the least work, in FP64 warp
+      // instructions per row and sample (an element takes about 14 and one for each
+      // bump within reach, U nbx nby / 32); 256 columns for every grid left a
+      // third of the lanes of 513 past its edge
+      int nchunk = 1;
+      double least = 0.0;
+      for (int k = cols / 32; k >= 1; --k) {
+        const int n = (grid->nf + 32 * k - 1) / (32 * k);
+        const double cost = n * (k * (14.0 + nbx) + nbx * field->nby / 32.0);
+        if (k == cols / 32 || cost < least) {
+          least = cost;
+          h.kw = k;
+          nchunk = n;
+        }
       }
-    }
-    auto pairs = [&](int r) { return (long long)((grid->nf + r - 1) / r) * nchunk * S; };
-    const long long blocks = 2LL * sms;
-    if (R > 64) R = 64;
-    while (R > 8 && pairs(R) < 4 * blocks) R >>= 1;
-    // strips of equal height (77 rows as 39 + 38, not 64 + 13: the blocks' shares
-    // count pairs)
-    const int nstrip = (grid->nf + R - 1) / R;
-    const long long npair = pairs(R);
-    R = (grid->nf + nstrip - 1) / nstrip;
-    // row groups share the bump values of their columns where these fit
-    const size_t own = (64 + (size_t)(field->nbx + field->nby) * R) * sizeof(double);
-    const size_t shared_gx = (size_t)nbx * 32 * kw * sizeof(double);
-    const int share = kw <= kCoefCols / 64 && own + shared_gx <= kCoefSmem;
-    const size_t bytes = own + (share ? shared_gx : 0);
-    const unsigned grd = (unsigned)(npair < blocks ? npair : blocks);
-#define LAUNCH(N)                                                                                               \
-  sample_coef_kernel<N><<<grd, kCoefCols, bytes, st>>>(grid->nf, field->kind, nbx, field->nby, R, nstrip, kw, share, S, npair, \
-                                                       field->width, field->scale, field->contrast_log,         \
-                                                       field->gain, xi, a)
-    if (nbx <= 4) LAUNCH(4);
-    else if (nbx <= 8) LAUNCH(8);
-    else if (nbx <= 16) LAUNCH(16);
-    else if (nbx <= 32) LAUNCH(32);
-    else LAUNCH(64);
+      auto pairs = [&](int r) { return (long long)((grid->nf + r - 1) / r) * nchunk * S; };
+      h.blocks = (nbx <= 32 ? 512LL : 256LL) / cols * sms;  // as many as are resident
+      h.R = R < 64 ? R : 64;
+      while (h.R > 8 && pairs(h.R) < 4 * h.blocks) h.R >>= 1;
+      // strips of equal height (77 rows as 39 + 38, not 64 + 13: the blocks' shares
+      // count pairs)
+      h.nstrip = (grid->nf + h.R - 1) / h.R;
+      h.npair = pairs(h.R);
+      h.R = (grid->nf + h.nstrip - 1) / h.nstrip;
+      // row groups share the bump values of their columns where these fit
+      const size_t own = (64 + (size_t)(nbx + field->nby) * h.R) * sizeof(double);
+      const size_t shared_gx = (size_t)nbx * 32 * h.kw * sizeof(double);
+      h.share = h.kw <= cols / 64 && own + shared_gx <= kCoefSmem;
+      h.bytes = own + (h.share ? shared_gx : 0);
+      return h;
+    };
+    // Blocks of 128 threads for more than 32 bumps a row (255 registers a thread:
+    // two blocks an SM, where one of 256 threads has no other to cover its
+    // barriers) and where there is at most one pair for every block of 256 (the
+    // pairs then run on twice as many).  256 against 128 threads, us: 20 samples
+    // of 128^2 with 64^2 bumps 338, 240; 100 of 16^2 with 33 x 8 bumps 130, 72; 200
+    // of 8^2 with 16^2 bumps 41.9, 31.3; 150 of 16^2 42.3, 31.3.
+    Shape h = shape(kCoefCols);
+    if (nbx > 32 || h.npair <= h.blocks) h = shape(kCoefCols / 2);
+    const unsigned grd = (unsigned)(h.npair < h.blocks ? h.npair : h.blocks);
+#define LAUNCH(N, C)                                                                                               \
+  sample_coef_kernel<N, C><<<grd, C, h.bytes, st>>>(grid->nf, field->kind, nbx, field->nby, h.R, h.nstrip, h.kw,   \
+                                                    h.share, S, h.npair, field->width, field->scale,               \
+                                                    field->contrast_log, field->gain, xi, a)
+#define LAUNCH2(N)                          \
+  do {                                      \
+    if (h.cols == kCoefCols)                \
+      LAUNCH(N, kCoefCols);                 \
+    else                                    \
+      LAUNCH(N, kCoefCols / 2);             \
+  } while (0)
+    if (nbx <= 4) LAUNCH2(4);
+    else if (nbx <= 8) LAUNCH2(8);
+    else if (nbx <= 16) LAUNCH2(16);
+    else if (nbx <= 32) LAUNCH2(32);
+    else LAUNCH(64, kCoefCols / 2);
+#undef LAUNCH2
 #undef LAUNCH
     STOMSFEM_TRY_CUDA(cudaGetLastError());
     return STOMSFEM_OK;
