@@ -1110,12 +1110,13 @@ int vcycle(MgLevel* lv, int L, int l, int S, const double* r, double* rz, cudaSt
 
 namespace stomsfem {
 
+// (room to move the start to a 16-byte boundary)
 size_t fine_mg_workspace_bytes(int nf, int S) {
   MgLevel lv[kMgMaxLevels];
   int L;
   double* vec[4];
   double* scal;
-  return mg_layout(nf, S, lv, &L, nullptr, vec, &scal);
+  return mg_layout(nf, S, lv, &L, nullptr, vec, &scal) + 16;
 }
 
 bool fine_mg_supported(int nf) {
@@ -1133,7 +1134,9 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
   int L;
   double* vec[4];
   double* scal;
-  const size_t need = mg_layout(nf, S, lv, &L, static_cast<unsigned char*>(workspace), vec, &scal);
+  // the stencils are stored and copied 16 bytes at a time
+  const size_t shift = (0 - reinterpret_cast<uintptr_t>(workspace)) & 15;
+  const size_t need = shift + mg_layout(nf, S, lv, &L, static_cast<unsigned char*>(workspace) + shift, vec, &scal);
   if (workspace_bytes < need)
     return set_error(STOMSFEM_ENOMEM, "fine FEM workspace %zu < %zu bytes", workspace_bytes, need);
   double *r = vec[0], *p = vec[1], *Ap = vec[2], *st64 = vec[3];

@@ -213,6 +213,26 @@ def test_small_systems(orc, nc, S):
         assert np.linalg.norm(uf[s].cpu().numpy() - ref) <= 1e-10 * np.linalg.norm(ref) + 1e-300
 
 
+@pytest.mark.parametrize("contrast", [1.0, 2e3])
+@pytest.mark.parametrize("shift", [0, 4, 8, 12])
+def test_fine_solver_workspace_alignment(orc, contrast, shift):
+    """A workspace of exactly the reported size at any place: the solver's 16-byte
+    accesses start at a boundary of their own."""
+    nf, S = 80, 3
+    a = np.exp(np.random.default_rng(nf).uniform(-1.0, 1.0, size=(S, nf, nf)))
+    a[:, 30:32, :] *= contrast
+    g = api.grid(nf, 1)
+    need = api.stomsfem_fine_fem_workspace_size(g, S)
+    buf = torch.full((need + 64,), 0xFF, dtype=torch.uint8, device=DEV)
+    assert buf.data_ptr() % 16 == 0
+    u = torch.zeros((S, (nf + 1) ** 2), dtype=torch.float64, device=DEV)
+    api.stomsfem_fine_fem(g, _t(a), u, workspace=buf[shift:shift + need])
+    assert bool((buf[shift + need:] == 0xFF).all()) and bool((buf[:shift] == 0xFF).all())
+    for s in range(S):
+        uo = orc.fine_fem(nf, 1.0, a[s]).reshape(-1)
+        assert np.linalg.norm(u[s].cpu().numpy() - uo) <= 1e-10 * np.linalg.norm(uo)
+
+
 # one and 32 threads per node; the rule turns at 48 samples and one more for each
 # 64 nodes
 @pytest.mark.parametrize("n", [9, 1089, 9409, 40001])
