@@ -51,7 +51,7 @@ __device__ __forceinline__ float mg_omega(int sweep) {
 // interval, where 60 Jacobi sweeps left 0.25 of the smoothest.
 constexpr int kMgCoarseSteps = 24;
 constexpr float kMgCoarseLo = 0.02f, kMgCoarseHi = 2.5f;
-constexpr int kMgSmall = 32;  // a level of at most this many elements per side and the one below run in one kernel
+constexpr int kMgSmall = 32;  // the level above the coarsest has at most this many elements per side; the two run in one kernel
 constexpr int kMgThreads = 256;
 // Coefficient contrast (max a / min a over the batch) above which the
 // transfers between levels use the operator-dependent prolongation; below
@@ -741,18 +741,18 @@ __global__ void __launch_bounds__(kMgWarps * 32) mgf_up_kernel(int nf, int rows,
   if (r) block_sum_to(acc, rz + s);
 }
 
-// ---- the last levels of one sample in one CTA: a level of at most 32 elements
-// per side (if the coarsest is not the only one left) and the coarsest.  A
-// thread holds one interior node of each (at most 961 and 225) with its
-// couplings in registers; the vectors live in shared memory.  As marches and
-// a kernel for the coarsest grid, three launches of 10 to 13 us; with the
-// level of 64 and loops over the nodes in here too, 40 us.
+// ---- the last two levels of one sample in one CTA: the coarsest (at most 16
+// elements per side) and the one above it (at most 32).  A thread holds one
+// interior node of each (at most 961 and 225) with its couplings in registers;
+// the vectors live in shared memory.  As marches and a kernel for the coarsest
+// grid, three launches of 10 to 13 us; with the level of 64 and loops over the
+// nodes in here too, 40 us.
 struct MgSmallArgs {
-  int nf;  // the upper level, 0: only the coarsest
+  int nf;  // the upper level
   const float *st, *P;
   int nfc;  // the coarsest level
   const float* stc;
-  const float* f;  // right-hand side of the first of them [S][N]
+  const float* f;  // right-hand side on the upper level [S][N]
   float* out;      // solution there [S][N]
 };
 constexpr int kMgSmallThreads = 992;  // 31 warps: 31^2 interior nodes
@@ -773,13 +773,12 @@ __global__ void __launch_bounds__(kMgSmallThreads) mgf_small_kernel(MgSmallArgs 
   constexpr int NF = (kMgSmall + 1) * (kMgSmall + 1), NC = 17 * 17;
   __shared__ float U[NF], V[NF], Uc[2][NC];
   const int s = blockIdx.x, tid = threadIdx.x;
-  const bool two = A.nf > 0;
   // the upper level's node (x, y) and the coarsest's (I, J)
   const int W = A.nf + 1, N = W * W, Wc = A.nfc + 1, Nc = Wc * Wc;
-  const int mx = max(A.nf - 1, 1), mc = A.nfc - 1;
+  const int mx = A.nf - 1, mc = A.nfc - 1;
   const int x = tid % mx + 1, y = tid / mx + 1, v = y * W + x;
   const int I = tid % mc + 1, J = tid / mc + 1, vc = J * Wc + I;
-  const bool in = two && tid < mx * mx, inc = tid < mc * mc;
+  const bool in = tid < mx * mx, inc = tid < mc * mc;
   for (int q = tid; q < NF; q += kMgSmallThreads) U[q] = V[q] = 0.f;
   for (int q = tid; q < NC; q += kMgSmallThreads) Uc[0][q] = Uc[1][q] = 0.f;
   float a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, c[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -792,34 +791,30 @@ __global__ void __launch_bounds__(kMgSmallThreads) mgf_small_kernel(MgSmallArgs 
   if (inc) {
     stencil9(A.stc + (size_t)s * st_stride(Nc), Nc, vc, Wc, c);
     rc = 1.f / jacobi_divisor(c);
-    if (!two) fc = A.f[(size_t)s * Nc + vc];
   }
   const float* ps = A.P + (size_t)s * 4 * N;
   __syncthreads();
-  float u = 0.f;
-  if (two) {
-    // two sweeps from zero, the residual and its restriction
-    u = mg_omega<OD>(0) * fv * rd;
-    if (in) V[v] = u;
-    __syncthreads();
-    if (in) {
-      u += mg_omega<OD>(1) * (fv - apply9s(a, V + v, W)) * rd;
-      U[v] = u;
-    }
-    __syncthreads();
-    if (in) V[v] = fv - apply9s(a, U + v, W);
-    __syncthreads();
-    if (inc) {
-      const float* q = V + 2 * J * W + 2 * I;
-      if constexpr (OD) {
+  // two sweeps from zero, the residual and its restriction
+  float u = mg_omega<OD>(0) * fv * rd;
+  if (in) V[v] = u;
+  __syncthreads();
+  if (in) {
+    u += mg_omega<OD>(1) * (fv - apply9s(a, V + v, W)) * rd;
+    U[v] = u;
+  }
+  __syncthreads();
+  if (in) V[v] = fv - apply9s(a, U + v, W);
+  __syncthreads();
+  if (inc) {
+    const float* q = V + 2 * J * W + 2 * I;
+    if constexpr (OD) {
 #pragma unroll
-        for (int dy = -1; dy <= 1; ++dy)
+      for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
-          for (int dx = -1; dx <= 1; ++dx)
-            fc = fmaf(pweight(ps, N, W, 2 * I + dx, 2 * J + dy, I, J), q[dy * W + dx], fc);
-      } else {
-        fc = q[0] + 0.5f * (q[-1] + q[1] + q[-W] + q[W]) + 0.25f * (q[-W - 1] + q[-W + 1] + q[W - 1] + q[W + 1]);
-      }
+        for (int dx = -1; dx <= 1; ++dx)
+          fc = fmaf(pweight(ps, N, W, 2 * I + dx, 2 * J + dy, I, J), q[dy * W + dx], fc);
+    } else {
+      fc = q[0] + 0.5f * (q[-1] + q[1] + q[-W] + q[W]) + 0.25f * (q[-W - 1] + q[-W + 1] + q[W - 1] + q[W + 1]);
     }
   }
   // the coarsest grid: Chebyshev steps from zero
@@ -837,10 +832,6 @@ __global__ void __launch_bounds__(kMgSmallThreads) mgf_small_kernel(MgSmallArgs 
     }
     rho = next;
     __syncthreads();
-  }
-  if (!two) {
-    for (int q = tid; q < Nc; q += kMgSmallThreads) A.out[(size_t)s * Nc + q] = Uc[(kMgCoarseSteps - 1) & 1][q];
-    return;
   }
   // prolongation and two sweeps
   if (in) {
@@ -1077,16 +1068,16 @@ dim3 mg_grid(int nf, int S, int useful, int rows) {
 }
 
 // z = V-cycle(r) on level l (f of level l holds the right-hand side; the
-// result in u2 of level l); on the finest level rz[s] += r . z.
+// result in u2 of level l); on the finest level rz[s] += r . z.  The level
+// above the coarsest has at most kMgSmall elements per side and is not the
+// finest (fine_mg_supported).
 template <bool OD>
 int vcycle(MgLevel* lv, int L, int l, int S, const double* r, double* rz, cudaStream_t st) {
   MgLevel& c = lv[l];
-  const int left = L - l;
-  if (left == 1 || (left == 2 && c.nf <= kMgSmall)) {
+  if (l == L - 2) {
     const MgLevel& last = lv[L - 1];
-    if (last.nf > 16) return set_error(STOMSFEM_EINVAL, "coarsest grid of %d elements per side", last.nf);
     MgSmallArgs A;
-    A.nf = left == 2 ? c.nf : 0;
+    A.nf = c.nf;
     A.st = c.st;
     A.P = c.P;
     A.nfc = last.nf;
@@ -1122,7 +1113,7 @@ size_t fine_mg_workspace_bytes(int nf, int S) {
 bool fine_mg_supported(int nf) {
   int nfs[kMgMaxLevels];
   const int L = mg_levels(nf, nfs);
-  return L >= 2 && nfs[L - 1] <= 16;
+  return nf > kMgSmall && nfs[L - 1] <= 16;  // (three levels at least)
 }
 
 // u [S][(nf+1)^2] (boundary 0) solves the Q1 system of each sample to
