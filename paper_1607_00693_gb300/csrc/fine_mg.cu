@@ -37,8 +37,17 @@ constexpr int kMgMaxLevels = 12;
 // Damping of the two sweeps before and after the coarse correction.  On the
 // bilinear levels the high-frequency eigenvalues of D^-1 A lie in [0.75, 1.5]
 // (Q1 stencil, constant coefficient): the two sweeps are the Chebyshev pair
-// of [0.8, 1.6] (largest factor on the former 0.09; 0.16 with 0.8 twice),
-// which converges for eigenvalues below 2.4.  The operator-dependent levels
+// of [0.8, 1.6] (largest factor on the former 0.09; 0.16 with 0.8 twice).  It
+// converges, and the cycle stays definite, for eigenvalues below 2.4.  A
+// bilinear level is the Q1 discretisation of its own elements with the fine
+// coefficient inside, so its largest eigenvalue is at most that of one element's
+// D^-1 A: 1.5 for a constant coefficient, and with a contrast of 1e3 (above it
+// the other transfers run) 2.386, the maximum over all coefficients of 2^2 ..
+// 64^2 fine cells an element (alternating between the vector and the bang-bang
+// coefficient that is best for it; the hot cells then fill an element's corner;
+// without a bound on the contrast it tends to 3).  The pair of [0.75, 1.75] would
+// converge up to 2.5 and took one CG iteration more on smooth media (constant 9
+// for 8, lognormal of contrast 900 18 for 17).  The operator-dependent levels
 // keep 0.8 (see mgf_divisor_kernel).
 constexpr float kMgOmega = 0.8f;
 template <bool OD>
@@ -515,7 +524,7 @@ struct MgStencil {
 // P^T (f - A u) at the next level's nodes.  OD: operator-dependent transfers,
 // whose coarse operators need not be diagonally dominant: the sweeps divide
 // by the divisor of mgf_divisor_kernel; with the bilinear transfers by the
-// diagonal entry, as the M-matrix levels allow.  rows: even.
+// diagonal entry, as the bound on their eigenvalues allows (mg_omega).  rows: even.
 template <bool OD>
 __global__ void __launch_bounds__(kMgWarps * 32, kMgBlocks) mgf_down_kernel(int nf, int rows, const float* __restrict__ st,
                                                                  const float* __restrict__ dv,

@@ -213,6 +213,30 @@ def test_small_systems(orc, nc, S):
         assert np.linalg.norm(uf[s].cpu().numpy() - ref) <= 1e-10 * np.linalg.norm(ref) + 1e-300
 
 
+@pytest.mark.parametrize("r,place", [(2, "corner"), (2, "edge")] +
+                         [(r, p) for r in (4, 8, 16) for p in ("corner", "edge", "centre")])
+def test_fine_solver_just_below_the_contrast_rule(orc, r, place):
+    """Inclusions of contrast 999, mirrored so that a bilinear level's elements of r^2
+    fine cells are all alike (largest eigenvalues of D^-1 A up to 2.354 on some
+    level): the bilinear cycle has to converge.  The residual is 1e-13 of the load's
+    and the load is smooth, so the solution's error is of that order; the direct
+    reference's rounding (about its condition number, 1e7, times 1e-16 at most) sets
+    the bound."""
+    nf = 128
+    a = np.ones((1, nf, nf))
+    x = np.arange(nf) % (2 * r)
+    m = np.minimum(x, 2 * r - 1 - x)  # 0 .. r - 1 from one mirror line to the other
+    side = max(1, r // 4)
+    low, mid = m < side, np.abs(m - (r - 1) / 2) < max(side, 1) / 2 + 0.25
+    hot = {"corner": low[:, None] & low[None, :], "edge": low[:, None] & mid[None, :],
+           "centre": mid[:, None] & mid[None, :]}[place]
+    a[0][hot] = 999.0
+    u = torch.zeros((1, (nf + 1) ** 2), dtype=torch.float64, device=DEV)
+    api.stomsfem_fine_fem(api.grid(nf, 1), _t(a), u)
+    uo = orc.fine_fem(nf, 1.0, a[0]).reshape(-1)
+    assert np.linalg.norm(u[0].cpu().numpy() - uo) <= 1e-9 * np.linalg.norm(uo)
+
+
 @pytest.mark.parametrize("contrast", [1.0, 2e3])
 @pytest.mark.parametrize("shift", [0, 4, 8, 12])
 def test_fine_solver_workspace_alignment(orc, contrast, shift):
