@@ -88,7 +88,6 @@ __device__ inline BlkSmem<float> tc_blk_view(const TcSmem& t) {
   s.RW = kTcRW;
   s.PW = 0;
   s.RP = 0;
-  s.RAWD = 4;
   return s;
 }
 

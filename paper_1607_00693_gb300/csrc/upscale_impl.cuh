@@ -83,42 +83,6 @@ struct PatchGen {
     j = q + 1;
     i = r - q * mx + 1;
   }
-  template <typename T>
-  __device__ __forceinline__ T coef(int r, int d) const {
-    if (d != 0 && d != 1 && d != mx - 1 && d != mx && d != mx + 1) return T(0);
-    int i, j;
-    node(r, i, j);
-    const T aSW = (T)ael(i - 1, j - 1), aSE = (T)ael(i, j - 1);
-    const T aNE = (T)ael(i, j), aNW = (T)ael(i - 1, j);
-    T v = T(0);
-    if (d == 0) v += (T(2) / T(3)) * (aSW + aSE + aNE + aNW);
-    if (d == 1 && i > 1) v -= (aSW + aNW) / T(6);                    // west
-    if (d == mx && j > 1) v -= (aSW + aSE) / T(6);                   // south
-    if (d == mx + 1 && i > 1 && j > 1) v -= aSW / T(3);              // south-west
-    if (d == mx - 1 && i < mx && j > 1) v -= aSE / T(3);             // south-east
-    return v;
-  }
-  // (A X), (A Y), (A XY) at interior node (i, j) for the patch coordinates
-  // X = i/Nx, Y = j/Ny; then -(A p_l) for p_SW = 1-X-Y+XY, p_SE = X-XY, p_NE = XY.
-  template <typename T>
-  __device__ __forceinline__ void ap(int i, int j, T& AX, T& AY, T& AXY) const {
-    const T aSW = (T)ael(i - 1, j - 1), aSE = (T)ael(i, j - 1);
-    const T aNE = (T)ael(i, j), aNW = (T)ael(i - 1, j);
-    AX = ((aSW + aNW) - (aSE + aNE)) / (T(2) * (T)Nx);
-    AY = ((aSW + aSE) - (aNW + aNE)) / (T(2) * (T)Ny);
-    const T Xc = (T)i / (T)Nx, Yc = (T)j / (T)Ny;
-    AXY = Xc * AY + Yc * AX + ((aSE + aNW) - (aNE + aSW)) / (T(3) * (T)Nx * (T)Ny);
-  }
-  template <typename T>
-  __device__ __forceinline__ T rhs(int r, int l) const {
-    int i, j;
-    node(r, i, j);
-    T AX, AY, AXY;
-    ap<T>(i, j, AX, AY, AXY);
-    if (l == 0) return AX + AY - AXY;
-    if (l == 1) return AXY - AX;
-    return -AXY;
-  }
   // Raw values of row r: the coefficient on the four elements around the node.
   struct Raw {
     double sw, se, ne, nw;
@@ -171,6 +135,8 @@ struct PatchGen {
     e[2] = (i < mx && j > 1) ? -aSE * r3 : T(0);
     e[3] = j > 1 ? -(aSW + aSE) * r6 : T(0);
     e[4] = (i > 1 && j > 1) ? -aSW * r3 : T(0);
+    // (A X), (A Y), (A XY) for the patch coordinates X = i/Nx, Y = j/Ny; then
+    // -(A p_l) for p_SW = 1 - X - Y + XY, p_SE = X - XY, p_NE = XY
     const T AX = T(0.5) * ((aSW + aNW) - (aSE + aNE)) * iNx;
     const T AY = T(0.5) * ((aSW + aSE) - (aNW + aNE)) * iNy;
     const T Xc = (T)i * iNx, Yc = (T)j * iNy;
@@ -1144,9 +1110,6 @@ static int upscale_engine(int requested, int precision, int rho, int bmax) {
 }
 // Lanes per unit of the resolved engine.
 static int upscale_engine_lanes(int engine) { return engine == kEngineBlocked ? 16 : 32; }
-static bool upscale_uses_tc(int precision, int rho, int bmax) {
-  return upscale_engine_lanes(upscale_engine(kEngineAuto, precision, rho, bmax)) == 32;
-}
 
 // The WIDE engine's launches (upscale_wide.cu; the Galerkin form without
 // the oscillatory data).  fp64_acc: TA = double (the FP32 + refinement form).
