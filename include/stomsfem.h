@@ -411,7 +411,7 @@ int stomsfem_local_kl_project(const stomsfem_local_kl* kl, const double* kappa, 
  * ------------------------------------------------------------------- */
 
 /* Scratch needed by stomsfem_fine_fem for S samples (nf <= 64: the banded
- * factors of the warps in flight; larger nf: the multigrid hierarchy, the
+ * factors of the systems in flight; larger nf: the multigrid hierarchy, the
  * CG vectors and the FP64 operator of all S samples, about 139 bytes per
  * fine node and sample).  EINVAL for an nf above 64 that does not halve down to 16 or
  * less. */
@@ -419,9 +419,9 @@ int stomsfem_fine_fem_workspace_size(const stomsfem_grid* grid, int32_t S, size_
 
 /* Standard Q1 FEM on the fine grid with zero Dirichlet data and load f
  * (element matrices a_e K_ref, load f h^2/4 per element corner).
- *  - nf <= 64: one CTA per sample on the banded solver of the coarse
- *    solve (NaN for a sample whose matrix is not positive
- *    definite); stream-ordered.
+ *  - nf <= 64: the banded solver of the coarse solve, one CTA per sample
+ *    (16 lanes up to nf = 5; NaN for a sample whose matrix is not
+ *    positive definite); stream-ordered.
  *  - nf > 64 (nf = c 2^k, c <= 16): conjugate gradients in FP64 on all S
  *    samples at once, preconditioned by one multigrid V-cycle in FP32
  *    (bilinear prolongation, or operator-dependent prolongation when the
@@ -432,8 +432,9 @@ int stomsfem_fine_fem_workspace_size(const stomsfem_grid* grid, int32_t S, size_
  *    ENOTSPD too as soon as a residual is not finite);
  *    the true residual b - A u then sits at the FP64 rounding floor
  *    (about eps || |A| |u| ||, e.g. 2e-11 of the load on a 1024^2
- *    lognormal medium); synchronises `stream` (convergence is checked on
- *    the host every four iterations).
+ *    lognormal medium); synchronises `stream` (the host checks
+ *    convergence at the fourth iteration and then where the reduction so
+ *    far predicts the end, at most four iterations apart).
  * a device [S][nf][nf], u device [S][(nf+1)^2] (boundary entries 0). */
 int stomsfem_fine_fem(const stomsfem_grid* grid, const double* a, int32_t S, double* u, void* workspace,
                       size_t workspace_bytes, stomsfem_stream_t stream);
@@ -524,9 +525,10 @@ int stomsfem_coarse_bc_workspace_size(const stomsfem_grid* grid, int32_t pg, int
  * carry the natural condition (zero flux on the boundary).  pg = 0:
  * Galerkin, K = Ke [S][nc*nc][10] and b = be [S][nc*nc][4] of
  * stomsfem_upscale, symmetric elimination of the prescribed nodes and the
- * blocked banded Cholesky (half bandwidth nc + 2); pg = 1:
- * Petrov-Galerkin, K [S][nc*nc][16] and b [S][nc*nc][4] of
- * stomsfem_upscale_pg, banded LU without pivoting.  One warp per sample.
+ * banded L D L^T of the coarse solve (half bandwidth nc + 2, one CTA per
+ * sample, 16 lanes up to nc = 3); pg = 1: Petrov-Galerkin, K
+ * [S][nc*nc][16] and b [S][nc*nc][4] of stomsfem_upscale_pg, banded LU
+ * without pivoting, one warp per sample.
  * u [S][(nc+1)^2] takes every node (g at the prescribed ones); mean, m2,
  * count as stomsfem_coarse_solve.  The caller makes the problem well posed
  * (at least one prescribed node in every part of the domain the cells

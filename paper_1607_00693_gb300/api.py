@@ -107,7 +107,8 @@ def stomsfem_upscale_workspace_size(g: Grid, max_oversample=0, precision=FP64):
 def stomsfem_upscale(g: Grid, a, Ke, be, oversample=None, max_oversample=0, precision=FP64,
                      refine_iters=2, phi=None, unit_status=None, workspace=None, stream=None, engine=None,
                      order=None):
-    """engine and order None: stomsfem_upscale (the default engine, cell
+    """engine and order None: stomsfem_upscale (the default engine; by patch
+    size where the call is large enough for its cell lists, else in cell
     order); otherwise stomsfem_upscale_engine with those STOMSFEM_ENGINE_*
     and STOMSFEM_ORDER_* values (None: AUTO, CELL)."""
     S = a.shape[0]

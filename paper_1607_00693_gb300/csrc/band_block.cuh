@@ -11,10 +11,12 @@
 //      entries, both columns of multipliers broadcast through a
 //      double-buffered shared vector, one warp sync per pair); the NR
 //      right-hand sides ride along, which is the forward substitution;
-//   2. applies the rank-nb update to the trailing b x b window with 4 x 4
-//      register tiles (128-bit shared loads of the transposed panel, which
-//      is kept in the ring slots of the rows just retired; each tile row
-//      read, updated and written back as one 128-bit access);
+//   2. applies the rank-nb update to the trailing b x b window in register
+//      tiles: 8 x 8 or 8 x 4, one a lane for the whole factorisation (FP32,
+//      G = 16, half bandwidths 25..40), 1 x 4 (FP64), 4 x 4 (the other FP32
+//      forms); 128-bit shared loads of the transposed panel, which is kept
+//      in the ring slots of the rows just retired, each tile row read,
+//      updated and written back in 128-bit accesses;
 //   3. clears the retired slots and writes the next rows from values the
 //      row generator copied into shared memory one block earlier.
 // The matrix lives only as a window of RW >= NB + b band rows in shared
@@ -401,7 +403,8 @@ __device__ __forceinline__ void panel_pair(T (&pr)[RPL][NB], T (&rh)[RPL][NR], T
     T l0q[RPL], l1q[RPL];
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
-      // rows at or above J hold no multiplier; rows past the panel are zero
+      // rows at or above J hold no multiplier (rows past the panel hold
+      // values that stay in their own lane's row and are never stored)
       const bool b0 = q > 0 || gl > J, b1 = q > 0 || gl > J1;
       const T l0 = b0 ? pr[q][J] * i0 : T(0);
       const T l1 = b1 ? (pr[q][J1] - l0 * l10) * i1 : T(0);
@@ -797,7 +800,7 @@ __device__ int blk_factor(const Gen& gen, int n, int b, int bmax, const BlkSmem<
       }
     }
     __syncwarp();
-    // ---- 2. trailing update A22 -= L21 L21^T with 4x4 register tiles
+    // ---- 2. trailing update A22 -= L21 L21^T in the form's register tiles
     const int nt = np - nb;
     if constexpr (kTiles8) {
       // (nt > 0 only after a full block: nb = NB)

@@ -405,8 +405,9 @@ __device__ __forceinline__ void block_sum_to(double v, double* acc) {
 // 1024^2, 8 samples: the whole solve, with the leaner CG and set-up, 12.0 ->
 // 6.84 ms; the finest level's passes 69 us down and 138 us up.
 constexpr int kMgWarps = 4;
-constexpr int kMgBlocks = 5;  // of the downward kernel, blocks an SM holds at least (102 registers a
-                              // thread; the upward one spills there: 196 against 138 us on the finest level)
+constexpr int kMgBlocks = 5;  // of the downward kernel, blocks an SM holds at least (96 registers a thread
+                              // and a spill of six words; the upward one spills more there: 196 against 138 us
+                              // on the finest level)
 
 // One strip and row segment of a level for the calling warp.
 struct MgMarch {

@@ -1346,7 +1346,7 @@ pod_solve_kernel(PodSolveArgs A) {
 // tile loads of eight units both meet eight bank groups), then a
 // left-looking tiled Cholesky with the four right-hand sides, the back
 // substitution and the sums of K_e and b_e run without any exchange between
-// the lanes.  74 KB per warp: three warps per SM, each with independent
+// the lanes.  72 KB per warp: three warps per SM, each with independent
 // tiles enough to issue; while one waits for its copies the others compute.
 // Every entry sees the operations of the warp form in the same order (also
 // its butterfly sums), so the results are the same bits.
