@@ -110,7 +110,14 @@ __device__ __forceinline__ float st_entry(const float* __restrict__ st, size_t N
 // west, south, south-west and south-east entries of a node are the east,
 // north, north-east and north-west entries of its neighbours there; zero
 // at the boundary nodes, whose values are zero in every CG vector).
-__global__ void mgf_fine_stencil_kernel(int nf, const double* __restrict__ a, float* __restrict__ st,
+// shift: the FP32 stencils are those of 2^shift a (a preconditioner may be
+// scaled by any constant), which keeps their entries and the entries'
+// reciprocals in range whatever the unit of the coefficient; 0 unless needed.
+__device__ __forceinline__ float narrow_shifted(double v, int shift) {
+  const int hi = __double2hiint(v);
+  return narrow((hi & 0x7ff00000) ? __hiloint2double(hi + (int)((unsigned)shift << 20), __double2loint(v)) : v);
+}
+__global__ void mgf_fine_stencil_kernel(int nf, int shift, const double* __restrict__ a, float* __restrict__ st,
                                         double* __restrict__ st64) {
   const int s = blockIdx.y;
   const int W = nf + 1, N = W * W;
@@ -133,8 +140,10 @@ __global__ void mgf_fine_stencil_kernel(int nf, const double* __restrict__ a, fl
       d[3] = -aNE * k3;
       d[4] = -aNW * k3;
     }
-    *reinterpret_cast<float4*>(ss + 4 * (size_t)v) = make_float4(narrow(d[0]), narrow(d[1]), narrow(d[2]), narrow(d[3]));
-    ss[4 * (size_t)N + v] = narrow(d[4]);
+    *reinterpret_cast<float4*>(ss + 4 * (size_t)v) =
+        make_float4(narrow_shifted(d[0], shift), narrow_shifted(d[1], shift), narrow_shifted(d[2], shift),
+                    narrow_shifted(d[3], shift));
+    ss[4 * (size_t)N + v] = narrow_shifted(d[4], shift);
 #pragma unroll
     for (int k = 0; k < 5; ++k) s64[(size_t)k * N + v] = d[k];
   }
@@ -1163,8 +1172,11 @@ int fine_mg_solve(int nf, double f, const double* a, int S, double* u, void* wor
   std::memcpy(&amax, &hrange[0], sizeof(double));
   std::memcpy(&amin, &hrange[1], sizeof(double));
   const bool od = amax > kMgOdContrast * amin;
+  int exponent = 0;  // of the FP32 hierarchy's unit
+  if (std::isfinite(amax) && (amax > 0x1p100 || amin < 0x1p-100))
+    exponent = -(std::ilogb(amax) + std::ilogb(amin)) / 2;
   // multigrid set-up: stencils of every level
-  mgf_fine_stencil_kernel<<<g0, kMgThreads, 0, st>>>(nf, a, lv[0].st, st64);
+  mgf_fine_stencil_kernel<<<g0, kMgThreads, 0, st>>>(nf, exponent, a, lv[0].st, st64);
   for (int l = 0; l + 1 < L; ++l) {
     if (od) {
       mgf_interp_kernel<<<grid2(lv[l].N, S), kMgThreads, 0, st>>>(lv[l].nf, lv[l].st, lv[l].P);

@@ -238,6 +238,23 @@ def test_fine_solver_just_below_the_contrast_rule(orc, r, place):
 
 
 @pytest.mark.parametrize("contrast", [1.0, 2e3])
+@pytest.mark.parametrize("unit", [2.0 ** 125, 2.0 ** -132, 1e-150, 1e150])
+def test_fine_solver_coefficient_units(orc, contrast, unit):
+    """A coefficient whose FP32 value or its reciprocal leaves the type's range; a load
+    of the same side keeps the solution's magnitude ordinary or the residual in
+    range."""
+    nf, S = 96, 2
+    a = np.exp(np.random.default_rng(nf).uniform(-1.0, 1.0, size=(S, nf, nf)))
+    a[:, 30:32, :] *= contrast
+    u = torch.zeros((S, (nf + 1) ** 2), dtype=torch.float64, device=DEV)
+    f = min(max(unit, 1e-20), 1e20)  # (the FP32 residual's range is the load's)
+    api.stomsfem_fine_fem(api.grid(nf, 1, f), _t(a * unit), u)
+    for s in range(S):
+        uo = orc.fine_fem(nf, 1.0, a[s]).reshape(-1)
+        assert np.linalg.norm(u[s].cpu().numpy() * (unit / f) - uo) <= 1e-10 * np.linalg.norm(uo)
+
+
+@pytest.mark.parametrize("contrast", [1.0, 2e3])
 @pytest.mark.parametrize("shift", [0, 4, 8, 12])
 def test_fine_solver_workspace_alignment(orc, contrast, shift):
     """A workspace of exactly the reported size at any place: the solver's 16-byte
