@@ -27,6 +27,8 @@
 // 32 samples of the 1024^2 grid: 2.25 -> 1.65 ms; 60 samples of 513^2 1.31 ->
 // 1.05 ms (1.43 with 256 columns in every block and strips of 64 rows); 64
 // samples of 32^2 with 32^2 narrow bumps 161 -> 89 us (187 without shared gx).
+#include <cmath>
+
 #include "common.cuh"
 #include "fexp.cuh"
 
@@ -62,8 +64,9 @@ __device__ __forceinline__ double sigmoid_scaled(double clog, double e) {
 
 template <int NBX, int COLS>
 __global__ void __launch_bounds__(COLS, (NBX <= 32 ? 512 : 256) / COLS)
-sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw, int share, int S, long long npair, double w, double scale,
-                   double clog, double gain, const double* __restrict__ xi, double* __restrict__ a) {
+sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw, int share, int S, int per_block,
+                   unsigned extra, double w, double amp, double scale, double clog, double gain,
+                   const double* __restrict__ xi, double* __restrict__ a) {
   extern __shared__ double csm[];
   double* tab = csm;                     // [64] 2^(j/64)
   double* gy = csm + 64;                 // [nby][R]
@@ -72,24 +75,22 @@ sample_coef_kernel(int nf, int kind, int nbx, int nby, int R, int nstrip, int kw
   const int tid = threadIdx.x;
   const double h = 1.0 / nf;
   const double iw2 = 1.0 / (w * w);
-  // the largest amplitude with which far bumps are left out: what they add
-  // stays below the rounding of the exponent, or of an affine field's mean
-  // level (whose field may be sampled with the mean zero: every bump counts then)
-  const double gain_z = kind == STOMSFEM_FIELD_EXP_SIGMOID ? 0.25 * fabs(clog * gain) : fabs(scale);
-  const double amp = kind == STOMSFEM_FIELD_AFFINE ? kCoefAmp * fabs(gain) / gain_z
-                                                   : (gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp);
   // the warps split into row groups of kw warps (32 kw columns); those left
   // over only help with the tables
   const int cols = 32 * kw, nrg = COLS / cols, rg = tid / cols, col = tid - rg * cols;
   exp_table_fill(tab);
-  // this block's (place, sample) pairs, the samples fastest
-  const long long u0 = npair * blockIdx.x / gridDim.x, u1 = npair * (blockIdx.x + 1) / gridDim.x;
+  // this block's (place, sample) pairs, the samples fastest: from npair b / grid
+  // on, with npair = per_block grid + extra (32-bit divisions: 64-bit ones run on
+  // the FP64 pipe, 2 us of a small call's 20)
+  auto first = [&](unsigned b) { return (long long)per_block * b + extra * b / gridDim.x; };
+  const long long u0 = first(blockIdx.x);
+  const int npair = (int)(first(blockIdx.x + 1) - u0);
+  int t = u0 <= 0x7fffffffll ? (int)((unsigned)u0 / (unsigned)S) : (int)(u0 / S), s = (int)(u0 - (long long)t * S);
   int place = -1, ey0 = 0, rows = 0, ex = 0;
   unsigned near = 0;    // groups of four bumps within reach of the warp's 32 columns
   unsigned have = 0;    // those that gx holds
   double gx[NBX];
-  for (long long u = u0; u < u1; ++u) {
-    const int t = (int)(u / S), s = (int)(u - (long long)t * S);
+  for (int k = 0; k < npair; ++k, t += s + 1 == S ? 1 : 0, s = s + 1 == S ? 0 : s + 1) {
     __syncthreads();  // (the table; gy and U of the pair before are no longer read)
     if (t != place) {
       place = t;
@@ -293,10 +294,18 @@ static int sample_coef_impl(const stomsfem_grid* grid, const stomsfem_field* fie
     Shape h = shape(kCoefCols);
     if (nbx > 32 || h.npair <= h.blocks) h = shape(kCoefCols / 2);
     const unsigned grd = (unsigned)(h.npair < h.blocks ? h.npair : h.blocks);
+    // the largest amplitude with which far bumps are left out: what they add
+    // stays below the rounding of the exponent, or of an affine field's mean
+    // level (whose field may be sampled with the mean zero: every bump counts then)
+    const double gain_z = field->kind == STOMSFEM_FIELD_EXP_SIGMOID ? 0.25 * std::fabs(field->contrast_log * field->gain)
+                                                                    : std::fabs(field->scale);
+    const double amp = field->kind == STOMSFEM_FIELD_AFFINE ? kCoefAmp * std::fabs(field->gain) / gain_z
+                                                            : (gain_z > 1.0 ? kCoefAmp / gain_z : kCoefAmp);
 #define LAUNCH(N, C)                                                                                               \
   sample_coef_kernel<N, C><<<grd, C, h.bytes, st>>>(grid->nf, field->kind, nbx, field->nby, h.R, h.nstrip, h.kw,   \
-                                                    h.share, S, h.npair, field->width, field->scale,               \
-                                                    field->contrast_log, field->gain, xi, a)
+                                                    h.share, S, (int)(h.npair / grd), (unsigned)(h.npair % grd),   \
+                                                    field->width, amp, field->scale, field->contrast_log,          \
+                                                    field->gain, xi, a)
 #define LAUNCH2(N)                          \
   do {                                      \
     if (h.cols == kCoefCols)                \
