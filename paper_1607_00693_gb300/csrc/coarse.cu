@@ -327,8 +327,9 @@ struct BcSystems {
 
 // Merge this batch's moments into the running ones (pairwise update of
 // Chan, Golub and LeVeque): batch mean/M2 two-pass, then combine.
-// A CTA takes NODES nodes, GROUPS threads each sharing the node's samples.
-template <int NODES, int GROUPS>
+// A CTA takes NODES nodes, GROUPS threads each sharing the node's samples, each
+// thread keeping SUMS sums.
+template <int NODES, int GROUPS, int SUMS>
 __global__ void __launch_bounds__(NODES * GROUPS)
 moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double* m2, const double* count) {
   __shared__ double part[GROUPS][NODES + 1];
@@ -347,17 +348,22 @@ moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double
     __syncthreads();
     return t;
   };
-  double mb = 0.0;
-  if (q < nn)
-    for (int s = g; s < S; s += GROUPS) mb += u[(size_t)s * nn + q];
-  mb = total(mb) / S;
-  double M2b = 0.0;
-  if (q < nn)
-    for (int s = g; s < S; s += GROUPS) {
-      const double d = u[(size_t)s * nn + q] - mb;
-      M2b += d * d;
+  auto sum = [&](auto term) {  // of this thread's samples
+    double c[SUMS] = {};
+    if (q < nn) {
+      int s = g;
+      for (; s + (SUMS - 1) * GROUPS < S; s += SUMS * GROUPS)
+#pragma unroll
+        for (int j = 0; j < SUMS; ++j) c[j] += term(u[(size_t)(s + j * GROUPS) * nn + q]);
+#pragma unroll
+      for (int j = 0; j < SUMS - 1; ++j)
+        if (s + j * GROUPS < S) c[j] += term(u[(size_t)(s + j * GROUPS) * nn + q]);
     }
-  M2b = total(M2b);
+    if constexpr (SUMS == 4) return (c[0] + c[1]) + (c[2] + c[3]);
+    return c[0];
+  };
+  const double mb = total(sum([](double v) { return v; })) / S;
+  const double M2b = total(sum([&](double v) { return (v - mb) * (v - mb); }));
   if (q >= nn || g != 0) return;
   const double na = count[0], nb = (double)S, nt = na + nb;
   const double delta = mb - mean[q];
@@ -368,19 +374,25 @@ moments_kernel(int nn, int S, const double* __restrict__ u, double* mean, double
 __global__ void count_kernel(double* count, int S) { count[0] += (double)S; }
 
 // Moments of a batch merged, then the count.  One thread per node is bound by
-// its two chains of S dependent additions (about 0.14 us a sample), 32 threads
-// per node by the barriers of their sums, 12 us for a CTA of 16 nodes and more once
-// the SMs hold several: the line lies where the chains have grown past that.  One
-// thread, 32 threads, us: 1089 nodes, 1 sample 6.7, 10.8; 16 8.7, 11.6; 100 20.4,
-// 13.2; 512 74, 19; 4225 nodes, 64 samples 15.3, 16.9; 100 19.8, 17.3; 9409 nodes,
-// 100 samples 20.6, 26.0; 200 32.9, 31.3; 16641 nodes, 16 samples 9.1, 31; 100 21, 39;
-// 512 76, 76; 1025^2 nodes, 16 samples 158, 1348.
+// its S loads a pass in turn (about 0.14 us a sample), 32 threads per node by the
+// barriers of their sums, 12 us for a CTA of 16 nodes and more once the SMs hold
+// several: the line lies where the one has grown past the other.  One thread, 32
+// threads, us: 1089 nodes, 1 sample 6.7, 10.8; 16 8.7, 11.6; 100 20.4, 13.2; 512 74,
+// 19; 2401 nodes, 64 samples 16.5, 14.1; 4225 nodes, 64 samples 15.3, 16.9; 100 19.8,
+// 17.3; 9409 nodes, 100 samples 20.6, 26.0; 200 32.9, 31.3; 16641 nodes, 16 samples
+// 9.1, 31; 100 21, 39; 512 76, 76; 1025^2 nodes, 16 samples 158, 1348.
+// The thread alone keeps four sums up to kFewNodes (every coarse grid): their
+// rounding is that of the shared sums (37 samples 1.9e-16 of the mean, 2.6e-16 in one
+// sum).  A fine grid's moments are bound by the FP64 pipe, where the additions of
+// four sums cost 158 -> 188 us.
 static int merge_moments(int nn, int S, const double* u, double* mean, double* m2, double* count, cudaStream_t st) {
-  constexpr int kNodes = 16, kGroups = 32, kThreads = 128;
-  if (S > 48 + nn / 64)
-    moments_kernel<kNodes, kGroups><<<(nn + kNodes - 1) / kNodes, kNodes * kGroups, 0, st>>>(nn, S, u, mean, m2, count);
+  constexpr int kNodes = 16, kGroups = 32, kThreads = 128, kFewNodes = 10000;
+  if (S > 48 + (nn > 2400 ? (nn - 2400) / 56 : 0))
+    moments_kernel<kNodes, kGroups, 1><<<(nn + kNodes - 1) / kNodes, kNodes * kGroups, 0, st>>>(nn, S, u, mean, m2, count);
+  else if (nn <= kFewNodes)
+    moments_kernel<kThreads, 1, 4><<<(nn + kThreads - 1) / kThreads, kThreads, 0, st>>>(nn, S, u, mean, m2, count);
   else
-    moments_kernel<kThreads, 1><<<(nn + kThreads - 1) / kThreads, kThreads, 0, st>>>(nn, S, u, mean, m2, count);
+    moments_kernel<kThreads, 1, 1><<<(nn + kThreads - 1) / kThreads, kThreads, 0, st>>>(nn, S, u, mean, m2, count);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
   count_kernel<<<1, 1, 0, st>>>(count, S);
   STOMSFEM_TRY_CUDA(cudaGetLastError());
